@@ -7,6 +7,7 @@
 #include <mutex>
 #include <vector>
 
+#include <cooperative_groups.h>
 #include <cuda_runtime.h>
 
 #include "../../include/wf.h"
@@ -58,56 +59,127 @@ wf_status cuda_fail(cudaError_t e) {
 // ---------------------------------------------------------------------------------------------
 // set-up kernels
 // ---------------------------------------------------------------------------------------------
-// One block: tau = min observed Ndiag (or the caller's), max_k P_k, input checks, lambda_0, levels.
-__device__ void prep_block(const float* __restrict__ d, const float* __restrict__ Ndiag,
-                           const uint8_t* __restrict__ mask, const float* __restrict__ Pk, int H, int W,
-                           double tau_user, double eta, wf::Scalars* sc) {
-  __shared__ float s_min[32], s_max[32];
-  __shared__ int s_obs[32], s_bad[32], s_neg[32];
-  float vmin = INFINITY, vmax = 0.0f;
-  int nobs = 0, bad = 0, neg = 0;
-  const int n = H * W, nm = H * (W / 2 + 1);
-  for (int i = threadIdx.x; i < n; i += blockDim.x) {
-    if (mask[i] == 0) {
-      const float nv = Ndiag[i], dv = d[i];
-      ++nobs;
-      if (!isfinite(nv) || !isfinite(dv)) bad = 1;
-      else if (!(nv > 0.0f)) neg = 1;
-      else vmin = fminf(vmin, nv);
-    }
+// Reductions of the set-up over the inputs: min observed Ndiag, max_k P_k, observed pixels, input checks. All
+// of them are exact and independent of the order, so the split over threads changes no result.
+struct PrepSums {
+  float vmin, vmax;
+  int nobs, bad, neg;
+  __device__ void pixel(uint32_t missing, float dv, float nv) {
+    if (missing) return;
+    ++nobs;
+    if (!isfinite(nv) || !isfinite(dv)) bad = 1;
+    else if (!(nv > 0.0f)) neg = 1;
+    else vmin = fminf(vmin, nv);
   }
-  for (int i = threadIdx.x; i < nm; i += blockDim.x) {
-    const float p = Pk[i];
+  __device__ void mode(float p) {
     if (!isfinite(p)) bad = 1;
     else if (p < 0.0f) neg = 1;
     else vmax = fmaxf(vmax, p);
   }
+  __device__ void merge(const PrepSums& o) {
+    vmin = fminf(vmin, o.vmin);
+    vmax = fmaxf(vmax, o.vmax);
+    nobs += o.nobs;
+    bad |= o.bad;
+    neg |= o.neg;
+  }
+};
+
+// One thread-block cluster (kPrepCluster CTAs from 256^2 up, else one CTA): tau = min observed Ndiag (or the
+// caller's), max_k P_k, input checks, lambda_0, levels. The pass is bounded by the loads' latency and by what
+// a few SMs can read: 16-byte loads of four pixels at a time (where the pointers allow it), all issued before
+// the checks, and eight SMs for the large images. Against one CTA with scalar loads, each waiting for its
+// mask, a whole 256^2 call got 29 us shorter (3 chains x 50 sweeps: 895 -> 866 us), a 512^2 call 380 us
+// (50 chains x 16 sweeps: 2666 -> 2286 us); up to 128^2 one CTA is as fast.
+constexpr int kPrepThreads = 1024, kPrepCluster = 8;
+int prep_cluster(int H) { return H >= 256 ? kPrepCluster : 1; }
+
+__device__ void prep_cluster_block(const float* __restrict__ d, const float* __restrict__ Ndiag,
+                                   const uint8_t* __restrict__ mask, const float* __restrict__ Pk, int H, int W,
+                                   double tau_user, double eta, wf::Scalars* sc) {
+  namespace cg = cooperative_groups;
+  cg::cluster_group cl = cg::this_cluster();
+  __shared__ PrepSums part[kPrepThreads / 32];
+  __shared__ PrepSums cta;
+  PrepSums r{INFINITY, 0.0f, 0, 0, 0};
+  const int n = H * W, nm = H * (W / 2 + 1);
+  const int g = int(cl.block_rank()) * int(blockDim.x) + int(threadIdx.x), stride = int(cl.num_blocks() * blockDim.x);
+  const bool wide = ((reinterpret_cast<uintptr_t>(d) | reinterpret_cast<uintptr_t>(Ndiag) |
+                      reinterpret_cast<uintptr_t>(Pk)) & 15) == 0 && (reinterpret_cast<uintptr_t>(mask) & 3) == 0;
+  if (wide) {  // n and nm are multiples of 16
+#pragma unroll 2
+    for (int i = g; i < n / 4; i += stride) {
+      const float4 nv = __ldg(reinterpret_cast<const float4*>(Ndiag) + i);
+      const float4 dv = __ldg(reinterpret_cast<const float4*>(d) + i);
+      const uint32_t m = __ldg(reinterpret_cast<const uint32_t*>(mask) + i);
+      r.pixel(m & 0xffu, dv.x, nv.x);
+      r.pixel(m & 0xff00u, dv.y, nv.y);
+      r.pixel(m & 0xff0000u, dv.z, nv.z);
+      r.pixel(m & 0xff000000u, dv.w, nv.w);
+    }
+#pragma unroll 2
+    for (int i = g; i < nm / 4; i += stride) {
+      const float4 p = __ldg(reinterpret_cast<const float4*>(Pk) + i);
+      r.mode(p.x);
+      r.mode(p.y);
+      r.mode(p.z);
+      r.mode(p.w);
+    }
+  } else {
+#pragma unroll 4
+    for (int i = g; i < n; i += stride) r.pixel(mask[i], __ldg(d + i), __ldg(Ndiag + i));
+#pragma unroll 4
+    for (int i = g; i < nm; i += stride) r.mode(__ldg(Pk + i));
+  }
   for (int o = 16; o > 0; o >>= 1) {
-    vmin = fminf(vmin, __shfl_xor_sync(0xffffffffu, vmin, o));
-    vmax = fmaxf(vmax, __shfl_xor_sync(0xffffffffu, vmax, o));
-    nobs += __shfl_xor_sync(0xffffffffu, nobs, o);
-    bad |= __shfl_xor_sync(0xffffffffu, bad, o);
-    neg |= __shfl_xor_sync(0xffffffffu, neg, o);
+    PrepSums q;
+    q.vmin = __shfl_xor_sync(0xffffffffu, r.vmin, o);
+    q.vmax = __shfl_xor_sync(0xffffffffu, r.vmax, o);
+    q.nobs = __shfl_xor_sync(0xffffffffu, r.nobs, o);
+    q.bad = __shfl_xor_sync(0xffffffffu, r.bad, o);
+    q.neg = __shfl_xor_sync(0xffffffffu, r.neg, o);
+    r.merge(q);
   }
-  const int w = threadIdx.x >> 5, l = threadIdx.x & 31, nw = int(blockDim.x >> 5);
-  if (l == 0) { s_min[w] = vmin; s_max[w] = vmax; s_obs[w] = nobs; s_bad[w] = bad; s_neg[w] = neg; }
+  if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = r;
   __syncthreads();
-  if (threadIdx.x != 0) return;
-  int total_obs = 0;
-  for (int i = 0; i < nw; ++i) {
-    vmin = fminf(vmin, s_min[i]);
-    vmax = fmaxf(vmax, s_max[i]);
-    total_obs += s_obs[i];
-    bad |= s_bad[i];
-    neg |= s_neg[i];
+  if (threadIdx.x == 0) {
+    for (int i = 1; i < int(blockDim.x >> 5); ++i) r.merge(part[i]);
+    cta = r;
   }
-  wf::Scalars r = wf::make_scalars(vmin, total_obs, vmax, bad, neg, tau_user, eta);
-  *sc = r;
+  if (cl.num_blocks() > 1) {
+    cl.sync();
+    if (cl.block_rank() == 0 && threadIdx.x == 0)
+      for (unsigned j = 1; j < cl.num_blocks(); ++j) r.merge(*cl.map_shared_rank(&cta, j));
+    cl.sync();  // every CTA's sums stay readable until they have been read
+  }
+  if (cl.block_rank() == 0 && threadIdx.x == 0)
+    *sc = wf::make_scalars(r.vmin, r.nobs, r.vmax, r.bad, r.neg, tau_user, eta);
 }
 
-__global__ void k_prep(const float* __restrict__ d, const float* __restrict__ Ndiag, const uint8_t* __restrict__ mask,
-                       const float* __restrict__ Pk, int H, int W, double tau_user, double eta, wf::Scalars* sc) {
-  prep_block(d, Ndiag, mask, Pk, H, W, tau_user, eta, sc);
+__global__ void __launch_bounds__(kPrepThreads) k_prep(const float* __restrict__ d, const float* __restrict__ Ndiag,
+                                                       const uint8_t* __restrict__ mask, const float* __restrict__ Pk,
+                                                       int H, int W, double tau_user, double eta, wf::Scalars* sc) {
+  prep_cluster_block(d, Ndiag, mask, Pk, H, W, tau_user, eta, sc);
+}
+
+// `blocks` clusters of prep_cluster(H) CTAs of a set-up kernel
+template <class... P, class... A>
+cudaError_t launch_prep_kernel(void (*kern)(P...), int blocks, int H, cudaStream_t st, A... args) {
+  cudaLaunchAttribute attr{};
+  attr.id = cudaLaunchAttributeClusterDimension;
+  attr.val.clusterDim.x = unsigned(prep_cluster(H));
+  attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(unsigned(blocks) * unsigned(prep_cluster(H)));
+  cfg.blockDim = dim3(kPrepThreads);
+  cfg.stream = st;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kern, static_cast<P>(args)...);
+}
+cudaError_t launch_prep(const float* d, const float* Ndiag, const uint8_t* mask, const float* Pk, int H, int W,
+                        double tau_user, double eta, wf::Scalars* sc, cudaStream_t st) {
+  return launch_prep_kernel(k_prep, 1, H, st, d, Ndiag, mask, Pk, H, W, tau_user, eta, sc);
 }
 
 // Per-pixel tables ([W][H], x-major so that row threads read consecutive addresses) and the
@@ -347,8 +419,7 @@ wf_status sample_global(const float* d, const float* Ndiag, const uint8_t* mask,
   auto* sc = reinterpret_cast<wf::Scalars*>(b + o_sc);
   auto* bar = reinterpret_cast<wf::GridBar*>(b + o_bar);
   WF_CUDA(cudaMemsetAsync(bar, 0, sizeof(wf::GridBar), st));
-  k_prep<<<1, 1024, 0, st>>>(d, Ndiag, mask, Pk, H, W, o.tau, 0.5, sc);
-  WF_CUDA(cudaGetLastError());
+  WF_CUDA(launch_prep(d, Ndiag, mask, Pk, H, W, o.tau, 0.5, sc, st));
   k_tables<<<int((n + nm + 255) / 256), 256, 0, st>>>(d, Ndiag, mask, Pk, H, W, sc,
                                                        reinterpret_cast<float2*>(b + o_aq), nullptr,
                                                        reinterpret_cast<float2*>(b + o_fg));
@@ -391,42 +462,52 @@ wf_status sample_global(const float* d, const float* Ndiag, const uint8_t* mask,
   return hb.err ? wf_status(hb.err) : WF_OK;
 }
 
+// Set-up shared by the solves of one refined Wiener filter: the scalars (on the device, and on the host for
+// the large images, whose level norms are sized by the number of levels) and the pixel table [W][H] (d, 1/N_bar).
+struct SolveSetup {
+  const wf::Scalars* sc = nullptr;
+  const float2* dn = nullptr;
+  wf::Scalars host{};
+};
+
 // Wiener filter for H >= 256: level norms (fields = levels), then the cooled iteration, field in
 // global memory.
 wf_status solve_global(const float* d, const float* Ndiag, const uint8_t* mask, const float* Pk, int H, int W,
                        const wf_solve_opts& o, float* out_s, int32_t* iters_out, double* resid_out, cudaStream_t st,
-                       wf::LaunchTimer* timer, const float2* rhs_tab = nullptr, const double* rhs_norms = nullptr) {
+                       wf::LaunchTimer* timer, const float2* rhs_tab = nullptr, const double* rhs_norms = nullptr,
+                       const SolveSetup* su = nullptr) {
   const size_t n = size_t(H) * W, nz = size_t(H) * (W / 2);
   // scalars first: the number of cooling levels sizes the level-norm pass
   Scratch s1;
   s1.st = st;
-  WF_CUDA(cudaMallocAsync(&s1.base, sizeof(wf::Scalars), st));
-  auto* sc1 = static_cast<wf::Scalars*>(s1.base);
-  k_prep<<<1, 1024, 0, st>>>(d, Ndiag, mask, Pk, H, W, o.tau, o.eta, sc1);
-  WF_CUDA(cudaGetLastError());
   wf::Scalars hsc;
-  WF_CUDA(cudaMemcpyAsync(&hsc, sc1, sizeof(hsc), cudaMemcpyDeviceToHost, st));
-  WF_CUDA(cudaStreamSynchronize(st));
+  const wf::Scalars* sc = su ? su->sc : nullptr;
+  if (su) {
+    hsc = su->host;
+  } else {
+    WF_CUDA(cudaMallocAsync(&s1.base, sizeof(wf::Scalars), st));
+    auto* sc1 = static_cast<wf::Scalars*>(s1.base);
+    WF_CUDA(launch_prep(d, Ndiag, mask, Pk, H, W, o.tau, o.eta, sc1, st));
+    WF_CUDA(cudaMemcpyAsync(&hsc, sc1, sizeof(hsc), cudaMemcpyDeviceToHost, st));
+    WF_CUDA(cudaStreamSynchronize(st));
+    sc = sc1;
+  }
   if (hsc.status != WF_OK) return wf_status(hsc.status);
   const int levels = hsc.n_levels;
+  const bool own_dn = !rhs_tab && !su;
   Carve cv;
-  const size_t o_sc = cv.take<wf::Scalars>(1), o_bar = cv.take<wf::GridBar>(2), o_dn = cv.take<float2>(n),
+  const size_t o_bar = cv.take<wf::GridBar>(2), o_bn = cv.take<double>(wf::kMaxLevels), o_acc = cv.take<double>(2),
+               o_st = cv.take<wf::SolveStatus>(1), zeroed = cv.off, o_dn = cv.take<float2>(own_dn ? n : 0),
                o_tr = cv.take<float2>(W / 2), o_tc = cv.take<float2>(H), o_tw = cv.take<float2>(W / 2),
-               o_bn = cv.take<double>(wf::kMaxLevels), o_acc = cv.take<double>(2), o_st = cv.take<wf::SolveStatus>(1),
                o_prev = cv.take<float2>(nz),
                o_z = cv.take<float2>(nz * size_t(levels > 1 && !rhs_tab ? levels : 1));
   Scratch scr;
   scr.st = st;
   WF_CUDA(cudaMallocAsync(&scr.base, cv.off, st));
   char* b = static_cast<char*>(scr.base);
-  auto* sc = reinterpret_cast<wf::Scalars*>(b + o_sc);
   auto* bar = reinterpret_cast<wf::GridBar*>(b + o_bar);
-  WF_CUDA(cudaMemcpyAsync(sc, &hsc, sizeof(hsc), cudaMemcpyHostToDevice, st));
-  WF_CUDA(cudaMemsetAsync(bar, 0, 2 * sizeof(wf::GridBar), st));
-  WF_CUDA(cudaMemsetAsync(b + o_bn, 0, wf::kMaxLevels * sizeof(double), st));
-  WF_CUDA(cudaMemsetAsync(b + o_acc, 0, 2 * sizeof(double), st));
-  WF_CUDA(cudaMemsetAsync(b + o_st, 0, sizeof(wf::SolveStatus), st));
-  if (!rhs_tab) {
+  WF_CUDA(cudaMemsetAsync(b, 0, zeroed, st));  // barriers, level norms, residual sums, status
+  if (own_dn) {
     k_tables<<<int((n + 255) / 256), 256, 0, st>>>(d, Ndiag, mask, Pk, H, W, sc, nullptr,
                                                    reinterpret_cast<float2*>(b + o_dn), nullptr);
     WF_CUDA(cudaGetLastError());
@@ -439,7 +520,7 @@ wf_status solve_global(const float* d, const float* Ndiag, const uint8_t* mask, 
   a.tw_row = reinterpret_cast<float2*>(b + o_tr);
   a.tw_col = reinterpret_cast<float2*>(b + o_tc);
   a.tw_real = reinterpret_cast<float2*>(b + o_tw);
-  a.dn = rhs_tab ? rhs_tab : reinterpret_cast<float2*>(b + o_dn);
+  a.dn = rhs_tab ? rhs_tab : (su ? su->dn : reinterpret_cast<float2*>(b + o_dn));
   a.Pk = Pk;
   a.sc = sc;
   a.bar = bar;
@@ -562,8 +643,7 @@ wf_status solve_cluster(const float* d, const float* Ndiag, const uint8_t* mask,
   char* b = static_cast<char*>(scr.base);
   auto* sc = reinterpret_cast<wf::Scalars*>(b + o_sc);
   auto* res = reinterpret_cast<wf::BatchResult*>(b + o_res);
-  k_prep<<<1, 1024, 0, st>>>(d, Ndiag, mask, Pk, H, W, o.tau, o.eta, sc);
-  WF_CUDA(cudaGetLastError());
+  WF_CUDA(launch_prep(d, Ndiag, mask, Pk, H, W, o.tau, o.eta, sc, st));
   const int rows = cluster_rows_of(H, 0);
   k_tables<<<int((n + nm + 255) / 256), 256, 0, st>>>(d, Ndiag, mask, Pk, H, W, sc, nullptr,
                                                       reinterpret_cast<float2*>(b + o_dn), nullptr, H / rows, rows,
@@ -602,32 +682,33 @@ wf_status solve_cluster(const float* d, const float* Ndiag, const uint8_t* mask,
 // with the table's r and the supplied per-level norms).
 wf_status solve_pass(const float* d, const float* Ndiag, const uint8_t* mask, const float* Pk, int32_t H, int32_t W,
                      const wf_solve_opts& o, float* out_s, int32_t* iters_out, double* resid_out, cudaStream_t st,
-                     wf::LaunchTimer* timer, const float2* rhs_tab = nullptr, const double* rhs_norms = nullptr) {
+                     wf::LaunchTimer* timer, const float2* rhs_tab = nullptr, const double* rhs_norms = nullptr,
+                     const SolveSetup* su = nullptr) {
   if (!size_on_chip(H)) {
     if (o.init_s) return WF_ERR_ARG;  // the large-image solve starts from zero
     if (!rhs_tab && use_cluster(H, 1))
       return solve_cluster(d, Ndiag, mask, Pk, H, W, o, out_s, iters_out, resid_out, st, timer);
-    return solve_global(d, Ndiag, mask, Pk, H, W, o, out_s, iters_out, resid_out, st, timer, rhs_tab, rhs_norms);
+    return solve_global(d, Ndiag, mask, Pk, H, W, o, out_s, iters_out, resid_out, st, timer, rhs_tab, rhs_norms, su);
   }
   const size_t n = size_t(H) * W, nm = size_t(H) * (W / 2 + 1);
   Carve cv;
   const size_t off_sc = cv.take<wf::Scalars>(1), off_st = cv.take<wf::SolveStatus>(1),
-               off_bn = cv.take<double>(kMaxLevels), off_dn = cv.take<float2>(n),
+               off_bn = cv.take<double>(kMaxLevels), off_dn = cv.take<float2>(su ? 0 : n),
                off_prev = cv.take<float2>(size_t(H) * (W / 2));
   Scratch scr;
   scr.st = st;
   WF_CUDA(cudaMallocAsync(&scr.base, cv.off, st));
   char* b = static_cast<char*>(scr.base);
-  auto* sc = reinterpret_cast<wf::Scalars*>(b + off_sc);
+  const wf::Scalars* sc = su ? su->sc : reinterpret_cast<wf::Scalars*>(b + off_sc);
   auto* sst = reinterpret_cast<wf::SolveStatus*>(b + off_st);
   auto* bn = reinterpret_cast<double*>(b + off_bn);
-  auto* dn = reinterpret_cast<float2*>(b + off_dn);
+  const float2* dn = su ? su->dn : reinterpret_cast<float2*>(b + off_dn);
   auto* prev = reinterpret_cast<float2*>(b + off_prev);
   WF_CUDA(cudaMemsetAsync(sst, 0, sizeof(wf::SolveStatus), st));
-  k_prep<<<1, 1024, 0, st>>>(d, Ndiag, mask, Pk, H, W, o.tau, o.eta, sc);
-  WF_CUDA(cudaGetLastError());
-  if (!rhs_tab) {
-    k_tables<<<int((n + nm + 255) / 256), 256, 0, st>>>(d, Ndiag, mask, Pk, H, W, sc, nullptr, dn, nullptr);
+  if (!su) {
+    WF_CUDA(launch_prep(d, Ndiag, mask, Pk, H, W, o.tau, o.eta, reinterpret_cast<wf::Scalars*>(b + off_sc), st));
+    k_tables<<<int((n + nm + 255) / 256), 256, 0, st>>>(d, Ndiag, mask, Pk, H, W, sc, nullptr,
+                                                        reinterpret_cast<float2*>(b + off_dn), nullptr);
     WF_CUDA(cudaGetLastError());
   }
   wf::SolveArgs a{};
@@ -677,9 +758,6 @@ wf_status solve_refined(const float* d, const float* Ndiag, const uint8_t* mask,
   first.tol = o.tol > 1e-5 ? o.tol : 1e-5;  // the FP32 iteration alone stops above its floor
   int32_t it = 0, total = 0;
   double rs = 0.0;
-  wf_status r = solve_pass(d, Ndiag, mask, Pk, H, W, first, out_s, &it, &rs, st, timer);
-  total += it;
-  if (r != WF_OK && r != WF_ERR_NOT_CONVERGED) return r;
   const size_t n = size_t(H) * W, nm = size_t(H) * (W / 2 + 1);
   Carve cv;
   const size_t o_sc = cv.take<wf::Scalars>(1), o_dn = cv.take<float2>(n), o_rt = cv.take<float2>(n),
@@ -690,11 +768,21 @@ wf_status solve_refined(const float* d, const float* Ndiag, const uint8_t* mask,
   WF_CUDA(cudaMallocAsync(&scr.base, cv.off, st));
   char* b = static_cast<char*>(scr.base);
   auto* sc = reinterpret_cast<wf::Scalars*>(b + o_sc);
-  k_prep<<<1, 1024, 0, st>>>(d, Ndiag, mask, Pk, H, W, o.tau, o.eta, sc);
-  WF_CUDA(cudaGetLastError());
+  // one set-up for the first solve, the residuals and every correction solve
+  SolveSetup su;
+  su.sc = sc;
+  su.dn = reinterpret_cast<float2*>(b + o_dn);
+  WF_CUDA(launch_prep(d, Ndiag, mask, Pk, H, W, o.tau, o.eta, sc, st));
   k_tables<<<int((n + nm + 255) / 256), 256, 0, st>>>(d, Ndiag, mask, Pk, H, W, sc, nullptr,
                                                        reinterpret_cast<float2*>(b + o_dn), nullptr);
   WF_CUDA(cudaGetLastError());
+  if (!size_on_chip(H)) {
+    WF_CUDA(cudaMemcpyAsync(&su.host, sc, sizeof(su.host), cudaMemcpyDeviceToHost, st));
+    WF_CUDA(cudaStreamSynchronize(st));
+  }
+  wf_status r = solve_pass(d, Ndiag, mask, Pk, H, W, first, out_s, &it, &rs, st, timer, nullptr, nullptr, &su);
+  total += it;
+  if (r != WF_OK && r != WF_ERR_NOT_CONVERGED) return r;
   double* norms = reinterpret_cast<double*>(b + o_nr);
   wf::RefineArgs ra{};
   ra.H = H;
@@ -729,7 +817,7 @@ wf_status solve_refined(const float* d, const float* Ndiag, const uint8_t* mask,
     if (!(rho == rho)) { status = WF_ERR_NONFINITE; break; }
     if (rho < o.tol) { status = WF_OK; break; }
     if (k == o.refine) break;
-    r = solve_pass(d, Ndiag, mask, Pk, H, W, corr, ev, &it, &rs, st, nullptr, ra.rtab, ra.level_norms);
+    r = solve_pass(d, Ndiag, mask, Pk, H, W, corr, ev, &it, &rs, st, nullptr, ra.rtab, ra.level_norms, &su);
     total += it;
     if (r != WF_OK && r != WF_ERR_NOT_CONVERGED) return r;
     if ((e = wf::refine_update(int(n), out_s, ev, st)) != cudaSuccess) return cuda_fail(e);
@@ -821,8 +909,7 @@ wf_status wf_sample_ex(const float* d, const float* Ndiag, const uint8_t* mask, 
   auto* sc = reinterpret_cast<wf::Scalars*>(b + off_sc);
   auto* aq = reinterpret_cast<float2*>(b + off_aq);
   auto* fg = reinterpret_cast<float2*>(b + off_fg);
-  k_prep<<<1, 1024, 0, st>>>(d, Ndiag, mask, Pk, H, W, o.tau, 0.5, sc);
-  WF_CUDA(cudaGetLastError());
+  WF_CUDA(launch_prep(d, Ndiag, mask, Pk, H, W, o.tau, 0.5, sc, st));
   k_tables<<<int((n + nm + 255) / 256), 256, 0, st>>>(d, Ndiag, mask, Pk, H, W, sc, aq, nullptr, fg,
                                                        cluster ? H / cluster_rows_of(H, 0) : 0,
                                                        cluster ? cluster_rows_of(H, 0) : 0);
@@ -993,8 +1080,7 @@ wf_status wf_sample_band(const float* d, const float* Ndiag, const uint8_t* mask
   auto* sc = reinterpret_cast<wf::Scalars*>(b + off_sc);
   auto* aq = reinterpret_cast<float2*>(b + off_aq);
   auto* fg = reinterpret_cast<float2*>(b + off_fg);
-  k_prep<<<1, 1024, 0, st>>>(d, Ndiag, mask, Pk, H, W, o.tau, 0.5, sc);
-  WF_CUDA(cudaGetLastError());
+  WF_CUDA(launch_prep(d, Ndiag, mask, Pk, H, W, o.tau, 0.5, sc, st));
   k_check_band<<<int((nm + n_bins + 255) / 256), 256, 0, st>>>(bins, int(nm), n_bins, P0, sc);
   WF_CUDA(cudaGetLastError());
   k_tables<<<int((n + nm + 255) / 256), 256, 0, st>>>(d, Ndiag, mask, Pk, H, W, sc, aq, nullptr, fg, perm, cm);
@@ -1092,8 +1178,8 @@ wf_status wf_sample_spin2(const float* d1, const float* d2, const float* N1, con
   auto* fgB = reinterpret_cast<float2*>(b + o_fb);
   // each component's set-up checks the caller's tau against its own noise (or finds its own minimum);
   // the pair then uses the caller's tau or the smaller minimum
-  k_prep<<<1, 1024, 0, st>>>(d1, N1, mask, PE, H, W, o.tau, 0.5, sc);
-  k_prep<<<1, 1024, 0, st>>>(d2, N2, mask, PB, H, W, o.tau, 0.5, sc + 1);
+  WF_CUDA(launch_prep(d1, N1, mask, PE, H, W, o.tau, 0.5, sc, st));
+  WF_CUDA(launch_prep(d2, N2, mask, PB, H, W, o.tau, 0.5, sc + 1, st));
   k_min_tau<<<1, 32, 0, st>>>(sc, sc + 1, o.tau);
   WF_CUDA(cudaGetLastError());
   // 256 and 512: both components of a chain in one thread-block cluster of 32-row CTAs, tables in the
@@ -1203,8 +1289,8 @@ wf_status wf_solve_spin2(const float* d1, const float* d2, const float* N1, cons
   auto* fgE = reinterpret_cast<float2*>(b + o_fe);
   auto* fgB = reinterpret_cast<float2*>(b + o_fb);
   auto* rn = reinterpret_cast<double*>(b + o_r);
-  k_prep<<<1, 1024, 0, st>>>(d1, N1, mask, PE, H, W, o.tau, o.eta, sc);
-  k_prep<<<1, 1024, 0, st>>>(d2, N2, mask, PB, H, W, o.tau, o.eta, sc + 1);
+  WF_CUDA(launch_prep(d1, N1, mask, PE, H, W, o.tau, o.eta, sc, st));
+  WF_CUDA(launch_prep(d2, N2, mask, PB, H, W, o.tau, o.eta, sc + 1, st));
   k_min_tau<<<1, 32, 0, st>>>(sc, sc + 1, o.tau);
   k_s2_quiet<<<1, 32, 0, st>>>(sc, sc + 2);
   WF_CUDA(cudaGetLastError());
@@ -1498,11 +1584,12 @@ std::vector<wf::GBField> small_fields(const SmallClass& c, const std::vector<wf:
   return v;
 }
 
-// per-field set-up: one block per field (as k_prep)
-__global__ void k_prep_fields(const wf::BatchItem* __restrict__ items, const int* __restrict__ idx, int H,
+// per-field set-up: one cluster per field (as k_prep)
+__global__ void __launch_bounds__(kPrepThreads) k_prep_fields(const wf::BatchItem* __restrict__ items, const int* __restrict__ idx, int H,
                               double tau_user, double eta, wf::Scalars* sc) {
-  const wf::BatchItem it = items[idx[blockIdx.x]];
-  prep_block(it.d, it.Ndiag, it.mask, it.Pk, H, H, tau_user, eta, sc + blockIdx.x);
+  const int f = int(blockIdx.x / cooperative_groups::this_cluster().num_blocks());
+  const wf::BatchItem it = items[idx[f]];
+  prep_cluster_block(it.d, it.Ndiag, it.mask, it.Pk, H, H, tau_user, eta, sc + f);
 }
 
 // per-field tables (as k_tables), grid-stride over fields x (n + nm)
@@ -1616,8 +1703,7 @@ wf_status run_small(const SmallClass& c, const wf::BatchItem* d_items, wf::Batch
   auto* fields = reinterpret_cast<wf::GBField*>(b + c.o_fields);
   auto* idx = reinterpret_cast<int*>(b + c.o_idx);
   auto* sc = reinterpret_cast<wf::Scalars*>(b + c.o_sc);
-  k_prep_fields<<<F, 1024, 0, st>>>(d_items, idx, H, o.tau, o.eta, sc);
-  WF_CUDA(cudaGetLastError());
+  WF_CUDA(launch_prep_kernel(k_prep_fields, F, H, st, d_items, idx, H, o.tau, o.eta, sc));
   const long long tab = (long long)F * (size_t(H) * H + size_t(H) * (H / 2 + 1));
   k_tables_fields<<<int((tab + 255) / 256 < 4096 ? (tab + 255) / 256 : 4096), 256, 0, st>>>(d_items, idx, fields,
                                                                                            sc, F, H, 0);
@@ -1660,8 +1746,7 @@ wf_status run_chunk(const GBChunk& c, const wf::BatchItem* d_items, wf::BatchRes
   auto* bn = reinterpret_cast<double*>(b + c.o_bn);
   auto* active = reinterpret_cast<int*>(b + c.o_active);
   auto* bar = reinterpret_cast<wf::GridBar*>(b + c.o_bar);
-  k_prep_fields<<<F, 1024, 0, st>>>(d_items, idx, H, o.tau, o.eta, sc);
-  WF_CUDA(cudaGetLastError());
+  WF_CUDA(launch_prep_kernel(k_prep_fields, F, H, st, d_items, idx, H, o.tau, o.eta, sc));
   const long long tab = (long long)F * (size_t(H) * H + size_t(H) * (H / 2 + 1));
   k_tables_fields<<<int((tab + 255) / 256 < 4096 ? (tab + 255) / 256 : 4096), 256, 0, st>>>(
       d_items, idx, fields, sc, F, H, c.cluster ? H / c.rows : 0, c.cluster ? c.rows : 0);
@@ -2660,8 +2745,7 @@ wf_status wf_sample_noalloc(const float* d, const float* Ndiag, const uint8_t* m
   auto* aq = reinterpret_cast<float2*>(b + off_aq);
   auto* fg = reinterpret_cast<float2*>(b + off_fg);
   // k_prep rewrites every field of sc and k_tables every table entry before the sampler reads them
-  k_prep<<<1, 1024, 0, st>>>(d, Ndiag, mask, Pk, H, W, o.tau, 0.5, sc);
-  WF_CUDA(cudaGetLastError());
+  WF_CUDA(launch_prep(d, Ndiag, mask, Pk, H, W, o.tau, 0.5, sc, st));
   k_tables<<<int((n + nm + 255) / 256), 256, 0, st>>>(d, Ndiag, mask, Pk, H, W, sc, aq, nullptr, fg);
   WF_CUDA(cudaGetLastError());
   wf::SampleArgs a{};
