@@ -190,7 +190,7 @@ cudaError_t launch_prep(const float* d, const float* Ndiag, const uint8_t* mask,
 __host__ __device__ inline int table_row(int y, int H, int perm) { return perm ? (y % perm) * (H / perm) + y / perm : y; }
 
 // Position of half-spectrum entry j = ky (W/2 + 1) + kx in a mode table: natural (cm = 0), or the column slot
-// order of the cluster kernels with cm rows per CTA (kx < W/2 at ky W/2 + t, t = (kx mod cm) R + kx / cm,
+// order of the cluster kernels with cm rows per CTA, and of the on-chip kernels with cm = core_cm(H) (kx < W/2 at ky W/2 + t, t = (kx mod cm) R + kx / cm,
 // R = (W/2) / cm, the slot holding kx; kx = W/2 at H W/2 + ky), so that a column unit's threads read
 // consecutive addresses.
 __host__ __device__ inline int mode_pos(int j, int H, int W, int cm) {
@@ -280,6 +280,14 @@ bool cluster_fits(int H, int rows) {
   }
   return known[k][dev] == 1;
 }
+
+// Order of the sampler's mode table at an on-chip size (mode_pos), which selects its kernel: several threads per
+// row, except for more 64 x 64 chains than one wave of that kernel (5 CTAs on each of 152 SMs), where the
+// one-thread-per-row kernel runs with fewer instructions (us per sweep, one thread per row / several: 600 chains
+// 9.77 / 8.99, 900 chains 13.3 / 14.9, 1216 chains 17.1 / 17.6, 2048 chains 29.3 / 29.7; both kernels are then bound by
+// instruction dispatch). At 32 and 128 several threads per row are faster or equal at every count (128, 1000
+// chains: 65.4 / 60.0; 32, 4864 chains: 17.0 / 16.8).
+int sample_cm(int H, int n_chains) { return H == 64 && n_chains > 760 ? 0 : wf::core_cm(H); }
 
 // An output the kernels may store to: device or managed memory, or page-locked host memory that is
 // mapped into the device address space at the same address (cudaHostAlloc, or cudaHostRegister with
@@ -467,6 +475,7 @@ wf_status sample_global(const float* d, const float* Ndiag, const uint8_t* mask,
 struct SolveSetup {
   const wf::Scalars* sc = nullptr;
   const float2* dn = nullptr;
+  const float* Pk = nullptr;  // P in the order of the size's solve kernel
   wf::Scalars host{};
 };
 
@@ -694,6 +703,7 @@ wf_status solve_pass(const float* d, const float* Ndiag, const uint8_t* mask, co
   Carve cv;
   const size_t off_sc = cv.take<wf::Scalars>(1), off_st = cv.take<wf::SolveStatus>(1),
                off_bn = cv.take<double>(kMaxLevels), off_dn = cv.take<float2>(su ? 0 : n),
+               off_pk = cv.take<float>(su ? 0 : nm),
                off_prev = cv.take<float2>(size_t(H) * (W / 2));
   Scratch scr;
   scr.st = st;
@@ -703,17 +713,19 @@ wf_status solve_pass(const float* d, const float* Ndiag, const uint8_t* mask, co
   auto* sst = reinterpret_cast<wf::SolveStatus*>(b + off_st);
   auto* bn = reinterpret_cast<double*>(b + off_bn);
   const float2* dn = su ? su->dn : reinterpret_cast<float2*>(b + off_dn);
+  const float* pk = su ? su->Pk : reinterpret_cast<float*>(b + off_pk);
   auto* prev = reinterpret_cast<float2*>(b + off_prev);
   WF_CUDA(cudaMemsetAsync(sst, 0, sizeof(wf::SolveStatus), st));
   if (!su) {
     WF_CUDA(launch_prep(d, Ndiag, mask, Pk, H, W, o.tau, o.eta, reinterpret_cast<wf::Scalars*>(b + off_sc), st));
     k_tables<<<int((n + nm + 255) / 256), 256, 0, st>>>(d, Ndiag, mask, Pk, H, W, sc, nullptr,
-                                                        reinterpret_cast<float2*>(b + off_dn), nullptr);
+                                                        reinterpret_cast<float2*>(b + off_dn), nullptr, 0,
+                                                        wf::core_cm(H), reinterpret_cast<float*>(b + off_pk));
     WF_CUDA(cudaGetLastError());
   }
   wf::SolveArgs a{};
   a.dn = rhs_tab ? rhs_tab : dn;
-  a.Pk = Pk;
+  a.Pk = pk;
   a.sc = sc;
   a.bnorm2 = rhs_tab ? rhs_norms : bn;
   a.init_s = o.init_s;
@@ -727,7 +739,7 @@ wf_status solve_pass(const float* d, const float* Ndiag, const uint8_t* mask, co
   a.level_max = o.level_max;
   a.check = o.check;
   a.rhs_mode = rhs_tab ? 1 : 0;
-  wf::BnormArgs bb{dn, Pk, sc, bn, o.eta};
+  wf::BnormArgs bb{dn, pk, sc, bn, o.eta};
   cudaError_t e = cudaSuccess;
   switch (H) {
     case 16: e = wf::launch_solve<16>(a, bb, st, timer); break;
@@ -762,6 +774,7 @@ wf_status solve_refined(const float* d, const float* Ndiag, const uint8_t* mask,
   Carve cv;
   const size_t o_sc = cv.take<wf::Scalars>(1), o_dn = cv.take<float2>(n), o_rt = cv.take<float2>(n),
                o_e = cv.take<float>(n), o_nr = cv.take<double>(4), o_ln = cv.take<double>(kMaxLevels),
+               o_pk = cv.take<float>(size_on_chip(H) ? nm : 0),
                o_fft = cv.take<char>(wf::refine_scratch_bytes(H, W));
   Scratch scr;
   scr.st = st;
@@ -772,9 +785,11 @@ wf_status solve_refined(const float* d, const float* Ndiag, const uint8_t* mask,
   SolveSetup su;
   su.sc = sc;
   su.dn = reinterpret_cast<float2*>(b + o_dn);
+  su.Pk = size_on_chip(H) ? reinterpret_cast<float*>(b + o_pk) : Pk;
   WF_CUDA(launch_prep(d, Ndiag, mask, Pk, H, W, o.tau, o.eta, sc, st));
-  k_tables<<<int((n + nm + 255) / 256), 256, 0, st>>>(d, Ndiag, mask, Pk, H, W, sc, nullptr,
-                                                       reinterpret_cast<float2*>(b + o_dn), nullptr);
+  k_tables<<<int((n + nm + 255) / 256), 256, 0, st>>>(
+      d, Ndiag, mask, Pk, H, W, sc, nullptr, reinterpret_cast<float2*>(b + o_dn), nullptr, 0, wf::core_cm(H),
+      size_on_chip(H) ? reinterpret_cast<float*>(b + o_pk) : nullptr);
   WF_CUDA(cudaGetLastError());
   if (!size_on_chip(H)) {
     WF_CUDA(cudaMemcpyAsync(&su.host, sc, sizeof(su.host), cudaMemcpyDeviceToHost, st));
@@ -912,7 +927,7 @@ wf_status wf_sample_ex(const float* d, const float* Ndiag, const uint8_t* mask, 
   WF_CUDA(launch_prep(d, Ndiag, mask, Pk, H, W, o.tau, 0.5, sc, st));
   k_tables<<<int((n + nm + 255) / 256), 256, 0, st>>>(d, Ndiag, mask, Pk, H, W, sc, aq, nullptr, fg,
                                                        cluster ? H / cluster_rows_of(H, 0) : 0,
-                                                       cluster ? cluster_rows_of(H, 0) : 0);
+                                                       cluster ? cluster_rows_of(H, 0) : sample_cm(H, o.n_chains));
   WF_CUDA(cudaGetLastError());
   wf::SampleArgs a{};
   a.aq = aq; a.fg = fg; a.sc = sc; a.init_s = o.init_s;
@@ -921,6 +936,7 @@ wf_status wf_sample_ex(const float* d, const float* Ndiag, const uint8_t* mask, 
   a.burn_in = o.burn_in; a.thin = o.thin; a.chain0 = o.chain_offset; a.step0 = o.start_step;
   a.key0 = uint32_t(seed & 0xffffffffu); a.key1 = uint32_t(seed >> 32);
   a.out_dtype = o.out_dtype;
+  a.cm = sample_cm(H, o.n_chains);
   KernelTimer timer(st);
   cudaError_t e = cudaSuccess;
   switch (H) {
@@ -1057,7 +1073,7 @@ wf_status wf_sample_band(const float* d, const float* Ndiag, const uint8_t* mask
   // and 512: thread-block clusters, as many as can be resident, each looping over chains, with tables in
   // the cluster kernels' orders)
   const bool cluster = !size_on_chip(H);
-  const int cm = cluster ? wf::cluster_rows(H) : 0, perm = cluster ? H / cm : 1;
+  const int cm = cluster ? wf::cluster_rows(H) : wf::core_cm(H), perm = cluster ? H / cm : 1;
   long long n_buf = 0;
   int n_cl = 0;
   if (cluster) {
@@ -1066,7 +1082,7 @@ wf_status wf_sample_band(const float* d, const float* Ndiag, const uint8_t* mask
     if (n_cl > o.n_chains) n_cl = o.n_chains;
     n_buf = n_cl;
   } else {
-    const int fpc = H >= 128 ? 1 : 128 / H;  // fields per CTA of k_sample_band
+    const int fpc = wf::core_size(H) ? 1 : 128 / H;  // fields per CTA
     n_buf = (o.n_chains + fpc - 1) / fpc * (long long)fpc;
   }
   Carve cv;
@@ -1184,7 +1200,7 @@ wf_status wf_sample_spin2(const float* d1, const float* d2, const float* N1, con
   WF_CUDA(cudaGetLastError());
   // 256 and 512: both components of a chain in one thread-block cluster of 32-row CTAs, tables in the
   // cluster kernels' orders
-  const int cm = size_on_chip(H) ? 0 : 32, perm = cm ? H / cm : 0;
+  const int cm = size_on_chip(H) ? wf::core_cm(H) : 32, perm = size_on_chip(H) ? 0 : H / cm;
   k_tables<<<int((n + nm + 255) / 256), 256, 0, st>>>(d1, N1, mask, PE, H, W, sc, aq, nullptr, fgE, perm, cm);
   k_tables<<<int((n + nm + 255) / 256), 256, 0, st>>>(d2, N2, mask, PB, H, W, sc, aq + n, nullptr, fgB, perm, cm);
   WF_CUDA(cudaGetLastError());
@@ -1311,7 +1327,8 @@ wf_status wf_solve_spin2(const float* d1, const float* d2, const float* N1, cons
   wf::Spin2Args a{};
   a.aq2 = aq; a.fgE = fgE; a.fgB = fgB; a.sc = sc + 2; a.init_s = out; a.init_stride = 0;
   a.out = out; a.n_samples = 1; a.n_chains = 1; a.burn_in = 0; a.thin = 1; a.out_dtype = 0;
-  const int cm = size_on_chip(H) ? 0 : 32, perm = cm ? H / cm : 0;  // 256, 512: the cluster sampler's orders
+  // the sampler kernels' table orders
+  const int cm = size_on_chip(H) ? wf::core_cm(H) : 32, perm = size_on_chip(H) ? 0 : H / cm;
   auto run = [&](double lam, int sweeps) -> wf_status {
     k_s2_level_tables<<<int((n + nm + 255) / 256), 256, 0, st>>>(d1, N1, mask, PE, H, W, sc, lam, aq, fgE, perm, cm);
     k_s2_level_tables<<<int((n + nm + 255) / 256), 256, 0, st>>>(d2, N2, mask, PB, H, W, sc, lam, aq + n, fgB, perm,
@@ -1541,7 +1558,7 @@ struct SmallClass {
   int H = 0;
   std::vector<int> items;
   size_t o_fields = 0, o_idx = 0, o_sc = 0, o_bn = 0, o_order = 0, o_data = 0, per_field = 0;
-  size_t f_aq = 0, f_dn = 0, f_fg = 0, f_prev = 0, f_sw = 0;
+  size_t f_aq = 0, f_dn = 0, f_fg = 0, f_prev = 0, f_sw = 0, f_pk = 0;
 };
 
 void layout_small(SmallClass& c, Carve& cv) {
@@ -1558,6 +1575,7 @@ void layout_small(SmallClass& c, Carve& cv) {
   c.f_fg = f.take<float2>(nm);
   c.f_prev = f.take<float2>(nz);
   c.f_sw = f.take<float>(n);
+  c.f_pk = f.take<float>(wf::core_cm(H) ? nm : 0);  // P in the mode tables' slot order
   c.per_field = f.off;
   c.o_data = cv.take<char>(c.per_field * size_t(F));
 }
@@ -1571,7 +1589,7 @@ std::vector<wf::GBField> small_fields(const SmallClass& c, const std::vector<wf:
     g.aq = reinterpret_cast<const float2*>(base + c.f_aq);
     g.dn = reinterpret_cast<const float2*>(base + c.f_dn);
     g.fg = reinterpret_cast<const float2*>(base + c.f_fg);
-    g.Pk = it.Pk;
+    g.Pk = wf::core_cm(c.H) ? reinterpret_cast<const float*>(base + c.f_pk) : it.Pk;
     g.Z = nullptr;
     g.prev = reinterpret_cast<float2*>(base + c.f_prev);
     g.out_wf = it.out_wf ? it.out_wf : reinterpret_cast<float*>(base + c.f_sw);  // s_W always kept
@@ -1593,8 +1611,8 @@ __global__ void __launch_bounds__(kPrepThreads) k_prep_fields(const wf::BatchIte
 }
 
 // per-field tables (as k_tables), grid-stride over fields x (n + nm)
-// cm > 0 (cluster chunks, cm rows per CTA): the mode table in the clusters' slot order, and a copy of P in
-// that order at the field's Pk (chunk scratch)
+// cm > 0: the mode table in the kernels' slot order (mode_pos), and a copy of P in that order at the field's Pk
+// (scratch of the chunk or class)
 __global__ void k_tables_fields(const wf::BatchItem* __restrict__ items, const int* __restrict__ idx,
                                 const wf::GBField* __restrict__ fields, const wf::Scalars* __restrict__ sc, int F,
                                 int H, int perm, int cm = 0) {
@@ -1706,7 +1724,8 @@ wf_status run_small(const SmallClass& c, const wf::BatchItem* d_items, wf::Batch
   WF_CUDA(launch_prep_kernel(k_prep_fields, F, H, st, d_items, idx, H, o.tau, o.eta, sc));
   const long long tab = (long long)F * (size_t(H) * H + size_t(H) * (H / 2 + 1));
   k_tables_fields<<<int((tab + 255) / 256 < 4096 ? (tab + 255) / 256 : 4096), 256, 0, st>>>(d_items, idx, fields,
-                                                                                           sc, F, H, 0);
+                                                                                           sc, F, H, 0,
+                                                                                           wf::core_cm(H));
   WF_CUDA(cudaGetLastError());
   wf::BSolveArgs sa{};
   sa.fields = fields;
@@ -2746,7 +2765,8 @@ wf_status wf_sample_noalloc(const float* d, const float* Ndiag, const uint8_t* m
   auto* fg = reinterpret_cast<float2*>(b + off_fg);
   // k_prep rewrites every field of sc and k_tables every table entry before the sampler reads them
   WF_CUDA(launch_prep(d, Ndiag, mask, Pk, H, W, o.tau, 0.5, sc, st));
-  k_tables<<<int((n + nm + 255) / 256), 256, 0, st>>>(d, Ndiag, mask, Pk, H, W, sc, aq, nullptr, fg);
+  k_tables<<<int((n + nm + 255) / 256), 256, 0, st>>>(d, Ndiag, mask, Pk, H, W, sc, aq, nullptr, fg, 0,
+                                                       sample_cm(H, o.n_chains));
   WF_CUDA(cudaGetLastError());
   wf::SampleArgs a{};
   a.aq = aq; a.fg = fg; a.sc = sc; a.init_s = o.init_s;
@@ -2755,6 +2775,7 @@ wf_status wf_sample_noalloc(const float* d, const float* Ndiag, const uint8_t* m
   a.burn_in = o.burn_in; a.thin = o.thin; a.chain0 = o.chain_offset; a.step0 = o.start_step;
   a.key0 = uint32_t(seed & 0xffffffffu); a.key1 = uint32_t(seed >> 32);
   a.out_dtype = o.out_dtype;
+  a.cm = sample_cm(H, o.n_chains);
   cudaError_t e = cudaSuccess;
   switch (H) {
     case 16: e = wf::launch_sample<16>(a, st, nullptr); break;

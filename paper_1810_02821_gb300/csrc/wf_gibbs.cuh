@@ -460,6 +460,8 @@ struct SampleArgs {
   uint32_t step0;
   uint32_t key0, key1;
   int out_dtype;         // OutType of out
+  int cm;                // order of fg (mode_pos); 0 at a size of the several-threads-per-row kernels selects the
+                         // one-thread-per-row kernel
   // hierarchical samplers (k_sample_band, k_csample_band) only
   int n_bins;
   const float* P0;       // [n_bins] initial band powers

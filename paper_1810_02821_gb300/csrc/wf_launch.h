@@ -10,6 +10,7 @@
 #include "wf_cluster.cuh"
 #include "wf_cluster_ext.cuh"
 #include "wf_bphase.cuh"
+#include "wf_core.cuh"
 
 namespace wf {
 
@@ -19,7 +20,8 @@ struct LaunchTimer {
   virtual void stop() = 0;
 };
 
-// fields (chains) per CTA of the sampler: 128 threads per CTA for every size
+// fields (chains) per CTA of the one-thread-per-row kernels (16 x 16; the fused batch kernel's class count):
+// 128 threads per CTA for every size
 template <int N>
 constexpr int fields_per_cta() { return N >= 128 ? 1 : 128 / N; }
 
@@ -85,66 +87,64 @@ cudaError_t launch_csample_spin2(const Spin2Args& a, cudaStream_t st, LaunchTime
 
 // definitions, included by the per-size translation units only
 #if defined(WF_LAUNCH_DEFINE)
-template <int N>
-cudaError_t launch_sample(const SampleArgs& a, cudaStream_t st, LaunchTimer* t) {
-  constexpr int FPC = fields_per_cta<N>();
-  const int smem = FPC * Geo<N>::FIELD_BYTES;
-  auto kern = k_sample<N, FPC>;
+// one launch of a kernel with dynamic shared memory, timed when t is given
+template <class Kern, class Args>
+cudaError_t launch_smem(Kern kern, dim3 grid, int threads, int smem, const Args& a, cudaStream_t st, LaunchTimer* t) {
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (e != cudaSuccess) return e;
-  const int blocks = (a.n_chains + FPC - 1) / FPC;
   if (t) t->start();
-  kern<<<blocks, N * FPC, smem, st>>>(a);
+  kern<<<grid, threads, smem, st>>>(a);
   if (t) t->stop();
   return cudaGetLastError();
+}
+
+template <int N>
+cudaError_t launch_sample(const SampleArgs& a, cudaStream_t st, LaunchTimer* t) {
+  if constexpr (core_size(N)) {
+    if (a.cm != 0) return launch_smem(k_msample<N>, a.n_chains, KGeo<N>::T, KGeo<N>::SMEM, a, st, t);
+  }
+  if constexpr (N == 16 || N == 64) {
+    constexpr int FPC = fields_per_cta<N>();
+    return launch_smem(k_sample<N, FPC>, (a.n_chains + FPC - 1) / FPC, N * FPC, FPC * Geo<N>::FIELD_BYTES, a, st, t);
+  }
+  return cudaErrorInvalidValue;
 }
 
 template <int N>
 cudaError_t launch_sample_band(const SampleArgs& a, cudaStream_t st, LaunchTimer* t) {
-  constexpr int FPC = fields_per_cta<N>();
-  const int smem = FPC * (Geo<N>::FIELD_BYTES + band_bytes(a.n_bins));
-  auto kern = k_sample_band<N, FPC>;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-  if (e != cudaSuccess) return e;
-  const int blocks = (a.n_chains + FPC - 1) / FPC;
-  if (t) t->start();
-  kern<<<blocks, N * FPC, smem, st>>>(a);
-  if (t) t->stop();
-  return cudaGetLastError();
+  if constexpr (core_size(N)) {
+    return launch_smem(k_mband<N>, a.n_chains, KGeo<N>::T, KGeo<N>::SMEM + band_bytes(a.n_bins), a, st, t);
+  } else {
+    constexpr int FPC = fields_per_cta<N>();
+    return launch_smem(k_sample_band<N, FPC>, (a.n_chains + FPC - 1) / FPC, N * FPC,
+                       FPC * (Geo<N>::FIELD_BYTES + band_bytes(a.n_bins)), a, st, t);
+  }
 }
 
 template <int N>
 cudaError_t launch_sample_spin2(const Spin2Args& a, cudaStream_t st, LaunchTimer* t) {
-  constexpr int FPC = fields_per_cta<N>();  // images per CTA; two component fields each
-  const int smem = 2 * FPC * Geo<N>::FIELD_BYTES;
-  auto kern = k_sample_spin2<N, FPC>;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-  if (e != cudaSuccess) return e;
-  const int blocks = (a.n_chains + FPC - 1) / FPC;
-  if (t) t->start();
-  kern<<<blocks, 2 * N * FPC, smem, st>>>(a);
-  if (t) t->stop();
-  return cudaGetLastError();
+  if constexpr (core_size(N)) {
+    return launch_smem(k_mspin2<N>, a.n_chains, 2 * KGeo<N>::T, kspin2_smem<N>(), a, st, t);
+  } else {
+    constexpr int FPC = fields_per_cta<N>();  // images per CTA; two component fields each
+    return launch_smem(k_sample_spin2<N, FPC>, (a.n_chains + FPC - 1) / FPC, 2 * N * FPC,
+                       2 * FPC * Geo<N>::FIELD_BYTES, a, st, t);
+  }
 }
 
 template <int N>
 cudaError_t launch_solve(const SolveArgs& a, const BnormArgs& b, cudaStream_t st, LaunchTimer* t) {
-  const int smem = Geo<N>::FIELD_BYTES + 33 * 8;
-  cudaError_t e = cudaFuncSetAttribute(k_bnorm<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-  if (e != cudaSuccess) return e;
-  e = cudaFuncSetAttribute(k_solve<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-  if (e != cudaSuccess) return e;
-  if (!a.rhs_mode) {  // rhs mode: the level norms are supplied
-    k_bnorm<N><<<kMaxLevels, N, smem, st>>>(b);
-    e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
+  cudaError_t e = cudaSuccess;
+  if constexpr (core_size(N)) {
+    if (!a.rhs_mode)  // rhs mode: the level norms are supplied
+      e = launch_smem(k_mbnorm<N>, kMaxLevels, KGeo<N>::T, ksolve_smem<N>(), b, st, nullptr);
+    return e != cudaSuccess ? e : launch_smem(k_msolve<N>, 1, KGeo<N>::T, ksolve_smem<N>(), a, st, t);
+  } else {
+    const int smem = Geo<N>::FIELD_BYTES + 33 * 8;
+    if (!a.rhs_mode) e = launch_smem(k_bnorm<N>, kMaxLevels, N, smem, b, st, nullptr);
+    return e != cudaSuccess ? e : launch_smem(k_solve<N>, 1, N, smem, a, st, t);
   }
-  if (t) t->start();
-  k_solve<N><<<1, N, smem, st>>>(a);
-  if (t) t->stop();
-  return cudaGetLastError();
 }
-
 
 template <int N>
 cudaError_t batch_grid(int n_items, int grid_pct, int* grid_out) {
@@ -174,40 +174,41 @@ cudaError_t launch_batch(const BatchArgs& b, int* grid_out, cudaStream_t st) {
 
 template <int N>
 cudaError_t launch_bsolve(const BSolveArgs& a, cudaStream_t st) {
-  const int smem = bsolve_smem_bytes<N>();
-  cudaError_t e = cudaFuncSetAttribute(k_blevels<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-  if (e != cudaSuccess) return e;
-  e = cudaFuncSetAttribute(k_bsolve<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-  if (e != cudaSuccess) return e;
-  if (a.F > 0) {
-    k_blevels<N><<<dim3(a.F, kLevelCtas), N, smem, st>>>(a);
-    k_bsolve<N><<<a.F, N, smem, st>>>(a);
+  if (a.F < 1) return cudaSuccess;
+  if constexpr (core_size(N)) {
+    const cudaError_t e = launch_smem(k_mblevels<N>, dim3(a.F, kLevelCtas), KGeo<N>::T, ksolve_smem<N>(), a, st, nullptr);
+    return e != cudaSuccess ? e : launch_smem(k_mbsolve<N>, a.F, KGeo<N>::T, ksolve_smem<N>(), a, st, nullptr);
+  } else {
+    const int smem = bsolve_smem_bytes<N>();
+    const cudaError_t e = launch_smem(k_blevels<N>, dim3(a.F, kLevelCtas), N, smem, a, st, nullptr);
+    return e != cudaSuccess ? e : launch_smem(k_bsolve<N>, a.F, N, smem, a, st, nullptr);
   }
-  return cudaGetLastError();
 }
 
 template <int N, int FPC>
 cudaError_t launch_bsample_fpc(const BSampleArgs& a, cudaStream_t st) {
-  const int smem = FPC * Geo<N>::FIELD_BYTES;
-  auto kern = k_bsample<N, FPC>;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-  if (e != cudaSuccess) return e;
-  if (a.F > 0 && a.n_samples > 0) kern<<<(a.F + FPC - 1) / FPC, N * FPC, smem, st>>>(a);
-  return cudaGetLastError();
+  if (a.F < 1 || a.n_samples < 1) return cudaSuccess;
+  return launch_smem(k_bsample<N, FPC>, (a.F + FPC - 1) / FPC, N * FPC, FPC * Geo<N>::FIELD_BYTES, a, st, nullptr);
 }
 
-// fields (images) per CTA fpc in 1 .. 128 / N (0: fields_per_cta<N>())
+// fields (images) per CTA fpc in 1 .. 128 / N (0: fields_per_cta<N>()); the kernels with several threads per row
+// always take one image per CTA
 template <int N>
 cudaError_t launch_bsample(const BSampleArgs& a, int fpc, cudaStream_t st) {
   if (fpc == 0) fpc = fields_per_cta<N>();
   if (fpc < 1 || fpc > fields_per_cta<N>()) return cudaErrorInvalidValue;
-  switch (fpc) {
-    case 1: return launch_bsample_fpc<N, 1>(a, st);
-    case 2: if constexpr (fields_per_cta<N>() >= 2) return launch_bsample_fpc<N, 2>(a, st); break;
-    case 4: if constexpr (fields_per_cta<N>() >= 4) return launch_bsample_fpc<N, 4>(a, st); break;
-    case 8: if constexpr (fields_per_cta<N>() >= 8) return launch_bsample_fpc<N, 8>(a, st); break;
+  if constexpr (core_size(N)) {
+    if (a.F < 1 || a.n_samples < 1) return cudaSuccess;
+    return launch_smem(k_mbsample<N>, a.F, KGeo<N>::T, KGeo<N>::SMEM, a, st, nullptr);
+  } else {
+    switch (fpc) {
+      case 1: return launch_bsample_fpc<N, 1>(a, st);
+      case 2: return launch_bsample_fpc<N, 2>(a, st);
+      case 4: return launch_bsample_fpc<N, 4>(a, st);
+      case 8: return launch_bsample_fpc<N, 8>(a, st);
+    }
+    return cudaErrorInvalidValue;
   }
-  return cudaErrorInvalidValue;
 }
 
 template <int N>

@@ -1,0 +1,86 @@
+"""CPU checks of the index algebra behind the on-chip kernels with several threads per row (32^2, 64^2 and
+128^2), restated in FP64 NumPy:
+
+* a transform of length B A in two in-place passes (B-point DFTs over the A-strided subsequences n0 + A m,
+  twiddle W^(n0 q) at position A q + n0, then A-point DFTs of unit q, X[q + B j] at position A q + j), and its
+  inverse run backwards;
+* the two units of a thread, q and B - q (0 and B/2 for the first), with the first thread's swap, hold every mode
+  pair (k, -k) once, in the pair pattern (p[j], q[A-1-j]), (q[j], p[A-1-j]) with the stated frequencies;
+* the slot order of the mode tables.
+"""
+import numpy as np
+import pytest
+
+SIZES = [32, 64, 128]
+
+
+def _geo(N):
+    A = 8 if N >= 64 else 4
+    return A, (N // 2) // A, N // A   # A, row radix BR, column radix BC
+
+
+def _forward(x, A, B):
+    n, buf = x.size, np.array(x, complex)
+    for n0 in range(A):
+        c = np.fft.fft(buf[n0 + A * np.arange(B)])
+        buf[n0 + A * np.arange(B)] = c * np.exp(-2j * np.pi * n0 * np.arange(B) / n)
+    for q in range(B):
+        buf[A * q:A * q + A] = np.fft.fft(buf[A * q:A * q + A])
+    return buf
+
+
+def _inverse(buf, A, B):
+    n, x = buf.size, np.array(buf, complex)
+    for q in range(B):
+        x[A * q:A * q + A] = np.fft.ifft(x[A * q:A * q + A]) * A * np.exp(2j * np.pi * q * np.arange(A) / n)
+    for n0 in range(A):
+        x[n0 + A * np.arange(B)] = np.fft.ifft(x[n0 + A * np.arange(B)]) * B
+    return x
+
+
+def _pairs(A, B, h):
+    """Frequency pairs of the thread with units (h, hb), in the order the kernels run them."""
+    hb = B // 2 if h == 0 else B - h
+    p, q = [h + B * j for j in range(A)], [hb + B * j for j in range(A)]
+    if h == 0:   # swap of the upper halves, unit 0's rotated
+        t = p[A // 2:]
+        p = p[:A // 2] + q[A // 2:]
+        q = q[:A // 2] + t[1:] + t[:1]
+    return [(p[j], q[A - 1 - j], h + B * j) for j in range(A // 2)] + \
+           [(q[j], p[A - 1 - j], hb + B * j) for j in range(A // 2)]
+
+
+@pytest.mark.parametrize("N", SIZES)
+def test_two_pass_transform_and_inverse(N):
+    A, BR, BC = _geo(N)
+    rng = np.random.default_rng(N)
+    for n, B in ((N // 2, BR), (N, BC)):
+        x = rng.standard_normal(n) + 1j * rng.standard_normal(n)
+        buf, X = _forward(x, A, B), np.fft.fft(x)
+        k = np.array([s // A + B * (s % A) for s in range(n)])   # frequency held by position s
+        assert np.allclose(buf, X[k], atol=1e-10)
+        assert np.allclose(_inverse(buf, A, B), n * x, atol=1e-9)
+
+
+@pytest.mark.parametrize("N", SIZES)
+def test_unit_pairs_cover_every_mode_pair_once(N):
+    A, BR, BC = _geo(N)
+    for n, B in ((N // 2, BR), (N, BC)):
+        seen, leads = [], []
+        for h in range(B // 2):
+            for a, b, lead in _pairs(A, B, h):
+                assert a == lead and (b == n - a if a else b == n // 2)
+                seen += [a, b]
+                leads.append(a)
+        assert sorted(seen) == list(range(n))
+        assert sorted(leads) == sorted(min(a, (n - a) % n) if a else 0 for a in leads)  # leads below n/2
+        assert sorted(leads) == list(range(n // 2))
+
+
+@pytest.mark.parametrize("N", SIZES)
+def test_slot_order_of_the_mode_tables(N):
+    A, BR, _ = _geo(N)
+    L = N // 2
+    for kx in range(L):   # mode_pos with cm = BR
+        slot = (kx % BR) * (L // BR) + kx // BR
+        assert slot // A + BR * (slot % A) == kx
