@@ -182,12 +182,20 @@ cudaError_t launch_prep(const float* d, const float* Ndiag, const uint8_t* mask,
   return launch_prep_kernel(k_prep, 1, H, st, d, Ndiag, mask, Pk, H, W, tau_user, eta, sc);
 }
 
+bool size_on_chip(int H) { return H <= 128; }
+
 // Per-pixel tables ([W][H], x-major so that row threads read consecutive addresses) and the
 // per-mode sample table (table_pixel, table_mode: within 2 ulp of the exact coefficients).
 // Pixel tables are x-major, aq[x*H + ty] and dn[x*H + ty], with ty = y, or with perm = P > 0 (the
 // cluster kernels, CTA b holding the rows y = P a + b) ty = (y mod P) H/P + y / P, so that the rows of one
 // CTA are contiguous and its row threads read consecutive addresses.
+// With perm < 0 (the global-memory kernels) they are row-major.
 __host__ __device__ inline int table_row(int y, int H, int perm) { return perm ? (y % perm) * (H / perm) + y / perm : y; }
+__host__ __device__ inline int pixel_pos(int y, int x, int H, int W, int perm) {
+  return perm < 0 ? y * W + x : x * H + table_row(y, H, perm);
+}
+// order of the pixel tables of the solve kernels without a cluster: row-major above 128 x 128
+int solve_perm(int H) { return size_on_chip(H) ? 0 : -1; }
 
 // Position of half-spectrum entry j = ky (W/2 + 1) + kx in a mode table: natural (cm = 0), or the column slot
 // order of the cluster kernels with cm rows per CTA, and of the on-chip kernels with cm = core_cm(H) (kx < W/2 at ky W/2 + t, t = (kx mod cm) R + kx / cm,
@@ -210,11 +218,11 @@ __global__ void k_tables(const float* __restrict__ d, const float* __restrict__ 
   const double inv_n = 1.0 / double(n);
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n + nm; i += gridDim.x * blockDim.x) {
     if (i < n) {
-      const int y = i / W, x = i % W, ty = table_row(y, H, perm);
+      const int at = pixel_pos(i / W, i % W, H, W, perm);
       float2 a2, d2;
       wf::table_pixel(d[i], Ndiag[i], mask[i] == 0, tau, &a2, &d2);
-      if (aq) aq[x * H + ty] = a2;
-      if (dn) dn[x * H + ty] = d2;
+      if (aq) aq[at] = a2;
+      if (dn) dn[at] = d2;
     } else {
       const int j = i - n, q = mode_pos(j, H, W, cm);
       if (fg) fg[q] = wf::table_mode(Pk[j], tau, inv_n);
@@ -229,7 +237,6 @@ __global__ void k_tables(const float* __restrict__ d, const float* __restrict__ 
 bool size_ok(int H, int W) {
   return H == W && (H == 16 || H == 32 || H == 64 || H == 128 || H == 256 || H == 512 || H == 1024);
 }
-bool size_on_chip(int H) { return H <= 128; }
 
 bool cluster_fits(int H, int rows = 0);
 
@@ -310,27 +317,6 @@ bool out_ptr_ok(const void* p) {
     return pageable != 0;
   }
   return true;
-}
-
-// Twiddle tables of the large-image path, in FP64 then rounded once:
-// tw_row[j] = exp(-2 pi i j / (W/2)), tw_col[j] = exp(-2 pi i j / H), tw_real[k] = exp(-2 pi i k / W).
-__global__ void k_twiddles(int H, int W, float2* tw_row, float2* tw_col, float2* tw_real) {
-  const int LR = W / 2;
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < LR + H + LR; i += gridDim.x * blockDim.x) {
-    double sn, cs;
-    if (i < LR) {
-      sincospi(-2.0 * double(i) / double(LR), &sn, &cs);
-      tw_row[i] = make_float2(float(cs), float(sn));
-    } else if (i < LR + H) {
-      const int j = i - LR;
-      sincospi(-2.0 * double(j) / double(H), &sn, &cs);
-      tw_col[j] = make_float2(float(cs), float(sn));
-    } else {
-      const int k = i - LR - H;
-      sincospi(-2.0 * double(k) / double(W), &sn, &cs);
-      tw_real[k] = make_float2(float(cs), float(sn));
-    }
-  }
 }
 
 cudaError_t launch_global_any(int H, const wf::GlobalArgs& a, cudaStream_t st, wf::LaunchTimer* t) {
@@ -418,8 +404,7 @@ wf_status sample_global(const float* d, const float* Ndiag, const uint8_t* mask,
   const size_t n = size_t(H) * W, nm = size_t(H) * (W / 2 + 1), nz = size_t(H) * (W / 2);
   Carve cv;
   const size_t o_sc = cv.take<wf::Scalars>(1), o_bar = cv.take<wf::GridBar>(1), o_aq = cv.take<float2>(n),
-               o_fg = cv.take<float2>(nm), o_tr = cv.take<float2>(W / 2), o_tc = cv.take<float2>(H),
-               o_tw = cv.take<float2>(W / 2), o_z = cv.take<float2>(nz * size_t(o.n_chains));
+               o_fg = cv.take<float2>(nm), o_z = cv.take<float2>(nz * size_t(o.n_chains));
   Scratch scr;
   scr.st = st;
   WF_CUDA(cudaMallocAsync(&scr.base, cv.off, st));
@@ -430,16 +415,10 @@ wf_status sample_global(const float* d, const float* Ndiag, const uint8_t* mask,
   WF_CUDA(launch_prep(d, Ndiag, mask, Pk, H, W, o.tau, 0.5, sc, st));
   k_tables<<<int((n + nm + 255) / 256), 256, 0, st>>>(d, Ndiag, mask, Pk, H, W, sc,
                                                        reinterpret_cast<float2*>(b + o_aq), nullptr,
-                                                       reinterpret_cast<float2*>(b + o_fg));
-  WF_CUDA(cudaGetLastError());
-  k_twiddles<<<8, 256, 0, st>>>(H, W, reinterpret_cast<float2*>(b + o_tr), reinterpret_cast<float2*>(b + o_tc),
-                                reinterpret_cast<float2*>(b + o_tw));
+                                                       reinterpret_cast<float2*>(b + o_fg), -1);
   WF_CUDA(cudaGetLastError());
   wf::GlobalArgs a{};
   a.Z = reinterpret_cast<float2*>(b + o_z);
-  a.tw_row = reinterpret_cast<float2*>(b + o_tr);
-  a.tw_col = reinterpret_cast<float2*>(b + o_tc);
-  a.tw_real = reinterpret_cast<float2*>(b + o_tw);
   a.aq = reinterpret_cast<float2*>(b + o_aq);
   a.fg = reinterpret_cast<float2*>(b + o_fg);
   a.Pk = Pk;
@@ -507,7 +486,6 @@ wf_status solve_global(const float* d, const float* Ndiag, const uint8_t* mask, 
   Carve cv;
   const size_t o_bar = cv.take<wf::GridBar>(2), o_bn = cv.take<double>(wf::kMaxLevels), o_acc = cv.take<double>(2),
                o_st = cv.take<wf::SolveStatus>(1), zeroed = cv.off, o_dn = cv.take<float2>(own_dn ? n : 0),
-               o_tr = cv.take<float2>(W / 2), o_tc = cv.take<float2>(H), o_tw = cv.take<float2>(W / 2),
                o_prev = cv.take<float2>(nz),
                o_z = cv.take<float2>(nz * size_t(levels > 1 && !rhs_tab ? levels : 1));
   Scratch scr;
@@ -518,17 +496,11 @@ wf_status solve_global(const float* d, const float* Ndiag, const uint8_t* mask, 
   WF_CUDA(cudaMemsetAsync(b, 0, zeroed, st));  // barriers, level norms, residual sums, status
   if (own_dn) {
     k_tables<<<int((n + 255) / 256), 256, 0, st>>>(d, Ndiag, mask, Pk, H, W, sc, nullptr,
-                                                   reinterpret_cast<float2*>(b + o_dn), nullptr);
+                                                   reinterpret_cast<float2*>(b + o_dn), nullptr, -1);
     WF_CUDA(cudaGetLastError());
   }
-  k_twiddles<<<8, 256, 0, st>>>(H, W, reinterpret_cast<float2*>(b + o_tr), reinterpret_cast<float2*>(b + o_tc),
-                                reinterpret_cast<float2*>(b + o_tw));
-  WF_CUDA(cudaGetLastError());
   wf::GlobalArgs a{};
   a.Z = reinterpret_cast<float2*>(b + o_z);
-  a.tw_row = reinterpret_cast<float2*>(b + o_tr);
-  a.tw_col = reinterpret_cast<float2*>(b + o_tc);
-  a.tw_real = reinterpret_cast<float2*>(b + o_tw);
   a.dn = rhs_tab ? rhs_tab : (su ? su->dn : reinterpret_cast<float2*>(b + o_dn));
   a.Pk = Pk;
   a.sc = sc;
@@ -788,8 +760,8 @@ wf_status solve_refined(const float* d, const float* Ndiag, const uint8_t* mask,
   su.Pk = size_on_chip(H) ? reinterpret_cast<float*>(b + o_pk) : Pk;
   WF_CUDA(launch_prep(d, Ndiag, mask, Pk, H, W, o.tau, o.eta, sc, st));
   k_tables<<<int((n + nm + 255) / 256), 256, 0, st>>>(
-      d, Ndiag, mask, Pk, H, W, sc, nullptr, reinterpret_cast<float2*>(b + o_dn), nullptr, 0, wf::core_cm(H),
-      size_on_chip(H) ? reinterpret_cast<float*>(b + o_pk) : nullptr);
+      d, Ndiag, mask, Pk, H, W, sc, nullptr, reinterpret_cast<float2*>(b + o_dn), nullptr, solve_perm(H),
+      wf::core_cm(H), size_on_chip(H) ? reinterpret_cast<float*>(b + o_pk) : nullptr);
   WF_CUDA(cudaGetLastError());
   if (!size_on_chip(H)) {
     WF_CUDA(cudaMemcpyAsync(&su.host, sc, sizeof(su.host), cudaMemcpyDeviceToHost, st));
@@ -810,6 +782,7 @@ wf_status solve_refined(const float* d, const float* Ndiag, const uint8_t* mask,
   ra.s = out_s;
   ra.dn = reinterpret_cast<float2*>(b + o_dn);
   ra.rtab = reinterpret_cast<float2*>(b + o_rt);
+  ra.row_major = solve_perm(H) < 0;
   ra.rnorm = norms;
   ra.bnorm = norms + 1;
   ra.level_norms = reinterpret_cast<double*>(b + o_ln);
@@ -1402,7 +1375,8 @@ wf_status wf_shear_to_convergence(const float* gamma, int64_t n_fields, int32_t 
 namespace {
 // a grid barrier that expects one arrival more than the grid: every CTA's wait runs out
 __global__ void k_wait_timeout(wf::GridBar* bar) {
-  wf::grid_barrier(bar, gridDim.x + 1);
+  unsigned int target = 0;
+  wf::grid_barrier(bar, gridDim.x + 1, target);
 }
 }  // namespace
 
@@ -1498,8 +1472,7 @@ struct GBChunk {
   bool cluster = false;
   int rows = 0;  // rows per CTA of the cluster kernels
   std::vector<int> items;  // batch item indices
-  size_t o_fields = 0, o_idx = 0, o_sc = 0, o_state = 0, o_acc = 0, o_bn = 0, o_active = 0, o_bar = 0, o_tr = 0,
-         o_tc = 0, o_tw = 0, o_data = 0, per_field = 0;
+  size_t o_fields = 0, o_idx = 0, o_sc = 0, o_state = 0, o_acc = 0, o_bn = 0, o_active = 0, o_bar = 0, o_data = 0, per_field = 0;
   size_t f_aq = 0, f_dn = 0, f_fg = 0, f_z = 0, f_prev = 0, f_pk = 0;
 };
 
@@ -1514,9 +1487,6 @@ void layout_chunk(GBChunk& c, Carve& cv) {
   c.o_bn = cv.take<double>(size_t(F) * wf::kMaxLevels);
   c.o_active = cv.take<int>(1);
   c.o_bar = cv.take<wf::GridBar>(1);
-  c.o_tr = cv.take<float2>(H / 2);
-  c.o_tc = cv.take<float2>(H);
-  c.o_tw = cv.take<float2>(H / 2);
   Carve f;
   c.f_aq = f.take<float2>(n);
   c.f_dn = f.take<float2>(n);
@@ -1627,11 +1597,11 @@ __global__ void k_tables_fields(const wf::BatchItem* __restrict__ items, const i
     const wf::BatchItem it = items[idx[f]];
     const wf::GBField fd = fields[f];
     if (i < n) {
-      const int y = int(i / H), x = int(i % H), ty = table_row(y, H, perm);
+      const int at = pixel_pos(int(i / H), int(i % H), H, H, perm);
       float2 a2, d2;
       wf::table_pixel(it.d[i], it.Ndiag[i], it.mask[i] == 0, s.tau, &a2, &d2);
-      const_cast<float2*>(fd.aq)[x * H + ty] = a2;
-      const_cast<float2*>(fd.dn)[x * H + ty] = d2;
+      const_cast<float2*>(fd.aq)[at] = a2;
+      const_cast<float2*>(fd.dn)[at] = d2;
     } else {
       const int j = int(i - n), q = mode_pos(j, H, H, cm);
       const_cast<float2*>(fd.fg)[q] = wf::table_mode(it.Pk[j], s.tau, inv_n);
@@ -1653,9 +1623,7 @@ __global__ void k_gb_init(wf::GBState* state, double* acc, double* bnorm, int* a
   if (blockIdx.x == 0 && threadIdx.x == 0) {
     *active = F;
     bar->count = 0;
-    bar->gen = 0;
     bar->err = 0;
-    bar->pad = 0;
   }
 }
 
@@ -1768,7 +1736,7 @@ wf_status run_chunk(const GBChunk& c, const wf::BatchItem* d_items, wf::BatchRes
   WF_CUDA(launch_prep_kernel(k_prep_fields, F, H, st, d_items, idx, H, o.tau, o.eta, sc));
   const long long tab = (long long)F * (size_t(H) * H + size_t(H) * (H / 2 + 1));
   k_tables_fields<<<int((tab + 255) / 256 < 4096 ? (tab + 255) / 256 : 4096), 256, 0, st>>>(
-      d_items, idx, fields, sc, F, H, c.cluster ? H / c.rows : 0, c.cluster ? c.rows : 0);
+      d_items, idx, fields, sc, F, H, c.cluster ? H / c.rows : -1, c.cluster ? c.rows : 0);
   WF_CUDA(cudaGetLastError());
   if (c.cluster) {
     wf::CBArgs cb{};
@@ -1791,9 +1759,6 @@ wf_status run_chunk(const GBChunk& c, const wf::BatchItem* d_items, wf::BatchRes
   k_gb_init<<<int((init_words + 255) / 256 < 1024 ? (init_words + 255) / 256 : 1024), 256, 0, st>>>(state, acc, bn,
                                                                                                    active, bar, F);
   WF_CUDA(cudaGetLastError());
-  k_twiddles<<<8, 256, 0, st>>>(H, H, reinterpret_cast<float2*>(b + c.o_tr), reinterpret_cast<float2*>(b + c.o_tc),
-                                reinterpret_cast<float2*>(b + c.o_tw));
-  WF_CUDA(cudaGetLastError());
   wf::GBArgs a{};
   a.fields = fields;
   a.sc = sc;
@@ -1803,9 +1768,6 @@ wf_status run_chunk(const GBChunk& c, const wf::BatchItem* d_items, wf::BatchRes
   a.res = d_res;
   a.active = active;
   a.bar = bar;
-  a.tw_row = reinterpret_cast<float2*>(b + c.o_tr);
-  a.tw_col = reinterpret_cast<float2*>(b + c.o_tc);
-  a.tw_real = reinterpret_cast<float2*>(b + c.o_tw);
   a.F = F;
   a.tol = o.tol;
   a.eta = o.eta;
@@ -2331,8 +2293,8 @@ cudaError_t spectral_power_dev(const float* a, const float* b, float sgn, int n_
   // large images: mode 3 of the cooperative kernel (tables and twiddles in a scratch block)
   const size_t nz = size_t(H) * (W / 2);
   Carve cv;
-  const size_t o_sc = cv.take<wf::Scalars>(1), o_bar = cv.take<wf::GridBar>(1), o_tr = cv.take<float2>(W / 2),
-               o_tc = cv.take<float2>(H), o_tw = cv.take<float2>(W / 2), o_z = cv.take<float2>(nz * size_t(n_fields));
+  const size_t o_sc = cv.take<wf::Scalars>(1), o_bar = cv.take<wf::GridBar>(1),
+               o_z = cv.take<float2>(nz * size_t(n_fields));
   void* base = nullptr;
   cudaError_t e = cudaMallocAsync(&base, cv.off, st);
   if (e != cudaSuccess) return e;
@@ -2345,16 +2307,11 @@ cudaError_t spectral_power_dev(const float* a, const float* b, float sgn, int n_
   if (e == cudaSuccess) e = cudaMemsetAsync(bb + o_bar, 0, sizeof(wf::GridBar), st);
   if (e == cudaSuccess) e = cudaMemsetAsync(dout, 0, sizeof(double) * size_t(n_fields) * nw, st);
   if (e == cudaSuccess) {
-    k_twiddles<<<8, 256, 0, st>>>(H, W, reinterpret_cast<float2*>(bb + o_tr), reinterpret_cast<float2*>(bb + o_tc),
-                                  reinterpret_cast<float2*>(bb + o_tw));
     e = cudaGetLastError();
   }
   if (e == cudaSuccess) {
     wf::GlobalArgs g{};
     g.Z = reinterpret_cast<float2*>(bb + o_z);
-    g.tw_row = reinterpret_cast<float2*>(bb + o_tr);
-    g.tw_col = reinterpret_cast<float2*>(bb + o_tc);
-    g.tw_real = reinterpret_cast<float2*>(bb + o_tw);
     g.sc = reinterpret_cast<wf::Scalars*>(bb + o_sc);
     g.bar = reinterpret_cast<wf::GridBar*>(bb + o_bar);
     g.mode = 3;

@@ -581,7 +581,7 @@ __device__ __forceinline__ void ct_update_wf(float2* row, int y, int h, const fl
   for (int x2 = h; x2 < G::W / 2; x2 += G::R) {
     float2 v = row[cphys<N, MR>(x2)];
     const float2 c0 = ldk(dn + (2 * x2) * G::H + y, pol), c1 = ldk(dn + (2 * x2 + 1) * G::H + y, pol);
-    const float w0 = wf_rcp(fmaf(lt_, c0.y, 1.0f)), w1 = wf_rcp(fmaf(lt_, c1.y, 1.0f));
+    const float w0 = wf_weight(lt_, c0.y), w1 = wf_weight(lt_, c1.y);
     v.x = fmaf(w0, v.x - c0.x, c0.x);
     v.y = fmaf(w1, v.y - c1.x, c1.x);
     row[cphys<N, MR>(x2)] = v;

@@ -28,24 +28,9 @@
 #pragma once
 
 #include "wf_bphase.cuh"
+#include "wf_units.cuh"
 
 namespace wf {
-
-// exp(-2 pi i j / 1024), rounded once from FP64, made at compile time
-struct TwTable {
-  float2 v[1024];
-};
-constexpr TwTable make_tw_table() {
-  TwTable t{};
-  for (int j = 0; j < 1024; ++j) {
-    t.v[j].x = float(cos2pi(j, 1024));
-    t.v[j].y = float(-sin2pi(j, 1024));
-  }
-  return t;
-}
-namespace {
-__device__ const TwTable g_tw1024 = make_tw_table();
-}
 
 // sizes with these kernels, and the mode tables' slot order for them (mode_pos with cm = BR; 0: natural order)
 WF_HD constexpr bool core_size(int N) { return N == 32 || N == 64 || N == 128; }
@@ -192,57 +177,6 @@ __device__ __forceinline__ void ktw_init() {
     t[i] = g_tw1024.v[k * (1024 / N)];
   }
   __syncthreads();
-}
-
-// the first thread's units 0 and B/2 hold their pairs (j, A - j) and (j, A - 1 - j) within each unit; swapping
-// the upper halves (and rotating unit 0's) makes them pairs (p[j], q[A-1-j]), (q[j], p[A-1-j]), j < A/2, as in
-// the other threads; the pair j = 0 of p is then (X[0], X[B A/2])
-template <int A>
-__device__ __forceinline__ void unit0_swap(float2 (&p)[A], float2 (&q)[A]) {
-  float2 t[A / 2];
-#pragma unroll
-  for (int i = 0; i < A / 2; ++i) t[i] = p[A / 2 + i];
-#pragma unroll
-  for (int i = 0; i < A / 2; ++i) p[A / 2 + i] = q[A / 2 + i];
-#pragma unroll
-  for (int i = 0; i < A / 2; ++i) q[A / 2 + i] = t[(i + 1) % (A / 2)];
-}
-template <int A>
-__device__ __forceinline__ void unit0_unswap(float2 (&p)[A], float2 (&q)[A]) {
-  float2 t[A / 2];
-#pragma unroll
-  for (int i = 0; i < A / 2; ++i) t[(i + 1) % (A / 2)] = q[A / 2 + i];
-#pragma unroll
-  for (int i = 0; i < A / 2; ++i) q[A / 2 + i] = p[A / 2 + i];
-#pragma unroll
-  for (int i = 0; i < A / 2; ++i) p[A / 2 + i] = t[i];
-}
-
-// real-transform passes of the pair (K, L - K), w = exp(-2 pi i K / W): the packed-complex spectrum C to the
-// half spectrum R, and back (unnormalised inverse)
-__device__ __forceinline__ void k_post(float2& a, float2& b, float2 w) {
-  const float2 E = cscale(cadd_conj(a, b), 0.5f);
-  const float2 O = cmul_mi(cscale(csub_conj(a, b), 0.5f));
-  const float2 WO = cmul(O, w);
-  a = cadd(E, WO);
-  b = cconj(csub(E, WO));
-}
-__device__ __forceinline__ void k_pre(float2& a, float2& b, float2 w) {
-  const float2 E = cadd_conj(a, b);
-  const float2 O = cmul(csub_conj(a, b), cconj(w));
-  a = cadd(E, cmul_i(O));
-  b = cadd(cconj(E), cmul_i(cconj(O)));
-}
-
-// c[k] *= w[k] (or its conjugate), k = 1 .. B-1, from a table row of B twiddles (16-byte aligned): two per load
-template <int B, bool INV>
-__device__ __forceinline__ void ktwiddle(float2 (&c)[B], const float2* w) {
-#pragma unroll
-  for (int k = 0; k < B; k += 2) {
-    const float4 v = *reinterpret_cast<const float4*>(w + k);
-    if (k > 0) c[k] = cmul(c[k], make_float2(v.x, INV ? -v.y : v.y));
-    c[k + 1] = cmul(c[k + 1], make_float2(v.z, INV ? -v.w : v.w));
-  }
 }
 
 // B twiddles of a table row (16-byte aligned), two per load
@@ -508,7 +442,7 @@ __device__ __forceinline__ void kt_update_wf(float2 (&x)[KGeo<N>::E],
     for (int m = 0; m < G::BR; ++m) {
       const int n = i + G::A * m;
       const float2 c0 = __ldg(tab + (2 * n) * G::H), c1 = __ldg(tab + (2 * n + 1) * G::H);
-      const float w0 = wf_rcp(fmaf(lt_, c0.y, 1.0f)), w1 = wf_rcp(fmaf(lt_, c1.y, 1.0f));
+      const float w0 = wf_weight(lt_, c0.y), w1 = wf_weight(lt_, c1.y);
       float2& v = x[i * G::BR + m];
       v.x = fmaf(w0, fmaf(-g, c0.x, v.x), h * c0.x);
       v.y = fmaf(w1, fmaf(-g, c1.x, v.y), h * c1.x);
@@ -617,13 +551,13 @@ __device__ __forceinline__ void ks_draw(const KCol<N>& t, float2 (&p)[KGeo<N>::A
 // Wiener-filter s-update at level lambda with its residual bookkeeping (s_update_wf_parked): P in slot order
 // (pks), previous iterate prev[ky L + slot]; returns the thread's share of the residual sum
 template <int N>
-__device__ __forceinline__ double ks_update_wf(const KCol<N>& t, float2 (&p)[KGeo<N>::A], float2 (&q)[KGeo<N>::A],
+__device__ __forceinline__ float ks_update_wf(const KCol<N>& t, float2 (&p)[KGeo<N>::A], float2 (&q)[KGeo<N>::A],
                                                const float* __restrict__ pks, float lt_, float2* __restrict__ prev,
                                                bool cmp, bool store) {
   using G = KGeo<N>;
   constexpr int L = G::L, HL = G::H * G::L;
   constexpr float INV_N = 1.0f / float(G::H * G::W);
-  const float inv_lt = 1.0f / lt_;
+  const float inv_lt = cmp ? 1.0f / lt_ : 0.0f;
   float acc = 0.0f;
   auto wres = [&](float P, float dre, float dim) -> float {
     const float g = fmaf(P, inv_lt, 1.0f);
@@ -677,12 +611,12 @@ __device__ __forceinline__ double ks_update_wf(const KCol<N>& t, float2 (&p)[KGe
           prev[ky2 * L] = y2;
         }
       });
-  return double(acc);
+  return acc;
 }
 
 // the thread's share of sum_k P^2 |V|^2 over the full spectrum (p2_power)
 template <int N>
-__device__ __forceinline__ double ks_p2(const KCol<N>& t, float2 (&p)[KGeo<N>::A], float2 (&q)[KGeo<N>::A],
+__device__ __forceinline__ float ks_p2(const KCol<N>& t, float2 (&p)[KGeo<N>::A], float2 (&q)[KGeo<N>::A],
                                         const float* __restrict__ pks) {
   using G = KGeo<N>;
   constexpr int L = G::L, HL = G::H * G::L;
@@ -704,7 +638,7 @@ __device__ __forceinline__ double ks_p2(const KCol<N>& t, float2 (&p)[KGeo<N>::A
           acc += 2.0f * (p2(__ldg(pks + ky1 * L), Am.x, Am.y) + p2(__ldg(pks + HL + ky1), Bm.x, Bm.y));
         }
       });
-  return double(acc);
+  return acc;
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -1028,12 +962,35 @@ __global__ void __launch_bounds__(2 * KGeo<N>::T, N == 64 ? 3 : (N == 32 ? 6 : 1
 // ---------------------------------------------------------------------------------------------
 // Wiener filter
 // ---------------------------------------------------------------------------------------------
+// Sums over the CTA and schedule decisions: every thread leaves its FP32 partial sum in shared memory, one warp adds
+// them in FP64 (T/32 per lane in order, then a fixed shuffle tree) and its first lane decides. With every thread
+// running the FP64 sum, division and square root, a check kept the SM's two FP64 lanes busy for several thousand
+// cycles.
+struct KSolveState {
+  double tot;
+  float ltau;
+  int lev, k, status;
+};
 template <int N>
-constexpr int ksolve_smem() { return KGeo<N>::SMEM + 34 * 8; }
+constexpr int ksolve_smem() { return KGeo<N>::SMEM + KGeo<N>::T * 4 + int(sizeof(KSolveState)); }
 template <int N>
-__device__ __forceinline__ double* kred() { return reinterpret_cast<double*>(kfield_smem() + KGeo<N>::SMEM); }
+__device__ __forceinline__ float* kpart() { return reinterpret_cast<float*>(kfield_smem() + KGeo<N>::SMEM); }
+template <int N>
+__device__ __forceinline__ KSolveState* kstate() { return reinterpret_cast<KSolveState*>(kpart<N>() + KGeo<N>::T); }
+// sum of the partial sums by one whole warp, valid in every lane
+template <int N>
+__device__ __forceinline__ double kwarp_total() {
+  const float* part = kpart<N>();
+  const int lane = threadIdx.x % 32;
+  double s = 0.0;
+#pragma unroll
+  for (int w = 0; w < KGeo<N>::T / 32; ++w) s += double(part[32 * w + lane]);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  return s;
+}
 
-// ||S N_lambda^-1 d||^2 of one cooling level, the same in every thread (ends with a CTA barrier)
+// ||S N_lambda^-1 d||^2 of one cooling level, valid in the first warp (ends with a CTA barrier)
 template <int N>
 __device__ __forceinline__ double klevel_norm(const float2* __restrict__ dn, const float* __restrict__ pks, float ltau) {
   using G = KGeo<N>;
@@ -1041,9 +998,13 @@ __device__ __forceinline__ double klevel_norm(const float2* __restrict__ dn, con
   kt_rhs<N>(x, dn, ltau);
   krow_fwd<N>(x);
   __syncthreads();
-  double acc = 0.0;
-  kcol<N, false>([&](const KCol<N>& t, float2 (&p)[G::A], float2 (&q)[G::A]) { acc = ks_p2<N>(t, p, q, pks); });
-  return block_sum(acc, kred<N>()) / double(G::H * G::W);
+  kcol<N, false>([&](const KCol<N>& t, float2 (&p)[G::A], float2 (&q)[G::A]) {
+    kpart<N>()[threadIdx.x] = ks_p2<N>(t, p, q, pks);
+  });
+  __syncthreads();
+  const double tot = threadIdx.x < 32 ? kwarp_total<N>() * (1.0 / double(G::H * G::W)) : 0.0;
+  __syncthreads();
+  return tot;
 }
 
 // The G -> 0 iteration with lambda-cooling (solve_sweeps): x holds the starting iterate on entry and the last
@@ -1068,31 +1029,49 @@ __device__ __forceinline__ int ksolve_sweeps(float2 (&x)[KGeo<N>::E], const floa
     kt_update_wf<N>(x, dn, ltau, rhs);
     krow_fwd<N>(x);
     __syncthreads();
-    double acc = 0.0;
     kcol<N, true>([&](const KCol<N>& t, float2 (&p)[G::A], float2 (&q)[G::A]) {
-      acc = ks_update_wf<N>(t, p, q, pks, ltau, prev, cmp, store);
+      const float acc = ks_update_wf<N>(t, p, q, pks, ltau, prev, cmp, store);
+      if (cmp) kpart<N>()[threadIdx.x] = acc;
     });
     __syncthreads();
-    if (cmp) {
-      const double tot = block_sum(acc, kred<N>()) * double(G::H * G::W);
-      const double bn = bnorm2[lev];
-      const double r2 = bn > 0.0 ? tot / bn : tot;
-      rho = sqrt(r2);
-      if (!(r2 == r2) || r2 > 1e300) {
-        status = 6;  // non-finite residual
-      } else if (lev < last_level) {
-        if (rho < level_tol || k >= level_max) {
-          ++lev;
-          ltau = float(level_lambda(sc, lev, eta) * sc.tau);
-          k = 0;
+    // the last warp decides while the others start the inverse rows; the next sweep needs the decision
+    if (cmp && threadIdx.x >= G::T - 32) {
+      const double tot = kwarp_total<N>() * double(G::H * G::W);
+      if (threadIdx.x == G::T - 32) {
+        // rho = sqrt(tot / bn) against the tolerances, without the division and the root
+        const double bn = bnorm2[lev], ref = bn > 0.0 ? bn : 1.0;
+        KSolveState d{tot, ltau, lev, k, 1};
+        if (!(tot == tot) || tot > 1e300 * ref) {
+          d.status = 6;  // non-finite residual
+        } else if (lev < last_level) {
+          if (tot < level_tol * level_tol * ref || k >= level_max) {
+            ++d.lev;
+            d.ltau = float(level_lambda(sc, d.lev, eta) * sc.tau);
+            d.k = 0;
+          }
+        } else if (tot < tol * tol * ref) {
+          d.status = 0;
         }
-      } else if (rho < tol) {
-        status = 0;
+        d.tot = tot / ref;
+        *kstate<N>() = d;
       }
+      __syncwarp();
+    }
+    krow_inv<N>(x);
+    if (cmp) {
+      __syncthreads();
+      const KSolveState& d = *kstate<N>();
+      rho = d.tot;
+      lev = d.lev;
+      ltau = d.ltau;
+      k = d.k;
+      status = d.status;
     }
     if (status == 1 && it >= max_iter) status = 5;  // not converged
-    krow_inv<N>(x);
-    if (status != 1) return status;
+    if (status != 1) {
+      rho = rho >= 0.0 ? sqrt(rho) : rho;  // of the last check (-1: never measured)
+      return status;
+    }
   }
 }
 

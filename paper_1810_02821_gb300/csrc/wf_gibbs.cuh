@@ -51,6 +51,21 @@ WF_HD float wf_rcp(float x) {
   return 1.0f / x;
 #endif
 }
+// Wiener-filter pixel weight w = N_bar / (N_bar + lambda tau) = 1 / (1 + lt inb), lt = lambda tau >= 0 and
+// inb = 1/N_bar in [0, inf]: the hardware reciprocal (1 ulp) with one Newton-Raphson step, r (2 - x r), without a
+// branch. The rounded library reciprocal branches on its special cases, which serialised a thread's pixels:
+// the pixel update of a 256^2 row phase took 3950 cycles, against 1650 for the sampler's with its draws. At
+// x = inf the residual is inf * 0 and the maximum drops the NaN, leaving w = 0.
+WF_HD float wf_weight(float lt, float inb) {
+#if defined(__CUDA_ARCH__)
+  const float x = fmaf(lt, inb, 1.0f);
+  float r;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return fmaf(r, fmaxf(fmaf(-x, r, 1.0f), -1.0f), r);
+#else
+  return 1.0f / (1.0f + lt * inb);
+#endif
+}
 // a / b with the fast device division (about 2 ulp); used where a few ulp do not matter
 WF_HD float wf_fdiv(float a, float b) {
 #if defined(__CUDA_ARCH__)
@@ -536,8 +551,8 @@ WF_HD void t_update_wf_staged(float* stg, int y, const float2* __restrict__ dn, 
     float2 p0 = row[2 * q], p1 = row[2 * q + 1];
     const float2 c0 = WF_LDG(dn + (4 * q) * G::H + y), c1 = WF_LDG(dn + (4 * q + 1) * G::H + y);
     const float2 c2 = WF_LDG(dn + (4 * q + 2) * G::H + y), c3 = WF_LDG(dn + (4 * q + 3) * G::H + y);
-    const float w0 = wf_rcp(fmaf(lt_, c0.y, 1.0f)), w1 = wf_rcp(fmaf(lt_, c1.y, 1.0f));
-    const float w2 = wf_rcp(fmaf(lt_, c2.y, 1.0f)), w3 = wf_rcp(fmaf(lt_, c3.y, 1.0f));
+    const float w0 = wf_weight(lt_, c0.y), w1 = wf_weight(lt_, c1.y);
+    const float w2 = wf_weight(lt_, c2.y), w3 = wf_weight(lt_, c3.y);
     p0.x = fmaf(w0, fmaf(-g, c0.x, p0.x), h * c0.x);
     p0.y = fmaf(w1, fmaf(-g, c1.x, p0.y), h * c1.x);
     p1.x = fmaf(w2, fmaf(-g, c2.x, p1.x), h * c2.x);

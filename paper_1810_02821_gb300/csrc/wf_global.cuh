@@ -3,203 +3,290 @@
 // The packed half spectrum Z[H][W/2] of every field (kx = 0 and W/2 packed as re/im of column 0) lives in
 // global memory (L2-resident when the working set allows). One persistent cooperative kernel runs every
 // sweep as two phases separated by a bounded grid barrier:
-//   row phase    (CTA = RB rows of one field): Z rows -> C2R -> s -> [sample write] -> t-draw -> R2C -> Z
-//   column phase (CTA = CB columns of one field): Z columns -> FFT -> s-draw -> inverse FFT -> Z
-// (Alg. 1 of the paper with A = I). Each 1D transform of length L = R * S (S = 64, or 32 at 1024^2) runs
-// in shared memory as R-point register DFTs on the S strided subsequences with twiddles W_L^(q n), then
-// S-point register FFTs (decimation in frequency), with 1 float2 of padding per 64 to keep the strided accesses
-// conflict-free. Every CTA uses 128 threads and 66,560 bytes of shared memory.
+//   row phase    (CTA = 8 rows of one field): Z rows -> C2R -> s -> [sample write] -> t-draw -> R2C -> Z
+//   column phase (CTA = 4 columns of one field): Z columns -> FFT -> s-draw -> inverse FFT -> Z
+// (Alg. 1 of the paper with A = I).
+//
+// Each transform of length n (rows W/2, columns H) is held by n/E threads of E = 2A elements (E = 8 at 256 and
+// 512, 16 at 1024) and runs in three or four in-place passes, n = 8 R2 [R3] A (decimation in frequency, L1 = n/8):
+//   pass 1: 8-point DFTs over m of x[n0 + L1 m], output q1, times W_n^(n0 q1);
+//   middle: within each block of length Lb (L1 first), R-point DFTs over m of n1 + (Lb/R) m, output q2 (q3), times
+//           W_Lb^(n1 q2);
+//   last:   per unit q = q1 + 8 (q2 + R2 q3), the A-point DFT: X[q + (n/A) j].
+// A thread owns the units q and n/A - q (0 and n/2A for the first), which hold every mode pair (k, -k), so the
+// real-transform passes of a row and the s-draw of a column run on registers, and so does the t-draw between the
+// inverse and the forward row transform: Z goes straight from global memory into the first pass's registers and
+// back from the last pass's, and only the exchanges inside a transform use shared memory (blocks of L1 + 2 float2
+// and the vector strides below leave the accesses free of conflicts). A row's threads share a warp, so its
+// exchanges need no CTA barrier.
+//
+// What bounds it: one field is only N^2/16 (1024: N^2/32) threads, so a phase is the latency of an L2 round trip, two
+// transforms whose instructions issue from one or two warps a scheduler, and a grid barrier, not bandwidth.
+// Measured at one field (us per sampler sweep / Wiener sweep), against 128-thread items with 8- to 16-point register
+// sub-transforms, draws through shared memory and a barrier with a generation word: 256^2 14.7 / 17.7 -> 6.8 / 7.3,
+// 512^2 20.5 / 23.3 -> 8.8 / 9.1, 1024^2 27.8 / 33.0 -> 13.1 / 13.8; 31 fields of 256^2 42.4 -> 24.0, 4 of 1024^2
+// 88 -> 34. Of a 256^2 sweep's 14K cycles a thread spends about 2.1K in each barrier and 2.5K on loads and stores of
+// Z; with 16 elements a thread (half as many warps) the same sweep took 9.6 us.
 #pragma once
 
 #include "wf_gibbs.cuh"
+#include "wf_units.cuh"
 
 namespace wf {
 
-// Length S of the register sub-transforms. A shorter S means fewer rows and columns per CTA and more work
-// items per phase, so a single field keeps more CTAs busy: with S = 16 a 1024^2 field has 256 row and 256
-// column items per phase (64 with S = 64). Measured on GB300 (one image): 1024^2 precision solve 3.27 s
-// (S = 64) -> 2.14 s (32) -> 1.84 s (16); 256^2 solve of 184 sweeps 15.0 -> 7.2 -> 4.4 ms.
-// Row and column sub-transform lengths measured on GB300 (one image, after the split of large step-A
-// DFTs), microseconds per Wiener-filter sweep at 256^2 / 512^2 / 1024^2 (and ms for 4 chains x 50 samples
-// at 256^2 / 512^2): rows 16, columns 16: 23.0 / 25.1 / 42.6 (0.97 / 1.56); rows 16, columns 32: 27.7 /
-// 28.3 / 42.5; rows 32, columns 16: 34.1 / 48.7 / 65.3; rows 8, columns 16: 18.0 / 20.9 / 52.7 (0.80 /
-// 2.14). So rows of 8-point sub-transforms at 256^2 and 16 elsewhere, columns 16.
 template <int N_>
 struct GGeo {
   static constexpr int N = N_, H = N_, W = N_;
-  static constexpr int SR = N_ == 256 ? 8 : 16;  // sub-transform length of the row transforms
-  static constexpr int SC = 16;                  // ... and of the column transforms
-  static constexpr int LR = W / 2;          // complex length of a row transform
-  static constexpr int RR = LR / SR;        // row radix
-  static constexpr int RC = H / SC;         // column radix
-  static constexpr int RB = 128 / RR;       // rows per CTA
-  static constexpr int CB = 128 / RC;       // columns per CTA
-  // float2 stride between vectors in shared memory: each vector carries 1 float2 of padding per 64 and
-  // room for the skewed blocks between the two steps of fft_smem (R blocks of S + 1), and the stride is odd
-  // (2 x odd when only 8 vectors share a half-warp) so that a half-warp reading the same element of
-  // consecutive vectors hits distinct banks
-  static constexpr int vstride(int len, int nv, int r) {
-    const int v0 = len + len / 64, v = v0 > len + r ? v0 : len + r;
-    return nv >= 16 ? (v % 2 == 1 ? v : v + 1) : (v % 16 == 2 ? v : v + ((18 - v % 16) % 16));
-  }
-  static constexpr int VROW = vstride(LR, 128 / RR, RR);
-  static constexpr int VCOL = vstride(H, 128 / RC, RC);
-  static constexpr int SMEM = (RB * VROW > CB * VCOL ? RB * VROW : CB * VCOL) * 8;
+  static constexpr int LR = W / 2;           // complex length of a row transform
+  static constexpr int E = N_ == 1024 ? 16 : 8, A = E / 2;  // elements per thread, length of the unit transforms
+  static constexpr int TR = LR / E, TC = H / E;    // threads per row and per column
+  static constexpr int RB = 8;                     // rows per CTA
+  static constexpr int T = RB * TR;                // threads per CTA
+  static constexpr int CB = T / TC;                // columns per CTA
+  static constexpr int BR = LR / A, BC = H / A;    // frequency strides of the units
+  // float2 strides of a row's and a column's vector: 8 blocks of L1 + 2; columns 4 modulo 16 apart (a half-warp
+  // holds four columns)
+  static constexpr int VROW = LR + 16 + 8, VCOL = H + 16 + 4;
+  static constexpr int VEC = RB * VROW > CB * VCOL ? RB * VROW : CB * VCOL;
+  // twiddle tables: T1 [q1][n0] (rows of n/8 + 2), T2 and T3 [q][n1] of the rows and columns, W_W^K (K < LR/2)
+  static constexpr int O_T1R = VEC, O_T2R = O_T1R + 8 * (LR / 8 + 2), O_T3R = O_T2R + LR / 8, O_T1C = O_T3R + 16,
+                       O_T2C = O_T1C + 8 * (H / 8 + 2), O_T3C = O_T2C + H / 8, O_W = O_T3C + 16, O_EDGE = O_W + LR / 2,
+                       SMEM_F2 = O_EDGE + H;
+  static constexpr int SMEM = SMEM_F2 * 8;
   static constexpr int ROW_ITEMS = H / RB;  // row-phase work items per field
   static constexpr int COL_ITEMS = LR / CB; // column-phase work items per field
   static constexpr int WH = W / 2 + 1;
+  // CTAs per SM the kernels are compiled for: up to 128 registers a thread with 16 elements, 80 with 8
+  static constexpr int MIN_CTAS = (E == 16 ? 512 : 768) / T;
+  static_assert(CB == 4 && TR <= 32 && VCOL % 16 == 4, "geometry");
 };
 
-WF_HD int padi(int i) { return i + (i >> 6); }
+// middle radices of a transform of length n
+template <int n, int E>
+struct GRad {
+  static constexpr int M = n / (4 * E);
+  static constexpr int R2 = M <= E ? M : 4, R3 = M / R2;
+  static constexpr int L1 = n / 8, S = L1 + 2, STEP2 = L1 / R2, STEP3 = STEP2 / R3;
+  static_assert(R2 * R3 == M && STEP3 == E / 2 && (R3 == 1 || STEP2 == 16), "passes");
+};
 
-// Forward DFT of length L = R*S of the padded vectors v_j = buf + j*V (j < NV), natural order in and out.
-// tw[j] = exp(-2 pi i j / L). INV: inverse via conjugation on the way in and out. 128 threads = NV * R.
-//   step A: for each n < S, the R-point DFT A[q] = sum_m x[n + S m] w_R^(q m), twiddled by W_L^(q n),
-//           stored at n + S q (block q);
-//   step C: for each q < R, the S-point FFT of block q; output k goes to q + R k (decimation in
-//           frequency: X[q + R k] = sum_n W_L^(q n) w_S^(n k) A_n[q]).
-// When NV * S < 128 (one or two warps would carry step A alone) the R-point DFTs are themselves split,
-// R = R1 R2 with m = m2 + R2 m1 and q = q1 + R1 q2:
-//   A1: for each (n, m2), B[q1] = sum_m1 x[n + S (m2 + R2 m1)] w_R1^(q1 m1), twiddled by w_R^(m2 q1),
-//       stored back at n + S (m2 + R2 q1);
-//   A2: for each (n, q1), A[q1 + R1 q2] = sum_m2 B'[m2][q1] w_R2^(q2 m2), twiddled by W_L^(q n) and
-//       stored in block q,
-// so every pass has NV S R2 or NV S R1 small DFTs spread over all 128 threads, consecutive threads on
-// consecutive n (contiguous addresses). A2 holds its inputs in registers across a CTA barrier anyway, so
-// it writes the blocks skewed by one float2 each (block q at q (S + 1), not padded): the threads of a warp,
-// each reading its own block in step C, then hit distinct banks.
-template <int R>
-__host__ __device__ constexpr int fft_smem_r1() { return R > 16 ? 8 : R; }
+__device__ __forceinline__ float2* gsmem() {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  return reinterpret_cast<float2*>(smem_raw);
+}
 
-template <int R, int NV, int V, bool INV, int S = 64>
-__device__ __forceinline__ void fft_smem(float2* buf, const float2* __restrict__ tw) {
-  static_assert(NV * R == 128, "one sub-transform per thread in step C");
-  constexpr int L = R * S;
-  constexpr bool SPLIT = !(NV * S >= 128 || R <= 16);
-  static_assert(!SPLIT || R * (S + 1) <= V, "room for the skewed blocks");
-  const int tid = threadIdx.x;
-  if constexpr (!SPLIT) {
-    // step A: R-point DFT across the S strided subsequences, twiddled by W_L^(q n), in place
-    for (int task = tid; task < NV * S; task += 128) {
-      const int j = task / S, n = task % S;
-      float2* v = buf + j * V;
-      float2 a[R];
-#pragma unroll
-      for (int m = 0; m < R; ++m) {
-        a[m] = v[padi(n + S * m)];
-        if (INV) a[m].y = -a[m].y;
-      }
-      fft<R, false>(a);
-#pragma unroll
-      for (int q = 0; q < R; ++q) v[padi(n + S * q)] = q == 0 ? a[0] : cmul(a[q], __ldg(tw + q * n));
-    }
-  } else {
-    constexpr int R1 = fft_smem_r1<R>(), R2 = R / R1;
-    static_assert(R1 * R2 == R && (NV * S * R2) % 128 == 0 && (NV * S * R1) % 128 == 0, "split step A");
-    // A1: R1-point DFTs over m1, twiddle w_R^(m2 q1) = W_L^((L/R) m2 q1), in place
-    for (int task = tid; task < NV * S * R2; task += 128) {
-      const int n = task % S, m2 = (task / S) % R2, j = task / (S * R2);
-      float2* v = buf + j * V;
-      float2 a[R1];
-#pragma unroll
-      for (int m1 = 0; m1 < R1; ++m1) {
-        a[m1] = v[padi(n + S * (m2 + R2 * m1))];
-        if (INV) a[m1].y = -a[m1].y;
-      }
-      fft<R1, false>(a);
-#pragma unroll
-      for (int q1 = 0; q1 < R1; ++q1)
-        v[padi(n + S * (m2 + R2 * q1))] = q1 == 0 ? a[0] : cmul(a[q1], __ldg(tw + (L / R) * m2 * q1));
-    }
-    __syncthreads();
-    // A2: R2-point DFTs over m2, twiddle W_L^(q n), q = q1 + R1 q2, to block q
-    constexpr int T2 = NV * S * R1 / 128;  // tasks per thread
-    float2 b[T2][R2];
-#pragma unroll
-    for (int t = 0; t < T2; ++t) {
-      const int task = tid + 128 * t;
-      const int n = task % S, q1 = (task / S) % R1, j = task / (S * R1);
-      const float2* v = buf + j * V;
-#pragma unroll
-      for (int m2 = 0; m2 < R2; ++m2) b[t][m2] = v[padi(n + S * (m2 + R2 * q1))];
-      fft<R2, false>(b[t]);
-    }
-    __syncthreads();
-#pragma unroll
-    for (int t = 0; t < T2; ++t) {
-      const int task = tid + 128 * t;
-      const int n = task % S, q1 = (task / S) % R1, j = task / (S * R1);
-      float2* v = buf + j * V;
-#pragma unroll
-      for (int q2 = 0; q2 < R2; ++q2) {
-        const int q = q1 + R1 * q2;
-        v[q * (S + 1) + n] = q == 0 ? b[t][q2] : cmul(b[t][q2], __ldg(tw + q * n));
-      }
-    }
+// the twiddle tables, by all threads (ends with a CTA barrier)
+template <int N>
+__device__ __forceinline__ void gtab_init() {
+  using G = GGeo<N>;
+  float2* s = gsmem();
+  auto w = [](int j) { return g_tw1024.v[(j * (1024 / N)) & 1023]; };  // exp(-2 pi i j / N)
+  for (int i = threadIdx.x; i < 8 * (G::LR / 8); i += G::T) {
+    const int q = i / (G::LR / 8), n0 = i % (G::LR / 8);
+    s[G::O_T1R + q * (G::LR / 8 + 2) + n0] = w(2 * n0 * q);
   }
-  __syncthreads();
-  // step C: S-point FFT of each twiddled subsequence q (block q); output k goes to position q + R k
-  // (consecutive threads take consecutive vectors)
-  const int j = tid % NV, q = tid / NV;
-  float2* v = buf + j * V;
-  float2 u[S];
-#pragma unroll
-  for (int n = 0; n < S; ++n) u[n] = SPLIT ? v[q * (S + 1) + n] : v[padi(S * q + n)];
-  __syncthreads();
-  fft<S, false>(u);
-#pragma unroll
-  for (int k = 0; k < S; ++k) {
-    float2 o = u[k];
-    if (INV) o.y = -o.y;
-    v[padi(q + R * k)] = o;
+  for (int i = threadIdx.x; i < 8 * (G::H / 8); i += G::T) {
+    const int q = i / (G::H / 8), n0 = i % (G::H / 8);
+    s[G::O_T1C + q * (G::H / 8 + 2) + n0] = w(n0 * q);
   }
+  constexpr int SR = GRad<G::LR, G::E>::STEP2, SC = GRad<G::H, G::E>::STEP2;
+  for (int i = threadIdx.x; i < G::LR / 8; i += G::T) s[G::O_T2R + i] = w(16 * (i / SR) * (i % SR));
+  for (int i = threadIdx.x; i < G::H / 8; i += G::T) s[G::O_T2C + i] = w(8 * (i / SC) * (i % SC));
+  for (int i = threadIdx.x; i < 16; i += G::T)  // blocks of length 16
+    s[G::O_T3R + i] = s[G::O_T3C + i] = w(N / 16 * (i / 4) * (i % 4));
+  for (int i = threadIdx.x; i < G::LR / 2; i += G::T) s[G::O_W + i] = w(i);
   __syncthreads();
 }
 
-// Bounded grid barrier for a cooperative launch: arrive on count, the last arrival bumps gen.
-// Gives up after 2^22 polls (a few seconds) and raises WF_ERR_TIMEOUT in *err; callers then leave.
+// twiddle tables of the row (ROW) or column transforms
+struct GTab {
+  const float2 *t1, *t2, *t3;
+};
+template <int N, bool ROW>
+__device__ __forceinline__ GTab gtab() {
+  using G = GGeo<N>;
+  const float2* s = gsmem();
+  return ROW ? GTab{s + G::O_T1R, s + G::O_T2R, s + G::O_T3R} : GTab{s + G::O_T1C, s + G::O_T2C, s + G::O_T3C};
+}
+
+// position of unit q's first value in a vector of length n, and the unit's twiddles W_Lb^(n1 q2 or q3)
+template <int n, int E>
+__device__ __forceinline__ int gunit(int q) {
+  using R = GRad<n, E>;
+  const int r = q / 8;
+  return (q % 8) * R::S + (R::R3 == 1 ? (E / 2) * r : R::STEP2 * (r % R::R2) + (E / 2) * (r / R::R2));
+}
+template <int n, int E>
+__device__ __forceinline__ const float2* gunit_tw(int q, const GTab& t) {
+  using R = GRad<n, E>;
+  return R::R3 == 1 ? t.t2 + (E / 2) * (q / 8) : t.t3 + (E / 2) * (q / 8 / R::R2);
+}
+
+// pass 1: x[i 8 + m] = element n0 + L1 m, n0 = (E/8) h + i
+template <int n, int E>
+__device__ __forceinline__ void gfwd1(float2* v, int h, const float2 (&x)[E], const GTab& t) {
+  constexpr int S = GRad<n, E>::S, NC = E / 8;
+  float2 a[NC][8];
+#pragma unroll
+  for (int i = 0; i < NC; ++i) {
+#pragma unroll
+    for (int m = 0; m < 8; ++m) a[i][m] = x[8 * i + m];
+    fft<8, false>(a[i]);
+  }
+#pragma unroll
+  for (int q = 0; q < 8; ++q) {
+    if constexpr (NC == 2) {
+      if (q > 0) {
+        const float4 w = *reinterpret_cast<const float4*>(t.t1 + q * S + 2 * h);
+        a[0][q] = cmul(a[0][q], make_float2(w.x, w.y));
+        a[1][q] = cmul(a[1][q], make_float2(w.z, w.w));
+      }
+      *reinterpret_cast<float4*>(v + q * S + 2 * h) = make_float4(a[0][q].x, a[0][q].y, a[1][q].x, a[1][q].y);
+    } else {
+      v[q * S + h] = q == 0 ? a[0][0] : cmul(a[0][q], t.t1[q * S + h]);
+    }
+  }
+}
+template <int n, int E>
+__device__ __forceinline__ void ginv1(const float2* v, int h, float2 (&x)[E]) {
+  constexpr int S = GRad<n, E>::S, NC = E / 8;
+  float2 a[NC][8];
+#pragma unroll
+  for (int q = 0; q < 8; ++q) {
+    if constexpr (NC == 2) {
+      const float4 w = *reinterpret_cast<const float4*>(v + q * S + 2 * h);
+      a[0][q] = make_float2(w.x, w.y);
+      a[1][q] = make_float2(w.z, w.w);
+    } else {
+      a[0][q] = v[q * S + h];
+    }
+  }
+#pragma unroll
+  for (int i = 0; i < NC; ++i) {
+    fft<8, true>(a[i]);
+#pragma unroll
+    for (int m = 0; m < 8; ++m) x[8 * i + m] = a[i][m];
+  }
+}
+// the middle passes (INV: backwards); a butterfly's index puts 8 blocks q1 and two offsets n1 in each half-warp
+template <int n, int E, bool INV, class Sync>
+__device__ __forceinline__ void gmid(float2* v, int h, const GTab& t, Sync&& sync) {
+  using R = GRad<n, E>;
+  auto pass2 = [&] {
+    constexpr int STEP = R::STEP2;
+#pragma unroll
+    for (int i = 0; i < E / R::R2; ++i) {
+      const int idx = h + (n / E) * i, n1 = (idx & 1) + 2 * (idx >> 4), q1 = (idx >> 1) & 7;
+      float2* u = v + q1 * R::S + n1;
+      float2 c[R::R2];
+#pragma unroll
+      for (int m = 0; m < R::R2; ++m) c[m] = u[STEP * m];
+      fft<R::R2, INV>(c);
+#pragma unroll
+      for (int m = 0; m < R::R2; ++m) {
+        if (!INV) u[STEP * m] = m == 0 ? c[0] : cmul(c[m], t.t2[STEP * m + n1]);
+        else u[STEP * m] = cmul(c[m], cconj(t.t1[q1 * R::S + n1 + STEP * m]));
+      }
+    }
+  };
+  auto pass3 = [&] {
+    if constexpr (R::R3 > 1) {
+      constexpr int STEP = R::STEP3;
+#pragma unroll
+      for (int i = 0; i < E / R::R3; ++i) {
+        const int idx = h + (n / E) * i, r = idx >> 4, q1 = (idx >> 1) & 7;
+        const int n1 = (idx & 1) + 2 * (r % (STEP / 2)), q2 = r / (STEP / 2);
+        float2* u = v + q1 * R::S + q2 * R::STEP2 + n1;
+        float2 c[R::R3];
+#pragma unroll
+        for (int m = 0; m < R::R3; ++m) c[m] = u[STEP * m];
+        fft<R::R3, INV>(c);
+#pragma unroll
+        for (int m = 0; m < R::R3; ++m) {
+          if (!INV) u[STEP * m] = m == 0 ? c[0] : cmul(c[m], t.t3[STEP * m + n1]);
+          else u[STEP * m] = cmul(c[m], cconj(t.t2[q2 * R::STEP2 + n1 + STEP * m]));
+        }
+      }
+    }
+  };
+  if constexpr (R::R3 == 1) {
+    pass2();
+  } else if constexpr (INV) {
+    pass3();
+    sync();
+    pass2();
+  } else {
+    pass2();
+    sync();
+    pass3();
+  }
+}
+// last pass: unit q's spectrum X[q + (n/A) j] into p[j]
+template <int n, int E>
+__device__ __forceinline__ void gfwd_unit(const float2* v, int q, float2 (&p)[E / 2]) {
+  const float2* u = v + gunit<n, E>(q);
+#pragma unroll
+  for (int j = 0; j < E / 2; j += 2) {
+    const float4 w = *reinterpret_cast<const float4*>(u + j);
+    p[j] = make_float2(w.x, w.y);
+    p[j + 1] = make_float2(w.z, w.w);
+  }
+  fft<E / 2, false>(p);
+}
+template <int n, int E>
+__device__ __forceinline__ void ginv_unit(float2* v, int q, float2 (&p)[E / 2], const GTab& t) {
+  fft<E / 2, true>(p);
+  ktwiddle<E / 2, true>(p, gunit_tw<n, E>(q, t));
+  float2* u = v + gunit<n, E>(q);
+#pragma unroll
+  for (int j = 0; j < E / 2; j += 2)
+    *reinterpret_cast<float4*>(u + j) = make_float4(p[j].x, p[j].y, p[j + 1].x, p[j + 1].y);
+}
+
+// Bounded grid barrier for a cooperative launch: every CTA adds one arrival to a running count (a release, so that
+// it follows the CTA's stores) and polls with acquire loads until the count reaches its own target, nblocks
+// further on at each barrier (target: the caller's, zero at the start of the launch; the comparison is by
+// difference, so the count may wrap). The arrival returns nothing, so its way to L2 and the first poll's overlap;
+// an atomic that waits for its old value and a generation word cost two more round trips. Gives up after 2^22 polls
+// (a few seconds) and raises WF_ERR_TIMEOUT in *err; callers then leave.
 struct GridBar {
   unsigned int count;
-  unsigned int gen;
+  unsigned int pad0;
   int err;
   int pad;
 };
 
-__device__ __forceinline__ bool grid_barrier(GridBar* gb, unsigned int nblocks) {
+// opened(): run by thread 0 once the barrier has opened, before the CTA goes on
+template <class F>
+__device__ __forceinline__ bool grid_barrier(GridBar* gb, unsigned int nblocks, unsigned int& target, F&& opened) {
   __syncthreads();
   __shared__ int s_ok;
+  target += nblocks;
   if (threadIdx.x == 0) {
-    __threadfence();
-    const unsigned int g = atomicAdd(&gb->gen, 0u);
-    if (atomicAdd(&gb->count, 1u) == nblocks - 1) {
-      atomicExch(&gb->count, 0u);
-      __threadfence();
-      atomicAdd(&gb->gen, 1u);
-      s_ok = 1;
-    } else {
-      int ok = 0;
-      for (long it = 0; it < (1L << 22); ++it) {
-        if (*reinterpret_cast<volatile unsigned int*>(&gb->gen) != g) { ok = 1; break; }
-        if (*reinterpret_cast<volatile int*>(&gb->err) != 0) break;
-        __nanosleep(64);
-      }
-      if (!ok) atomicExch(&gb->err, 7);  // WF_ERR_TIMEOUT
-      s_ok = ok;
+    asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(&gb->count), "r"(1u) : "memory");
+    int ok = 0;
+    for (long it = 0; !ok && it < (1L << 22); ++it) {
+      unsigned int c;
+      asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(c) : "l"(&gb->count) : "memory");
+      ok = int(c - target) >= 0;
+      if (!ok && (it & 255) == 255 && *reinterpret_cast<volatile int*>(&gb->err) != 0) break;
     }
-    __threadfence();
+    if (ok) opened();
+    else atomicExch(&gb->err, 7);  // WF_ERR_TIMEOUT
+    s_ok = ok;
   }
   __syncthreads();
   return s_ok != 0;
 }
+__device__ __forceinline__ bool grid_barrier(GridBar* gb, unsigned int nblocks, unsigned int& target) {
+  return grid_barrier(gb, nblocks, target, [] {});
+}
 
 struct GlobalArgs {
   float2* Z;               // [n_fields][H][W/2] packed half spectra (state)
-  const float2* tw_row;    // exp(-2 pi i j / (W/2)), j < W/2
-  const float2* tw_col;    // exp(-2 pi i j / H), j < H
-  const float2* tw_real;   // exp(-2 pi i k / W), k < W/2
-  const float2* aq;        // sampler pixel table [W][H] (a, q)
+  const float2* aq;        // sampler pixel table [H][W] (a, q)
   const float2* fg;        // sampler mode table [H][W/2+1]
-  const float2* dn;        // Wiener-filter pixel table [W][H] (d, 1/N_bar)
+  const float2* dn;        // Wiener-filter pixel table [H][W] (d, 1/N_bar)
   const float* Pk;         // [H][W/2+1]
   const Scalars* sc;
   GridBar* bar;
@@ -236,404 +323,548 @@ struct GlobalArgs {
   int out_dtype;           // mode 0: OutType of the samples
 };
 
-// R2C post-processing / C2R pre-processing of one padded row vector (pairs k <-> LR - k), all threads of
-// the CTA over all rows in it. Same arithmetic as r2c_post_pair / c2r_pre_pair with run-time twiddles.
-template <int N, bool POST>
-__device__ __forceinline__ void real_pass(float2* buf, int nrows, const float2* __restrict__ tw_real) {
+// ---------------------------------------------------------------------------------------------
+// row phase: thread tid of a row item holds row tid / TR, unit pair (h, hb), h = tid % TR
+// ---------------------------------------------------------------------------------------------
+// row y of Z (natural order) -> x (x[8 i + m] = pixel pair (E/8) h + i + (LR/8) m), unnormalised inverse transform
+template <int N>
+__device__ __forceinline__ void grow_inv(const float2* Zrow, float2 (&x)[GGeo<N>::E]) {
   using G = GGeo<N>;
-  constexpr int L = G::LR;
-  for (int task = threadIdx.x; task < nrows * (L / 2 + 1); task += 128) {
-    const int j = task / (L / 2 + 1), k = task % (L / 2 + 1);
-    float2* v = buf + j * G::VROW;
-    if (k == 0) {
-      const float2 c0 = v[0];
-      v[0] = make_float2(c0.x + c0.y, c0.x - c0.y);
-    } else if (2 * k == L) {
-      const float2 c = v[padi(k)];
-      v[padi(k)] = POST ? cconj(c) : cscale(cconj(c), 2.0f);
-    } else if (k < L / 2) {
-      const float2 w = __ldg(tw_real + k);  // exp(-2 pi i k / W)
-      float2 a = v[padi(k)], b = cconj(v[padi(L - k)]);
-      if (POST) {
-        const float2 E = cscale(cadd(a, b), 0.5f);
-        const float2 O = cmul_mi(cscale(csub(a, b), 0.5f));
-        const float2 WO = cmul(O, w);
-        v[padi(k)] = cadd(E, WO);
-        v[padi(L - k)] = cconj(csub(E, WO));
-      } else {
-        const float2 E = cadd(a, b);
-        const float2 O = cmul(csub(a, b), cconj(w));
-        v[padi(k)] = cadd(E, cmul_i(O));
-        v[padi(L - k)] = cadd(cconj(E), cmul_i(cconj(O)));
-      }
+  constexpr int LR = G::LR, BR = G::BR, E = G::E, A = G::A;
+  const int h = threadIdx.x % G::TR, hb = h == 0 ? BR / 2 : BR - h;
+  const GTab t = gtab<N, true>();
+  float2* v = gsmem() + (threadIdx.x / G::TR) * G::VROW;
+  {
+    float2 p[A], q[A];
+#pragma unroll
+    for (int j = 0; j < A; ++j) p[j] = __ldcg(Zrow + h + BR * j);
+#pragma unroll
+    for (int j = 0; j < A; ++j) q[j] = __ldcg(Zrow + hb + BR * j);
+    const float2* w = gsmem() + G::O_W;
+    if (h == 0) {
+      unit0_swap<A>(p, q);
+      p[0] = make_float2(p[0].x + p[0].y, p[0].x - p[0].y);
+      q[A - 1] = cscale(cconj(q[A - 1]), 2.0f);
+    } else {
+      k_pre(p[0], q[A - 1], w[h]);
     }
+#pragma unroll
+    for (int j = 1; j < A / 2; ++j) k_pre(p[j], q[A - 1 - j], w[h + BR * j]);
+#pragma unroll
+    for (int j = 0; j < A / 2; ++j) k_pre(q[j], p[A - 1 - j], w[hb + BR * j]);
+    if (h == 0) unit0_unswap<A>(p, q);
+    ginv_unit<LR, E>(v, h, p, t);
+    ginv_unit<LR, E>(v, hb, q, t);
   }
-  __syncthreads();
+  __syncwarp();
+  gmid<LR, E, true>(v, h, t, [] { __syncwarp(); });
+  __syncwarp();
+  ginv1<LR, E>(v, h, x);
 }
 
-// Row-phase pixel update of rows y0 .. y0+RB-1 held in buf as (s[2m], s[2m+1]) pairs (then a CTA barrier):
+// x -> half spectrum of the row, to Z
+template <int N>
+__device__ __forceinline__ void grow_fwd(const float2 (&x)[GGeo<N>::E], float2* Zrow) {
+  using G = GGeo<N>;
+  constexpr int LR = G::LR, BR = G::BR, E = G::E, A = G::A;
+  const int h = threadIdx.x % G::TR, hb = h == 0 ? BR / 2 : BR - h;
+  const GTab t = gtab<N, true>();
+  float2* v = gsmem() + (threadIdx.x / G::TR) * G::VROW;
+  gfwd1<LR, E>(v, h, x, t);
+  __syncwarp();
+  gmid<LR, E, false>(v, h, t, [] { __syncwarp(); });
+  __syncwarp();
+  float2 p[A], q[A];
+  gfwd_unit<LR, E>(v, h, p);
+  gfwd_unit<LR, E>(v, hb, q);
+  const float2* w = gsmem() + G::O_W;
+  if (h == 0) {
+    unit0_swap<A>(p, q);
+    p[0] = make_float2(p[0].x + p[0].y, p[0].x - p[0].y);  // (R[0], R[LR])
+    q[A - 1] = cconj(q[A - 1]);                            // K = LR/2
+  } else {
+    k_post(p[0], q[A - 1], w[h]);
+  }
+#pragma unroll
+  for (int j = 1; j < A / 2; ++j) k_post(p[j], q[A - 1 - j], w[h + BR * j]);
+#pragma unroll
+  for (int j = 0; j < A / 2; ++j) k_post(q[j], p[A - 1 - j], w[hb + BR * j]);
+  if (h == 0) unit0_unswap<A>(p, q);
+#pragma unroll
+  for (int j = 0; j < A; ++j) __stcg(Zrow + h + BR * j, p[j]);
+#pragma unroll
+  for (int j = 0; j < A; ++j) __stcg(Zrow + hb + BR * j, q[j]);
+  __syncwarp();  // the row's vector is rewritten by the next item
+}
+
+// f(x, e): pixel pair e (pixels 2e and 2e + 1) of the row, for each of the thread's pairs
+template <int N, class F>
+__device__ __forceinline__ void gpixels(float2 (&x)[GGeo<N>::E], F&& f) {
+  using G = GGeo<N>;
+  constexpr int NC = G::E / 8;
+  const int h = threadIdx.x % G::TR;
+#pragma unroll
+  for (int m = 0; m < 8; ++m)
+#pragma unroll
+    for (int i = 0; i < NC; ++i) f(x[8 * i + m], NC * h + i + (G::LR / 8) * m);
+}
+
+// a row of a row-major real image (nullptr: zeros)
+template <int N>
+__device__ __forceinline__ void grow_load(float2 (&x)[GGeo<N>::E], const float* row) {
+  gpixels<N>(x, [&](float2& v, int e) {
+    v = row != nullptr ? __ldg(reinterpret_cast<const float2*>(row) + e) : make_float2(0.f, 0.f);
+  });
+}
+// x to row y of an image of element type ot
+template <int N>
+__device__ __forceinline__ void grow_store(float2 (&x)[GGeo<N>::E], void* img, long long y, int ot) {
+  gpixels<N>(x, [&](float2& v, int e) { store_pair(img, y * (N / 2) + e, v, ot); });
+}
+
+// Pixel update of row y (pixel tables row-major):
 //   mode 0: sampler t-draw t = (1 - w) d + sqrt(w) (sqrt(w) s + sqrt(tau) xi) with the (a, q) table, Philox
 //           counter (pixel group (y W + x) / 4, step, chain, stream 0);
 //   mode 1: Wiener-filter t-update t = w (s - d) + d, w = 1 / (1 + lambda tau / N_bar) from the (d, 1/N_bar)
 //           table (rhs_mode: t = w s + lambda tau r with r in place of d);
 //   mode 2: the level right-hand side N_lambda^-1 d with N_lambda = N_bar + lt2 (s ignored).
+// The two pairs of a Philox group are in one thread (E = 16), or in neighbouring lanes (E = 8): there each lane
+// draws half of the groups and the two exchange the halves they need.
 template <int N>
-__device__ __forceinline__ void pixel_update(int mode, float2* buf, int y0, const float2* __restrict__ aq,
+__device__ __forceinline__ void pixel_update(int mode, float2 (&x)[GGeo<N>::E], int y, const float2* __restrict__ aq,
                                              const float2* __restrict__ dn, uint32_t step, uint32_t chain,
                                              uint32_t key0, uint32_t key1, float sqrt_tau, float ltau, int rhs_mode,
                                              float lt2) {
   using G = GGeo<N>;
-  for (int task = threadIdx.x; task < G::RB * (G::W / 4); task += 128) {
-    const int j = task / (G::W / 4), q = task % (G::W / 4);
-    const int y = y0 + j;
-    float2* v = buf + j * G::VROW;
-    float2 p0 = v[padi(2 * q)], p1 = v[padi(2 * q + 1)];
-    float s4[4] = {p0.x, p0.y, p1.x, p1.y};
-    if (mode == 0) {
-      float z[4];
-      normals4(uint32_t(y * (G::W / 4) + q), step, chain, 0u, key0, key1, z);
+  const float4* tab = reinterpret_cast<const float4*>((mode == 0 ? aq : dn) + (long long)y * G::W);
+  if (mode == 0) {
+    const int h = threadIdx.x % G::TR;
+    auto upd = [&](float2& v, float4 c, float z0, float z1) {
+      v.x = fmaf(c.y, fmaf(c.y, v.x, sqrt_tau * z0), c.x);
+      v.y = fmaf(c.w, fmaf(c.w, v.y, sqrt_tau * z1), c.z);
+    };
+    if constexpr (G::E == 16) {
 #pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        const float2 co = __ldg(aq + (4 * q + e) * G::H + y);
-        s4[e] = fmaf(co.y, fmaf(co.y, s4[e], sqrt_tau * z[e]), co.x);
-      }
-    } else if (mode == 1) {
-      const float g = rhs_mode ? 0.0f : 1.0f, h = rhs_mode ? ltau : 1.0f;
-#pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        const float2 co = __ldg(dn + (4 * q + e) * G::H + y);
-        const float w = wf_rcp(fmaf(ltau, co.y, 1.0f));
-        s4[e] = fmaf(w, fmaf(-g, co.x, s4[e]), h * co.x);
+      for (int m = 0; m < 8; ++m) {
+        const int e = 2 * h + (G::LR / 8) * m;
+        const float4 c0 = __ldg(tab + e), c1 = __ldg(tab + e + 1);
+        float z[4];
+        normals4(uint32_t(y * (G::W / 4) + e / 2), step, chain, 0u, key0, key1, z);
+        upd(x[m], c0, z[0], z[1]);
+        upd(x[8 + m], c1, z[2], z[3]);
       }
     } else {
+      const bool odd = h & 1;
 #pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        const float2 co = __ldg(dn + (4 * q + e) * G::H + y);
-        const float nbar = co.y > 0.0f ? wf_rcp(co.y) : wf_inf();
-        s4[e] = co.x / (nbar + lt2);
+      for (int i = 0; i < 4; ++i) {
+        const int e0 = h + (G::LR / 8) * i, e1 = h + (G::LR / 8) * (4 + i);
+        const float4 c0 = __ldg(tab + e0), c1 = __ldg(tab + e1);
+        float z[4];  // even lanes: the group of pair e0, odd lanes: that of e1
+        normals4(uint32_t(y * (G::W / 4) + (odd ? e1 : e0) / 2), step, chain, 0u, key0, key1, z);
+        const float r0 = __shfl_xor_sync(0xffffffffu, odd ? z[0] : z[2], 1);
+        const float r1 = __shfl_xor_sync(0xffffffffu, odd ? z[1] : z[3], 1);
+        upd(x[i], c0, odd ? r0 : z[0], odd ? r1 : z[1]);
+        upd(x[4 + i], c1, odd ? z[2] : r0, odd ? z[3] : r1);
       }
     }
-    v[padi(2 * q)] = make_float2(s4[0], s4[1]);
-    v[padi(2 * q + 1)] = make_float2(s4[2], s4[3]);
+  } else if (mode == 1) {
+    const float g = rhs_mode ? 0.0f : 1.0f, hh = rhs_mode ? ltau : 1.0f;
+    auto upd = [&](float& v, float dv, float inb) {
+      const float w = wf_weight(ltau, inb);
+      v = fmaf(w, fmaf(-g, dv, v), hh * dv);
+    };
+    gpixels<N>(x, [&](float2& v, int e) {
+      const float4 c = __ldg(tab + e);
+      upd(v.x, c.x, c.y);
+      upd(v.y, c.z, c.w);
+    });
+  } else {
+    auto rhs = [&](float dv, float inb) { return dv / ((inb > 0.0f ? wf_rcp(inb) : wf_inf()) + lt2); };
+    gpixels<N>(x, [&](float2& v, int e) {
+      const float4 c = __ldg(tab + e);
+      v = make_float2(rhs(c.x, c.y), rhs(c.z, c.w));
+    });
   }
-  __syncthreads();
 }
 
 // Row phase on one work item: rows y0 .. y0+RB-1 of field f. first: start from the real state s0.
 template <int N>
-__device__ void row_item(const GlobalArgs& a, float2* buf, int f, int y0, int done, bool first, bool emit_only,
-                         float ltau, const Scalars& sc) {
+__device__ void row_item(const GlobalArgs& a, int f, int y0, int done, bool first, bool emit_only, float ltau,
+                         const Scalars& sc) {
   using G = GGeo<N>;
-  constexpr int L = G::LR;
-  float2* Zf = a.Z + (long long)f * G::H * L;
-  const int nthr = 128;
-  if (first) {
-    for (int e = threadIdx.x; e < G::RB * L; e += nthr) {
-      const int j = e / L, m = e % L;
-      float2 v = make_float2(0.f, 0.f);
-      if (a.mode == 0 && a.init_s != nullptr)
-        v = reinterpret_cast<const float2*>(a.init_s + f * a.init_stride + (long long)(y0 + j) * G::W)[m];
-      if (a.mode == 3) {
-        const long long o = (long long)f * G::H * G::W + (long long)(y0 + j) * G::W;
-        v = reinterpret_cast<const float2*>(a.va + o)[m];
-        if (a.vb) {
-          const float2 u = reinterpret_cast<const float2*>(a.vb + o)[m];
-          v = make_float2(fmaf(a.vsign, u.x, v.x), fmaf(a.vsign, u.y, v.y));
-        }
-      }
-      buf[j * G::VROW + padi(m)] = v;
-    }
-    __syncthreads();
+  const int y = y0 + int(threadIdx.x) / G::TR;
+  float2* Zrow = a.Z + ((long long)f * G::H + y) * G::LR;
+  float2 x[G::E];
+  if (!first) {
+    grow_inv<N>(Zrow, x);
+  } else if (a.mode == 3) {
+    const long long o = ((long long)f * G::H + y) * G::W;
+    grow_load<N>(x, a.va + o);
+    if (a.vb)
+      gpixels<N>(x, [&](float2& v, int e) {
+        const float2 u = __ldg(reinterpret_cast<const float2*>(a.vb + o) + e);
+        v = make_float2(fmaf(a.vsign, u.x, v.x), fmaf(a.vsign, u.y, v.y));
+      });
   } else {
-    for (int e = threadIdx.x; e < G::RB * L; e += nthr) {
-      const int j = e / L, m = e % L;
-      buf[j * G::VROW + padi(m)] = __ldcg(Zf + (long long)(y0 + j) * L + m);
-    }
-    __syncthreads();
-    real_pass<N, false>(buf, G::RB, a.tw_real);
-    fft_smem<G::RR, G::RB, G::VROW, true, G::SR>(buf, a.tw_row);
+    grow_load<N>(x, a.mode == 0 && a.init_s ? a.init_s + f * a.init_stride + (long long)y * G::W : nullptr);
   }
-  // buf rows hold (s[2m], s[2m+1]) (scaled as the fused kernels: unnormalised transforms, the 1/n and
-  // 1/sqrt(2n) factors are in the Fourier-space tables)
+  // x holds the row's pixels (unnormalised transforms, the 1/n and 1/sqrt(2n) factors are in the Fourier-space
+  // tables)
   if (a.mode == 0 && !first) {
     const int d1 = done;  // sweeps completed
-    if (d1 > a.burn_in && (d1 - a.burn_in) % a.thin == 0 && f < a.n_fields) {
+    if (d1 > a.burn_in && (d1 - a.burn_in) % a.thin == 0) {
       const long long ms = (d1 - a.burn_in) / a.thin - 1;
-      const long long base = ((long long)f * a.n_samples + ms) * (long long)(G::H * G::W) / 2;  // pairs
-      for (int e = threadIdx.x; e < G::RB * L; e += nthr) {
-        const int j = e / L, m = e % L;
-        store_pair(a.out, base + (long long)(y0 + j) * (G::W / 2) + m, buf[j * G::VROW + padi(m)], a.out_dtype);
-      }
+      grow_store<N>(x, a.out, ((long long)f * a.n_samples + ms) * G::H + y, a.out_dtype);
     }
-    __syncthreads();  // the pixel update below maps threads to other elements of buf
   }
   if (emit_only) {
-    if (a.mode == 1) {  // Wiener filter: final state to out
-      for (int e = threadIdx.x; e < G::RB * L; e += nthr) {
-        const int j = e / L, m = e % L;
-        reinterpret_cast<float2*>(a.out + (long long)(y0 + j) * G::W)[m] = buf[j * G::VROW + padi(m)];
-      }
-    }
-    __syncthreads();
+    if (a.mode == 1) grow_store<N>(x, a.out, y, kOutF32);  // Wiener filter: final state to out
     return;
   }
-  // pixel-space update on 4-pixel groups (Philox group (y W + x)/4 in the sampler); mode 3 transforms
-  // the field as loaded
-  if (a.mode != 3)
-    pixel_update<N>(a.mode, buf, y0, a.aq, a.dn, a.step0 + uint32_t(done), a.chain0 + uint32_t(f), a.key0, a.key1,
+  if (a.mode != 3)  // mode 3 transforms the field as loaded
+    pixel_update<N>(a.mode, x, y, a.aq, a.dn, a.step0 + uint32_t(done), a.chain0 + uint32_t(f), a.key0, a.key1,
                     sc.sqrt_tau, ltau, a.rhs_mode, a.mode == 2 ? float(level_lambda(sc, f, a.eta) * sc.tau) : 0.f);
-  else
-    __syncthreads();
-  fft_smem<G::RR, G::RB, G::VROW, false, G::SR>(buf, a.tw_row);
-  real_pass<N, true>(buf, G::RB, a.tw_real);
-  for (int e = threadIdx.x; e < G::RB * L; e += nthr) {
-    const int j = e / L, m = e % L;
-    __stcg(Zf + (long long)(y0 + j) * L + m, buf[j * G::VROW + padi(m)]);
+  grow_fwd<N>(x, Zrow);
+}
+
+// ---------------------------------------------------------------------------------------------
+// column phase: thread tid of a column item holds column c0 + tid % CB, unit pair (h, hb), h = tid / CB
+// ---------------------------------------------------------------------------------------------
+// Columns c0 .. c0 + CB - 1 of Z: forward transform, f(p, q) on the thread's units (after unit0_swap: mode
+// pairs (p[j], q[A-1-j]) at ky1 = h + BC j and (q[j], p[A-1-j]) at ky1 = hb + BC j, j < A/2), and with INV the inverse
+// transform back to Z.
+template <int N, bool INV, class F>
+__device__ __forceinline__ void gcol(float2* Z, int c0, F&& f) {
+  using G = GGeo<N>;
+  constexpr int H = G::H, LR = G::LR, BC = G::BC, E = G::E, A = G::A, NC = E / 8;
+  const int c = threadIdx.x % G::CB, h = threadIdx.x / G::CB, hb = h == 0 ? BC / 2 : BC - h;
+  const GTab t = gtab<N, false>();
+  float2* v = gsmem() + c * G::VCOL;
+  float2* Zc = Z + (long long)(NC * h) * LR + c0 + c;
+  {
+    float2 x[E];
+#pragma unroll
+    for (int m = 0; m < 8; ++m)
+#pragma unroll
+      for (int i = 0; i < NC; ++i) x[8 * i + m] = __ldcg(Zc + (long long)(H / 8 * m + i) * LR);
+    gfwd1<H, E>(v, h, x, t);
+  }
+  __syncthreads();
+  gmid<H, E, false>(v, h, t, [] { __syncthreads(); });
+  __syncthreads();
+  {
+    float2 p[A], q[A];
+    gfwd_unit<H, E>(v, h, p);
+    gfwd_unit<H, E>(v, hb, q);
+    if (h == 0) unit0_swap<A>(p, q);
+    f(p, q, c0 + c, h, hb);
+    if (!INV) {
+      __syncthreads();  // the vectors are rewritten by the next item
+      return;
+    }
+    if (h == 0) unit0_unswap<A>(p, q);
+    ginv_unit<H, E>(v, h, p, t);
+    ginv_unit<H, E>(v, hb, q, t);
+  }
+  __syncthreads();
+  gmid<H, E, true>(v, h, t, [] { __syncthreads(); });
+  __syncthreads();
+  {
+    float2 x[E];
+    ginv1<H, E>(v, h, x);
+#pragma unroll
+    for (int m = 0; m < 8; ++m)
+#pragma unroll
+      for (int i = 0; i < NC; ++i) __stcg(Zc + (long long)(H / 8 * m + i) * LR, x[8 * i + m]);
   }
   __syncthreads();
 }
 
-// Column-phase spectral update of columns c0 .. c0+CB-1 held in buf (after the forward column FFT), over
-// the mode pairs (j, H - j) of each column (j = 0 pairs ky = 0 with ky = H/2), then a CTA barrier:
+// inter(y1, y2, ky1, ky2) on the mode pairs of an interior column; the H/2 pairs of the packed edge column (column
+// 0: kx = 0 as A and kx = W/2 as B in Y = A + i B) are shared out over all threads of its CTA
+template <int N, class I, class X>
+__device__ __forceinline__ void gpairs(float2 (&p)[GGeo<N>::A], float2 (&q)[GGeo<N>::A], int col, int h, int hb, int c0, I&& inter,
+                                       X&& edge) {
+  using G = GGeo<N>;
+  constexpr int H = G::H, BC = G::BC, A = G::A;
+  float2* e = gsmem() + G::O_EDGE;
+  if (c0 == 0) {  // the same in every thread of the CTA
+    if (col == 0) {
+#pragma unroll
+      for (int j = 0; j < A / 2; ++j) {
+        e[2 * (h + BC * j)] = p[j];
+        e[2 * (h + BC * j) + 1] = q[A - 1 - j];
+        e[2 * (hb + BC * j)] = q[j];
+        e[2 * (hb + BC * j) + 1] = p[A - 1 - j];
+      }
+    }
+    __syncthreads();
+    for (int k = threadIdx.x; k < H / 2; k += G::T) {
+      float2 y1 = e[2 * k], y2 = e[2 * k + 1];
+      edge(y1, y2, k, k == 0 ? H / 2 : H - k);
+      e[2 * k] = y1;
+      e[2 * k + 1] = y2;
+    }
+  }
+  if (col != 0) {
+#pragma unroll
+    for (int j = 0; j < A / 2; ++j) {
+      const int ky1 = h + BC * j;
+      inter(p[j], q[A - 1 - j], ky1, ky1 == 0 ? H / 2 : H - ky1);
+    }
+#pragma unroll
+    for (int j = 0; j < A / 2; ++j) inter(q[j], p[A - 1 - j], hb + BC * j, H - hb - BC * j);
+  }
+  if (c0 == 0) {
+    __syncthreads();
+    if (col == 0) {
+#pragma unroll
+      for (int j = 0; j < A / 2; ++j) {
+        p[j] = e[2 * (h + BC * j)];
+        q[A - 1 - j] = e[2 * (h + BC * j) + 1];
+        q[j] = e[2 * (hb + BC * j)];
+        p[A - 1 - j] = e[2 * (hb + BC * j) + 1];
+      }
+    }
+  }
+}
+
+// Column-phase spectral update of columns c0 .. c0+CB-1 (tables in natural order):
 //   mode 0: sampler s-draw s_hat = f t_hat + g zeta with the (f/n, g/sqrt(2n)) table and Philox counter
-//           (column pair group col H/2 + j, step, chain, stream 1; edge column shared as in the on-chip kernel);
-//   mode 1: Wiener-filter update s_hat = P/(P + lambda tau) t_hat / n; with cmp, returns this CTA's part of
+//           (column pair group col H/2 + j, step, chain, stream 1; edge column as in the on-chip kernel);
+//   mode 1: Wiener-filter update s_hat = P/(P + lambda tau) t_hat / n; with cmp, returns this thread's part of
 //           sum_k |s_hat - prev|^2 ((P + lambda tau)/(lambda tau))^2 (the residual from consecutive
 //           iterates); with store, keeps s_hat in prev;
-//   mode 2: returns sum_k P^2 |t_hat|^2 of the level right-hand side (buf unchanged).
+//   mode 2: returns this thread's part of sum_k P^2 |t_hat|^2 of the level right-hand side (Z unchanged).
+// Per-mode terms and a thread's partial sum in FP32, the CTA and grid sums in FP64.
 template <int N>
-__device__ __forceinline__ double col_update(int mode, float2* buf, int c0, const float2* __restrict__ fg,
-                                             const float* __restrict__ Pk, float2* prev, uint32_t step,
-                                             uint32_t chain, uint32_t key0, uint32_t key1, float ltau, bool cmp,
-                                             bool store) {
+__device__ __forceinline__ float gcol_update(int mode, float2* Z, int c0, const float2* __restrict__ fg,
+                                              const float* __restrict__ Pk, float2* prev, uint32_t step,
+                                              uint32_t chain, uint32_t key0, uint32_t key1, float ltau, bool cmp,
+                                              bool store) {
   using G = GGeo<N>;
   constexpr int L = G::LR, H = G::H, WH = G::WH;
   constexpr float INV_N = 1.0f / float(G::H * G::W);
-  float acc = 0.0f;  // this thread's tasks in FP32; the CTA and grid sums are FP64
-  // mode pairs (j, H - j) of each column, j in [0, H/2); j = 0 pairs ky = 0 with ky = H/2
-  for (int task = threadIdx.x; task < G::CB * (H / 2); task += 128) {
-    const int jc = task / (H / 2), j = task % (H / 2);
-    const int col = c0 + jc;
-    const int ky1 = j, ky2 = j == 0 ? H / 2 : H - j;
-    float2* v = buf + jc * G::VCOL;
-    float2 y1 = v[padi(ky1)], y2 = v[padi(ky2)];
-    if (mode == 0) {
-      float z[4];
-      normals4(uint32_t(col * (H / 2) + j), step, chain, 1u, key0, key1, z);
-      if (col != 0) {
-        const float2 m1 = __ldg(fg + ky1 * WH + col), m2 = __ldg(fg + ky2 * WH + col);
-        y1 = make_float2(fmaf(m1.x, y1.x, m1.y * z[0]), fmaf(m1.x, y1.y, m1.y * z[1]));
-        y2 = make_float2(fmaf(m2.x, y2.x, m2.y * z[2]), fmaf(m2.x, y2.y, m2.y * z[3]));
-      } else {
-        const float2 a1 = __ldg(fg + ky1 * WH), b1 = __ldg(fg + ky1 * WH + G::W / 2);
-        if (j == 0) {
-          const float2 a2 = __ldg(fg + ky2 * WH), b2 = __ldg(fg + ky2 * WH + G::W / 2);
-          constexpr float R2 = 1.41421356237309505f;
-          y1 = make_float2(fmaf(a1.x, y1.x, R2 * a1.y * z[0]), fmaf(b1.x, y1.y, R2 * b1.y * z[2]));
-          y2 = make_float2(fmaf(a2.x, y2.x, R2 * a2.y * z[1]), fmaf(b2.x, y2.y, R2 * b2.y * z[3]));
-        } else {
-          const float2 y2c = cconj(y2);
-          const float2 A = cscale(cadd(y1, y2c), 0.5f);
-          const float2 B = cmul_mi(cscale(csub(y1, y2c), 0.5f));
-          const float2 Ap = make_float2(fmaf(a1.x, A.x, a1.y * z[0]), fmaf(a1.x, A.y, a1.y * z[1]));
-          const float2 Bp = make_float2(fmaf(b1.x, B.x, b1.y * z[2]), fmaf(b1.x, B.y, b1.y * z[3]));
-          y1 = cadd(Ap, cmul_i(Bp));
-          y2 = cadd(cconj(Ap), cmul_i(cconj(Bp)));
-        }
-      }
-    } else if (mode == 1) {
-      // per-mode residual terms and the thread's partial sum in FP32, CTA and grid sums in FP64 (as
-      // s_update_wf_parked)
-      const float inv_lt = 1.0f / ltau;
-      auto wres = [&](float P, float dre, float dim) -> float {
-        const float g = fmaf(P, inv_lt, 1.0f);
-        return fmaf(dre, dre, dim * dim) * (g * g);
-      };
-      if (col != 0) {
-        const float P1 = __ldg(Pk + ky1 * WH + col), P2 = __ldg(Pk + ky2 * WH + col);
-        const float2 n1 = cscale(y1, wf_fdiv(P1, P1 + ltau) * INV_N), n2 = cscale(y2, wf_fdiv(P2, P2 + ltau) * INV_N);
-        if (cmp) {
-          const float2 o1 = prev[ky1 * L + col], o2 = prev[ky2 * L + col];
-          acc += 2.0f * (wres(P1, n1.x - o1.x, n1.y - o1.y) + wres(P2, n2.x - o2.x, n2.y - o2.y));
-        }
-        y1 = n1;
-        y2 = n2;
-      } else {
-        const float Pa1 = __ldg(Pk + ky1 * WH), Pb1 = __ldg(Pk + ky1 * WH + G::W / 2);
-        const float Pa2 = __ldg(Pk + ky2 * WH), Pb2 = __ldg(Pk + ky2 * WH + G::W / 2);
-        const float fa1 = wf_fdiv(Pa1, Pa1 + ltau) * INV_N, fb1 = wf_fdiv(Pb1, Pb1 + ltau) * INV_N;
-        const float fa2 = wf_fdiv(Pa2, Pa2 + ltau) * INV_N, fb2 = wf_fdiv(Pb2, Pb2 + ltau) * INV_N;
-        if (j == 0) {
-          const float2 n1 = make_float2(fa1 * y1.x, fb1 * y1.y), n2 = make_float2(fa2 * y2.x, fb2 * y2.y);
-          if (cmp) {
-            const float2 o1 = prev[ky1 * L], o2 = prev[ky2 * L];
-            acc += wres(Pa1, n1.x - o1.x, 0.f) + wres(Pb1, n1.y - o1.y, 0.f) + wres(Pa2, n2.x - o2.x, 0.f) +
-                   wres(Pb2, n2.y - o2.y, 0.f);
-          }
-          y1 = n1;
-          y2 = n2;
-        } else {
-          const float2 y2c = cconj(y2);
-          const float2 A = cscale(cscale(cadd(y1, y2c), 0.5f), fa1);
-          const float2 B = cscale(cmul_mi(cscale(csub(y1, y2c), 0.5f)), fb1);
-          if (cmp) {
-            const float2 o1 = prev[ky1 * L], o2c = cconj(prev[ky2 * L]);
-            const float2 oA = cscale(cadd(o1, o2c), 0.5f);
-            const float2 oB = cmul_mi(cscale(csub(o1, o2c), 0.5f));
-            acc += 2.0f * (wres(Pa1, A.x - oA.x, A.y - oA.y) + wres(Pb1, B.x - oB.x, B.y - oB.y));
-          }
-          y1 = cadd(A, cmul_i(B));
-          y2 = cadd(cconj(A), cmul_i(cconj(B)));
-        }
-      }
-      if (store) {
-        prev[ky1 * L + col] = y1;
-        prev[ky2 * L + col] = y2;
-      }
-    } else {
-      auto p2 = [](float P, float re, float im) -> float { return P * P * fmaf(re, re, im * im); };
-      if (col != 0) {
-        acc += 2.0f * (p2(__ldg(Pk + ky1 * WH + col), y1.x, y1.y) + p2(__ldg(Pk + ky2 * WH + col), y2.x, y2.y));
-      } else if (j == 0) {
-        acc += p2(__ldg(Pk + ky1 * WH), y1.x, 0.f) + p2(__ldg(Pk + ky1 * WH + G::W / 2), y1.y, 0.f) +
-               p2(__ldg(Pk + ky2 * WH), y2.x, 0.f) + p2(__ldg(Pk + ky2 * WH + G::W / 2), y2.y, 0.f);
-      } else {
-        const float2 y2c = cconj(y2);
-        const float2 A = cscale(cadd(y1, y2c), 0.5f);
-        const float2 B = cmul_mi(cscale(csub(y1, y2c), 0.5f));
-        acc += 2.0f * (p2(__ldg(Pk + ky1 * WH), A.x, A.y) + p2(__ldg(Pk + ky1 * WH + G::W / 2), B.x, B.y));
-      }
-    }
-    v[padi(ky1)] = y1;
-    v[padi(ky2)] = y2;
+  float acc = 0.0f;
+  if (mode == 0) {
+    gcol<N, true>(Z, c0, [&](float2 (&p)[G::A], float2 (&q)[G::A], int col, int h, int hb) {
+      gpairs<N>(
+          p, q, col, h, hb, c0,
+          [&](float2& y1, float2& y2, int ky1, int ky2) {
+            const float2 m1 = __ldg(fg + ky1 * WH + col), m2 = __ldg(fg + ky2 * WH + col);
+            float z[4];
+            normals4(uint32_t(col * (H / 2) + ky1), step, chain, 1u, key0, key1, z);
+            y1 = make_float2(fmaf(m1.x, y1.x, m1.y * z[0]), fmaf(m1.x, y1.y, m1.y * z[1]));
+            y2 = make_float2(fmaf(m2.x, y2.x, m2.y * z[2]), fmaf(m2.x, y2.y, m2.y * z[3]));
+          },
+          [&](float2& y1, float2& y2, int ky1, int ky2) {
+            const float2 a1 = __ldg(fg + ky1 * WH), b1 = __ldg(fg + ky1 * WH + G::W / 2);
+            float z[4];
+            normals4(uint32_t(ky1), step, chain, 1u, key0, key1, z);
+            if (ky1 == 0) {
+              const float2 a2 = __ldg(fg + ky2 * WH), b2 = __ldg(fg + ky2 * WH + G::W / 2);
+              constexpr float R2 = 1.41421356237309505f;
+              y1 = make_float2(fmaf(a1.x, y1.x, R2 * a1.y * z[0]), fmaf(b1.x, y1.y, R2 * b1.y * z[2]));
+              y2 = make_float2(fmaf(a2.x, y2.x, R2 * a2.y * z[1]), fmaf(b2.x, y2.y, R2 * b2.y * z[3]));
+            } else {
+              const float2 y2c = cconj(y2);
+              const float2 A = cscale(cadd(y1, y2c), 0.5f);
+              const float2 B = cmul_mi(cscale(csub(y1, y2c), 0.5f));
+              const float2 Ap = make_float2(fmaf(a1.x, A.x, a1.y * z[0]), fmaf(a1.x, A.y, a1.y * z[1]));
+              const float2 Bp = make_float2(fmaf(b1.x, B.x, b1.y * z[2]), fmaf(b1.x, B.y, b1.y * z[3]));
+              y1 = cadd(Ap, cmul_i(Bp));
+              y2 = cadd(cconj(Ap), cmul_i(cconj(Bp)));
+            }
+          });
+    });
+  } else if (mode == 1) {
+    const float inv_lt = cmp ? 1.0f / ltau : 0.0f;
+    auto wres = [&](float P, float dre, float dim) -> float {
+      const float g = fmaf(P, inv_lt, 1.0f);
+      return fmaf(dre, dre, dim * dim) * (g * g);
+    };
+    auto fcoef = [&](float P) { return wf_fdiv(P, P + ltau) * INV_N; };
+    gcol<N, true>(Z, c0, [&](float2 (&p)[G::A], float2 (&q)[G::A], int col, int h, int hb) {
+      gpairs<N>(
+          p, q, col, h, hb, c0,
+          [&](float2& y1, float2& y2, int ky1, int ky2) {
+            const float P1 = __ldg(Pk + ky1 * WH + col), P2 = __ldg(Pk + ky2 * WH + col);
+            y1 = cscale(y1, fcoef(P1));
+            y2 = cscale(y2, fcoef(P2));
+            if (cmp) {
+              const float2 o1 = prev[ky1 * L + col], o2 = prev[ky2 * L + col];
+              acc += 2.0f * (wres(P1, y1.x - o1.x, y1.y - o1.y) + wres(P2, y2.x - o2.x, y2.y - o2.y));
+            }
+            if (store) {
+              prev[ky1 * L + col] = y1;
+              prev[ky2 * L + col] = y2;
+            }
+          },
+          [&](float2& y1, float2& y2, int ky1, int ky2) {
+            const float Pa1 = __ldg(Pk + ky1 * WH), Pb1 = __ldg(Pk + ky1 * WH + G::W / 2);
+            const float fa1 = fcoef(Pa1), fb1 = fcoef(Pb1);
+            if (ky1 == 0) {
+              const float Pa2 = __ldg(Pk + ky2 * WH), Pb2 = __ldg(Pk + ky2 * WH + G::W / 2);
+              y1 = make_float2(fa1 * y1.x, fb1 * y1.y);
+              y2 = make_float2(fcoef(Pa2) * y2.x, fcoef(Pb2) * y2.y);
+              if (cmp) {
+                const float2 o1 = prev[0], o2 = prev[ky2 * L];
+                acc += wres(Pa1, y1.x - o1.x, 0.f) + wres(Pb1, y1.y - o1.y, 0.f) + wres(Pa2, y2.x - o2.x, 0.f) +
+                       wres(Pb2, y2.y - o2.y, 0.f);
+              }
+            } else {
+              const float2 y2c = cconj(y2);
+              const float2 A = cscale(cscale(cadd(y1, y2c), 0.5f), fa1);
+              const float2 B = cscale(cmul_mi(cscale(csub(y1, y2c), 0.5f)), fb1);
+              y1 = cadd(A, cmul_i(B));
+              y2 = cadd(cconj(A), cmul_i(cconj(B)));
+              if (cmp) {
+                const float2 o1 = prev[ky1 * L], o2c = cconj(prev[ky2 * L]);
+                const float2 oA = cscale(cadd(o1, o2c), 0.5f);
+                const float2 oB = cmul_mi(cscale(csub(o1, o2c), 0.5f));
+                acc += 2.0f * (wres(Pa1, A.x - oA.x, A.y - oA.y) + wres(Pb1, B.x - oB.x, B.y - oB.y));
+              }
+            }
+            if (store) {
+              prev[ky1 * L] = y1;
+              prev[ky2 * L] = y2;
+            }
+          });
+    });
+  } else {
+    auto p2 = [](float P, float re, float im) -> float { return P * P * fmaf(re, re, im * im); };
+    gcol<N, false>(Z, c0, [&](float2 (&p)[G::A], float2 (&q)[G::A], int col, int h, int hb) {
+      gpairs<N>(
+          p, q, col, h, hb, c0,
+          [&](float2& y1, float2& y2, int ky1, int ky2) {
+            acc += 2.0f * (p2(__ldg(Pk + ky1 * WH + col), y1.x, y1.y) + p2(__ldg(Pk + ky2 * WH + col), y2.x, y2.y));
+          },
+          [&](float2& y1, float2& y2, int ky1, int ky2) {
+            if (ky1 == 0) {
+              acc += p2(__ldg(Pk), y1.x, 0.f) + p2(__ldg(Pk + G::W / 2), y1.y, 0.f) +
+                     p2(__ldg(Pk + ky2 * WH), y2.x, 0.f) + p2(__ldg(Pk + ky2 * WH + G::W / 2), y2.y, 0.f);
+            } else {
+              const float2 y2c = cconj(y2);
+              const float2 A = cscale(cadd(y1, y2c), 0.5f);
+              const float2 B = cmul_mi(cscale(csub(y1, y2c), 0.5f));
+              acc += 2.0f * (p2(__ldg(Pk + ky1 * WH), A.x, A.y) + p2(__ldg(Pk + ky1 * WH + G::W / 2), B.x, B.y));
+            }
+          });
+    });
   }
-  __syncthreads();
-  return double(acc);
-}
-
-// Column phase on one work item: columns c0 .. c0+CB-1 of field f.
-// mode 0: s-draw; mode 1: s_hat = f_lambda t_hat with residual bookkeeping (returns this CTA's partial
-// sum when cmp); mode 2: P^2 |V|^2 power of the level right-hand side (no write-back).
-template <int N>
-__device__ double col_item(const GlobalArgs& a, float2* buf, int f, int c0, int done, float ltau, bool cmp,
-                           bool store) {
-  using G = GGeo<N>;
-  constexpr int L = G::LR, H = G::H;
-  float2* Zf = a.Z + (long long)f * H * L;
-  for (int e = threadIdx.x; e < G::CB * H; e += 128) {
-    const int j = e % G::CB, y = e / G::CB;  // consecutive threads: consecutive columns of a row
-    buf[j * G::VCOL + padi(y)] = __ldcg(Zf + (long long)y * L + c0 + j);
-  }
-  __syncthreads();
-  fft_smem<G::RC, G::CB, G::VCOL, false, G::SC>(buf, a.tw_col);
-  const double acc = col_update<N>(a.mode, buf, c0, a.fg, a.Pk, a.prev, a.step0 + uint32_t(done),
-                                   a.chain0 + uint32_t(f), a.key0, a.key1, ltau, cmp, store);
-  if (a.mode == 2) return acc;
-  fft_smem<G::RC, G::CB, G::VCOL, true, G::SC>(buf, a.tw_col);
-  for (int e = threadIdx.x; e < G::CB * H; e += 128) {
-    const int j = e % G::CB, y = e / G::CB;
-    __stcg(Zf + (long long)y * L + c0 + j, buf[j * G::VCOL + padi(y)]);
-  }
-  __syncthreads();
   return acc;
 }
 
 // mode 3: weighted power sums of CB columns of field f into acc[j], j < nw
 template <int N>
-__device__ void col_wpower(const GlobalArgs& a, float2* buf, int f, int c0, double (&acc)[4]) {
+__device__ void col_wpower(const GlobalArgs& a, int f, int c0, double (&acc)[4]) {
   using G = GGeo<N>;
-  constexpr int L = G::LR, H = G::H, WH = G::WH, TS = G::H * G::WH;
-  const float2* Zf = a.Z + (long long)f * H * L;
-  for (int e = threadIdx.x; e < G::CB * H; e += 128) {
-    const int j = e % G::CB, y = e / G::CB;
-    buf[j * G::VCOL + padi(y)] = __ldcg(Zf + (long long)y * L + c0 + j);
-  }
-  __syncthreads();
-  fft_smem<G::RC, G::CB, G::VCOL, false, G::SC>(buf, a.tw_col);
+  constexpr int WH = G::WH, TS = G::H * G::WH;
   auto sq = [](float p, float q) -> double { return double(p) * p + double(q) * q; };
-  for (int task = threadIdx.x; task < G::CB * (H / 2); task += 128) {
-    const int jc = task / (H / 2), j = task % (H / 2);
-    const int col = c0 + jc;
-    const int ky1 = j, ky2 = j == 0 ? H / 2 : H - j;
-    const float2* v = buf + jc * G::VCOL;
-    const float2 y1 = v[padi(ky1)], y2 = v[padi(ky2)];
-    for (int t = 0; t < a.nw; ++t) {
-      const float* wt = a.wts + t * TS;
-      double s;
-      if (col != 0) {
-        s = 2.0 * (__ldg(wt + ky1 * WH + col) * sq(y1.x, y1.y) + __ldg(wt + ky2 * WH + col) * sq(y2.x, y2.y));
-      } else if (j == 0) {
-        s = __ldg(wt + ky1 * WH) * sq(y1.x, 0.f) + __ldg(wt + ky1 * WH + G::W / 2) * sq(y1.y, 0.f) +
-            __ldg(wt + ky2 * WH) * sq(y2.x, 0.f) + __ldg(wt + ky2 * WH + G::W / 2) * sq(y2.y, 0.f);
-      } else {
-        const float2 y2c = cconj(y2);
-        const float2 A = cscale(cadd(y1, y2c), 0.5f);
-        const float2 B = cmul_mi(cscale(csub(y1, y2c), 0.5f));
-        s = 2.0 * (__ldg(wt + ky1 * WH) * sq(A.x, A.y) + __ldg(wt + ky1 * WH + G::W / 2) * sq(B.x, B.y));
-      }
-      acc[t] += s;
-    }
-  }
-  __syncthreads();
+  gcol<N, false>(a.Z + (long long)f * G::H * G::LR, c0, [&](float2 (&p)[G::A], float2 (&q)[G::A], int col, int h, int hb) {
+    gpairs<N>(
+        p, q, col, h, hb, c0,
+        [&](float2& y1, float2& y2, int ky1, int ky2) {
+          for (int t = 0; t < a.nw; ++t) {
+            const float* wt = a.wts + t * TS;
+            acc[t] += 2.0 * (__ldg(wt + ky1 * WH + col) * sq(y1.x, y1.y) + __ldg(wt + ky2 * WH + col) * sq(y2.x, y2.y));
+          }
+        },
+        [&](float2& y1, float2& y2, int ky1, int ky2) {
+          for (int t = 0; t < a.nw; ++t) {
+            const float* wt = a.wts + t * TS;
+            if (ky1 == 0) {
+              acc[t] += __ldg(wt) * sq(y1.x, 0.f) + __ldg(wt + G::W / 2) * sq(y1.y, 0.f) +
+                        __ldg(wt + ky2 * WH) * sq(y2.x, 0.f) + __ldg(wt + ky2 * WH + G::W / 2) * sq(y2.y, 0.f);
+            } else {
+              const float2 y2c = cconj(y2);
+              const float2 A = cscale(cadd(y1, y2c), 0.5f);
+              const float2 B = cmul_mi(cscale(csub(y1, y2c), 0.5f));
+              acc[t] += 2.0 * (__ldg(wt + ky1 * WH) * sq(A.x, A.y) + __ldg(wt + ky1 * WH + G::W / 2) * sq(B.x, B.y));
+            }
+          }
+        });
+  });
 }
 
-__device__ __forceinline__ double block_sum_128(double v, double* red) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
+// CTA sum in a fixed order, valid in the first warp: the threads' values through shared memory (T doubles), one warp
+// adds them (with every thread in the shuffle tree the SM's two FP64 lanes are busy for several hundred cycles)
+template <int T>
+__device__ __forceinline__ double gblock_sum(double v, double* red) {
+  red[threadIdx.x] = v;
   __syncthreads();
-  const double s = red[0] + red[1] + red[2] + red[3];
+  double s = 0.0;
+  if (threadIdx.x < 32) {
+#pragma unroll
+    for (int w = 0; w < T / 32; ++w) s += red[32 * w + threadIdx.x];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  }
   __syncthreads();
   return s;
 }
 
+// schedule of the cooled solve, decided by one thread per CTA (every CTA the same way) and shared
+struct GSolveState {
+  double rho2;  // of the last check (-1: none)
+  float ltau;
+  int lev, k, status;
+};
+
 template <int N>
-__global__ void __launch_bounds__(128, 3) k_global(GlobalArgs a) {
+__global__ void __launch_bounds__(GGeo<N>::T, GGeo<N>::MIN_CTAS) k_global(const __grid_constant__ GlobalArgs a) {
   using G = GGeo<N>;
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  float2* buf = reinterpret_cast<float2*>(smem_raw);
-  __shared__ double red[4];
+  __shared__ double red[G::T];
+  __shared__ GSolveState dec;
   const Scalars sc = *a.sc;
   if (sc.status != 0) {
     if (a.mode == 1 && blockIdx.x == 0 && threadIdx.x == 0) a.st->status = sc.status;
     return;
   }
+  gtab_init<N>();
   const unsigned int nb = gridDim.x;
+  unsigned int target = 0;  // of the grid barrier
   const int row_items = G::ROW_ITEMS * a.n_fields, col_items = G::COL_ITEMS * a.n_fields;
 
   auto rows = [&](int done, bool first, bool emit_only, float ltau) {
     for (int it = blockIdx.x; it < row_items; it += nb) {
       const int f = it / G::ROW_ITEMS;
       if (a.mode == 2 && f >= sc.n_levels) continue;  // level fields past the schedule
-      row_item<N>(a, buf, f, (it % G::ROW_ITEMS) * G::RB, done, first, emit_only, ltau, sc);
+      row_item<N>(a, f, (it % G::ROW_ITEMS) * G::RB, done, first, emit_only, ltau, sc);
     }
+  };
+  auto col = [&](int f, int it, int done, float ltau, bool cmp, bool store) -> float {
+    return gcol_update<N>(a.mode, a.Z + (long long)f * G::H * G::LR, (it % G::COL_ITEMS) * G::CB, a.fg, a.Pk, a.prev,
+                          a.step0 + uint32_t(done), a.chain0 + uint32_t(f), a.key0, a.key1, ltau, cmp, store);
   };
   auto cols = [&](int done, float ltau, bool cmp, bool store) -> double {
     double acc = 0.0;
-    for (int it = blockIdx.x; it < col_items; it += nb)
-      acc += col_item<N>(a, buf, it / G::COL_ITEMS, (it % G::COL_ITEMS) * G::CB, done, ltau, cmp, store);
+    for (int it = blockIdx.x; it < col_items; it += nb) {
+      const float v = col(it / G::COL_ITEMS, it, done, ltau, cmp, store);
+      if (cmp) acc += double(v);
+    }
     return acc;
   };
 
   if (a.mode == 0) {
     rows(0, true, false, 0.f);
     for (int i = 0; i < a.n_sweeps; ++i) {
-      if (!grid_barrier(a.bar, nb)) return;
+      if (!grid_barrier(a.bar, nb, target)) return;
       cols(i, 0.f, false, false);
-      if (!grid_barrier(a.bar, nb)) return;
+      if (!grid_barrier(a.bar, nb, target)) return;
       rows(i + 1, false, i + 1 == a.n_sweeps, 0.f);
     }
     return;
   }
   if (a.mode == 3) {  // weighted power of given fields
     rows(0, true, false, 0.f);
-    if (!grid_barrier(a.bar, nb)) return;
+    if (!grid_barrier(a.bar, nb, target)) return;
     for (int it = blockIdx.x; it < col_items; it += nb) {
       const int f = it / G::COL_ITEMS;
       double acc[4] = {0.0, 0.0, 0.0, 0.0};
-      col_wpower<N>(a, buf, f, (it % G::COL_ITEMS) * G::CB, acc);
+      col_wpower<N>(a, f, (it % G::COL_ITEMS) * G::CB, acc);
       for (int t = 0; t < a.nw; ++t) {
-        const double s = block_sum_128(acc[t], red);
+        const double s = gblock_sum<G::T>(acc[t], red);
         if (threadIdx.x == 0) atomicAdd(a.wout + f * a.nw + t, s / double(G::H * G::W));
       }
     }
@@ -641,61 +872,71 @@ __global__ void __launch_bounds__(128, 3) k_global(GlobalArgs a) {
   }
   if (a.mode == 2) {  // level norms, fields = levels
     rows(0, true, false, 0.f);
-    if (!grid_barrier(a.bar, nb)) return;
+    if (!grid_barrier(a.bar, nb, target)) return;
     for (int it = blockIdx.x; it < col_items; it += nb) {
       const int f = it / G::COL_ITEMS;
       if (f >= sc.n_levels) continue;
-      const double s = block_sum_128(col_item<N>(a, buf, f, (it % G::COL_ITEMS) * G::CB, 0, 0.f, false, false), red);
+      const double s = gblock_sum<G::T>(col(f, it, 0, 0.f, false, false), red);
       if (threadIdx.x == 0) atomicAdd(a.bnorm_out + f, s / double(G::H * G::W));
     }
     return;
   }
   // Wiener filter with lambda-cooling, one field; every CTA follows the same schedule
-  const double tau = sc.tau;
-  int lev = 0;
-  double lam = sc.lam0;
-  float ltau = float(lam * tau);
   const int last_level = sc.n_levels - 1;
-  int it = 0, k = 0, status = 1, parity = 0;
-  double rho = -1.0;
+  int lev = 0, it = 0, k = 0, status = 1, parity = 0;
+  float ltau = float(sc.lam0 * sc.tau);
+  double rho2 = -1.0;
   rows(0, true, false, ltau);
   while (true) {
     ++k;
     ++it;
     const bool cmp = (k % a.check == 0) && k >= 2;
     const bool store = ((k + 1) % a.check == 0);
-    if (!grid_barrier(a.bar, nb)) return;
-    const double part = block_sum_128(cols(it, ltau, cmp, store), red);
-    if (cmp && threadIdx.x == 0) atomicAdd(a.acc + parity, part);
-    if (!grid_barrier(a.bar, nb)) return;
+    if (!grid_barrier(a.bar, nb, target)) return;
+    const double mine = cols(it, ltau, cmp, store);
     if (cmp) {
-      const double tot = __ldcg(a.acc + parity) * double(G::H * G::W);
-      if (blockIdx.x == 0 && threadIdx.x == 0) a.acc[parity ^ 1] = 0.0;  // next check's accumulator
-      parity ^= 1;
-      const double bn = a.bnorm2[lev];
-      const double r2 = bn > 0.0 ? tot / bn : tot;
-      rho = sqrt(r2);
-      if (!(r2 == r2) || r2 > 1e300) {
-        status = 6;
-      } else if (lev < last_level) {
-        if (rho < a.level_tol || k >= a.level_max) {
-          ++lev;
-          lam = level_lambda(sc, lev, a.eta);
-          ltau = float(lam * tau);
-          k = 0;
-        }
-      } else if (rho < a.tol) {
-        status = 0;
-      }
+      const double part = gblock_sum<G::T>(mine, red);
+      if (threadIdx.x == 0) atomicAdd(a.acc + parity, part);
     }
-    if (status == 1 && it >= a.max_iter) status = 5;
+    // a check's decision by the thread that waits for the barrier: rho = sqrt(tot / bn) against the tolerances,
+    // without the division and the root (run by every thread these took about 4000 cycles a check)
+    const bool open = grid_barrier(a.bar, nb, target, [&] {
+      if (!cmp) return;
+      const double tot = __ldcg(a.acc + parity) * double(G::H * G::W);
+      const double bn = a.bnorm2[lev], ref = bn > 0.0 ? bn : 1.0;
+      if (blockIdx.x == 0) a.acc[parity ^ 1] = 0.0;  // next check's accumulator
+      GSolveState d{tot, ltau, lev, k, 1};
+      if (!(tot == tot) || tot > 1e300 * ref) {
+        d.status = 6;  // non-finite residual
+      } else if (lev < last_level) {
+        if (tot < a.level_tol * a.level_tol * ref || k >= a.level_max) {
+          ++d.lev;
+          d.ltau = float(level_lambda(sc, d.lev, a.eta) * sc.tau);
+          d.k = 0;
+        }
+      } else if (tot < a.tol * a.tol * ref) {
+        d.status = 0;
+      }
+      if (blockIdx.x == 0) d.rho2 = tot / ref;
+      dec = d;
+    });
+    if (!open) return;
+    if (cmp) {
+      parity ^= 1;
+      rho2 = dec.rho2;
+      lev = dec.lev;
+      ltau = dec.ltau;
+      k = dec.k;
+      status = dec.status;
+    }
+    if (status == 1 && it >= a.max_iter) status = 5;  // not converged
     rows(it, false, status != 1, ltau);
     if (status != 1) break;
   }
   if (blockIdx.x == 0 && threadIdx.x == 0) {
     a.st->status = status;
     a.st->iters = it;
-    a.st->resid = rho;
+    a.st->resid = rho2 >= 0.0 ? sqrt(rho2) : rho2;
   }
 }
 

@@ -241,7 +241,7 @@ cudaError_t launch_global(const GlobalArgs& a, cudaStream_t st, LaunchTimer* t) 
   int dev = 0, sms = 0, per_sm = 0;
   if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
   if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-  if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_global<N>, 128, G::SMEM)) != cudaSuccess) return e;
+  if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_global<N>, G::T, G::SMEM)) != cudaSuccess) return e;
   if (per_sm < 1) return cudaErrorInvalidConfiguration;
   const long long items = (long long)(G::ROW_ITEMS > G::COL_ITEMS ? G::ROW_ITEMS : G::COL_ITEMS) * a.n_fields;
   long long full = (long long)per_sm * sms;
@@ -250,7 +250,7 @@ cudaError_t launch_global(const GlobalArgs& a, cudaStream_t st, LaunchTimer* t) 
   GlobalArgs arg = a;
   void* args[] = {&arg};
   if (t) t->start();
-  e = cudaLaunchCooperativeKernel(reinterpret_cast<void*>(k_global<N>), dim3(grid), dim3(128), args, G::SMEM, st);
+  e = cudaLaunchCooperativeKernel(reinterpret_cast<void*>(k_global<N>), dim3(grid), dim3(G::T), args, G::SMEM, st);
   if (t) t->stop();
   if (e != cudaSuccess) return e;
   return cudaGetLastError();
@@ -263,7 +263,7 @@ cudaError_t launch_gbatch(const GBArgs& a, cudaStream_t st) {
   int dev = 0, sms = 0, per_sm = 0;
   if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
   if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-  if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_gbatch<N>, 128, G::SMEM)) != cudaSuccess) return e;
+  if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_gbatch<N>, G::T, G::SMEM)) != cudaSuccess) return e;
   if (per_sm < 1) return cudaErrorInvalidConfiguration;
   const long long items = (long long)(G::ROW_ITEMS > G::COL_ITEMS ? G::ROW_ITEMS : G::COL_ITEMS) * a.F;
   long long full = (long long)per_sm * sms;
@@ -271,7 +271,7 @@ cudaError_t launch_gbatch(const GBArgs& a, cudaStream_t st) {
   const int grid = int(items < full ? items : full);
   GBArgs arg = a;
   void* args[] = {&arg};
-  e = cudaLaunchCooperativeKernel(reinterpret_cast<void*>(k_gbatch<N>), dim3(grid), dim3(128), args, G::SMEM, st);
+  e = cudaLaunchCooperativeKernel(reinterpret_cast<void*>(k_gbatch<N>), dim3(grid), dim3(G::T), args, G::SMEM, st);
   if (e != cudaSuccess) return e;
   return cudaGetLastError();
 }

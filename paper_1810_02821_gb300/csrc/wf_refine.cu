@@ -93,15 +93,16 @@ __global__ void k_ir_divp(int H, int W, const float* __restrict__ Pk, double2* X
   if ((threadIdx.x & 31) == 0 && acc != 0.0) atomicAdd(out, acc);
 }
 
-// r = rpix - Re(q); xr = (r, 0); rtab[x*H + y] = (float(r), 1/N_bar) for the correction solve
+// r = rpix - Re(q); xr = (r, 0); rtab = (float(r), 1/N_bar) for the correction solve, in dn's order (x-major, or
+// row-major with row_major)
 __global__ void k_ir_finish(int H, int W, const double* __restrict__ rpix, const double2* __restrict__ q,
-                            const float2* __restrict__ dn, double2* xr, float2* rtab) {
+                            const float2* __restrict__ dn, int row_major, double2* xr, float2* rtab) {
   const int n = H * W;
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
     const double r = rpix[i] - q[i].x;
     xr[i] = make_double2(r, 0.0);
-    const int y = i / W, x = i % W;
-    rtab[x * H + y] = make_float2(float(r), dn[x * H + y].y);
+    const int at = row_major ? i : (i % W) * H + i / W;
+    rtab[at] = make_float2(float(r), dn[at].y);
   }
 }
 
@@ -194,7 +195,7 @@ cudaError_t refine_residual(const RefineArgs& a, cudaStream_t st) {
   double2* q = nullptr;
   if ((e = fft2_f64(X, other, a.H, a.W, +1, st, &q)) != cudaSuccess) return e;  // q = S^-1 s
   double2* xr = q == xa ? xb : xa;
-  k_ir_finish<<<grid_for(n), 256, 0, st>>>(a.H, a.W, rpix, q, a.dn, xr, a.rtab);
+  k_ir_finish<<<grid_for(n), 256, 0, st>>>(a.H, a.W, rpix, q, a.dn, a.row_major, xr, a.rtab);
   double2* other2 = xr == xa ? xb : xa;
   double2* R = nullptr;
   if ((e = fft2_f64(xr, other2, a.H, a.W, -1, st, &R)) != cudaSuccess) return e;

@@ -16,8 +16,9 @@ struct RefineArgs {
   const float* A;        // diagonal pixel response of d = A s + n, or null for A = I
   const float* Pk;       // [H][W/2+1]
   const float* s;        // current FP32 iterate [H][W]
-  const float2* dn;      // Wiener-filter pixel table [W][H] (d, 1/N_bar)
-  float2* rtab;          // out: correction right-hand-side table [W][H] (r, 1/N_bar)
+  const float2* dn;      // Wiener-filter pixel table (d, 1/N_bar), [W][H] or, with row_major, [H][W]
+  float2* rtab;          // out: correction right-hand-side table (r, 1/N_bar) in the same order
+  int row_major;
   double* rnorm;         // out: ||S r||^2
   double* bnorm;         // out (refine_bnorm): ||S N^-1 d||^2
   double* level_norms;   // out: rnorm copied into n_levels entries
