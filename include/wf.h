@@ -229,11 +229,11 @@ wf_status wf_shear_to_convergence(const float* gamma, int64_t n, int32_t H, int3
  *   - Images up to 128 x 128, per size (opts->small_path): by default in phases (per-image set-up and
  *     tables, the level norms, one CTA per image for the cooled solve, then the samplers with several
  *     images per CTA), or as one persistent launch in which every CTA keeps one image's field in shared
- *     memory and takes images from an atomic work counter. 256 x 256 and 512 x 512 images: one
- *     thread-block cluster per image runs its whole pipeline with the field in distributed shared memory;
- *     1024 x 1024 images, small chunks and devices without room for a cluster: one cooperative launch per
- *     chunk with the fields in global memory. The size classes and the chunks of the large classes run
- *     on their own streams (`large_streams` per large class) and overlap. All of it is ordered after the
+ *     memory and takes images from an atomic work counter. Larger images: one
+ *     cooperative launch per size class with the fields in global memory, or, from 400 images of 256 x 256,
+ *     one thread-block cluster per image that runs its whole pipeline with the field in distributed shared
+ *     memory (wf_set_large_image_sampler forces either). The size classes, and the chunks of a class on
+ *     clusters, run on their own streams (up to `large_streams`) and overlap. All of it is ordered after the
  *     work already on `stream` and the call returns when everything has finished.
  *   - items: HOST array; the pointers inside are DEVICE pointers owned by the caller; out_wf may be NULL
  *     (then the filter is not written), out_samples may be NULL when n_samples == 0.
@@ -262,7 +262,8 @@ typedef struct {
   double tol, eta, level_tol;
   int32_t level_max, check, max_iter;
   int32_t n_samples;   /* samples per image (>= 0) */
-  int32_t large_streams; /* concurrent pipelines for images above 128 x 128 (>= 1) */
+  int32_t large_streams; /* concurrent pipelines for images above 128 x 128 (>= 1): chunks of a class on clusters, and
+                            streams that the classes on the global-memory kernels (one launch each) share */
   int32_t small_grid_pct; /* launch shape: persistent CTAs of each size class up to 128 x 128, in percent of
                              the occupancy limit (1..100; 0 = 100) */
   int32_t large_grid_pct; /* launch shape: CTAs of each cooperative launch for larger images, in percent of
@@ -277,7 +278,8 @@ typedef struct {
                                  0 = 32 */
   int32_t small_fields_per_cta; /* phased path: images per CTA of the sampler launch of each size class up
                                    to 128 x 128, 1, 2, 4 or 8, capped at 128 / H (128 threads per CTA);
-                                   0 = the cap */
+                                   0 = the cap. In effect at 16 x 16: the larger sizes run several threads
+                                   per row, one image per CTA */
 } wf_batch_opts;
 
 void wf_batch_opts_default(wf_batch_opts* o);
@@ -446,9 +448,9 @@ double wf_last_kernel_ms(void);
  * rounding): thread-block clusters, each holding one chain's or image's field in distributed shared memory
  * (N / 64 or N / 32 CTAs; a batch image runs its level norms, cooled solve and samples in one cluster),
  * and the global-memory kernels (fields in global memory, cooperative launches with many CTAs per field).
- * mode 0 (default, automatic): clusters when a call holds at least 32 chains at 256 x 256 or 8 at
- * 512 x 512 (a batch chunk as many images) and the device can host the cluster, otherwise the
- * global-memory kernels, which are faster for few fields; mode 1: always the global-memory kernels;
+ * mode 0 (default, automatic): clusters when a call holds at least 400 chains at 256 x 256 (a batch as many
+ * images) and the device can host the cluster, otherwise the global-memory kernels, which are faster for
+ * fewer fields and at 512 x 512; mode 1: always the global-memory kernels;
  * mode 2: clusters wherever the device can host them. Returns the previous mode.
  */
 int32_t wf_set_large_image_sampler(int32_t mode);

@@ -240,12 +240,15 @@ bool size_ok(int H, int W) {
 
 bool cluster_fits(int H, int rows = 0);
 
-// Path for `units` independent fields (chains or images) of H x H, H in {256, 512}: one thread-block
-// cluster per field, or the global-memory kernels. Automatic choice (measured on GB300, 50 sweeps): the
-// global-memory kernels (16-point sub-transforms, many CTAs per field) are faster for few fields, the
-// clusters from about 32 fields at 256^2 (24 chains: 1.40 vs 1.84 ms; 32 chains: 2.46 vs 1.88 ms) and
-// from about 8 at 512^2 (4 chains: 1.39 vs 1.58 ms; 8 chains: 2.88 vs 2.07 ms).
-int cluster_min_units(int H) { return H == 256 ? 32 : 8; }
+// Path for `units` independent fields (chains or images) of H x H, H in {256, 512}: one thread-block cluster per
+// field, or the global-memory kernels. Automatic choice, measured on GB300 (us per sampler sweep of all chains,
+// global-memory / cluster): 256^2: 16 chains 11.9 / 29.4, 64 chains 34.4 / 33.3, 228 chains 88 / 100, 342 chains
+// 131 / 136, 400 chains 161 / 147, 1000 chains 380 / 354; 512^2: 4 chains 12.5 / 25.2, 50 chains 90 / 134, 152 chains
+// 265 / 370, 600 chains 1005 / 1443. So clusters from 400 fields at 256^2 (every SM full of clusters either way, and
+// the fields no longer fit L2 with their tables) and the global-memory kernels at every count at 512^2. A batch's
+// classes cross over at the same counts (Wiener solve and 16 samples, ms: 77 images of 256^2 5.5 / 7.3, 307 images
+// 17.5 / 17.6; 102 images of 512^2 21.9 / 26.4).
+int cluster_min_units(int H) { return H == 256 ? 400 : 1 << 30; }
 
 // rows per CTA of the cluster kernels: 64 at 256; at 512 the caller's choice of 32 or 64 (0: the default)
 int cluster_rows_of(int H, int rows) { return H == 512 && (rows == 32 || rows == 64) ? rows : wf::cluster_rows(H); }
@@ -1865,24 +1868,28 @@ wf_status plan_batch(const wf_batch_item* items, int n_items, const wf_batch_opt
     if (e != cudaSuccess) return cuda_fail(e);
     p->o_slot[c] = cv.take<char>(size_t(grid) * size_t(batch_slot_any(kBatchSizes[c])));
   }
-  // large images: each size class split into up to large_streams chunks, chunk k on stream k
+  // Large images. Cluster classes are split into up to large_streams chunks, chunk k on stream k. A class on the
+  // global-memory kernels is one chunk (its grid already fills the GPU; eight chunks on eight streams took turns:
+  // 154 images of 256^2 16.5 ms against 9.5 ms in one), each class on its own stream so that small ones overlap.
   p->chunks.clear();
   p->nls = 0;
   for (int c = 4; c < 7; ++c) {
     const int nc = int(p->cls[c].size());
     if (!nc) continue;
-    const int parts = o.large_streams < nc ? o.large_streams : nc;
+    const bool cluster = use_cluster(kBatchSizes[c], nc, o.large_cluster_rows);
+    const int parts = cluster ? (o.large_streams < nc ? o.large_streams : nc) : 1;
+    const int first = cluster ? 0 : (c - 4) % o.large_streams;
     for (int k = 0; k < parts; ++k) {
       GBChunk ch;
       ch.H = kBatchSizes[c];
-      ch.stream = k;
+      ch.stream = first + k;
       for (int i = k * nc / parts; i < (k + 1) * nc / parts; ++i) ch.items.push_back(p->cls[c][i]);
-      ch.cluster = use_cluster(ch.H, int(ch.items.size()), o.large_cluster_rows);
+      ch.cluster = cluster;
       ch.rows = cluster_rows_of(ch.H, o.large_cluster_rows);
       layout_chunk(ch, cv);
       p->chunks.push_back(std::move(ch));
     }
-    if (parts > p->nls) p->nls = parts;
+    if (first + parts > p->nls) p->nls = first + parts;
   }
   p->order.clear();
   for (int c = 0; c < 7; ++c) p->order.insert(p->order.end(), p->cls[c].begin(), p->cls[c].end());

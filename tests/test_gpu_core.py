@@ -1,5 +1,5 @@
-"""GPU checks of the on-chip sampler's kernel choice: the one-thread-per-row kernel (many 64 x 64 chains) and the
-kernel with several threads per row draw the same chains."""
+"""GPU checks of the sampler's kernel choice by chain count: the one-thread-per-row kernel (many 64 x 64 chains) and the
+kernel with several threads per row, and the cluster and global-memory kernels at 256 x 256, draw the same chains."""
 import pytest
 
 from gpu_common import need_gpu, rel, to_dev
@@ -8,7 +8,8 @@ from paper_1810_02821_gb300 import build, synth, wf
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("H,chains", [(32, 1), (32, 67), (64, 1), (64, 760), (64, 761), (64, 1217), (128, 305)])
+@pytest.mark.parametrize("H,chains", [(32, 1), (32, 67), (64, 1), (64, 760), (64, 761), (64, 1217), (128, 305), (256, 399),
+                                      (256, 400), (512, 9)])
 def test_chain_does_not_depend_on_the_chain_count(H, chains):
     """Chain c of a call with many chains equals the call for that chain alone. Each kernel is within 5e-7
     relative L2 of the exact chain (FP32 rounding over these sweeps), so the two agree to 2e-6."""
