@@ -748,7 +748,7 @@ wf_status solve_refined(const float* d, const float* Ndiag, const uint8_t* mask,
   const size_t n = size_t(H) * W, nm = size_t(H) * (W / 2 + 1);
   Carve cv;
   const size_t o_sc = cv.take<wf::Scalars>(1), o_dn = cv.take<float2>(n), o_rt = cv.take<float2>(n),
-               o_e = cv.take<float>(n), o_nr = cv.take<double>(4), o_ln = cv.take<double>(kMaxLevels),
+               o_e = cv.take<float>(n), o_nr = cv.take<double>(4),
                o_pk = cv.take<float>(size_on_chip(H) ? nm : 0),
                o_fft = cv.take<char>(wf::refine_scratch_bytes(H, W));
   Scratch scr;
@@ -788,8 +788,6 @@ wf_status solve_refined(const float* d, const float* Ndiag, const uint8_t* mask,
   ra.row_major = solve_perm(H) < 0;
   ra.rnorm = norms;
   ra.bnorm = norms + 1;
-  ra.level_norms = reinterpret_cast<double*>(b + o_ln);
-  ra.n_levels = kMaxLevels;
   ra.scratch = b + o_fft;
   cudaError_t e = wf::refine_bnorm(ra, st);
   if (e != cudaSuccess) return cuda_fail(e);
@@ -808,7 +806,8 @@ wf_status solve_refined(const float* d, const float* Ndiag, const uint8_t* mask,
     if (!(rho == rho)) { status = WF_ERR_NONFINITE; break; }
     if (rho < o.tol) { status = WF_OK; break; }
     if (k == o.refine) break;
-    r = solve_pass(d, Ndiag, mask, Pk, H, W, corr, ev, &it, &rs, st, nullptr, ra.rtab, ra.level_norms, &su);
+    if ((e = wf::refine_correction(ra, st)) != cudaSuccess) return cuda_fail(e);
+    r = solve_pass(d, Ndiag, mask, Pk, H, W, corr, ev, &it, &rs, st, nullptr, ra.rtab, ra.rnorm, &su);
     total += it;
     if (r != WF_OK && r != WF_ERR_NOT_CONVERGED) return r;
     if ((e = wf::refine_update(int(n), out_s, ev, st)) != cudaSuccess) return cuda_fail(e);
@@ -1271,7 +1270,7 @@ wf_status wf_solve_spin2(const float* d1, const float* d2, const float* N1, cons
   const size_t n = size_t(H) * W, nm = size_t(H) * (W / 2 + 1);
   Carve cv;
   const size_t o_sc = cv.take<wf::Scalars>(3), o_aq = cv.take<float2>(2 * n), o_fe = cv.take<float2>(nm),
-               o_fb = cv.take<float2>(nm), o_r = cv.take<double>(2), o_x = cv.take<double2>(8 * n);
+               o_fb = cv.take<float2>(nm), o_r = cv.take<double>(2), o_x = cv.take<double2>(2 * n);
   Scratch scr;
   scr.st = st;
   WF_CUDA(cudaMallocAsync(&scr.base, cv.off, st));
@@ -1289,7 +1288,6 @@ wf_status wf_solve_spin2(const float* d1, const float* d2, const float* N1, cons
   wf::Scalars hs[2];
   WF_CUDA(cudaMemcpyAsync(hs, sc, 2 * sizeof(wf::Scalars), cudaMemcpyDeviceToHost, st));
   WF_CUDA(cudaMemsetAsync(out, 0, 2 * n * sizeof(float), st));
-  WF_CUDA(cudaMemsetAsync(rn, 0, 2 * sizeof(double), st));
   WF_CUDA(cudaStreamSynchronize(st));
   if (hs[0].status != WF_OK) return wf_status(hs[0].status);
   const double tau = hs[0].tau, pmax = hs[0].pmax > hs[1].pmax ? hs[0].pmax : hs[1].pmax;
@@ -1339,7 +1337,6 @@ wf_status wf_solve_spin2(const float* d1, const float* d2, const float* N1, cons
     const int k = o.check < o.max_iter - iters ? o.check : o.max_iter - iters;
     if ((r = run(1.0, k)) != WF_OK) return r;
     iters += k;
-    WF_CUDA(cudaMemsetAsync(rn, 0, sizeof(double), st));
     e = wf::spin2_residual_f64(out, d1, d2, N1, N2, mask, PE, PB, H, W, false, rn, b + o_x, st);
     if (e != cudaSuccess) return cuda_fail(e);
     double h;
@@ -1360,13 +1357,16 @@ wf_status wf_shear_to_convergence(const float* gamma, int64_t n_fields, int32_t 
   if (!size_ok(H, W)) return WF_ERR_SHAPE;
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
   const size_t n = size_t(H) * W;
+  // as many fields per launch as fit 64 MiB of scratch (half of L2)
+  const int64_t most = int64_t((64u << 20) / (n * sizeof(double2)));
+  const int64_t chunk = n_fields < most ? n_fields : most;
   Scratch scr;
   scr.st = st;
-  WF_CUDA(cudaMallocAsync(&scr.base, 4 * n * sizeof(double2), st));
-  for (int64_t i = 0; i < n_fields; ++i) {
-    const float* g = gamma + i * 2 * n;
-    float* k = kappa + i * 2 * n;
-    cudaError_t e = wf::shear_to_convergence_f64(g, g + n, H, W, k, k + n, scr.base, st);
+  if (n_fields > 0) WF_CUDA(cudaMallocAsync(&scr.base, size_t(chunk) * n * sizeof(double2), st));
+  for (int64_t i = 0; i < n_fields; i += chunk) {
+    const int64_t f = n_fields - i < chunk ? n_fields - i : chunk;
+    const cudaError_t e =
+        wf::shear_to_convergence_f64(gamma + i * 2 * n, int(f), H, W, kappa + i * 2 * n, scr.base, st);
     if (e != cudaSuccess) return cuda_fail(e);
   }
   WF_CUDA(cudaStreamSynchronize(st));
@@ -2602,7 +2602,7 @@ wf_status wf_wiener_vjp(const float* d, const float* sigma2, const uint8_t* mask
   Carve cv;
   const size_t o_P = cv.take<float>(3 * nm), o_N = cv.take<float>(n), o_s = cv.take<float>(n), o_x = cv.take<float>(n),
                o_b = cv.take<float>(n), o_y = cv.take<float>(n), o_w = cv.take<float>(n), o_sum = cv.take<double>(4),
-               o_pow = cv.take<double>(8), o_f64 = cv.take<double2>(2 * n);
+               o_pow = cv.take<double>(8), o_f64 = cv.take<double2>(n);
   Scratch scr;
   scr.st = st;
   WF_CUDA(cudaMallocAsync(&scr.base, cv.off, st));

@@ -1039,7 +1039,7 @@ __device__ __forceinline__ int ksolve_sweeps(float2 (&x)[KGeo<N>::E], const floa
       const double tot = kwarp_total<N>() * double(G::H * G::W);
       if (threadIdx.x == G::T - 32) {
         // rho = sqrt(tot / bn) against the tolerances, without the division and the root
-        const double bn = bnorm2[lev], ref = bn > 0.0 ? bn : 1.0;
+        const double bn = bnorm2[rhs ? 0 : lev], ref = bn > 0.0 ? bn : 1.0;
         KSolveState d{tot, ltau, lev, k, 1};
         if (!(tot == tot) || tot > 1e300 * ref) {
           d.status = 6;  // non-finite residual

@@ -1183,7 +1183,7 @@ struct SolveArgs {
   const float2* dn;      // [W][H] pixel table (d, 1/N_bar), or (r, 1/N_bar) in rhs mode
   const float* Pk;       // [H][W/2+1]
   const Scalars* sc;
-  const double* bnorm2;  // [n_levels] ||S N_lambda^-1 d||^2 per level (rhs mode: ||S r||^2)
+  const double* bnorm2;  // [n_levels] ||S N_lambda^-1 d||^2 per level (rhs mode: ||S r||^2 for every level)
   const float* init_s;   // nullptr -> zeros
   float2* prev;          // [H][W/2] scratch: previous s_hat at check sweeps
   float* out;            // [H][W]
@@ -1248,7 +1248,7 @@ __device__ __forceinline__ int solve_sweeps(float2* S, double* red, int lt, floa
       unpark_modes<N>(S, lt, c);
       if (cmp) {
         const double tot = block_sum(acc, red) * double(G::H * G::W);
-        const double bn = bnorm2[lev];
+        const double bn = bnorm2[rhs ? 0 : lev];
         const double r2 = bn > 0.0 ? tot / bn : tot;
         rho = sqrt(r2);
         if (!(r2 == r2) || r2 > 1e300) {

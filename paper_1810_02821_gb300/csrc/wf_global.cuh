@@ -303,7 +303,7 @@ struct GlobalArgs {
   uint32_t step0;
   uint32_t key0, key1;
   // Wiener filter (n_fields == 1)
-  const double* bnorm2;
+  const double* bnorm2;    // level norms (rhs_mode: one norm for every level)
   double* acc;             // [2] residual accumulators (alternating)
   float2* prev;            // [H][W/2]
   SolveStatus* st;
@@ -903,7 +903,7 @@ __global__ void __launch_bounds__(GGeo<N>::T, GGeo<N>::MIN_CTAS) k_global(const 
     const bool open = grid_barrier(a.bar, nb, target, [&] {
       if (!cmp) return;
       const double tot = __ldcg(a.acc + parity) * double(G::H * G::W);
-      const double bn = a.bnorm2[lev], ref = bn > 0.0 ? bn : 1.0;
+      const double bn = a.bnorm2[a.rhs_mode ? 0 : lev], ref = bn > 0.0 ? bn : 1.0;
       if (blockIdx.x == 0) a.acc[parity ^ 1] = 0.0;  // next check's accumulator
       GSolveState d{tot, ltau, lev, k, 1};
       if (!(tot == tot) || tot > 1e300 * ref) {
