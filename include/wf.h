@@ -188,9 +188,10 @@ wf_status wf_sample_band(const float* d, const float* Ndiag, const uint8_t* mask
  * (zeta_E stream 1, zeta_B stream 9, the counter layout of wf_sample), and the rotation back. tau = the
  * minimum observed noise variance of both components unless opts->tau > 0. out: device
  * [n_chains][n_samples][2][H][W] shear samples (element type opts->out_dtype); opts->init_s, when given,
- * is [2][H][W] (or [n_chains][2][H][W] with init_per_chain). Sizes up to 512 x 512 (256 and 512: both
- * components of a chain in one thread-block cluster of 32-row CTAs; WF_ERR_CUDA with
- * cudaErrorNotSupported where the device cannot host such a cluster). opts->A, when given, is one pixel
+ * is [2][H][W] (or [n_chains][2][H][W] with init_per_chain). Sizes up to 512 x 512 (256 and 512: the
+ * fields in global memory, or, from 24 chains at 256 x 256, both components of a chain in one thread-block
+ * cluster of 32-row CTAs; wf_set_large_image_sampler forces either, and the forced clusters answer WF_ERR_CUDA
+ * with cudaErrorNotSupported where the device cannot host one). opts->A, when given, is one pixel
  * response for both components (as in wf_sample_ex: d_c = A gamma_c + n_c, A = 0 meaning no data).
  */
 wf_status wf_sample_spin2(const float* d1, const float* d2, const float* N1, const float* N2, const uint8_t* mask,
@@ -204,7 +205,7 @@ wf_status wf_sample_spin2(const float* d1, const float* d2, const float* N1, con
  * lambda = 1 the FP64 relative residual ||g + S N^-1 (g - d)|| / ||S N^-1 d|| (S the shear covariance of
  * the E/B spectra) is evaluated every opts->check sweeps until it is below opts->tol or opts->max_iter
  * sweeps have run (WF_ERR_NOT_CONVERGED). out: device [2][H][W]; iters_out, resid_out: HOST, may be NULL.
- * Sizes up to 512 x 512 (256 and 512 on wf_sample_spin2's thread-block clusters); opts may be NULL
+ * Sizes up to 512 x 512 (on wf_sample_spin2's kernels, without the draws); opts may be NULL
  * (defaults); opts->A, when given, is one pixel response for both components (the filter and its residual
  * are those of the response problem); opts->refine and init_s are not used.
  */
@@ -443,14 +444,15 @@ double wf_last_kernel_ms(void);
 
 /*
  * Path for 256 x 256 and 512 x 512 images (wf_sample, wf_sample_ex, the first pass of wf_solve /
- * wf_solve_ex, and the large images of wf_batch_run and the batch graphs), per host thread. Two kernel
+ * wf_solve_ex, wf_sample_spin2, wf_solve_spin2, and the large images of wf_batch_run and the batch graphs),
+ * per host thread. Two kernel
  * families compute the same chain and the same filter (the same draws and schedule; FP32 results agree to
  * rounding): thread-block clusters, each holding one chain's or image's field in distributed shared memory
  * (N / 64 or N / 32 CTAs; a batch image runs its level norms, cooled solve and samples in one cluster),
  * and the global-memory kernels (fields in global memory, cooperative launches with many CTAs per field).
  * mode 0 (default, automatic): clusters when a call holds at least 400 chains at 256 x 256 (a batch as many
  * images) and the device can host the cluster, otherwise the global-memory kernels, which are faster for
- * fewer fields and at 512 x 512; mode 1: always the global-memory kernels;
+ * fewer fields and at 512 x 512 (spin-2: clusters from 24 chains at 256 x 256); mode 1: always the global-memory kernels;
  * mode 2: clusters wherever the device can host them. Returns the previous mode.
  */
 int32_t wf_set_large_image_sampler(int32_t mode);

@@ -250,6 +250,15 @@ bool cluster_fits(int H, int rows = 0);
 // 17.5 / 17.6; 102 images of 512^2 21.9 / 26.4).
 int cluster_min_units(int H) { return H == 256 ? 400 : 1 << 30; }
 
+// Path of the spin-2 sampler and filter at 256 and 512: the global-memory kernels, or clusters from 24 chains at 256^2
+// (us per sweep of all chains, global-memory / cluster: 256^2: 1 chain 8.4 / 23.5, 16 chains 29.9 / 31.3, 32 chains
+// 43.1 / 33.1, 456 chains 460 / 402; 512^2: 1 chain 11.4 / 46.7, 36 chains 168 / 275, 150 chains 653 / 1017).
+int spin2_cluster_min(int H) { return H == 256 ? 24 : 1 << 30; }
+bool spin2_use_cluster(int H, int chains) {
+  if (g_large_sampler != 0) return g_large_sampler == 2;
+  return chains >= spin2_cluster_min(H) && cluster_fits(H);
+}
+
 // rows per CTA of the cluster kernels: 64 at 256; at 512 the caller's choice of 32 or 64 (0: the default)
 int cluster_rows_of(int H, int rows) { return H == 512 && (rows == 32 || rows == 64) ? rows : wf::cluster_rows(H); }
 
@@ -1118,6 +1127,45 @@ wf_status wf_sample_band(const float* d, const float* Ndiag, const uint8_t* mask
 }  // extern "C"
 
 namespace {
+// one launch of the spin-2 sweeps (tables in the order of spin2_orders); Z, bar: scratch of the global-memory form
+struct Spin2Path {
+  bool global = false;
+  int cm = 0, perm = 0;  // table orders (k_tables)
+  size_t z_count = 0;    // float2 of Z
+};
+Spin2Path spin2_path(int H, int chains) {
+  Spin2Path p;
+  if (size_on_chip(H)) {
+    p.cm = wf::core_cm(H);
+  } else if (spin2_use_cluster(H, chains)) {
+    p.cm = 32;
+    p.perm = H / 32;
+  } else {
+    p.global = true;
+    p.perm = -1;
+    p.z_count = size_t(chains) * H * H;
+  }
+  return p;
+}
+cudaError_t launch_spin2_any(int H, const Spin2Path& p, const wf::Spin2Args& a, float2* Z, wf::GridBar* bar,
+                             cudaStream_t st, wf::LaunchTimer* t) {
+  if (p.global) {
+    const cudaError_t e = cudaMemsetAsync(&bar->count, 0, sizeof(bar->count), st);  // err collects over launches
+    if (e != cudaSuccess) return e;
+    const wf::GSpin2Args g{a, Z, bar};
+    return H == 256 ? wf::launch_gspin2<256>(g, st, t) : wf::launch_gspin2<512>(g, st, t);
+  }
+  switch (H) {
+    case 16: return wf::launch_sample_spin2<16>(a, st, t);
+    case 32: return wf::launch_sample_spin2<32>(a, st, t);
+    case 64: return wf::launch_sample_spin2<64>(a, st, t);
+    case 128: return wf::launch_sample_spin2<128>(a, st, t);
+    case 256: return wf::launch_csample_spin2<256, 32>(a, st, t);
+    case 512: return wf::launch_csample_spin2<512, 32>(a, st, t);
+  }
+  return cudaErrorInvalidValue;
+}
+
 // the spin-2 messenger variance: the smaller of the two components' minima (statuses combined)
 __global__ void k_min_tau(wf::Scalars* a, const wf::Scalars* b, double tau_user) {
   if (threadIdx.x != 0 || blockIdx.x != 0) return;
@@ -1156,9 +1204,10 @@ wf_status wf_sample_spin2(const float* d1, const float* d2, const float* N1, con
     mask = r1.mask;
   }
   const size_t n = size_t(H) * W, nm = size_t(H) * (W / 2 + 1);
+  const Spin2Path path = spin2_path(H, o.n_chains);
   Carve cv;
-  const size_t o_sc = cv.take<wf::Scalars>(2), o_aq = cv.take<float2>(2 * n), o_fe = cv.take<float2>(nm),
-               o_fb = cv.take<float2>(nm);
+  const size_t o_sc = cv.take<wf::Scalars>(2), o_bar = cv.take<wf::GridBar>(1), o_aq = cv.take<float2>(2 * n),
+               o_fe = cv.take<float2>(nm), o_fb = cv.take<float2>(nm), o_z = cv.take<float2>(path.z_count);
   Scratch scr;
   scr.st = st;
   WF_CUDA(cudaMallocAsync(&scr.base, cv.off, st));
@@ -1173,9 +1222,7 @@ wf_status wf_sample_spin2(const float* d1, const float* d2, const float* N1, con
   WF_CUDA(launch_prep(d2, N2, mask, PB, H, W, o.tau, 0.5, sc + 1, st));
   k_min_tau<<<1, 32, 0, st>>>(sc, sc + 1, o.tau);
   WF_CUDA(cudaGetLastError());
-  // 256 and 512: both components of a chain in one thread-block cluster of 32-row CTAs, tables in the
-  // cluster kernels' orders
-  const int cm = size_on_chip(H) ? wf::core_cm(H) : 32, perm = size_on_chip(H) ? 0 : H / cm;
+  const int cm = path.cm, perm = path.perm;
   k_tables<<<int((n + nm + 255) / 256), 256, 0, st>>>(d1, N1, mask, PE, H, W, sc, aq, nullptr, fgE, perm, cm);
   k_tables<<<int((n + nm + 255) / 256), 256, 0, st>>>(d2, N2, mask, PB, H, W, sc, aq + n, nullptr, fgB, perm, cm);
   WF_CUDA(cudaGetLastError());
@@ -1187,20 +1234,17 @@ wf_status wf_sample_spin2(const float* d1, const float* d2, const float* N1, con
   a.key0 = uint32_t(seed & 0xffffffffu); a.key1 = uint32_t(seed >> 32);
   a.out_dtype = o.out_dtype;
   KernelTimer timer(st);
-  cudaError_t e = cudaSuccess;
-  switch (H) {
-    case 16: e = wf::launch_sample_spin2<16>(a, st, &timer); break;
-    case 32: e = wf::launch_sample_spin2<32>(a, st, &timer); break;
-    case 64: e = wf::launch_sample_spin2<64>(a, st, &timer); break;
-    case 128: e = wf::launch_sample_spin2<128>(a, st, &timer); break;
-    case 256: e = wf::launch_csample_spin2<256, 32>(a, st, &timer); break;
-    case 512: e = wf::launch_csample_spin2<512, 32>(a, st, &timer); break;
-  }
+  auto* bar = reinterpret_cast<wf::GridBar*>(b + o_bar);
+  WF_CUDA(cudaMemsetAsync(bar, 0, sizeof(wf::GridBar), st));
+  const cudaError_t e = launch_spin2_any(H, path, a, reinterpret_cast<float2*>(b + o_z), bar, st, &timer);
   if (e != cudaSuccess) return cuda_fail(e);
   wf::Scalars hsc;
+  wf::GridBar hb{};
   WF_CUDA(cudaMemcpyAsync(&hsc, sc, sizeof(hsc), cudaMemcpyDeviceToHost, st));
+  if (path.global) WF_CUDA(cudaMemcpyAsync(&hb, bar, sizeof(hb), cudaMemcpyDeviceToHost, st));
   WF_CUDA(cudaStreamSynchronize(st));
   timer.collect();
+  if (hsc.status == WF_OK && hb.err) return wf_status(hb.err);
   return wf_status(hsc.status);
 }
 
@@ -1225,7 +1269,7 @@ __global__ void k_s2_level_tables(const float* __restrict__ d, const float* __re
         w = nb / (nb + lt);
         a = (1.0 - w) * double(d[i]);
       }
-      aq[x * H + table_row(y, H, perm)] = make_float2(float(a), float(sqrt(w)));
+      aq[pixel_pos(y, x, H, W, perm)] = make_float2(float(a), float(sqrt(w)));
     } else {
       const int j = i - n;
       const double P = double(Pk[j]);
@@ -1269,8 +1313,10 @@ wf_status wf_solve_spin2(const float* d1, const float* d2, const float* N1, cons
   }
   const size_t n = size_t(H) * W, nm = size_t(H) * (W / 2 + 1);
   Carve cv;
-  const size_t o_sc = cv.take<wf::Scalars>(3), o_aq = cv.take<float2>(2 * n), o_fe = cv.take<float2>(nm),
-               o_fb = cv.take<float2>(nm), o_r = cv.take<double>(2), o_x = cv.take<double2>(2 * n);
+  const Spin2Path path = spin2_path(H, 1);
+  const size_t o_sc = cv.take<wf::Scalars>(3), o_bar = cv.take<wf::GridBar>(1), o_aq = cv.take<float2>(2 * n),
+               o_fe = cv.take<float2>(nm), o_fb = cv.take<float2>(nm), o_r = cv.take<double>(2),
+               o_x = cv.take<double2>(2 * n), o_z = cv.take<float2>(path.z_count);
   Scratch scr;
   scr.st = st;
   WF_CUDA(cudaMallocAsync(&scr.base, cv.off, st));
@@ -1301,8 +1347,10 @@ wf_status wf_solve_spin2(const float* d1, const float* d2, const float* N1, cons
   wf::Spin2Args a{};
   a.aq2 = aq; a.fgE = fgE; a.fgB = fgB; a.sc = sc + 2; a.init_s = out; a.init_stride = 0;
   a.out = out; a.n_samples = 1; a.n_chains = 1; a.burn_in = 0; a.thin = 1; a.out_dtype = 0;
-  // the sampler kernels' table orders
-  const int cm = size_on_chip(H) ? wf::core_cm(H) : 32, perm = size_on_chip(H) ? 0 : H / cm;
+  a.quiet = 1;
+  auto* bar = reinterpret_cast<wf::GridBar*>(b + o_bar);
+  WF_CUDA(cudaMemsetAsync(bar, 0, sizeof(wf::GridBar), st));
+  const int cm = path.cm, perm = path.perm;
   auto run = [&](double lam, int sweeps) -> wf_status {
     k_s2_level_tables<<<int((n + nm + 255) / 256), 256, 0, st>>>(d1, N1, mask, PE, H, W, sc, lam, aq, fgE, perm, cm);
     k_s2_level_tables<<<int((n + nm + 255) / 256), 256, 0, st>>>(d2, N2, mask, PB, H, W, sc, lam, aq + n, fgB, perm,
@@ -1310,15 +1358,7 @@ wf_status wf_solve_spin2(const float* d1, const float* d2, const float* N1, cons
     WF_CUDA(cudaGetLastError());
     a.n_sweeps = sweeps;
     a.thin = sweeps;  // the state after the last sweep is the only sample
-    cudaError_t e2 = cudaSuccess;
-    switch (H) {
-      case 16: e2 = wf::launch_sample_spin2<16>(a, st, nullptr); break;
-      case 32: e2 = wf::launch_sample_spin2<32>(a, st, nullptr); break;
-      case 64: e2 = wf::launch_sample_spin2<64>(a, st, nullptr); break;
-      case 128: e2 = wf::launch_sample_spin2<128>(a, st, nullptr); break;
-      case 256: e2 = wf::launch_csample_spin2<256, 32>(a, st, nullptr); break;
-      case 512: e2 = wf::launch_csample_spin2<512, 32>(a, st, nullptr); break;
-    }
+    const cudaError_t e2 = launch_spin2_any(H, path, a, reinterpret_cast<float2*>(b + o_z), bar, st, nullptr);
     if (e2 != cudaSuccess) return cuda_fail(e2);
     return WF_OK;
   };
@@ -1340,8 +1380,11 @@ wf_status wf_solve_spin2(const float* d1, const float* d2, const float* N1, cons
     e = wf::spin2_residual_f64(out, d1, d2, N1, N2, mask, PE, PB, H, W, false, rn, b + o_x, st);
     if (e != cudaSuccess) return cuda_fail(e);
     double h;
+    wf::GridBar hb{};
     WF_CUDA(cudaMemcpyAsync(&h, rn, sizeof(double), cudaMemcpyDeviceToHost, st));
+    if (path.global) WF_CUDA(cudaMemcpyAsync(&hb, bar, sizeof(hb), cudaMemcpyDeviceToHost, st));
     WF_CUDA(cudaStreamSynchronize(st));
+    if (hb.err) return wf_status(hb.err);
     rho = bnorm > 0.0 ? sqrt(h / bnorm) : sqrt(h);
     if (!(rho == rho)) { status = WF_ERR_NONFINITE; break; }
     if (rho < o.tol) { status = WF_OK; break; }

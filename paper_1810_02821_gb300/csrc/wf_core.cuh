@@ -402,7 +402,7 @@ __device__ __forceinline__ void kpairs(const KCol<N>& t, float2 (&p)[KGeo<N>::A]
 // pointwise updates on registers
 // ---------------------------------------------------------------------------------------------
 // t-draw (t_draw_staged): x[i BR + m], x[(i+1) BR + m] (i even) are the four pixels of group n / 2
-template <int N, int NF = 1>
+template <int N, int NF = 1, bool DRAW = true>
 __device__ __forceinline__ void kt_draw(float2 (&x)[KGeo<N>::E], const float2* __restrict__ aq,
                                         float sqrt_tau, uint32_t step, uint32_t chain, uint32_t k0, uint32_t k1,
                                         uint32_t stream) {
@@ -417,8 +417,8 @@ __device__ __forceinline__ void kt_draw(float2 (&x)[KGeo<N>::E], const float2* _
       const int n = 2 * a + G::A * m;  // pixel pair relative to the thread's first
       const float2 c0 = __ldg(tab + (2 * n) * G::H), c1 = __ldg(tab + (2 * n + 1) * G::H);
       const float2 c2 = __ldg(tab + (2 * n + 2) * G::H), c3 = __ldg(tab + (2 * n + 3) * G::H);
-      float z[4];
-      normals4(grp + uint32_t(n / 2), step, chain, stream, k0, k1, z);
+      float z[4] = {0.f, 0.f, 0.f, 0.f};
+      if (DRAW) normals4(grp + uint32_t(n / 2), step, chain, stream, k0, k1, z);
       float2& p0 = x[2 * a * G::BR + m];
       float2& p1 = x[(2 * a + 1) * G::BR + m];
       p0.x = fmaf(c0.y, fmaf(c0.y, p0.x, sqrt_tau * z[0]), c0.x);
@@ -839,7 +839,7 @@ __global__ void __launch_bounds__(KGeo<N>::T, kcore_min_ctas<N>()) k_mband(Sampl
 // first unit for both components, component 1's those led by the second (rotation into E and B, the two scalar
 // draws, rotation back, as spin2_interior and spin2_edge), and each thread reloads its own.
 // ---------------------------------------------------------------------------------------------
-template <int N>
+template <int N, bool DRAW>
 __device__ __forceinline__ void ks_draw_spin2(const KCol<N, 2>& t, float2 (&p)[KGeo<N>::A], float2 (&q)[KGeo<N>::A],
                                               const float2* __restrict__ fgE, const float2* __restrict__ fgB,
                                               uint32_t step, uint32_t chain, uint32_t k0, uint32_t k1) {
@@ -861,9 +861,11 @@ __device__ __forceinline__ void ks_draw_spin2(const KCol<N, 2>& t, float2 (&p)[K
       const int i1 = (A * lead + j) * SP + t.slot, i2 = (A * mate + A - 1 - j) * SP + t.slot;
       float2 a1 = c0[i1], b1 = c1[i1], a2 = c0[i2], b2 = c1[i2];
       const uint32_t grp = uint32_t(t.kx() * (G::H / 2) + ky1);
-      float zE[4], zB[4];
-      normals4(grp, step, chain, 1u, k0, k1, zE);
-      normals4(grp, step, chain, 9u, k0, k1, zB);
+      float zE[4] = {0.f, 0.f, 0.f, 0.f}, zB[4] = {0.f, 0.f, 0.f, 0.f};
+      if (DRAW) {
+        normals4(grp, step, chain, 1u, k0, k1, zE);
+        normals4(grp, step, chain, 9u, k0, k1, zB);
+      }
       const int m1 = ky1 * L + t.slot, m2 = ky2 * L + t.slot;
       float c, s;
       ks_rot<N>(ky1, t.kx(), c, s);
@@ -884,9 +886,11 @@ __device__ __forceinline__ void ks_draw_spin2(const KCol<N, 2>& t, float2 (&p)[K
     const int ky1 = el + G::BC * j, ky2 = ky1 == 0 ? G::H / 2 : G::H - ky1;
     const int i1 = (A * el + j) * SP, i2 = (A * em + A - 1 - j) * SP;
     float2 y1a = c0[i1], y2a = c0[i2], y1b = c1[i1], y2b = c1[i2];
-    float zE[4], zB[4];
-    normals4(uint32_t(ky1), step, chain, 1u, k0, k1, zE);
-    normals4(uint32_t(ky1), step, chain, 9u, k0, k1, zB);
+    float zE[4] = {0.f, 0.f, 0.f, 0.f}, zB[4] = {0.f, 0.f, 0.f, 0.f};
+    if (DRAW) {
+      normals4(uint32_t(ky1), step, chain, 1u, k0, k1, zE);
+      normals4(uint32_t(ky1), step, chain, 9u, k0, k1, zB);
+    }
     if (ky1 == 0) {
       // four real modes, each on k = 0 or a Nyquist line: no rotation, real draws with variance g^2
       constexpr float R2 = 1.41421356237309505f;
@@ -928,7 +932,8 @@ __device__ __forceinline__ void ks_draw_spin2(const KCol<N, 2>& t, float2 (&p)[K
 template <int N>
 constexpr int kspin2_smem() { return 2 * KGeo<N>::FIELD_BYTES + KGeo<N>::NTW * 8; }
 
-template <int N>
+// DRAW false (the shear Wiener filter): the draws are left out, their scales are zero
+template <int N, bool DRAW>
 __global__ void __launch_bounds__(2 * KGeo<N>::T, N == 64 ? 3 : (N == 32 ? 6 : 1)) k_mspin2(Spin2Args a) {
   using G = KGeo<N>;
   if (a.sc->status != 0) return;  // uniform over the grid
@@ -941,12 +946,12 @@ __global__ void __launch_bounds__(2 * KGeo<N>::T, N == 64 ? 3 : (N == 32 ? 6 : 1
   const int eb = out_elem_bytes(a.out_dtype);
   for (int done = 0; done < a.n_sweeps;) {
     const uint32_t step = a.step0 + uint32_t(done);
-    kt_draw<N, 2>(x, a.aq2 + (threadIdx.x / G::T) * n, a.sc->sqrt_tau, step, chain, a.key0, a.key1,
-                  8u * (threadIdx.x / G::T));
+    kt_draw<N, 2, DRAW>(x, a.aq2 + (threadIdx.x / G::T) * n, a.sc->sqrt_tau, step, chain, a.key0, a.key1,
+                        8u * (threadIdx.x / G::T));
     krow_fwd<N, 2>(x);
     __syncthreads();
     kcol<N, true, 2>([&](const KCol<N, 2>& t, float2 (&p)[G::A], float2 (&q)[G::A]) {
-      ks_draw_spin2<N>(t, p, q, a.fgE, a.fgB, step, chain, a.key0, a.key1);
+      ks_draw_spin2<N, DRAW>(t, p, q, a.fgE, a.fgB, step, chain, a.key0, a.key1);
     });
     __syncthreads();
     krow_inv<N, 2>(x);

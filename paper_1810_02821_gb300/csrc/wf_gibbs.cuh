@@ -1147,6 +1147,7 @@ struct Spin2Args {
   uint32_t step0;
   uint32_t key0, key1;
   int out_dtype;
+  int quiet;             // 1: no draws (every draw scale is zero: the shear Wiener filter)
 };
 
 template <int N, int FPC>

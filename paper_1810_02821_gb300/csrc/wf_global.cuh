@@ -424,7 +424,8 @@ __device__ __forceinline__ void grow_store(float2 (&x)[GGeo<N>::E], void* img, l
 
 // Pixel update of row y (pixel tables row-major):
 //   mode 0: sampler t-draw t = (1 - w) d + sqrt(w) (sqrt(w) s + sqrt(tau) xi) with the (a, q) table, Philox
-//           counter (pixel group (y W + x) / 4, step, chain, stream 0);
+//           counter (pixel group (y W + x) / 4, step, chain, stream);
+//   mode 4: its mean t = a + q^2 s (no draw);
 //   mode 1: Wiener-filter t-update t = w (s - d) + d, w = 1 / (1 + lambda tau / N_bar) from the (d, 1/N_bar)
 //           table (rhs_mode: t = w s + lambda tau r with r in place of d);
 //   mode 2: the level right-hand side N_lambda^-1 d with N_lambda = N_bar + lt2 (s ignored).
@@ -434,9 +435,9 @@ template <int N>
 __device__ __forceinline__ void pixel_update(int mode, float2 (&x)[GGeo<N>::E], int y, const float2* __restrict__ aq,
                                              const float2* __restrict__ dn, uint32_t step, uint32_t chain,
                                              uint32_t key0, uint32_t key1, float sqrt_tau, float ltau, int rhs_mode,
-                                             float lt2) {
+                                             float lt2, uint32_t stream = 0u) {
   using G = GGeo<N>;
-  const float4* tab = reinterpret_cast<const float4*>((mode == 0 ? aq : dn) + (long long)y * G::W);
+  const float4* tab = reinterpret_cast<const float4*>((mode == 0 || mode == 4 ? aq : dn) + (long long)y * G::W);
   if (mode == 0) {
     const int h = threadIdx.x % G::TR;
     auto upd = [&](float2& v, float4 c, float z0, float z1) {
@@ -449,7 +450,7 @@ __device__ __forceinline__ void pixel_update(int mode, float2 (&x)[GGeo<N>::E], 
         const int e = 2 * h + (G::LR / 8) * m;
         const float4 c0 = __ldg(tab + e), c1 = __ldg(tab + e + 1);
         float z[4];
-        normals4(uint32_t(y * (G::W / 4) + e / 2), step, chain, 0u, key0, key1, z);
+        normals4(uint32_t(y * (G::W / 4) + e / 2), step, chain, stream, key0, key1, z);
         upd(x[m], c0, z[0], z[1]);
         upd(x[8 + m], c1, z[2], z[3]);
       }
@@ -460,13 +461,19 @@ __device__ __forceinline__ void pixel_update(int mode, float2 (&x)[GGeo<N>::E], 
         const int e0 = h + (G::LR / 8) * i, e1 = h + (G::LR / 8) * (4 + i);
         const float4 c0 = __ldg(tab + e0), c1 = __ldg(tab + e1);
         float z[4];  // even lanes: the group of pair e0, odd lanes: that of e1
-        normals4(uint32_t(y * (G::W / 4) + (odd ? e1 : e0) / 2), step, chain, 0u, key0, key1, z);
+        normals4(uint32_t(y * (G::W / 4) + (odd ? e1 : e0) / 2), step, chain, stream, key0, key1, z);
         const float r0 = __shfl_xor_sync(0xffffffffu, odd ? z[0] : z[2], 1);
         const float r1 = __shfl_xor_sync(0xffffffffu, odd ? z[1] : z[3], 1);
         upd(x[i], c0, odd ? r0 : z[0], odd ? r1 : z[1]);
         upd(x[4 + i], c1, odd ? z[2] : r0, odd ? z[3] : r1);
       }
     }
+  } else if (mode == 4) {
+    gpixels<N>(x, [&](float2& v, int e) {
+      const float4 c = __ldg(tab + e);
+      v.x = fmaf(c.y, c.y * v.x, c.x);
+      v.y = fmaf(c.w, c.w * v.y, c.z);
+    });
   } else if (mode == 1) {
     const float g = rhs_mode ? 0.0f : 1.0f, hh = rhs_mode ? ltau : 1.0f;
     auto upd = [&](float& v, float dv, float inb) {

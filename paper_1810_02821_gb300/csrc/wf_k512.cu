@@ -6,4 +6,5 @@
 
 namespace wf {
 WF_INSTANTIATE_GLOBAL(512)
+WF_INSTANTIATE_GSPIN2(512)
 }  // namespace wf

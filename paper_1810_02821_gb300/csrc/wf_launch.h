@@ -11,6 +11,7 @@
 #include "wf_cluster_ext.cuh"
 #include "wf_bphase.cuh"
 #include "wf_core.cuh"
+#include "wf_gspin2.cuh"
 
 namespace wf {
 
@@ -61,6 +62,10 @@ cudaError_t launch_global(const GlobalArgs& a, cudaStream_t st, LaunchTimer* t);
 // batched large images (N >= 256): one cooperative launch of k_gbatch<N> over all fields of a size class
 template <int N>
 cudaError_t launch_gbatch(const GBArgs& a, cudaStream_t st);
+
+// spin-2 sampler with the fields in global memory (N in {256, 512}): one cooperative launch of k_gspin2<N>
+template <int N>
+cudaError_t launch_gspin2(const GSpin2Args& a, cudaStream_t st, LaunchTimer* t);
 
 // cluster-resident sampler (N in {256, 512}): one cluster of N / MR CTAs of MR rows each per chain
 // (MR = 64 at 256; 32 or 64 at 512). cudaErrorNotSupported when no cluster of that shape can be resident.
@@ -124,7 +129,8 @@ cudaError_t launch_sample_band(const SampleArgs& a, cudaStream_t st, LaunchTimer
 template <int N>
 cudaError_t launch_sample_spin2(const Spin2Args& a, cudaStream_t st, LaunchTimer* t) {
   if constexpr (core_size(N)) {
-    return launch_smem(k_mspin2<N>, a.n_chains, 2 * KGeo<N>::T, kspin2_smem<N>(), a, st, t);
+    return a.quiet ? launch_smem(k_mspin2<N, false>, a.n_chains, 2 * KGeo<N>::T, kspin2_smem<N>(), a, st, t)
+                   : launch_smem(k_mspin2<N, true>, a.n_chains, 2 * KGeo<N>::T, kspin2_smem<N>(), a, st, t);
   } else {
     constexpr int FPC = fields_per_cta<N>();  // images per CTA; two component fields each
     return launch_smem(k_sample_spin2<N, FPC>, (a.n_chains + FPC - 1) / FPC, 2 * N * FPC,
@@ -275,6 +281,29 @@ cudaError_t launch_gbatch(const GBArgs& a, cudaStream_t st) {
   if (e != cudaSuccess) return e;
   return cudaGetLastError();
 }
+template <int N>
+cudaError_t launch_gspin2(const GSpin2Args& a, cudaStream_t st, LaunchTimer* t) {
+  using G = GGeo<N>;
+  auto kern = a.s.quiet ? k_gspin2<N, false> : k_gspin2<N, true>;
+  const int smem = gspin2_smem<N>();
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  if (e != cudaSuccess) return e;
+  int dev = 0, sms = 0, per_sm = 0;
+  if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
+  if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
+  if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, G::T, smem)) != cudaSuccess) return e;
+  if (per_sm < 1) return cudaErrorInvalidConfiguration;
+  const long long items = (long long)(G::LR / 2) * a.s.n_chains;  // column items (more than row items)
+  const long long full = (long long)per_sm * sms;
+  GSpin2Args arg = a;
+  void* args[] = {&arg};
+  if (t) t->start();
+  e = cudaLaunchCooperativeKernel(reinterpret_cast<void*>(kern), dim3(unsigned(items < full ? items : full)),
+                                  dim3(G::T), args, smem, st);
+  if (t) t->stop();
+  return e != cudaSuccess ? e : cudaGetLastError();
+}
+#define WF_INSTANTIATE_GSPIN2(N) template cudaError_t launch_gspin2<N>(const GSpin2Args&, cudaStream_t, LaunchTimer*);
 #define WF_INSTANTIATE_GLOBAL(N)                                                               \
   template cudaError_t launch_global<N>(const GlobalArgs&, cudaStream_t, LaunchTimer*);         \
   template cudaError_t launch_gbatch<N>(const GBArgs&, cudaStream_t);

@@ -21,3 +21,23 @@ def test_chain_does_not_depend_on_the_chain_count(H, chains):
     for c in sorted({0, chains // 2, chains - 1}):
         one = wf.wf_sample_ex(*dev, seed=7, n_samples=2, n_chains=1, chain_offset=c, burn_in=2, thin=3)
         assert rel(many[c].cpu().numpy(), one[0].cpu().numpy()) < 2e-6, (H, chains, c)
+
+
+@pytest.mark.parametrize("H,chains", [(32, 3), (64, 2), (128, 2), (256, 23), (256, 24), (512, 2)])
+def test_shear_chain_does_not_depend_on_the_chain_count_or_path(H, chains):
+    """Both kernels of the spin-2 sampler draw the same chains (2e-6: FP32 rounding of either)."""
+    need_gpu()
+    build.build()
+    p = synth.make_problem(H, seed=H, mask_frac=0.1)
+    q = synth.make_problem(H, seed=H + 1, mask_frac=0.1)
+    d, N, m, P = to_dev(p)
+    d2, N2 = to_dev(q)[:2]
+    args = (d, d2, N, N2, m, P, (0.2 * P).contiguous())
+    many = wf.wf_sample_spin2(*args, seed=7, n_samples=2, n_chains=chains, burn_in=1, thin=2)
+    for mode in ("auto", "global", "cluster"):
+        prev = wf.wf_set_large_image_sampler(mode)
+        try:
+            one = wf.wf_sample_spin2(*args, seed=7, n_samples=2, chain_offset=chains - 1, burn_in=1, thin=2)
+        finally:
+            wf.wf_set_large_image_sampler(prev)
+        assert rel(many[chains - 1].cpu().numpy(), one[0].cpu().numpy()) < 2e-6, (H, chains, mode)
