@@ -182,7 +182,16 @@ cudaError_t launch_prep(const float* d, const float* Ndiag, const uint8_t* mask,
   return launch_prep_kernel(k_prep, 1, H, st, d, Ndiag, mask, Pk, H, W, tau_user, eta, sc);
 }
 
+constexpr int kFew128 = 36, kFewSpin2 = 40;  // chains from which the on-chip kernels run at 128^2
 bool size_on_chip(int H) { return H <= 128; }
+// Whether fields of an on-chip size run on the on-chip kernels, one CTA per field, or on the global-memory kernels, one
+// cooperative launch that spreads each field over 16 SMs. At 128^2 the latter has less latency for few fields (us per
+// sweep of all chains, global-memory / on-chip): sampler 1 chain 6.4 / 9.6, 16 chains 6.9 / 9.7, 32 chains 8.7 / 9.7,
+// 39 chains 10.1 / 9.7; spin-2 1 chain 7.6 / 22.9, 39 chains 20.6 / 22.9; a Wiener filter 6.8 / 8.0 (from zero only: the
+// global-memory solve takes no starting iterate).
+bool sample_on_chip(int H, int units) { return size_on_chip(H) && !(H == 128 && units < kFew128); }
+bool spin2_on_chip(int H, int units) { return size_on_chip(H) && !(H == 128 && units < kFewSpin2); }
+bool solve_on_chip(int H, bool from_zero) { return size_on_chip(H) && !(H == 128 && from_zero); }
 
 // Per-pixel tables ([W][H], x-major so that row threads read consecutive addresses) and the
 // per-mode sample table (table_pixel, table_mode: within 2 ulp of the exact coefficients).
@@ -194,8 +203,6 @@ __host__ __device__ inline int table_row(int y, int H, int perm) { return perm ?
 __host__ __device__ inline int pixel_pos(int y, int x, int H, int W, int perm) {
   return perm < 0 ? y * W + x : x * H + table_row(y, H, perm);
 }
-// order of the pixel tables of the solve kernels without a cluster: row-major above 128 x 128
-int solve_perm(int H) { return size_on_chip(H) ? 0 : -1; }
 
 // Position of half-spectrum entry j = ky (W/2 + 1) + kx in a mode table: natural (cm = 0), or the column slot
 // order of the cluster kernels with cm rows per CTA, and of the on-chip kernels with cm = core_cm(H) (kx < W/2 at ky W/2 + t, t = (kx mod cm) R + kx / cm,
@@ -333,6 +340,7 @@ bool out_ptr_ok(const void* p) {
 
 cudaError_t launch_global_any(int H, const wf::GlobalArgs& a, cudaStream_t st, wf::LaunchTimer* t) {
   switch (H) {
+    case 128: return wf::launch_global<128>(a, st, t);
     case 256: return wf::launch_global<256>(a, st, t);
     case 512: return wf::launch_global<512>(a, st, t);
     case 1024: return wf::launch_global<1024>(a, st, t);
@@ -466,7 +474,8 @@ wf_status sample_global(const float* d, const float* Ndiag, const uint8_t* mask,
 struct SolveSetup {
   const wf::Scalars* sc = nullptr;
   const float2* dn = nullptr;
-  const float* Pk = nullptr;  // P in the order of the size's solve kernel
+  const float* Pk = nullptr;  // P in the order of the solve kernel
+  bool chip = false;          // every solve on the on-chip kernels, else on the global-memory kernels
   wf::Scalars host{};
 };
 
@@ -677,7 +686,7 @@ wf_status solve_pass(const float* d, const float* Ndiag, const uint8_t* mask, co
                      const wf_solve_opts& o, float* out_s, int32_t* iters_out, double* resid_out, cudaStream_t st,
                      wf::LaunchTimer* timer, const float2* rhs_tab = nullptr, const double* rhs_norms = nullptr,
                      const SolveSetup* su = nullptr) {
-  if (!size_on_chip(H)) {
+  if (!(su ? su->chip : solve_on_chip(H, o.init_s == nullptr))) {
     if (o.init_s) return WF_ERR_ARG;  // the large-image solve starts from zero
     if (!rhs_tab && use_cluster(H, 1))
       return solve_cluster(d, Ndiag, mask, Pk, H, W, o, out_s, iters_out, resid_out, st, timer);
@@ -755,10 +764,11 @@ wf_status solve_refined(const float* d, const float* Ndiag, const uint8_t* mask,
   int32_t it = 0, total = 0;
   double rs = 0.0;
   const size_t n = size_t(H) * W, nm = size_t(H) * (W / 2 + 1);
+  const bool chip = solve_on_chip(H, o.init_s == nullptr);  // of the first solve; the corrections run the same kernels
   Carve cv;
   const size_t o_sc = cv.take<wf::Scalars>(1), o_dn = cv.take<float2>(n), o_rt = cv.take<float2>(n),
                o_e = cv.take<float>(n), o_nr = cv.take<double>(4),
-               o_pk = cv.take<float>(size_on_chip(H) ? nm : 0),
+               o_pk = cv.take<float>(chip ? nm : 0),
                o_fft = cv.take<char>(wf::refine_scratch_bytes(H, W));
   Scratch scr;
   scr.st = st;
@@ -769,13 +779,14 @@ wf_status solve_refined(const float* d, const float* Ndiag, const uint8_t* mask,
   SolveSetup su;
   su.sc = sc;
   su.dn = reinterpret_cast<float2*>(b + o_dn);
-  su.Pk = size_on_chip(H) ? reinterpret_cast<float*>(b + o_pk) : Pk;
+  su.Pk = chip ? reinterpret_cast<float*>(b + o_pk) : Pk;
+  su.chip = chip;
   WF_CUDA(launch_prep(d, Ndiag, mask, Pk, H, W, o.tau, o.eta, sc, st));
   k_tables<<<int((n + nm + 255) / 256), 256, 0, st>>>(
-      d, Ndiag, mask, Pk, H, W, sc, nullptr, reinterpret_cast<float2*>(b + o_dn), nullptr, solve_perm(H),
-      wf::core_cm(H), size_on_chip(H) ? reinterpret_cast<float*>(b + o_pk) : nullptr);
+      d, Ndiag, mask, Pk, H, W, sc, nullptr, reinterpret_cast<float2*>(b + o_dn), nullptr, chip ? 0 : -1,
+      wf::core_cm(H), chip ? reinterpret_cast<float*>(b + o_pk) : nullptr);
   WF_CUDA(cudaGetLastError());
-  if (!size_on_chip(H)) {
+  if (!chip) {
     WF_CUDA(cudaMemcpyAsync(&su.host, sc, sizeof(su.host), cudaMemcpyDeviceToHost, st));
     WF_CUDA(cudaStreamSynchronize(st));
   }
@@ -794,7 +805,7 @@ wf_status solve_refined(const float* d, const float* Ndiag, const uint8_t* mask,
   ra.s = out_s;
   ra.dn = reinterpret_cast<float2*>(b + o_dn);
   ra.rtab = reinterpret_cast<float2*>(b + o_rt);
-  ra.row_major = solve_perm(H) < 0;
+  ra.row_major = !chip;
   ra.rnorm = norms;
   ra.bnorm = norms + 1;
   ra.scratch = b + o_fft;
@@ -892,7 +903,7 @@ wf_status wf_sample_ex(const float* d, const float* Ndiag, const uint8_t* mask, 
   }
   // 256 and 512: one cluster per chain when the device can host the cluster, else the field in global memory
   const bool cluster = use_cluster(H, o.n_chains);
-  if (!size_on_chip(H) && !cluster) {
+  if (!sample_on_chip(H, o.n_chains) && !cluster) {
     KernelTimer gt(st);
     const wf_status r = sample_global(d, Ndiag, mask, Pk, H, W, seed, o, sweeps, out, st, &gt);
     gt.collect();
@@ -1135,9 +1146,9 @@ struct Spin2Path {
 };
 Spin2Path spin2_path(int H, int chains) {
   Spin2Path p;
-  if (size_on_chip(H)) {
+  if (spin2_on_chip(H, chains)) {
     p.cm = wf::core_cm(H);
-  } else if (spin2_use_cluster(H, chains)) {
+  } else if (H >= 256 && spin2_use_cluster(H, chains)) {
     p.cm = 32;
     p.perm = H / 32;
   } else {
@@ -1153,7 +1164,12 @@ cudaError_t launch_spin2_any(int H, const Spin2Path& p, const wf::Spin2Args& a, 
     const cudaError_t e = cudaMemsetAsync(&bar->count, 0, sizeof(bar->count), st);  // err collects over launches
     if (e != cudaSuccess) return e;
     const wf::GSpin2Args g{a, Z, bar};
-    return H == 256 ? wf::launch_gspin2<256>(g, st, t) : wf::launch_gspin2<512>(g, st, t);
+    switch (H) {
+      case 128: return wf::launch_gspin2<128>(g, st, t);
+      case 256: return wf::launch_gspin2<256>(g, st, t);
+      case 512: return wf::launch_gspin2<512>(g, st, t);
+    }
+    return cudaErrorInvalidValue;
   }
   switch (H) {
     case 16: return wf::launch_sample_spin2<16>(a, st, t);

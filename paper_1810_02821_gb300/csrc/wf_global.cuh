@@ -1,4 +1,5 @@
-// Messenger-field sweeps for images too large to keep a field in one SM (N in {256, 512, 1024}).
+// Messenger-field sweeps of fields in global memory: images too large for one SM (N in {256, 512, 1024}), and
+// few fields of 128^2, which one SM each would run with more latency.
 //
 // The packed half spectrum Z[H][W/2] of every field (kx = 0 and W/2 packed as re/im of column 0) lives in
 // global memory (L2-resident when the working set allows). One persistent cooperative kernel runs every
@@ -7,8 +8,8 @@
 //   column phase (CTA = 4 columns of one field): Z columns -> FFT -> s-draw -> inverse FFT -> Z
 // (Alg. 1 of the paper with A = I).
 //
-// Each transform of length n (rows W/2, columns H) is held by n/E threads of E = 2A elements (E = 8 at 256 and
-// 512, 16 at 1024) and runs in three or four in-place passes, n = 8 R2 [R3] A (decimation in frequency, L1 = n/8):
+// Each transform of length n (rows W/2, columns H) is held by n/E threads of E = 2A elements (E = 8 up to 512,
+// 16 at 1024: 8 there was 4% faster for one Wiener filter but 25% slower for several chains) and runs in three or four in-place passes, n = 8 R2 [R3] A (decimation in frequency, L1 = n/8):
 //   pass 1: 8-point DFTs over m of x[n0 + L1 m], output q1, times W_n^(n0 q1);
 //   middle: within each block of length Lb (L1 first), R-point DFTs over m of n1 + (Lb/R) m, output q2 (q3), times
 //           W_Lb^(n1 q2);

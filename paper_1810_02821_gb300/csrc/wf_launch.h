@@ -304,8 +304,9 @@ cudaError_t launch_gspin2(const GSpin2Args& a, cudaStream_t st, LaunchTimer* t) 
   return e != cudaSuccess ? e : cudaGetLastError();
 }
 #define WF_INSTANTIATE_GSPIN2(N) template cudaError_t launch_gspin2<N>(const GSpin2Args&, cudaStream_t, LaunchTimer*);
+#define WF_INSTANTIATE_GLOBAL_ONE(N) template cudaError_t launch_global<N>(const GlobalArgs&, cudaStream_t, LaunchTimer*);
 #define WF_INSTANTIATE_GLOBAL(N)                                                               \
-  template cudaError_t launch_global<N>(const GlobalArgs&, cudaStream_t, LaunchTimer*);         \
+  WF_INSTANTIATE_GLOBAL_ONE(N)                                                                  \
   template cudaError_t launch_gbatch<N>(const GBArgs&, cudaStream_t);
 #endif
 

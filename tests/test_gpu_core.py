@@ -8,7 +8,7 @@ from paper_1810_02821_gb300 import build, synth, wf
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("H,chains", [(32, 1), (32, 67), (64, 1), (64, 760), (64, 761), (64, 1217), (128, 305), (256, 399),
+@pytest.mark.parametrize("H,chains", [(32, 1), (32, 67), (64, 1), (64, 760), (64, 761), (64, 1217), (128, 35), (128, 36), (128, 305), (256, 399),
                                       (256, 400), (512, 9)])
 def test_chain_does_not_depend_on_the_chain_count(H, chains):
     """Chain c of a call with many chains equals the call for that chain alone. Each kernel is within 5e-7
@@ -23,7 +23,7 @@ def test_chain_does_not_depend_on_the_chain_count(H, chains):
         assert rel(many[c].cpu().numpy(), one[0].cpu().numpy()) < 2e-6, (H, chains, c)
 
 
-@pytest.mark.parametrize("H,chains", [(32, 3), (64, 2), (128, 2), (256, 23), (256, 24), (512, 2)])
+@pytest.mark.parametrize("H,chains", [(32, 3), (64, 2), (128, 39), (128, 40), (256, 23), (256, 24), (512, 2)])
 def test_shear_chain_does_not_depend_on_the_chain_count_or_path(H, chains):
     """Both kernels of the spin-2 sampler draw the same chains (2e-6: FP32 rounding of either)."""
     need_gpu()
@@ -41,3 +41,16 @@ def test_shear_chain_does_not_depend_on_the_chain_count_or_path(H, chains):
         finally:
             wf.wf_set_large_image_sampler(prev)
         assert rel(many[chains - 1].cpu().numpy(), one[0].cpu().numpy()) < 2e-6, (H, chains, mode)
+
+
+def test_128_filter_starts_on_either_path():
+    """A 128 x 128 filter from zero runs on the global-memory kernels, one with a starting iterate on chip: both reach
+    the same map (to the refined tolerance, 1e-7 of the right-hand side in the residual norm)."""
+    need_gpu()
+    build.build()
+    p = synth.config_paper128(3)
+    dev = to_dev(p)
+    r0 = wf.wf_solve_ex(*dev, tol=1e-7, refine=8)
+    r1 = wf.wf_solve_ex(*dev, tol=1e-7, refine=8, init_s=(0.5 * dev[0]).contiguous())
+    assert r0.resid < 1e-7 and r1.resid < 1e-7
+    assert rel(r0.s.cpu().numpy(), r1.s.cpu().numpy()) < 1e-5
