@@ -933,12 +933,13 @@ wf_status wf_sample_ex(const float* d, const float* Ndiag, const uint8_t* mask, 
   a.out_dtype = o.out_dtype;
   a.cm = sample_cm(H, o.n_chains);
   KernelTimer timer(st);
+  int timeout = 0;
   cudaError_t e = cudaSuccess;
   switch (H) {
-    case 16: e = wf::launch_sample<16>(a, st, &timer); break;
-    case 32: e = wf::launch_sample<32>(a, st, &timer); break;
-    case 64: e = wf::launch_sample<64>(a, st, &timer); break;
-    case 128: e = wf::launch_sample<128>(a, st, &timer); break;
+    case 16: e = wf::launch_sample<16>(a, st, &timer, &timeout); break;
+    case 32: e = wf::launch_sample<32>(a, st, &timer, &timeout); break;
+    case 64: e = wf::launch_sample<64>(a, st, &timer, &timeout); break;
+    case 128: e = wf::launch_sample<128>(a, st, &timer, &timeout); break;
     case 256:
     case 512: e = launch_csample_any(H, cluster_rows_of(H, 0), a, st, &timer); break;
   }
@@ -947,6 +948,7 @@ wf_status wf_sample_ex(const float* d, const float* Ndiag, const uint8_t* mask, 
   WF_CUDA(cudaMemcpyAsync(&hsc, sc, sizeof(hsc), cudaMemcpyDeviceToHost, st));
   WF_CUDA(cudaStreamSynchronize(st));
   timer.collect();
+  if (hsc.status == WF_OK && timeout) return wf_status(timeout);
   return wf_status(hsc.status);
 }
 
@@ -1118,12 +1120,13 @@ wf_status wf_sample_band(const float* d, const float* Ndiag, const uint8_t* mask
   a.band_map = bmap; a.band_off = band_off; a.band_lo = band_lo;
   a.band_buf = reinterpret_cast<float2*>(b + off_buf); a.band_clusters = n_cl;
   KernelTimer timer(st);
+  int timeout = 0;
   cudaError_t e = cudaSuccess;
   switch (H) {
-    case 16: e = wf::launch_sample_band<16>(a, st, &timer); break;
-    case 32: e = wf::launch_sample_band<32>(a, st, &timer); break;
-    case 64: e = wf::launch_sample_band<64>(a, st, &timer); break;
-    case 128: e = wf::launch_sample_band<128>(a, st, &timer); break;
+    case 16: e = wf::launch_sample_band<16>(a, st, &timer, &timeout); break;
+    case 32: e = wf::launch_sample_band<32>(a, st, &timer, &timeout); break;
+    case 64: e = wf::launch_sample_band<64>(a, st, &timer, &timeout); break;
+    case 128: e = wf::launch_sample_band<128>(a, st, &timer, &timeout); break;
     case 256: e = wf::launch_csample_band<256, 64>(a, st, &timer); break;
     case 512: e = wf::launch_csample_band<512, 32>(a, st, &timer); break;
   }
@@ -1132,6 +1135,7 @@ wf_status wf_sample_band(const float* d, const float* Ndiag, const uint8_t* mask
   WF_CUDA(cudaMemcpyAsync(&hsc, sc, sizeof(hsc), cudaMemcpyDeviceToHost, st));
   WF_CUDA(cudaStreamSynchronize(st));
   timer.collect();
+  if (hsc.status == WF_OK && timeout) return wf_status(timeout);
   return wf_status(hsc.status);
 }
 
@@ -1159,7 +1163,7 @@ Spin2Path spin2_path(int H, int chains) {
   return p;
 }
 cudaError_t launch_spin2_any(int H, const Spin2Path& p, const wf::Spin2Args& a, float2* Z, wf::GridBar* bar,
-                             cudaStream_t st, wf::LaunchTimer* t) {
+                             cudaStream_t st, wf::LaunchTimer* t, int* timeout) {
   if (p.global) {
     const cudaError_t e = cudaMemsetAsync(&bar->count, 0, sizeof(bar->count), st);  // err collects over launches
     if (e != cudaSuccess) return e;
@@ -1172,10 +1176,10 @@ cudaError_t launch_spin2_any(int H, const Spin2Path& p, const wf::Spin2Args& a, 
     return cudaErrorInvalidValue;
   }
   switch (H) {
-    case 16: return wf::launch_sample_spin2<16>(a, st, t);
-    case 32: return wf::launch_sample_spin2<32>(a, st, t);
-    case 64: return wf::launch_sample_spin2<64>(a, st, t);
-    case 128: return wf::launch_sample_spin2<128>(a, st, t);
+    case 16: return wf::launch_sample_spin2<16>(a, st, t, timeout);
+    case 32: return wf::launch_sample_spin2<32>(a, st, t, timeout);
+    case 64: return wf::launch_sample_spin2<64>(a, st, t, timeout);
+    case 128: return wf::launch_sample_spin2<128>(a, st, t, timeout);
     case 256: return wf::launch_csample_spin2<256, 32>(a, st, t);
     case 512: return wf::launch_csample_spin2<512, 32>(a, st, t);
   }
@@ -1252,7 +1256,8 @@ wf_status wf_sample_spin2(const float* d1, const float* d2, const float* N1, con
   KernelTimer timer(st);
   auto* bar = reinterpret_cast<wf::GridBar*>(b + o_bar);
   WF_CUDA(cudaMemsetAsync(bar, 0, sizeof(wf::GridBar), st));
-  const cudaError_t e = launch_spin2_any(H, path, a, reinterpret_cast<float2*>(b + o_z), bar, st, &timer);
+  int timeout = 0;
+  const cudaError_t e = launch_spin2_any(H, path, a, reinterpret_cast<float2*>(b + o_z), bar, st, &timer, &timeout);
   if (e != cudaSuccess) return cuda_fail(e);
   wf::Scalars hsc;
   wf::GridBar hb{};
@@ -1261,6 +1266,7 @@ wf_status wf_sample_spin2(const float* d1, const float* d2, const float* N1, con
   WF_CUDA(cudaStreamSynchronize(st));
   timer.collect();
   if (hsc.status == WF_OK && hb.err) return wf_status(hb.err);
+  if (hsc.status == WF_OK && timeout) return wf_status(timeout);
   return wf_status(hsc.status);
 }
 
@@ -1367,6 +1373,7 @@ wf_status wf_solve_spin2(const float* d1, const float* d2, const float* N1, cons
   auto* bar = reinterpret_cast<wf::GridBar*>(b + o_bar);
   WF_CUDA(cudaMemsetAsync(bar, 0, sizeof(wf::GridBar), st));
   const int cm = path.cm, perm = path.perm;
+  int timeout = 0;  // one chain: never a balanced launch
   auto run = [&](double lam, int sweeps) -> wf_status {
     k_s2_level_tables<<<int((n + nm + 255) / 256), 256, 0, st>>>(d1, N1, mask, PE, H, W, sc, lam, aq, fgE, perm, cm);
     k_s2_level_tables<<<int((n + nm + 255) / 256), 256, 0, st>>>(d2, N2, mask, PB, H, W, sc, lam, aq + n, fgB, perm,
@@ -1374,7 +1381,7 @@ wf_status wf_solve_spin2(const float* d1, const float* d2, const float* N1, cons
     WF_CUDA(cudaGetLastError());
     a.n_sweeps = sweeps;
     a.thin = sweeps;  // the state after the last sweep is the only sample
-    const cudaError_t e2 = launch_spin2_any(H, path, a, reinterpret_cast<float2*>(b + o_z), bar, st, nullptr);
+    const cudaError_t e2 = launch_spin2_any(H, path, a, reinterpret_cast<float2*>(b + o_z), bar, st, nullptr, &timeout);
     if (e2 != cudaSuccess) return cuda_fail(e2);
     return WF_OK;
   };
@@ -2801,10 +2808,10 @@ wf_status wf_sample_noalloc(const float* d, const float* Ndiag, const uint8_t* m
   a.cm = sample_cm(H, o.n_chains);
   cudaError_t e = cudaSuccess;
   switch (H) {
-    case 16: e = wf::launch_sample<16>(a, st, nullptr); break;
-    case 32: e = wf::launch_sample<32>(a, st, nullptr); break;
-    case 64: e = wf::launch_sample<64>(a, st, nullptr); break;
-    case 128: e = wf::launch_sample<128>(a, st, nullptr); break;
+    case 16: e = wf::launch_sample<16>(a, st, nullptr, nullptr); break;
+    case 32: e = wf::launch_sample<32>(a, st, nullptr, nullptr); break;
+    case 64: e = wf::launch_sample<64>(a, st, nullptr, nullptr); break;
+    case 128: e = wf::launch_sample<128>(a, st, nullptr, nullptr); break;
   }
   if (e != cudaSuccess) return cuda_fail(e);
   wf::Scalars hsc;

@@ -645,8 +645,8 @@ __device__ __forceinline__ float ks_p2(const KCol<N>& t, float2 (&p)[KGeo<N>::A]
 // field input and output
 // ---------------------------------------------------------------------------------------------
 // the thread's pixel pairs of a row-major [H][W] image (nullptr: zeros), through the field buffer so that the
-// loads coalesce
-template <int N, int NF = 1>
+// loads coalesce; NC false: an image that another CTA wrote during this launch
+template <int N, int NF = 1, bool NC = true>
 __device__ __forceinline__ void kload(float2 (&x)[KGeo<N>::E], const float* src) {
   using G = KGeo<N>;
   if (src == nullptr) {
@@ -656,7 +656,8 @@ __device__ __forceinline__ void kload(float2 (&x)[KGeo<N>::E], const float* src)
   }
   const KField<N, NF> k;
   for (int e = k.lt; e < G::H * G::L; e += G::T)
-    k.S()[(e / G::L) * G::SP + e % G::L] = __ldg(reinterpret_cast<const float2*>(src) + e);
+    k.S()[(e / G::L) * G::SP + e % G::L] =
+        NC ? __ldg(reinterpret_cast<const float2*>(src) + e) : __ldcg(reinterpret_cast<const float2*>(src) + e);
   __syncthreads();
   const KRow<N, NF> t;
   const float2* row = t.row + t.h * G::NR;
@@ -689,17 +690,17 @@ __device__ __forceinline__ void kstore(const float2 (&x)[KGeo<N>::E], void* out,
   __syncthreads();
 }
 
-// Sampler sweeps from the state in x. Per sweep: t-draw, forward rows, column transforms around the s-draw,
-// inverse rows; post() after the column barrier (the band draw), emit(m) after sample m has been stored to
+// Sampler sweeps d0 .. d1 - 1 of a chain from the state in x. Per sweep: t-draw, forward rows, column transforms
+// around the s-draw, inverse rows; post() after the column barrier (the band draw), emit(m) after sample m has been stored to
 // out + m H W elements (CTA barriers before and after the store).
 template <int N, class C, class Post, class Emit>
 __device__ __forceinline__ void ksweeps(float2 (&x)[KGeo<N>::E], const float2* __restrict__ aq,
                                         const C& cf, float sqrt_tau, uint32_t step0, uint32_t chain, uint32_t k0,
-                                        uint32_t k1, int n_sweeps, int burn_in, int thin, void* out, int ot,
+                                        uint32_t k1, int d0, int d1, int burn_in, int thin, void* out, int ot,
                                         Post&& post, Emit&& emit) {
   using G = KGeo<N>;
   const int eb = out_elem_bytes(ot);
-  for (int done = 0; done < n_sweeps;) {
+  for (int done = d0; done < d1;) {
     const uint32_t step = step0 + uint32_t(done);
     kt_draw<N>(x, aq, sqrt_tau, step, chain, k0, k1, 0u);
     krow_fwd<N>(x);
@@ -717,24 +718,144 @@ __device__ __forceinline__ void ksweeps(float2 (&x)[KGeo<N>::E], const float2* _
   }
 }
 
+// ---------------------------------------------------------------------------------------------
+// Balanced chains. With one CTA per chain, a few chains more than fit at once cost another whole round (200 shear
+// pairs on 152 SMs: two rounds of 22.9 us a sweep). Here as many CTAs as are resident take equal shares of all chains'
+// sweeps, laid end to end: CTA i runs sweeps [i W / R, (i + 1) W / R) of the W in all. A share starts and ends inside a
+// chain. The CTA runs the start of its last chain first and hands the state over, then its whole chains, and the rest
+// of its first chain last, from the state that CTA i - 1 handed over at the start of the launch: nobody waits in
+// practice, and the wait is bounded (cooperative launch: all CTAs are resident). A share is at least as long as a chain,
+// so a chain has at most two parts, and the first ends before the second starts. Measured at 128^2, us per sweep of all
+// chains: 200 shear pairs 45.8 -> 30.8; scalar 350 chains 27 -> 20.4, 1000 chains 59.0 -> 57.8.
+// ---------------------------------------------------------------------------------------------
+struct KBalance {
+  int shares;         // R: CTAs of the launch; 0: one CTA per chain
+  float* slot;        // [R][slot_floats] states handed over
+  int slot_floats;
+  unsigned int* flag; // [R] 1 once slot i is complete; zeroed before the launch
+  int* err;           // set to WF_ERR_TIMEOUT when a wait gives up; zeroed before the launch
+};
+// part `s` of CTA `i`: sweeps [d0, d1) of chain c; save: hand the state over; load: start from the state handed over
+struct KPart {
+  long long c;
+  int d0, d1;
+  bool load, save;
+};
+// false: no such part
+WF_HD bool kpart_of(int i, int s, int shares, long long n_chains, int n_sweeps, KPart* p) {
+  if (shares == 0) {
+    *p = KPart{i, 0, n_sweeps, false, false};
+    return s == 0;
+  }
+  const long long S = n_sweeps, W = n_chains * S;
+  // i W / R without overflow: W may be close to 2^62
+  const long long q = W / shares, r = W % shares;
+  const long long a = q * i + r * i / shares, b = q * (i + 1) + r * (i + 1) / shares;
+  const int head = int(b % S), tail = int(a % S);
+  if (head > 0) {
+    if (s == 0) {
+      *p = KPart{b / S, 0, head, false, true};
+      return true;
+    }
+    --s;
+  }
+  const long long first = (a + S - 1) / S, whole = b / S - first;
+  if (s < whole) {
+    *p = KPart{first + s, 0, n_sweeps, false, false};
+    return true;
+  }
+  *p = KPart{a / S, tail, n_sweeps, true, false};
+  return s == whole && tail > 0;
+}
+// the CTA's part s, formed by one thread in shared memory (read from there where it is needed: the sweeps' registers
+// are full); CTA barriers on both sides
+struct KPartShared {
+  KPart p;
+  int more;
+};
+__device__ __forceinline__ KPartShared& kpart_shared() {
+  __shared__ KPartShared sp;
+  return sp;
+}
+__device__ __forceinline__ bool knext_part(int s, const KBalance& bal, int n_chains, int n_sweeps) {
+  KPartShared& sp = kpart_shared();
+  __syncthreads();
+  if (threadIdx.x == 0) sp.more = kpart_of(blockIdx.x, s, bal.shares, n_chains, n_sweeps, &sp.p);
+  __syncthreads();
+  return sp.more != 0;
+}
+// the state in slot i is complete (all threads of the CTA have stored; called by all)
+__device__ __forceinline__ void kpublish(const KBalance& b, int i) {
+  __syncthreads();
+  if (threadIdx.x == 0)
+    asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(b.flag + i), "r"(1u) : "memory");
+}
+// waits for slot i (2^22 polls at most); false: gave up
+__device__ __forceinline__ bool kawait(const KBalance& b, int i) {
+  __shared__ int s_ok;
+  if (threadIdx.x == 0) {
+    unsigned int v = 0;
+    for (long it = 0; v == 0 && it < (1L << 22); ++it)
+      asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(b.flag + i) : "memory");
+    if (v == 0) atomicExch(b.err, 7);  // WF_ERR_TIMEOUT
+    s_ok = v != 0;
+  }
+  __syncthreads();
+  return s_ok != 0;
+}
+
+// CTA i's chain in a launch of one CTA per chain: nothing is handed over, and the compiler sees that
+struct KWhole {
+  long long c;
+  int d1;
+  static constexpr int d0 = 0;
+  static constexpr bool load = false, save = false;
+};
+// f(part) for the CTA's parts in order, until one returns false. BAL is a template parameter: with run-time parts the
+// 64-register kernels spill 28 (sampler) to 230 bytes, 1.5% of the band sampler's time
+template <bool BAL, class F>
+__device__ __forceinline__ void kparts(const KBalance& bal, int n_chains, int n_sweeps, F&& f) {
+  if constexpr (BAL) {
+    const volatile KPart& p = kpart_shared().p;
+    for (int s = 0; knext_part(s, bal, n_chains, n_sweeps); ++s)
+      if (!f(p)) return;
+  } else {
+    f(KWhole{blockIdx.x, n_sweeps});
+  }
+}
+
 // resident CTAs the kernels are compiled for: 64 registers a thread at 128^2 (two fields of 67 KB and 16 warps an
 // SM); at 64^2 and 32^2 five and ten CTAs with up to 96 registers measured as fast as eight and sixteen with 64
 // (the SM is bound by dispatch), and faster for a single chain (64^2: 4.5 -> 4.1 us per sweep)
 template <int N>
 constexpr int kcore_min_ctas() { return N == 64 ? 5 : (N == 32 ? 10 : 2); }
 
-template <int N>
-__global__ void __launch_bounds__(KGeo<N>::T, kcore_min_ctas<N>()) k_msample(SampleArgs a) {
+template <int N, class Part>
+__device__ __forceinline__ bool ksample_part(const SampleArgs& a, const KBalance& bal, const Part& p) {
   using G = KGeo<N>;
+  float2 x[G::E];
+  if (p.load) {
+    if (!kawait(bal, blockIdx.x - 1)) return false;
+    kload<N, 1, false>(x, bal.slot + (blockIdx.x - 1LL) * bal.slot_floats);
+  } else {
+    kload<N>(x, a.init_s ? a.init_s + p.c * a.init_stride : nullptr);
+  }
+  ksweeps<N>(x, a.aq, KTabCoef{a.fg}, a.sc->sqrt_tau, a.step0, a.chain0 + uint32_t(p.c), a.key0, a.key1, p.d0, p.d1,
+             a.burn_in, a.thin,
+             reinterpret_cast<char*>(a.out) + p.c * a.n_samples * (long long)(G::H * G::W) * out_elem_bytes(a.out_dtype),
+             a.out_dtype, [] {}, [](long long) {});
+  if (p.save) {
+    kstore<N>(x, bal.slot + (long long)blockIdx.x * bal.slot_floats, kOutF32);
+    kpublish(bal, blockIdx.x);
+  }
+  return true;
+}
+template <int N, bool BAL>
+__global__ void __launch_bounds__(KGeo<N>::T, kcore_min_ctas<N>()) k_msample(const __grid_constant__ SampleArgs a,
+                                                                            const __grid_constant__ KBalance bal) {
   if (a.sc->status != 0) return;  // uniform over the grid
   ktw_init<N>();
-  const long long ci = blockIdx.x;
-  float2 x[G::E];
-  kload<N>(x, a.init_s ? a.init_s + ci * a.init_stride : nullptr);
-  ksweeps<N>(x, a.aq, KTabCoef{a.fg}, a.sc->sqrt_tau, a.step0, a.chain0 + uint32_t(ci), a.key0, a.key1, a.n_sweeps,
-             a.burn_in, a.thin,
-             reinterpret_cast<char*>(a.out) + ci * a.n_samples * (long long)(G::H * G::W) * out_elem_bytes(a.out_dtype),
-             a.out_dtype, [] {}, [](long long) {});
+  kparts<BAL>(bal, a.n_chains, a.n_sweeps, [&](const auto& p) { return ksample_part<N>(a, bal, p); });
 }
 
 // every image's chain from its s_W (images whose set-up failed write nothing)
@@ -746,7 +867,7 @@ __global__ void __launch_bounds__(KGeo<N>::T, kcore_min_ctas<N>()) k_mbsample(BS
   ktw_init<N>();
   float2 x[G::E];
   kload<N>(x, fd.out_wf);
-  ksweeps<N>(x, fd.aq, KTabCoef{fd.fg}, a.sc[blockIdx.x].sqrt_tau, 0u, fd.chain, fd.key0, fd.key1, a.n_samples, 0, 1,
+  ksweeps<N>(x, fd.aq, KTabCoef{fd.fg}, a.sc[blockIdx.x].sqrt_tau, 0u, fd.chain, fd.key0, fd.key1, 0, a.n_samples, 0, 1,
              fd.out_samples, kOutF32, [] {}, [](long long) {});
 }
 
@@ -802,10 +923,11 @@ __device__ __forceinline__ void kband_update(const float2* __restrict__ buf, con
 }
 
 // The hierarchical sampler: the per-band draw coefficients [n_bins] float2 and band powers [n_bins] floats follow
-// the field; one bin-ordered statistics buffer per chain. The band draw runs after the column barrier; its
+// the field; one bin-ordered statistics buffer per CTA. The band draw runs after the column barrier; its
 // results are read after the next one.
-template <int N>
-__global__ void __launch_bounds__(KGeo<N>::T, kcore_min_ctas<N>()) k_mband(SampleArgs a) {
+template <int N, bool BAL>
+__global__ void __launch_bounds__(KGeo<N>::T, kcore_min_ctas<N>()) k_mband(const __grid_constant__ SampleArgs a,
+                                                                          const __grid_constant__ KBalance bal) {
   using G = KGeo<N>;
   if (a.sc->status != 0) return;  // uniform over the grid
   ktw_init<N>();
@@ -813,24 +935,41 @@ __global__ void __launch_bounds__(KGeo<N>::T, kcore_min_ctas<N>()) k_mband(Sampl
   float* Pb = reinterpret_cast<float*>(cb + a.n_bins);
   const float tau = float(a.sc->tau);
   constexpr float NPIX = float(G::H * G::W);
-  for (int b = threadIdx.x; b < a.n_bins; b += G::T) {
-    Pb[b] = a.P0[b];
-    cb[b] = band_coef(a.P0[b], tau, 1.0f / NPIX);
-  }
-  const long long ci = blockIdx.x;
-  float2* buf = a.band_buf + ci * (a.n_bins > 0 ? a.band_off[a.n_bins] : 0);
-  __syncthreads();
-  float2 x[G::E];
-  kload<N>(x, a.init_s ? a.init_s + ci * a.init_stride : nullptr);
-  float* outP = a.out_P ? a.out_P + ci * a.n_samples * (long long)a.n_bins : nullptr;
-  ksweeps<N>(x, a.aq, KBandCoef{a.fg, a.band_map, cb, buf, NPIX}, a.sc->sqrt_tau, a.step0, a.chain0 + uint32_t(ci),
-             a.key0, a.key1, a.n_sweeps, a.burn_in, a.thin,
-             reinterpret_cast<char*>(a.out) + ci * a.n_samples * (long long)(G::H * G::W) * out_elem_bytes(a.out_dtype),
-             a.out_dtype, [&] { kband_update<G::T>(buf, a.band_off, a.n_bins, cb, Pb, tau, 1.0f / NPIX); },
-             [&](long long m) {
-               if (outP)
-                 for (int b = threadIdx.x; b < a.n_bins; b += G::T) outP[m * a.n_bins + b] = Pb[b];
-             });
+  // one statistics buffer per CTA
+  float2* buf = a.band_buf + (long long)blockIdx.x * (a.n_bins > 0 ? a.band_off[a.n_bins] : 0);
+  kparts<BAL>(bal, a.n_chains, a.n_sweeps, [&](const auto& p) {
+    float2 x[G::E];
+    const float* P = a.P0;  // the part's band powers
+    if (p.load) {
+      if (!kawait(bal, blockIdx.x - 1)) return false;
+      P = bal.slot + (blockIdx.x - 1LL) * bal.slot_floats + G::H * G::W;
+    }
+    for (int b = threadIdx.x; b < a.n_bins; b += G::T) {
+      const float v = __ldcg(P + b);
+      Pb[b] = v;
+      cb[b] = band_coef(v, tau, 1.0f / NPIX);
+    }
+    __syncthreads();
+    if (p.load) kload<N, 1, false>(x, bal.slot + (blockIdx.x - 1LL) * bal.slot_floats);
+    else kload<N>(x, a.init_s ? a.init_s + p.c * a.init_stride : nullptr);
+    float* outP = a.out_P ? a.out_P + p.c * a.n_samples * (long long)a.n_bins : nullptr;
+    ksweeps<N>(x, a.aq, KBandCoef{a.fg, a.band_map, cb, buf, NPIX}, a.sc->sqrt_tau, a.step0, a.chain0 + uint32_t(p.c),
+               a.key0, a.key1, p.d0, p.d1, a.burn_in, a.thin,
+               reinterpret_cast<char*>(a.out) +
+                   p.c * a.n_samples * (long long)(G::H * G::W) * out_elem_bytes(a.out_dtype),
+               a.out_dtype, [&] { kband_update<G::T>(buf, a.band_off, a.n_bins, cb, Pb, tau, 1.0f / NPIX); },
+               [&](long long m) {
+                 if (outP)
+                   for (int b = threadIdx.x; b < a.n_bins; b += G::T) outP[m * a.n_bins + b] = Pb[b];
+               });
+    if (p.save) {
+      float* slot = bal.slot + (long long)blockIdx.x * bal.slot_floats;
+      kstore<N>(x, slot, kOutF32);  // its barriers order the last band draw before the reads below
+      for (int b = threadIdx.x; b < a.n_bins; b += G::T) slot[G::H * G::W + b] = Pb[b];
+      kpublish(bal, blockIdx.x);
+    }
+    return true;
+  });
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -933,35 +1072,47 @@ template <int N>
 constexpr int kspin2_smem() { return 2 * KGeo<N>::FIELD_BYTES + KGeo<N>::NTW * 8; }
 
 // DRAW false (the shear Wiener filter): the draws are left out, their scales are zero
-template <int N, bool DRAW>
-__global__ void __launch_bounds__(2 * KGeo<N>::T, N == 64 ? 3 : (N == 32 ? 6 : 1)) k_mspin2(Spin2Args a) {
+template <int N, bool DRAW, bool BAL>
+__global__ void __launch_bounds__(2 * KGeo<N>::T, N == 64 ? 3 : (N == 32 ? 6 : 1)) k_mspin2(
+    const __grid_constant__ Spin2Args a, const __grid_constant__ KBalance bal) {
   using G = KGeo<N>;
   if (a.sc->status != 0) return;  // uniform over the grid
   ktw_init<N, 2>();
-  const int comp = threadIdx.x / G::T;
-  const long long ci = blockIdx.x, n = G::H * G::W;
-  float2 x[G::E];
-  kload<N, 2>(x, a.init_s ? a.init_s + ci * a.init_stride + comp * n : nullptr);
-  const uint32_t chain = a.chain0 + uint32_t(ci);
+  constexpr long long n = G::H * G::W;
   const int eb = out_elem_bytes(a.out_dtype);
-  for (int done = 0; done < a.n_sweeps;) {
-    const uint32_t step = a.step0 + uint32_t(done);
-    kt_draw<N, 2, DRAW>(x, a.aq2 + (threadIdx.x / G::T) * n, a.sc->sqrt_tau, step, chain, a.key0, a.key1,
-                        8u * (threadIdx.x / G::T));
-    krow_fwd<N, 2>(x);
-    __syncthreads();
-    kcol<N, true, 2>([&](const KCol<N, 2>& t, float2 (&p)[G::A], float2 (&q)[G::A]) {
-      ks_draw_spin2<N, DRAW>(t, p, q, a.fgE, a.fgB, step, chain, a.key0, a.key1);
-    });
-    __syncthreads();
-    krow_inv<N, 2>(x);
-    ++done;
-    if (done > a.burn_in && (done - a.burn_in) % a.thin == 0) {
-      const long long m = (done - a.burn_in) / a.thin - 1;
-      kstore<N, 2>(x, reinterpret_cast<char*>(a.out) + ((ci * a.n_samples + m) * 2 + threadIdx.x / G::T) * n * eb,
-                   a.out_dtype);
+  kparts<BAL>(bal, a.n_chains, a.n_sweeps, [&](const auto& p) {
+    float2 x[G::E];
+    if (p.load) {
+      if (!kawait(bal, blockIdx.x - 1)) return false;
+      kload<N, 2, false>(x, bal.slot + (blockIdx.x - 1LL) * bal.slot_floats + (threadIdx.x / G::T) * n);
+    } else {
+      kload<N, 2>(x, a.init_s ? a.init_s + p.c * a.init_stride + (threadIdx.x / G::T) * n : nullptr);
     }
-  }
+    const uint32_t chain = a.chain0 + uint32_t(p.c);
+    for (int done = p.d0; done < p.d1;) {
+      const uint32_t step = a.step0 + uint32_t(done);
+      kt_draw<N, 2, DRAW>(x, a.aq2 + (threadIdx.x / G::T) * n, a.sc->sqrt_tau, step, chain, a.key0, a.key1,
+                          8u * (threadIdx.x / G::T));
+      krow_fwd<N, 2>(x);
+      __syncthreads();
+      kcol<N, true, 2>([&](const KCol<N, 2>& t, float2 (&u)[G::A], float2 (&v)[G::A]) {
+        ks_draw_spin2<N, DRAW>(t, u, v, a.fgE, a.fgB, step, chain, a.key0, a.key1);
+      });
+      __syncthreads();
+      krow_inv<N, 2>(x);
+      ++done;
+      if (done > a.burn_in && (done - a.burn_in) % a.thin == 0) {
+        const long long m = (done - a.burn_in) / a.thin - 1;
+        kstore<N, 2>(x, reinterpret_cast<char*>(a.out) + ((p.c * a.n_samples + m) * 2 + threadIdx.x / G::T) * n * eb,
+                     a.out_dtype);
+      }
+    }
+    if (p.save) {
+      kstore<N, 2>(x, bal.slot + (long long)blockIdx.x * bal.slot_floats + (threadIdx.x / G::T) * n, kOutF32);
+      kpublish(bal, blockIdx.x);
+    }
+    return true;
+  });
 }
 
 // ---------------------------------------------------------------------------------------------

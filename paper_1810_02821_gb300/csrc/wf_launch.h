@@ -26,14 +26,16 @@ struct LaunchTimer {
 template <int N>
 constexpr int fields_per_cta() { return N >= 128 ? 1 : 128 / N; }
 
+// Samplers up to 128 x 128. *timeout (host, set to 0 by the caller) receives WF_ERR_TIMEOUT, once st has passed, when a
+// wait of a balanced launch gave up; launch_sample with timeout null allocates nothing
 template <int N>
-cudaError_t launch_sample(const SampleArgs& a, cudaStream_t st, LaunchTimer* t);
+cudaError_t launch_sample(const SampleArgs& a, cudaStream_t st, LaunchTimer* t, int* timeout);
 
 template <int N>
-cudaError_t launch_sample_band(const SampleArgs& a, cudaStream_t st, LaunchTimer* t);
+cudaError_t launch_sample_band(const SampleArgs& a, cudaStream_t st, LaunchTimer* t, int* timeout);
 
 template <int N>
-cudaError_t launch_sample_spin2(const Spin2Args& a, cudaStream_t st, LaunchTimer* t);
+cudaError_t launch_sample_spin2(const Spin2Args& a, cudaStream_t st, LaunchTimer* t, int* timeout);
 
 template <int N>
 cudaError_t launch_solve(const SolveArgs& a, const BnormArgs& b, cudaStream_t st, LaunchTimer* t);
@@ -102,11 +104,62 @@ cudaError_t launch_smem(Kern kern, dim3 grid, int threads, int smem, const Args&
   if (t) t->stop();
   return cudaGetLastError();
 }
+// One CTA per chain, or, with more chains than are resident at once, a cooperative launch of equal shares (KBalance)
+// whose scratch (slots, flags) comes from st's memory pool. A last round of 0.92 to 1 CTA per SM at two CTAs per SM
+// keeps one CTA per chain: alone on their SMs those run at twice the pace, and shares would not be faster.
+template <class Kern, class Args>
+cudaError_t launch_chains(Kern whole, Kern balanced, int n_chains, int threads, int smem, int slot_floats,
+                          const Args& a, cudaStream_t st, LaunchTimer* t, int* timeout) {
+  cudaError_t e = cudaFuncSetAttribute(balanced, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  if (e != cudaSuccess) return e;
+  int dev = 0, sms = 0, per_sm = 0;
+  if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
+  if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
+  if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, balanced, threads, smem)) != cudaSuccess) return e;
+  const int R = per_sm * sms, over = R > 0 ? n_chains % R : 0;
+  KBalance b{};
+  void* base = nullptr;
+  const size_t flags = (size_t(R) + 1) * sizeof(unsigned int), off = (flags + 255) / 256 * 256;
+  bool bal = timeout && R > 0 && n_chains > R && over != 0 && !(per_sm == 2 && over <= sms && over > sms - sms / 12);
+  if (bal) {
+    e = cudaMallocAsync(&base, off + size_t(R) * size_t(slot_floats) * sizeof(float), st);
+    if (e == cudaErrorMemoryAllocation) {  // no room for the states handed over: one CTA per chain needs none
+      cudaGetLastError();
+      bal = false;
+    } else if (e != cudaSuccess) {
+      return e;
+    }
+  }
+  if (!bal) {
+    if ((e = cudaFuncSetAttribute(whole, cudaFuncAttributeMaxDynamicSharedMemorySize, smem)) != cudaSuccess) return e;
+    if (t) t->start();
+    whole<<<n_chains, threads, smem, st>>>(a, b);
+    if (t) t->stop();
+    return cudaGetLastError();
+  }
+  b.shares = R;
+  b.slot_floats = slot_floats;
+  b.flag = static_cast<unsigned int*>(base);
+  b.err = reinterpret_cast<int*>(b.flag + R);
+  b.slot = reinterpret_cast<float*>(static_cast<char*>(base) + off);
+  e = cudaMemsetAsync(base, 0, flags, st);
+  Args arg = a;
+  void* args[] = {&arg, &b};
+  if (t) t->start();
+  if (e == cudaSuccess)
+    e = cudaLaunchCooperativeKernel(reinterpret_cast<void*>(balanced), dim3(R), dim3(threads), args, smem, st);
+  if (t) t->stop();
+  if (e == cudaSuccess) e = cudaMemcpyAsync(timeout, b.err, sizeof(int), cudaMemcpyDeviceToHost, st);
+  const cudaError_t e2 = cudaFreeAsync(base, st);
+  return e != cudaSuccess ? e : e2;
+}
 
 template <int N>
-cudaError_t launch_sample(const SampleArgs& a, cudaStream_t st, LaunchTimer* t) {
+cudaError_t launch_sample(const SampleArgs& a, cudaStream_t st, LaunchTimer* t, int* timeout) {
   if constexpr (core_size(N)) {
-    if (a.cm != 0) return launch_smem(k_msample<N>, a.n_chains, KGeo<N>::T, KGeo<N>::SMEM, a, st, t);
+    if (a.cm != 0)
+      return launch_chains(k_msample<N, false>, k_msample<N, true>, a.n_chains, KGeo<N>::T, KGeo<N>::SMEM, N * N, a, st,
+                           t, timeout);
   }
   if constexpr (N == 16 || N == 64) {
     constexpr int FPC = fields_per_cta<N>();
@@ -116,9 +169,10 @@ cudaError_t launch_sample(const SampleArgs& a, cudaStream_t st, LaunchTimer* t) 
 }
 
 template <int N>
-cudaError_t launch_sample_band(const SampleArgs& a, cudaStream_t st, LaunchTimer* t) {
+cudaError_t launch_sample_band(const SampleArgs& a, cudaStream_t st, LaunchTimer* t, int* timeout) {
   if constexpr (core_size(N)) {
-    return launch_smem(k_mband<N>, a.n_chains, KGeo<N>::T, KGeo<N>::SMEM + band_bytes(a.n_bins), a, st, t);
+    return launch_chains(k_mband<N, false>, k_mband<N, true>, a.n_chains, KGeo<N>::T,
+                         KGeo<N>::SMEM + band_bytes(a.n_bins), N * N + (a.n_bins + 3) / 4 * 4, a, st, t, timeout);
   } else {
     constexpr int FPC = fields_per_cta<N>();
     return launch_smem(k_sample_band<N, FPC>, (a.n_chains + FPC - 1) / FPC, N * FPC,
@@ -127,10 +181,11 @@ cudaError_t launch_sample_band(const SampleArgs& a, cudaStream_t st, LaunchTimer
 }
 
 template <int N>
-cudaError_t launch_sample_spin2(const Spin2Args& a, cudaStream_t st, LaunchTimer* t) {
+cudaError_t launch_sample_spin2(const Spin2Args& a, cudaStream_t st, LaunchTimer* t, int* timeout) {
   if constexpr (core_size(N)) {
-    return a.quiet ? launch_smem(k_mspin2<N, false>, a.n_chains, 2 * KGeo<N>::T, kspin2_smem<N>(), a, st, t)
-                   : launch_smem(k_mspin2<N, true>, a.n_chains, 2 * KGeo<N>::T, kspin2_smem<N>(), a, st, t);
+    // the filter (quiet) is one chain
+    return launch_chains(a.quiet ? k_mspin2<N, false, false> : k_mspin2<N, true, false>, k_mspin2<N, true, true>,
+                         a.n_chains, 2 * KGeo<N>::T, kspin2_smem<N>(), 2 * N * N, a, st, t, a.quiet ? nullptr : timeout);
   } else {
     constexpr int FPC = fields_per_cta<N>();  // images per CTA; two component fields each
     return launch_smem(k_sample_spin2<N, FPC>, (a.n_chains + FPC - 1) / FPC, 2 * N * FPC,
@@ -227,9 +282,9 @@ cudaError_t launch_wpower(const WpowerArgs& p, cudaStream_t st) {
 }
 
 #define WF_INSTANTIATE(N)                                                              \
-  template cudaError_t launch_sample<N>(const SampleArgs&, cudaStream_t, LaunchTimer*); \
-  template cudaError_t launch_sample_band<N>(const SampleArgs&, cudaStream_t, LaunchTimer*); \
-  template cudaError_t launch_sample_spin2<N>(const Spin2Args&, cudaStream_t, LaunchTimer*); \
+  template cudaError_t launch_sample<N>(const SampleArgs&, cudaStream_t, LaunchTimer*, int*); \
+  template cudaError_t launch_sample_band<N>(const SampleArgs&, cudaStream_t, LaunchTimer*, int*); \
+  template cudaError_t launch_sample_spin2<N>(const Spin2Args&, cudaStream_t, LaunchTimer*, int*); \
   template cudaError_t launch_solve<N>(const SolveArgs&, const BnormArgs&, cudaStream_t, LaunchTimer*); \
   template cudaError_t launch_batch<N>(const BatchArgs&, int*, cudaStream_t);                     \
   template cudaError_t batch_grid<N>(int, int, int*);                                                   \

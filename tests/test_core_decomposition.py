@@ -84,3 +84,42 @@ def test_slot_order_of_the_mode_tables(N):
     for kx in range(L):   # mode_pos with cm = BR
         slot = (kx % BR) * (L // BR) + kx // BR
         assert slot // A + BR * (slot % A) == kx
+
+
+def _parts(i, R, n_chains, S):
+    """Parts (chain, first sweep, end, load, save) of CTA i, in the order it runs them."""
+    W = n_chains * S
+    q, r = divmod(W, R)
+    a, b = q * i + r * i // R, q * (i + 1) + r * (i + 1) // R
+    out = []
+    if b % S:
+        out.append((b // S, 0, b % S, False, True))
+    out += [(c, 0, S, False, False) for c in range((a + S - 1) // S, b // S)]
+    if a % S:
+        out.append((a // S, a % S, S, True, False))
+    return out
+
+
+@pytest.mark.parametrize("R,n_chains,S", [(152, 200, 30), (304, 1000, 7), (304, 305, 1), (5, 6, 100), (7, 13, 3), (3, 3, 4)])
+def test_balanced_shares_cover_every_sweep_once_and_hand_over_in_time(R, n_chains, S):
+    """Equal shares of all chains' sweeps: every sweep once, at most two parts a chain, the first part of a split chain
+    at the start of its CTA and the second at the end of the next one, never before the first has finished."""
+    seen, loads, length = {}, {}, []
+    for i in range(R):
+        t = 0
+        for k, (c, d0, d1, load, save) in enumerate(_parts(i, R, n_chains, S)):
+            assert d0 < d1
+            seen.setdefault(c, []).append((d0, d1))
+            if save:
+                assert k == 0
+                loads.setdefault(c, {})["ready"] = (i, d1)
+            if load:
+                loads.setdefault(c, {})["start"] = (i, t)
+            t += d1 - d0
+        length.append(t)
+    for c in range(n_chains):
+        spans = sorted(seen[c])
+        assert len(spans) <= 2 and spans[0][0] == 0 and spans[-1][1] == S and all(x[1] == y[0] for x, y in zip(spans, spans[1:]))
+    for c, v in loads.items():
+        assert v["start"][0] == v["ready"][0] + 1 and v["start"][1] >= v["ready"][1] - 1   # equal shares to one sweep
+    assert max(length) - min(length) <= 1
