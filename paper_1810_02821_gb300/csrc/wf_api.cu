@@ -182,14 +182,21 @@ cudaError_t launch_prep(const float* d, const float* Ndiag, const uint8_t* mask,
   return launch_prep_kernel(k_prep, 1, H, st, d, Ndiag, mask, Pk, H, W, tau_user, eta, sc);
 }
 
+int gcluster_max(int H, bool solve);
+
 constexpr int kFew128 = 36, kFewSpin2 = 40;  // chains from which the on-chip kernels run at 128^2
 bool size_on_chip(int H) { return H <= 128; }
-// Whether fields of an on-chip size run on the on-chip kernels, one CTA per field, or on the global-memory kernels, one
-// cooperative launch that spreads each field over 16 SMs. At 128^2 the latter has less latency for few fields (us per
-// sweep of all chains, global-memory / on-chip): sampler 1 chain 6.4 / 9.6, 16 chains 6.9 / 9.7, 32 chains 8.7 / 9.7,
-// 39 chains 10.1 / 9.7; spin-2 1 chain 7.6 / 22.9, 39 chains 20.6 / 22.9; a Wiener filter 6.8 / 8.0 (from zero only: the
-// global-memory solve takes no starting iterate).
-bool sample_on_chip(int H, int units) { return size_on_chip(H) && !(H == 128 && units < kFew128); }
+// Whether fields of an on-chip size run on the on-chip kernels, one CTA per field, or spread over several SMs. At 128^2
+// the latter has less latency for few fields (us per sweep of all chains): the sampler in clusters of 8 CTAs takes 3.8
+// for up to 14 chains, 4.8 for 36 and 5.6 for the 48 that are resident at once, on chip 9.6 (60 chains, two rounds of
+// clusters: as long). On a device without such clusters the global-memory kernel takes 6.4 to 9.2 for up to 36 chains.
+// Spin-2, global-memory / on chip: 1 chain 7.6 / 22.9, 39 chains 20.6 / 22.9. A Wiener filter 4.0 (cluster) / 8.0 (from
+// zero only: the other paths take no starting iterate).
+bool sample_on_chip(int H, int units) {
+  if (H != 128) return size_on_chip(H);
+  const int few = gcluster_max(H, false);
+  return units > (few > 0 ? few : kFew128 - 1);
+}
 bool spin2_on_chip(int H, int units) { return size_on_chip(H) && !(H == 128 && units < kFewSpin2); }
 bool solve_on_chip(int H, bool from_zero) { return size_on_chip(H) && !(H == 128 && from_zero); }
 
@@ -338,7 +345,39 @@ bool out_ptr_ok(const void* p) {
   return true;
 }
 
+// Fields of a launch up to which k_gcluster takes the place of k_global: as many clusters as are resident at once on
+// the device (0: none). us per sweep of all chains, k_global / k_gcluster, the same results bit for bit: 128^2 1 chain
+// 6.5 / 3.8, 12 chains 6.8 / 3.8, 35 chains 9.2 / 4.8; 256^2 1 chain 7.0 / 5.3, 7 chains 8.1 / 5.3, 14 chains 10.2 / 7.4;
+// Wiener filter 128^2 7.0 / 4.0, 256^2 7.3 / 5.5. A second round of clusters would cost as much as the first (256^2, 16
+// chains: 11.8 on k_global).
+int gcluster_max(int H, bool solve) {
+  if (H != 128 && H != 256) return 0;
+  static std::mutex mu;
+  static int known[2][2][64] = {};  // clusters + 1
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) {
+    cudaGetLastError();
+    return 0;
+  }
+  std::lock_guard<std::mutex> lock(mu);
+  int& k = known[H == 256][solve][dev];
+  if (k == 0) {
+    int n = 0;
+    const cudaError_t e = H == 128 ? wf::gcluster_count<128>(solve, &n) : wf::gcluster_count<256>(solve, &n);
+    if (e != cudaSuccess) {
+      cudaGetLastError();
+      n = 0;
+    }
+    k = n + 1;
+  }
+  return k - 1;
+}
+
 cudaError_t launch_global_any(int H, const wf::GlobalArgs& a, cudaStream_t st, wf::LaunchTimer* t) {
+  if (a.mode <= 1 && g_large_sampler == 0 && a.n_fields <= gcluster_max(H, a.mode == 1)) {
+    if (H == 128) return wf::launch_gcluster<128>(a, st, t);
+    return wf::launch_gcluster<256>(a, st, t);
+  }
   switch (H) {
     case 128: return wf::launch_global<128>(a, st, t);
     case 256: return wf::launch_global<256>(a, st, t);

@@ -112,7 +112,7 @@ __global__ void __launch_bounds__(GGeo<N>::T, GGeo<N>::MIN_CTAS) k_gbatch(const 
       float2 x[G::E];
       pixel_update<N>(2, x, y0 + ty, fd.aq, fd.dn, 0u, 0u, 0u, 0u, 0.f, 0.f, 0,
                       float(level_lambda(sc, l, a.eta) * sc.tau));
-      grow_fwd<N>(x, fd.Z + (long long)(y0 + ty) * G::LR);
+      grow_fwd<N>(x, ZRow{fd.Z + (long long)(y0 + ty) * G::LR});
     }
     if (!grid_barrier(a.bar, nb, target)) return;
     for (int it = blockIdx.x; it < col_items; it += nb) {
@@ -190,10 +190,10 @@ __global__ void __launch_bounds__(GGeo<N>::T, GGeo<N>::MIN_CTAS) k_gbatch(const 
         if (S.status == 1 && S.it >= a.max_iter) S.status = 5;
       }
       const int y = y0 + ty;
-      float2* Zrow = fd.Z + (long long)y * G::LR;
+      const ZRow z{fd.Z + (long long)y * G::LR};
       float2 x[G::E];
       if (fresh) grow_load<N>(x, nullptr);
-      else grow_inv<N>(Zrow, x);
+      else grow_inv<N>(z, x);
       bool finished = false;
       if (S.phase == 0 && S.status != 1) {  // solve done: s_W out, then samples from it
         if (fd.out_wf) grow_store<N>(x, fd.out_wf, y, kOutF32);
@@ -227,7 +227,7 @@ __global__ void __launch_bounds__(GGeo<N>::T, GGeo<N>::MIN_CTAS) k_gbatch(const 
       } else {
         pixel_update<N>(0, x, y, fd.aq, fd.dn, uint32_t(S.d), fd.chain, fd.key0, fd.key1, sc.sqrt_tau, 0.f, 0, 0.f);
       }
-      grow_fwd<N>(x, Zrow);
+      grow_fwd<N>(x, z);
       if (owner) nxt[f] = S;
     }
     if (!grid_barrier(a.bar, nb, target)) return;

@@ -1,5 +1,5 @@
 // Messenger-field sweeps of fields in global memory: images too large for one SM (N in {256, 512, 1024}), and
-// few fields of 128^2, which one SM each would run with more latency.
+// few fields of 128^2 (spin-2, and where clusters cannot run), which one SM each would run with more latency.
 //
 // The packed half spectrum Z[H][W/2] of every field (kx = 0 and W/2 packed as re/im of column 0) lives in
 // global memory (L2-resident when the working set allows). One persistent cooperative kernel runs every
@@ -35,19 +35,20 @@
 
 namespace wf {
 
-template <int N_>
+// RB: rows per CTA
+template <int N_, int RB_ = 8>
 struct GGeo {
   static constexpr int N = N_, H = N_, W = N_;
   static constexpr int LR = W / 2;           // complex length of a row transform
   static constexpr int E = N_ == 1024 ? 16 : 8, A = E / 2;  // elements per thread, length of the unit transforms
   static constexpr int TR = LR / E, TC = H / E;    // threads per row and per column
-  static constexpr int RB = 8;                     // rows per CTA
+  static constexpr int RB = RB_;
   static constexpr int T = RB * TR;                // threads per CTA
-  static constexpr int CB = T / TC;                // columns per CTA
+  static constexpr int CB = T / TC;                // columns per CTA (RB / 2)
   static constexpr int BR = LR / A, BC = H / A;    // frequency strides of the units
-  // float2 strides of a row's and a column's vector: 8 blocks of L1 + 2; columns 4 modulo 16 apart (a half-warp
-  // holds four columns)
-  static constexpr int VROW = LR + 16 + 8, VCOL = H + 16 + 4;
+  // float2 strides of a row's and a column's vector: 8 blocks of L1 + 2; columns 16/CB modulo 16 apart (a half-warp
+  // holds CB columns)
+  static constexpr int VROW = LR + 16 + 8, VCOL = H + 16 + 16 / CB;
   static constexpr int VEC = RB * VROW > CB * VCOL ? RB * VROW : CB * VCOL;
   // twiddle tables: T1 [q1][n0] (rows of n/8 + 2), T2 and T3 [q][n1] of the rows and columns, W_W^K (K < LR/2)
   static constexpr int O_T1R = VEC, O_T2R = O_T1R + 8 * (LR / 8 + 2), O_T3R = O_T2R + LR / 8, O_T1C = O_T3R + 16,
@@ -59,7 +60,7 @@ struct GGeo {
   static constexpr int WH = W / 2 + 1;
   // CTAs per SM the kernels are compiled for: up to 128 registers a thread with 16 elements, 80 with 8
   static constexpr int MIN_CTAS = (E == 16 ? 512 : 768) / T;
-  static_assert(CB == 4 && TR <= 32 && VCOL % 16 == 4, "geometry");
+  static_assert((CB == 4 || CB == 8) && TR <= 32 && VCOL % 16 == 16 / CB, "geometry");
 };
 
 // middle radices of a transform of length n
@@ -77,9 +78,9 @@ __device__ __forceinline__ float2* gsmem() {
 }
 
 // the twiddle tables, by all threads (ends with a CTA barrier)
-template <int N>
+template <int N, int RB = 8>
 __device__ __forceinline__ void gtab_init() {
-  using G = GGeo<N>;
+  using G = GGeo<N, RB>;
   float2* s = gsmem();
   auto w = [](int j) { return g_tw1024.v[(j * (1024 / N)) & 1023]; };  // exp(-2 pi i j / N)
   for (int i = threadIdx.x; i < 8 * (G::LR / 8); i += G::T) {
@@ -103,9 +104,9 @@ __device__ __forceinline__ void gtab_init() {
 struct GTab {
   const float2 *t1, *t2, *t3;
 };
-template <int N, bool ROW>
+template <int N, bool ROW, int RB = 8>
 __device__ __forceinline__ GTab gtab() {
-  using G = GGeo<N>;
+  using G = GGeo<N, RB>;
   const float2* s = gsmem();
   return ROW ? GTab{s + G::O_T1R, s + G::O_T2R, s + G::O_T3R} : GTab{s + G::O_T1C, s + G::O_T2C, s + G::O_T3C};
 }
@@ -327,20 +328,27 @@ struct GlobalArgs {
 // ---------------------------------------------------------------------------------------------
 // row phase: thread tid of a row item holds row tid / TR, unit pair (h, hb), h = tid % TR
 // ---------------------------------------------------------------------------------------------
-// row y of Z (natural order) -> x (x[8 i + m] = pixel pair (E/8) h + i + (LR/8) m), unnormalised inverse transform
-template <int N>
-__device__ __forceinline__ void grow_inv(const float2* Zrow, float2 (&x)[GGeo<N>::E]) {
-  using G = GGeo<N>;
+// a row of Z in global memory: ld and st of the entry at kx
+struct ZRow {
+  float2* p;
+  __device__ __forceinline__ float2 ld(int kx) const { return __ldcg(p + kx); }
+  __device__ __forceinline__ void st(int kx, float2 v) const { __stcg(p + kx, v); }
+};
+
+// the row of z (natural order) -> x (x[8 i + m] = pixel pair (E/8) h + i + (LR/8) m), unnormalised inverse transform
+template <int N, int RB = 8, class Z>
+__device__ __forceinline__ void grow_inv(const Z& z, float2 (&x)[GGeo<N>::E]) {
+  using G = GGeo<N, RB>;
   constexpr int LR = G::LR, BR = G::BR, E = G::E, A = G::A;
   const int h = threadIdx.x % G::TR, hb = h == 0 ? BR / 2 : BR - h;
-  const GTab t = gtab<N, true>();
+  const GTab t = gtab<N, true, RB>();
   float2* v = gsmem() + (threadIdx.x / G::TR) * G::VROW;
   {
     float2 p[A], q[A];
 #pragma unroll
-    for (int j = 0; j < A; ++j) p[j] = __ldcg(Zrow + h + BR * j);
+    for (int j = 0; j < A; ++j) p[j] = z.ld(h + BR * j);
 #pragma unroll
-    for (int j = 0; j < A; ++j) q[j] = __ldcg(Zrow + hb + BR * j);
+    for (int j = 0; j < A; ++j) q[j] = z.ld(hb + BR * j);
     const float2* w = gsmem() + G::O_W;
     if (h == 0) {
       unit0_swap<A>(p, q);
@@ -363,13 +371,13 @@ __device__ __forceinline__ void grow_inv(const float2* Zrow, float2 (&x)[GGeo<N>
   ginv1<LR, E>(v, h, x);
 }
 
-// x -> half spectrum of the row, to Z
-template <int N>
-__device__ __forceinline__ void grow_fwd(const float2 (&x)[GGeo<N>::E], float2* Zrow) {
-  using G = GGeo<N>;
+// x -> half spectrum of the row, to z
+template <int N, int RB = 8, class Z>
+__device__ __forceinline__ void grow_fwd(const float2 (&x)[GGeo<N>::E], const Z& z) {
+  using G = GGeo<N, RB>;
   constexpr int LR = G::LR, BR = G::BR, E = G::E, A = G::A;
   const int h = threadIdx.x % G::TR, hb = h == 0 ? BR / 2 : BR - h;
-  const GTab t = gtab<N, true>();
+  const GTab t = gtab<N, true, RB>();
   float2* v = gsmem() + (threadIdx.x / G::TR) * G::VROW;
   gfwd1<LR, E>(v, h, x, t);
   __syncwarp();
@@ -392,9 +400,9 @@ __device__ __forceinline__ void grow_fwd(const float2 (&x)[GGeo<N>::E], float2* 
   for (int j = 0; j < A / 2; ++j) k_post(q[j], p[A - 1 - j], w[hb + BR * j]);
   if (h == 0) unit0_unswap<A>(p, q);
 #pragma unroll
-  for (int j = 0; j < A; ++j) __stcg(Zrow + h + BR * j, p[j]);
+  for (int j = 0; j < A; ++j) z.st(h + BR * j, p[j]);
 #pragma unroll
-  for (int j = 0; j < A; ++j) __stcg(Zrow + hb + BR * j, q[j]);
+  for (int j = 0; j < A; ++j) z.st(hb + BR * j, q[j]);
   __syncwarp();  // the row's vector is rewritten by the next item
 }
 
@@ -431,14 +439,19 @@ __device__ __forceinline__ void grow_store(float2 (&x)[GGeo<N>::E], void* img, l
 //           table (rhs_mode: t = w s + lambda tau r with r in place of d);
 //   mode 2: the level right-hand side N_lambda^-1 d with N_lambda = N_bar + lt2 (s ignored).
 // The two pairs of a Philox group are in one thread (E = 16), or in neighbouring lanes (E = 8): there each lane
-// draws half of the groups and the two exchange the halves they need.
+// draws half of the groups and the two exchange the halves they need. tab(e): the table's entries of pixels 2e and
+// 2e + 1; draw(i, z): the normals of the thread's i-th group (pixel_group).
 template <int N>
-__device__ __forceinline__ void pixel_update(int mode, float2 (&x)[GGeo<N>::E], int y, const float2* __restrict__ aq,
-                                             const float2* __restrict__ dn, uint32_t step, uint32_t chain,
-                                             uint32_t key0, uint32_t key1, float sqrt_tau, float ltau, int rhs_mode,
-                                             float lt2, uint32_t stream = 0u) {
+__device__ __forceinline__ uint32_t pixel_group(int y, int i) {
   using G = GGeo<N>;
-  const float4* tab = reinterpret_cast<const float4*>((mode == 0 || mode == 4 ? aq : dn) + (long long)y * G::W);
+  const int h = threadIdx.x % G::TR;
+  if constexpr (G::E == 16) return uint32_t(y * (G::W / 4) + h + (G::LR / 16) * i);
+  else return uint32_t(y * (G::W / 4) + (h + (G::LR / 8) * ((h & 1) ? 4 + i : i)) / 2);
+}
+template <int N, class T, class D>
+__device__ __forceinline__ void pixel_update(int mode, float2 (&x)[GGeo<N>::E], T&& tab, D&& draw, float sqrt_tau,
+                                             float ltau, int rhs_mode, float lt2) {
+  using G = GGeo<N>;
   if (mode == 0) {
     const int h = threadIdx.x % G::TR;
     auto upd = [&](float2& v, float4 c, float z0, float z1) {
@@ -449,9 +462,9 @@ __device__ __forceinline__ void pixel_update(int mode, float2 (&x)[GGeo<N>::E], 
 #pragma unroll
       for (int m = 0; m < 8; ++m) {
         const int e = 2 * h + (G::LR / 8) * m;
-        const float4 c0 = __ldg(tab + e), c1 = __ldg(tab + e + 1);
+        const float4 c0 = tab(e), c1 = tab(e + 1);
         float z[4];
-        normals4(uint32_t(y * (G::W / 4) + e / 2), step, chain, stream, key0, key1, z);
+        draw(m, z);
         upd(x[m], c0, z[0], z[1]);
         upd(x[8 + m], c1, z[2], z[3]);
       }
@@ -460,9 +473,9 @@ __device__ __forceinline__ void pixel_update(int mode, float2 (&x)[GGeo<N>::E], 
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
         const int e0 = h + (G::LR / 8) * i, e1 = h + (G::LR / 8) * (4 + i);
-        const float4 c0 = __ldg(tab + e0), c1 = __ldg(tab + e1);
+        const float4 c0 = tab(e0), c1 = tab(e1);
         float z[4];  // even lanes: the group of pair e0, odd lanes: that of e1
-        normals4(uint32_t(y * (G::W / 4) + (odd ? e1 : e0) / 2), step, chain, stream, key0, key1, z);
+        draw(i, z);
         const float r0 = __shfl_xor_sync(0xffffffffu, odd ? z[0] : z[2], 1);
         const float r1 = __shfl_xor_sync(0xffffffffu, odd ? z[1] : z[3], 1);
         upd(x[i], c0, odd ? r0 : z[0], odd ? r1 : z[1]);
@@ -471,7 +484,7 @@ __device__ __forceinline__ void pixel_update(int mode, float2 (&x)[GGeo<N>::E], 
     }
   } else if (mode == 4) {
     gpixels<N>(x, [&](float2& v, int e) {
-      const float4 c = __ldg(tab + e);
+      const float4 c = tab(e);
       v.x = fmaf(c.y, c.y * v.x, c.x);
       v.y = fmaf(c.w, c.w * v.y, c.z);
     });
@@ -482,17 +495,31 @@ __device__ __forceinline__ void pixel_update(int mode, float2 (&x)[GGeo<N>::E], 
       v = fmaf(w, fmaf(-g, dv, v), hh * dv);
     };
     gpixels<N>(x, [&](float2& v, int e) {
-      const float4 c = __ldg(tab + e);
+      const float4 c = tab(e);
       upd(v.x, c.x, c.y);
       upd(v.y, c.z, c.w);
     });
   } else {
     auto rhs = [&](float dv, float inb) { return dv / ((inb > 0.0f ? wf_rcp(inb) : wf_inf()) + lt2); };
     gpixels<N>(x, [&](float2& v, int e) {
-      const float4 c = __ldg(tab + e);
+      const float4 c = tab(e);
       v = make_float2(rhs(c.x, c.y), rhs(c.z, c.w));
     });
   }
+}
+
+// with the tables in global memory and the draws on the spot
+template <int N>
+__device__ __forceinline__ void pixel_update(int mode, float2 (&x)[GGeo<N>::E], int y, const float2* __restrict__ aq,
+                                             const float2* __restrict__ dn, uint32_t step, uint32_t chain,
+                                             uint32_t key0, uint32_t key1, float sqrt_tau, float ltau, int rhs_mode,
+                                             float lt2, uint32_t stream = 0u) {
+  const float4* tab =
+      reinterpret_cast<const float4*>((mode == 0 || mode == 4 ? aq : dn) + (long long)y * GGeo<N>::W);
+  pixel_update<N>(
+      mode, x, [&](int e) { return __ldg(tab + e); },
+      [&](int i, float (&z)[4]) { normals4(pixel_group<N>(y, i), step, chain, stream, key0, key1, z); }, sqrt_tau,
+      ltau, rhs_mode, lt2);
 }
 
 // Row phase on one work item: rows y0 .. y0+RB-1 of field f. first: start from the real state s0.
@@ -501,10 +528,10 @@ __device__ void row_item(const GlobalArgs& a, int f, int y0, int done, bool firs
                          const Scalars& sc) {
   using G = GGeo<N>;
   const int y = y0 + int(threadIdx.x) / G::TR;
-  float2* Zrow = a.Z + ((long long)f * G::H + y) * G::LR;
+  const ZRow z{a.Z + ((long long)f * G::H + y) * G::LR};
   float2 x[G::E];
   if (!first) {
-    grow_inv<N>(Zrow, x);
+    grow_inv<N>(z, x);
   } else if (a.mode == 3) {
     const long long o = ((long long)f * G::H + y) * G::W;
     grow_load<N>(x, a.va + o);
@@ -532,29 +559,40 @@ __device__ void row_item(const GlobalArgs& a, int f, int y0, int done, bool firs
   if (a.mode != 3)  // mode 3 transforms the field as loaded
     pixel_update<N>(a.mode, x, y, a.aq, a.dn, a.step0 + uint32_t(done), a.chain0 + uint32_t(f), a.key0, a.key1,
                     sc.sqrt_tau, ltau, a.rhs_mode, a.mode == 2 ? float(level_lambda(sc, f, a.eta) * sc.tau) : 0.f);
-  grow_fwd<N>(x, Zrow);
+  grow_fwd<N>(x, z);
 }
 
 // ---------------------------------------------------------------------------------------------
 // column phase: thread tid of a column item holds column c0 + tid % CB, unit pair (h, hb), h = tid / CB
 // ---------------------------------------------------------------------------------------------
-// Columns c0 .. c0 + CB - 1 of Z: forward transform, f(p, q) on the thread's units (after unit0_swap: mode
+// the CTA's columns of Z in global memory: at(y0, c): column c from row y0, with ld and st of row y0 + dy
+template <int N>
+struct ZCols {
+  float2* p;  // of column 0
+  struct Col {
+    float2* p;
+    __device__ __forceinline__ float2 ld(int dy) const { return __ldcg(p + (long long)dy * (N / 2)); }
+    __device__ __forceinline__ void st(int dy, float2 v) const { __stcg(p + (long long)dy * (N / 2), v); }
+  };
+  __device__ __forceinline__ Col at(int y0, int c) const { return Col{p + (long long)y0 * (N / 2) + c}; }
+};
+// Columns c0 .. c0 + CB - 1 of z: forward transform, f(p, q) on the thread's units (after unit0_swap: mode
 // pairs (p[j], q[A-1-j]) at ky1 = h + BC j and (q[j], p[A-1-j]) at ky1 = hb + BC j, j < A/2), and with INV the inverse
 // transform back to Z.
-template <int N, bool INV, class F>
-__device__ __forceinline__ void gcol(float2* Z, int c0, F&& f) {
-  using G = GGeo<N>;
-  constexpr int H = G::H, LR = G::LR, BC = G::BC, E = G::E, A = G::A, NC = E / 8;
+template <int N, bool INV, int RB = 8, class Z, class F>
+__device__ __forceinline__ void gcol(const Z& z, int c0, F&& f) {
+  using G = GGeo<N, RB>;
+  constexpr int H = G::H, BC = G::BC, E = G::E, A = G::A, NC = E / 8;
   const int c = threadIdx.x % G::CB, h = threadIdx.x / G::CB, hb = h == 0 ? BC / 2 : BC - h;
-  const GTab t = gtab<N, false>();
+  const GTab t = gtab<N, false, RB>();
   float2* v = gsmem() + c * G::VCOL;
-  float2* Zc = Z + (long long)(NC * h) * LR + c0 + c;
+  const auto zc = z.at(NC * h, c);
   {
     float2 x[E];
 #pragma unroll
     for (int m = 0; m < 8; ++m)
 #pragma unroll
-      for (int i = 0; i < NC; ++i) x[8 * i + m] = __ldcg(Zc + (long long)(H / 8 * m + i) * LR);
+      for (int i = 0; i < NC; ++i) x[8 * i + m] = zc.ld(H / 8 * m + i);
     gfwd1<H, E>(v, h, x, t);
   }
   __syncthreads();
@@ -583,17 +621,17 @@ __device__ __forceinline__ void gcol(float2* Z, int c0, F&& f) {
 #pragma unroll
     for (int m = 0; m < 8; ++m)
 #pragma unroll
-      for (int i = 0; i < NC; ++i) __stcg(Zc + (long long)(H / 8 * m + i) * LR, x[8 * i + m]);
+      for (int i = 0; i < NC; ++i) zc.st(H / 8 * m + i, x[8 * i + m]);
   }
   __syncthreads();
 }
 
 // inter(y1, y2, ky1, ky2) on the mode pairs of an interior column; the H/2 pairs of the packed edge column (column
 // 0: kx = 0 as A and kx = W/2 as B in Y = A + i B) are shared out over all threads of its CTA
-template <int N, class I, class X>
-__device__ __forceinline__ void gpairs(float2 (&p)[GGeo<N>::A], float2 (&q)[GGeo<N>::A], int col, int h, int hb, int c0, I&& inter,
-                                       X&& edge) {
-  using G = GGeo<N>;
+template <int N, int RB = 8, class I, class X>
+__device__ __forceinline__ void gpairs(float2 (&p)[GGeo<N>::A], float2 (&q)[GGeo<N>::A], int col, int h, int hb,
+                                       int c0, I&& inter, X&& edge) {
+  using G = GGeo<N, RB>;
   constexpr int H = G::H, BC = G::BC, A = G::A;
   float2* e = gsmem() + G::O_EDGE;
   if (c0 == 0) {  // the same in every thread of the CTA
@@ -645,32 +683,33 @@ __device__ __forceinline__ void gpairs(float2 (&p)[GGeo<N>::A], float2 (&q)[GGeo
 //           iterates); with store, keeps s_hat in prev;
 //   mode 2: returns this thread's part of sum_k P^2 |t_hat|^2 of the level right-hand side (Z unchanged).
 // Per-mode terms and a thread's partial sum in FP32, the CTA and grid sums in FP64.
-template <int N>
-__device__ __forceinline__ float gcol_update(int mode, float2* Z, int c0, const float2* __restrict__ fg,
-                                              const float* __restrict__ Pk, float2* prev, uint32_t step,
-                                              uint32_t chain, uint32_t key0, uint32_t key1, float ltau, bool cmp,
-                                              bool store) {
-  using G = GGeo<N>;
-  constexpr int L = G::LR, H = G::H, WH = G::WH;
+// z: the CTA's columns; fg(ky, kx), Pk(ky, kx), prev(ky, kx): the tables; draw(i, g, z): the normals of the thread's
+// i-th pair, group g; edraw(ky, z): those of a pair of the edge column.
+template <int N, int RB = 8, class Z, class FG, class PK, class PV, class D, class X>
+__device__ __forceinline__ float gcol_update(int mode, const Z& z, int c0, FG&& fg, PK&& Pk, PV&& prev, D&& draw,
+                                             X&& edraw, float ltau, bool cmp, bool store) {
+  using G = GGeo<N, RB>;
+  constexpr int H = G::H, EW = G::W / 2;
   constexpr float INV_N = 1.0f / float(G::H * G::W);
   float acc = 0.0f;
   if (mode == 0) {
-    gcol<N, true>(Z, c0, [&](float2 (&p)[G::A], float2 (&q)[G::A], int col, int h, int hb) {
-      gpairs<N>(
+    gcol<N, true, RB>(z, c0, [&](float2 (&p)[G::A], float2 (&q)[G::A], int col, int h, int hb) {
+      int i = 0;
+      gpairs<N, RB>(
           p, q, col, h, hb, c0,
           [&](float2& y1, float2& y2, int ky1, int ky2) {
-            const float2 m1 = __ldg(fg + ky1 * WH + col), m2 = __ldg(fg + ky2 * WH + col);
+            const float2 m1 = fg(ky1, col), m2 = fg(ky2, col);
             float z[4];
-            normals4(uint32_t(col * (H / 2) + ky1), step, chain, 1u, key0, key1, z);
+            draw(i++, uint32_t(col * (H / 2) + ky1), z);
             y1 = make_float2(fmaf(m1.x, y1.x, m1.y * z[0]), fmaf(m1.x, y1.y, m1.y * z[1]));
             y2 = make_float2(fmaf(m2.x, y2.x, m2.y * z[2]), fmaf(m2.x, y2.y, m2.y * z[3]));
           },
           [&](float2& y1, float2& y2, int ky1, int ky2) {
-            const float2 a1 = __ldg(fg + ky1 * WH), b1 = __ldg(fg + ky1 * WH + G::W / 2);
+            const float2 a1 = fg(ky1, 0), b1 = fg(ky1, EW);
             float z[4];
-            normals4(uint32_t(ky1), step, chain, 1u, key0, key1, z);
+            edraw(ky1, z);
             if (ky1 == 0) {
-              const float2 a2 = __ldg(fg + ky2 * WH), b2 = __ldg(fg + ky2 * WH + G::W / 2);
+              const float2 a2 = fg(ky2, 0), b2 = fg(ky2, EW);
               constexpr float R2 = 1.41421356237309505f;
               y1 = make_float2(fmaf(a1.x, y1.x, R2 * a1.y * z[0]), fmaf(b1.x, y1.y, R2 * b1.y * z[2]));
               y2 = make_float2(fmaf(a2.x, y2.x, R2 * a2.y * z[1]), fmaf(b2.x, y2.y, R2 * b2.y * z[3]));
@@ -692,31 +731,31 @@ __device__ __forceinline__ float gcol_update(int mode, float2* Z, int c0, const 
       return fmaf(dre, dre, dim * dim) * (g * g);
     };
     auto fcoef = [&](float P) { return wf_fdiv(P, P + ltau) * INV_N; };
-    gcol<N, true>(Z, c0, [&](float2 (&p)[G::A], float2 (&q)[G::A], int col, int h, int hb) {
-      gpairs<N>(
+    gcol<N, true, RB>(z, c0, [&](float2 (&p)[G::A], float2 (&q)[G::A], int col, int h, int hb) {
+      gpairs<N, RB>(
           p, q, col, h, hb, c0,
           [&](float2& y1, float2& y2, int ky1, int ky2) {
-            const float P1 = __ldg(Pk + ky1 * WH + col), P2 = __ldg(Pk + ky2 * WH + col);
+            const float P1 = Pk(ky1, col), P2 = Pk(ky2, col);
             y1 = cscale(y1, fcoef(P1));
             y2 = cscale(y2, fcoef(P2));
             if (cmp) {
-              const float2 o1 = prev[ky1 * L + col], o2 = prev[ky2 * L + col];
+              const float2 o1 = prev(ky1, col), o2 = prev(ky2, col);
               acc += 2.0f * (wres(P1, y1.x - o1.x, y1.y - o1.y) + wres(P2, y2.x - o2.x, y2.y - o2.y));
             }
             if (store) {
-              prev[ky1 * L + col] = y1;
-              prev[ky2 * L + col] = y2;
+              prev(ky1, col) = y1;
+              prev(ky2, col) = y2;
             }
           },
           [&](float2& y1, float2& y2, int ky1, int ky2) {
-            const float Pa1 = __ldg(Pk + ky1 * WH), Pb1 = __ldg(Pk + ky1 * WH + G::W / 2);
+            const float Pa1 = Pk(ky1, 0), Pb1 = Pk(ky1, EW);
             const float fa1 = fcoef(Pa1), fb1 = fcoef(Pb1);
             if (ky1 == 0) {
-              const float Pa2 = __ldg(Pk + ky2 * WH), Pb2 = __ldg(Pk + ky2 * WH + G::W / 2);
+              const float Pa2 = Pk(ky2, 0), Pb2 = Pk(ky2, EW);
               y1 = make_float2(fa1 * y1.x, fb1 * y1.y);
               y2 = make_float2(fcoef(Pa2) * y2.x, fcoef(Pb2) * y2.y);
               if (cmp) {
-                const float2 o1 = prev[0], o2 = prev[ky2 * L];
+                const float2 o1 = prev(0, 0), o2 = prev(ky2, 0);
                 acc += wres(Pa1, y1.x - o1.x, 0.f) + wres(Pb1, y1.y - o1.y, 0.f) + wres(Pa2, y2.x - o2.x, 0.f) +
                        wres(Pb2, y2.y - o2.y, 0.f);
               }
@@ -727,40 +766,56 @@ __device__ __forceinline__ float gcol_update(int mode, float2* Z, int c0, const 
               y1 = cadd(A, cmul_i(B));
               y2 = cadd(cconj(A), cmul_i(cconj(B)));
               if (cmp) {
-                const float2 o1 = prev[ky1 * L], o2c = cconj(prev[ky2 * L]);
+                const float2 o1 = prev(ky1, 0), o2c = cconj(prev(ky2, 0));
                 const float2 oA = cscale(cadd(o1, o2c), 0.5f);
                 const float2 oB = cmul_mi(cscale(csub(o1, o2c), 0.5f));
                 acc += 2.0f * (wres(Pa1, A.x - oA.x, A.y - oA.y) + wres(Pb1, B.x - oB.x, B.y - oB.y));
               }
             }
             if (store) {
-              prev[ky1 * L] = y1;
-              prev[ky2 * L] = y2;
+              prev(ky1, 0) = y1;
+              prev(ky2, 0) = y2;
             }
           });
     });
   } else {
     auto p2 = [](float P, float re, float im) -> float { return P * P * fmaf(re, re, im * im); };
-    gcol<N, false>(Z, c0, [&](float2 (&p)[G::A], float2 (&q)[G::A], int col, int h, int hb) {
-      gpairs<N>(
+    gcol<N, false, RB>(z, c0, [&](float2 (&p)[G::A], float2 (&q)[G::A], int col, int h, int hb) {
+      gpairs<N, RB>(
           p, q, col, h, hb, c0,
           [&](float2& y1, float2& y2, int ky1, int ky2) {
-            acc += 2.0f * (p2(__ldg(Pk + ky1 * WH + col), y1.x, y1.y) + p2(__ldg(Pk + ky2 * WH + col), y2.x, y2.y));
+            acc += 2.0f * (p2(Pk(ky1, col), y1.x, y1.y) + p2(Pk(ky2, col), y2.x, y2.y));
           },
           [&](float2& y1, float2& y2, int ky1, int ky2) {
             if (ky1 == 0) {
-              acc += p2(__ldg(Pk), y1.x, 0.f) + p2(__ldg(Pk + G::W / 2), y1.y, 0.f) +
-                     p2(__ldg(Pk + ky2 * WH), y2.x, 0.f) + p2(__ldg(Pk + ky2 * WH + G::W / 2), y2.y, 0.f);
+              acc += p2(Pk(0, 0), y1.x, 0.f) + p2(Pk(0, EW), y1.y, 0.f) +
+                     p2(Pk(ky2, 0), y2.x, 0.f) + p2(Pk(ky2, EW), y2.y, 0.f);
             } else {
               const float2 y2c = cconj(y2);
               const float2 A = cscale(cadd(y1, y2c), 0.5f);
               const float2 B = cmul_mi(cscale(csub(y1, y2c), 0.5f));
-              acc += 2.0f * (p2(__ldg(Pk + ky1 * WH), A.x, A.y) + p2(__ldg(Pk + ky1 * WH + G::W / 2), B.x, B.y));
+              acc += 2.0f * (p2(Pk(ky1, 0), A.x, A.y) + p2(Pk(ky1, EW), B.x, B.y));
             }
           });
     });
   }
   return acc;
+}
+
+// with the tables in global memory and the draws on the spot
+template <int N>
+__device__ __forceinline__ float gcol_update(int mode, float2* Z, int c0, const float2* __restrict__ fg,
+                                             const float* __restrict__ Pk, float2* prev, uint32_t step,
+                                             uint32_t chain, uint32_t key0, uint32_t key1, float ltau, bool cmp,
+                                             bool store) {
+  constexpr int L = N / 2, WH = N / 2 + 1;
+  auto draw = [&](uint32_t g, float (&z)[4]) { normals4(g, step, chain, 1u, key0, key1, z); };
+  return gcol_update<N>(
+      mode, ZCols<N>{Z + c0}, c0, [&](int ky, int kx) { return __ldg(fg + ky * WH + kx); },
+      [&](int ky, int kx) { return __ldg(Pk + ky * WH + kx); },
+      [&](int ky, int kx) -> float2& { return prev[ky * L + kx]; },
+      [&](int, uint32_t g, float (&z)[4]) { draw(g, z); }, [&](int ky, float (&z)[4]) { draw(uint32_t(ky), z); }, ltau,
+      cmp, store);
 }
 
 // mode 3: weighted power sums of CB columns of field f into acc[j], j < nw
@@ -769,7 +824,7 @@ __device__ void col_wpower(const GlobalArgs& a, int f, int c0, double (&acc)[4])
   using G = GGeo<N>;
   constexpr int WH = G::WH, TS = G::H * G::WH;
   auto sq = [](float p, float q) -> double { return double(p) * p + double(q) * q; };
-  gcol<N, false>(a.Z + (long long)f * G::H * G::LR, c0, [&](float2 (&p)[G::A], float2 (&q)[G::A], int col, int h, int hb) {
+  gcol<N, false>(ZCols<N>{a.Z + (long long)f * G::H * G::LR + c0}, c0, [&](float2 (&p)[G::A], float2 (&q)[G::A], int col, int h, int hb) {
     gpairs<N>(
         p, q, col, h, hb, c0,
         [&](float2& y1, float2& y2, int ky1, int ky2) {

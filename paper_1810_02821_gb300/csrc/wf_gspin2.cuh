@@ -188,12 +188,12 @@ __global__ void __launch_bounds__(GGeo<N>::T, GGeo<N>::MIN_CTAS) k_gspin2(const 
   for (int done = 0;; ++done) {  // sweeps completed
     for (int it = blockIdx.x; it < row_items; it += nb) {
       const int f = it / G::ROW_ITEMS, comp = f & 1, ci = f / 2, y = (it % G::ROW_ITEMS) * G::RB + ty;
-      float2* Zrow = a.Z + f * nz + (long long)y * G::LR;
+      const ZRow z{a.Z + f * nz + (long long)y * G::LR};
       float2 x[G::E];
       if (done == 0)
         grow_load<N>(x, a.s.init_s ? a.s.init_s + ci * a.s.init_stride + comp * n + (long long)y * G::W : nullptr);
       else
-        grow_inv<N>(Zrow, x);
+        grow_inv<N>(z, x);
       if (done > a.s.burn_in && (done - a.s.burn_in) % a.s.thin == 0) {
         const long long m = (done - a.s.burn_in) / a.s.thin - 1;
         grow_store<N>(x, a.s.out, ((ci * a.s.n_samples + m) * 2 + comp) * G::H + y, a.s.out_dtype);
@@ -201,7 +201,7 @@ __global__ void __launch_bounds__(GGeo<N>::T, GGeo<N>::MIN_CTAS) k_gspin2(const 
       if (done == a.s.n_sweeps) continue;
       pixel_update<N>(DRAW ? 0 : 4, x, y, a.s.aq2 + comp * n, nullptr, a.s.step0 + uint32_t(done),
                       a.s.chain0 + uint32_t(ci), a.s.key0, a.s.key1, sqrt_tau, 0.f, 0, 0.f, 8u * uint32_t(comp));
-      grow_fwd<N>(x, Zrow);
+      grow_fwd<N>(x, z);
     }
     if (done == a.s.n_sweeps) return;
     if (!grid_barrier(a.bar, nb, target)) return;

@@ -12,6 +12,7 @@
 #include "wf_bphase.cuh"
 #include "wf_core.cuh"
 #include "wf_gspin2.cuh"
+#include "wf_gcluster.cuh"
 
 namespace wf {
 
@@ -60,6 +61,13 @@ cudaError_t batch_grid(int n_items, int grid_pct, int* grid_out);
 // large images (N >= 256): one cooperative launch of k_global<N> (all CTAs co-resident)
 template <int N>
 cudaError_t launch_global(const GlobalArgs& a, cudaStream_t st, LaunchTimer* t);
+
+// the same sampler (mode 0) and Wiener filter (mode 1) with each field in one cluster (N in {128, 256}; a.Z, a.bar, a.acc
+// and a.prev unused); gcluster_count: clusters resident at once on the current device, 0 if they cannot run
+template <int N>
+cudaError_t launch_gcluster(const GlobalArgs& a, cudaStream_t st, LaunchTimer* t);
+template <int N>
+cudaError_t gcluster_count(bool solve, int* clusters);
 
 // batched large images (N >= 256): one cooperative launch of k_gbatch<N> over all fields of a size class
 template <int N>
@@ -363,6 +371,54 @@ cudaError_t launch_gspin2(const GSpin2Args& a, cudaStream_t st, LaunchTimer* t) 
 #define WF_INSTANTIATE_GLOBAL(N)                                                               \
   WF_INSTANTIATE_GLOBAL_ONE(N)                                                                  \
   template cudaError_t launch_gbatch<N>(const GBArgs&, cudaStream_t);
+#endif
+
+#if defined(WF_LAUNCH_DEFINE_GCLUSTER)
+template <int N>
+cudaError_t gcluster_config(bool solve, int n_fields, cudaStream_t st, cudaLaunchConfig_t* cfg,
+                            cudaLaunchAttribute* attr) {
+  using K = GCl<N>;
+  auto kern = solve ? k_gcluster<N, true> : k_gcluster<N, false>;
+  const int smem = solve ? K::SMEM_SOLVE : K::SMEM_SAMPLE;
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  if (e != cudaSuccess) return e;
+  if (K::C > 8 && (e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1)) != cudaSuccess)
+    return e;
+  attr->id = cudaLaunchAttributeClusterDimension;
+  attr->val.clusterDim.x = K::C;
+  attr->val.clusterDim.y = attr->val.clusterDim.z = 1;
+  *cfg = cudaLaunchConfig_t{};
+  cfg->gridDim = dim3(unsigned(n_fields) * K::C);
+  cfg->blockDim = dim3(K::T);
+  cfg->dynamicSmemBytes = smem;
+  cfg->stream = st;
+  cfg->attrs = attr;
+  cfg->numAttrs = 1;
+  return cudaSuccess;
+}
+template <int N>
+cudaError_t gcluster_count(bool solve, int* clusters) {
+  cudaLaunchConfig_t cfg;
+  cudaLaunchAttribute attr;
+  const cudaError_t e = gcluster_config<N>(solve, 1, nullptr, &cfg, &attr);
+  if (e != cudaSuccess) return e;
+  return solve ? cudaOccupancyMaxActiveClusters(clusters, k_gcluster<N, true>, &cfg)
+               : cudaOccupancyMaxActiveClusters(clusters, k_gcluster<N, false>, &cfg);
+}
+template <int N>
+cudaError_t launch_gcluster(const GlobalArgs& a, cudaStream_t st, LaunchTimer* t) {
+  cudaLaunchConfig_t cfg;
+  cudaLaunchAttribute attr;
+  cudaError_t e = gcluster_config<N>(a.mode == 1, a.n_fields, st, &cfg, &attr);
+  if (e != cudaSuccess) return e;
+  if (t) t->start();
+  e = a.mode == 1 ? cudaLaunchKernelEx(&cfg, k_gcluster<N, true>, a) : cudaLaunchKernelEx(&cfg, k_gcluster<N, false>, a);
+  if (t) t->stop();
+  return e != cudaSuccess ? e : cudaGetLastError();
+}
+#define WF_INSTANTIATE_GCLUSTER(N)                                                          \
+  template cudaError_t gcluster_count<N>(bool, int*);                                        \
+  template cudaError_t launch_gcluster<N>(const GlobalArgs&, cudaStream_t, LaunchTimer*);
 #endif
 
 #if defined(WF_LAUNCH_DEFINE_CLUSTER)
