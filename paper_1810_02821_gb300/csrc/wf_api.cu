@@ -182,19 +182,21 @@ cudaError_t launch_prep(const float* d, const float* Ndiag, const uint8_t* mask,
   return launch_prep_kernel(k_prep, 1, H, st, d, Ndiag, mask, Pk, H, W, tau_user, eta, sc);
 }
 
-int gcluster_max(int H, bool solve);
+int few_max(int H, bool solve);
 
-constexpr int kFew128 = 36, kFewSpin2 = 40;  // chains from which the on-chip kernels run at 128^2
+constexpr int kFew64 = 115, kFew128 = 36, kFewSpin2 = 40;  // chains from which the on-chip kernels run
 bool size_on_chip(int H) { return H <= 128; }
-// Whether fields of an on-chip size run on the on-chip kernels, one CTA per field, or spread over several SMs. At 128^2
-// the latter has less latency for few fields (us per sweep of all chains): the sampler in clusters of 8 CTAs takes 3.8
-// for up to 14 chains, 4.8 for 36 and 5.6 for the 48 that are resident at once, on chip 9.6 (60 chains, two rounds of
-// clusters: as long). On a device without such clusters the global-memory kernel takes 6.4 to 9.2 for up to 36 chains.
-// Spin-2, global-memory / on chip: 1 chain 7.6 / 22.9, 39 chains 20.6 / 22.9. A Wiener filter 4.0 (cluster) / 8.0 (from
-// zero only: the other paths take no starting iterate).
+// Whether fields of an on-chip size run on the on-chip kernels, one CTA per field, or spread over several SMs (k_few:
+// clusters, where the device has them; else k_global at 128^2), with less latency for few fields. us per sweep of all
+// chains: sampler 64^2 clusters / on chip 1 chain 3.2 / 3.9, 114 chains 4.3 / 4.6, 152 chains 4.8 / 4.7; 128^2 clusters 3.8
+// for up to 14 chains, 4.8 for 36, 5.6 for the 48 that are resident at once, on chip 9.6 (60 chains, two rounds of
+// clusters: as long), k_global 6.4 to 9.2 for up to 36. A Wiener filter 64^2 3.3 / 3.1, 128^2 3.9 / 8.0 (from zero only: the
+// other paths take no starting iterate). Spin-2 128^2, k_few2 / on chip: 1 chain 5.7 / 22.9, 36 chains 8.2 / 22.9; without
+// clusters k_gspin2 takes 7.6 for 1 chain, 20.6 for 39.
 bool sample_on_chip(int H, int units) {
+  if (H == 64) return g_large_sampler != 0 || units >= kFew64 || units > few_max(64, false);
   if (H != 128) return size_on_chip(H);
-  const int few = gcluster_max(H, false);
+  const int few = few_max(H, false);
   return units > (few > 0 ? few : kFew128 - 1);
 }
 bool spin2_on_chip(int H, int units) { return size_on_chip(H) && !(H == 128 && units < kFewSpin2); }
@@ -345,38 +347,72 @@ bool out_ptr_ok(const void* p) {
   return true;
 }
 
-// Fields of a launch up to which k_gcluster takes the place of k_global: as many clusters as are resident at once on
-// the device (0: none). us per sweep of all chains, k_global / k_gcluster, the same results bit for bit: 128^2 1 chain
-// 6.5 / 3.8, 12 chains 6.8 / 3.8, 35 chains 9.2 / 4.8; 256^2 1 chain 7.0 / 5.3, 7 chains 8.1 / 5.3, 14 chains 10.2 / 7.4;
-// Wiener filter 128^2 7.0 / 4.0, 256^2 7.3 / 5.5. A second round of clusters would cost as much as the first (256^2, 16
-// chains: 11.8 on k_global).
-int gcluster_max(int H, bool solve) {
-  if (H != 128 && H != 256) return 0;
-  static std::mutex mu;
-  static int known[2][2][64] = {};  // clusters + 1
+// fields resident at once on the current device, queried once per device (known: fields + 1)
+template <class F>
+int resident_fields(std::mutex& mu, int (&known)[64], F&& query) {
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) {
     cudaGetLastError();
     return 0;
   }
   std::lock_guard<std::mutex> lock(mu);
-  int& k = known[H == 256][solve][dev];
-  if (k == 0) {
+  if (known[dev] == 0) {
     int n = 0;
-    const cudaError_t e = H == 128 ? wf::gcluster_count<128>(solve, &n) : wf::gcluster_count<256>(solve, &n);
-    if (e != cudaSuccess) {
+    if (query(&n) != cudaSuccess) {
       cudaGetLastError();
       n = 0;
     }
-    k = n + 1;
+    known[dev] = n + 1;
   }
-  return k - 1;
+  return known[dev] - 1;
+}
+
+// Fields of a launch up to which k_few takes the place of k_global: as many as are resident at once on the device (0: it
+// cannot run). us per sweep of all chains, k_global / k_few, the same results bit for bit: 128^2 1 chain 6.5 / 3.8, 12 chains
+// 6.8 / 3.8, 35 chains 9.2 / 4.8; 256^2 1 chain 7.1 / 5.3, 7 chains 8.3 / 5.4, 14 chains 10.2 / 7.4; 512^2 1 chain 8.8 / 7.0,
+// 4 chains 11.8 / 9.4; 1024^2 1 chain 13.1 / 10.7; Wiener filter 128^2 6.9 / 3.9, 256^2 7.5 / 5.3, 512^2 9.2 / 7.7, 1024^2
+// 13.9 / 11.3. A second round of clusters would cost as much as the first (256^2, 16 chains: 11.8 on k_global).
+int few_max(int H, bool solve) {
+  static std::mutex mu;
+  static int known[5][2][64] = {};  // fields + 1
+  auto count = [=](int* n) {
+    switch (H) {
+      case 64: return wf::few_count<64>(solve, n);
+      case 128: return wf::few_count<128>(solve, n);
+      case 256: return wf::few_count<256>(solve, n);
+      case 512: return wf::few_count<512>(solve, n);
+      default: return wf::few_count<1024>(solve, n);
+    }
+  };
+  if (H < 64) return 0;
+  return resident_fields(mu, known[H == 64 ? 0 : H == 128 ? 1 : H == 256 ? 2 : H == 512 ? 3 : 4][solve], count);
+}
+// The same for the spin-2 sampler and (quiet) filter, k_gspin2 / k_few2: 128^2 1 pair 7.4 / 5.7, 30 pairs 16.8 / 8.1; 256^2
+// 1 pair 8.1 / 6.0, 9 pairs 14.8 / 11.6 (a cluster of 16 CTAs per pair took 9.7 for up to 7 pairs: four warps a scheduler);
+// 512^2 1 pair 10.7 / 8.1, 2 pairs 14.2 / 11.3.
+int few2_max(int H, bool quiet) {
+  static std::mutex mu;
+  static int known[3][2][64] = {};
+  auto count = [=](int* n) {
+    switch (H) {
+      case 128: return wf::few2_count<128>(quiet, n);
+      case 256: return wf::few2_count<256>(quiet, n);
+      default: return wf::few2_count<512>(quiet, n);
+    }
+  };
+  if (H < 128 || H > 512) return 0;
+  return resident_fields(mu, known[H == 128 ? 0 : H == 256 ? 1 : 2][quiet], count);
 }
 
 cudaError_t launch_global_any(int H, const wf::GlobalArgs& a, cudaStream_t st, wf::LaunchTimer* t) {
-  if (a.mode <= 1 && g_large_sampler == 0 && a.n_fields <= gcluster_max(H, a.mode == 1)) {
-    if (H == 128) return wf::launch_gcluster<128>(a, st, t);
-    return wf::launch_gcluster<256>(a, st, t);
+  if (a.mode <= 1 && g_large_sampler == 0 && a.n_fields <= few_max(H, a.mode == 1)) {
+    switch (H) {
+      case 64: return wf::launch_few<64>(a, st, t);  // sampler only
+      case 128: return wf::launch_few<128>(a, st, t);
+      case 256: return wf::launch_few<256>(a, st, t);
+      case 512: return wf::launch_few<512>(a, st, t);
+      case 1024: return wf::launch_few<1024>(a, st, t);
+    }
   }
   switch (H) {
     case 128: return wf::launch_global<128>(a, st, t);
@@ -1183,13 +1219,17 @@ wf_status wf_sample_band(const float* d, const float* Ndiag, const uint8_t* mask
 namespace {
 // one launch of the spin-2 sweeps (tables in the order of spin2_orders); Z, bar: scratch of the global-memory form
 struct Spin2Path {
-  bool global = false;
+  bool global = false, few = false;  // the global-memory kernels; k_few2 in their place
   int cm = 0, perm = 0;  // table orders (k_tables)
   size_t z_count = 0;    // float2 of Z
 };
-Spin2Path spin2_path(int H, int chains) {
+Spin2Path spin2_path(int H, int chains, bool quiet) {
   Spin2Path p;
-  if (spin2_on_chip(H, chains)) {
+  if (g_large_sampler == 0 && chains <= few2_max(H, quiet)) {
+    p.few = p.global = true;
+    p.perm = -1;
+    p.z_count = size_t(chains) * H * H;
+  } else if (spin2_on_chip(H, chains)) {
     p.cm = wf::core_cm(H);
   } else if (H >= 256 && spin2_use_cluster(H, chains)) {
     p.cm = 32;
@@ -1207,6 +1247,11 @@ cudaError_t launch_spin2_any(int H, const Spin2Path& p, const wf::Spin2Args& a, 
     const cudaError_t e = cudaMemsetAsync(&bar->count, 0, sizeof(bar->count), st);  // err collects over launches
     if (e != cudaSuccess) return e;
     const wf::GSpin2Args g{a, Z, bar};
+    if (p.few) switch (H) {
+      case 128: return wf::launch_few2<128>(g, st, t);
+      case 256: return wf::launch_few2<256>(g, st, t);
+      case 512: return wf::launch_few2<512>(g, st, t);
+    }
     switch (H) {
       case 128: return wf::launch_gspin2<128>(g, st, t);
       case 256: return wf::launch_gspin2<256>(g, st, t);
@@ -1263,7 +1308,7 @@ wf_status wf_sample_spin2(const float* d1, const float* d2, const float* N1, con
     mask = r1.mask;
   }
   const size_t n = size_t(H) * W, nm = size_t(H) * (W / 2 + 1);
-  const Spin2Path path = spin2_path(H, o.n_chains);
+  const Spin2Path path = spin2_path(H, o.n_chains, false);
   Carve cv;
   const size_t o_sc = cv.take<wf::Scalars>(2), o_bar = cv.take<wf::GridBar>(1), o_aq = cv.take<float2>(2 * n),
                o_fe = cv.take<float2>(nm), o_fb = cv.take<float2>(nm), o_z = cv.take<float2>(path.z_count);
@@ -1374,7 +1419,7 @@ wf_status wf_solve_spin2(const float* d1, const float* d2, const float* N1, cons
   }
   const size_t n = size_t(H) * W, nm = size_t(H) * (W / 2 + 1);
   Carve cv;
-  const Spin2Path path = spin2_path(H, 1);
+  const Spin2Path path = spin2_path(H, 1, true);
   const size_t o_sc = cv.take<wf::Scalars>(3), o_bar = cv.take<wf::GridBar>(1), o_aq = cv.take<float2>(2 * n),
                o_fe = cv.take<float2>(nm), o_fb = cv.take<float2>(nm), o_r = cv.take<double>(2),
                o_x = cv.take<double2>(2 * n), o_z = cv.take<float2>(path.z_count);

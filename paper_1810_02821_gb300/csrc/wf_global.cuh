@@ -46,9 +46,10 @@ struct GGeo {
   static constexpr int T = RB * TR;                // threads per CTA
   static constexpr int CB = T / TC;                // columns per CTA (RB / 2)
   static constexpr int BR = LR / A, BC = H / A;    // frequency strides of the units
-  // float2 strides of a row's and a column's vector: 8 blocks of L1 + 2; columns 16/CB modulo 16 apart (a half-warp
-  // holds CB columns)
-  static constexpr int VROW = LR + 16 + 8, VCOL = H + 16 + 16 / CB;
+  // float2 strides of a row's and a column's vector: 8 blocks of L1 + 2; short rows TR, columns 4 or 2 modulo 16 apart (a half-warp
+  // holds 4 or 8 columns)
+  static constexpr int CW = CB < 8 ? CB : 8;
+  static constexpr int VROW = LR + 16 + (TR < 8 ? TR : 8), VCOL = H + 16 + 16 / CW;
   static constexpr int VEC = RB * VROW > CB * VCOL ? RB * VROW : CB * VCOL;
   // twiddle tables: T1 [q1][n0] (rows of n/8 + 2), T2 and T3 [q][n1] of the rows and columns, W_W^K (K < LR/2)
   static constexpr int O_T1R = VEC, O_T2R = O_T1R + 8 * (LR / 8 + 2), O_T3R = O_T2R + LR / 8, O_T1C = O_T3R + 16,
@@ -60,13 +61,13 @@ struct GGeo {
   static constexpr int WH = W / 2 + 1;
   // CTAs per SM the kernels are compiled for: up to 128 registers a thread with 16 elements, 80 with 8
   static constexpr int MIN_CTAS = (E == 16 ? 512 : 768) / T;
-  static_assert((CB == 4 || CB == 8) && TR <= 32 && VCOL % 16 == 16 / CB, "geometry");
+  static_assert((CB == 4 || CB % 8 == 0) && TR <= 32 && VCOL % 16 == 16 / CW, "geometry");
 };
 
 // middle radices of a transform of length n
 template <int n, int E>
 struct GRad {
-  static constexpr int M = n / (4 * E);
+  static constexpr int M = n / (4 * E);  // 1: no middle pass
   static constexpr int R2 = M <= E ? M : 4, R3 = M / R2;
   static constexpr int L1 = n / 8, S = L1 + 2, STEP2 = L1 / R2, STEP3 = STEP2 / R3;
   static_assert(R2 * R3 == M && STEP3 == E / 2 && (R3 == 1 || STEP2 == 16), "passes");
@@ -121,7 +122,7 @@ __device__ __forceinline__ int gunit(int q) {
 template <int n, int E>
 __device__ __forceinline__ const float2* gunit_tw(int q, const GTab& t) {
   using R = GRad<n, E>;
-  return R::R3 == 1 ? t.t2 + (E / 2) * (q / 8) : t.t3 + (E / 2) * (q / 8 / R::R2);
+  return R::R2 == 1 ? t.t1 + R::S * q : R::R3 == 1 ? t.t2 + (E / 2) * (q / 8) : t.t3 + (E / 2) * (q / 8 / R::R2);
 }
 
 // pass 1: x[i 8 + m] = element n0 + L1 m, n0 = (E/8) h + i
@@ -175,19 +176,21 @@ template <int n, int E, bool INV, class Sync>
 __device__ __forceinline__ void gmid(float2* v, int h, const GTab& t, Sync&& sync) {
   using R = GRad<n, E>;
   auto pass2 = [&] {
-    constexpr int STEP = R::STEP2;
+    if constexpr (R::R2 > 1) {
+      constexpr int STEP = R::STEP2;
 #pragma unroll
-    for (int i = 0; i < E / R::R2; ++i) {
-      const int idx = h + (n / E) * i, n1 = (idx & 1) + 2 * (idx >> 4), q1 = (idx >> 1) & 7;
-      float2* u = v + q1 * R::S + n1;
-      float2 c[R::R2];
+      for (int i = 0; i < E / R::R2; ++i) {
+        const int idx = h + (n / E) * i, n1 = (idx & 1) + 2 * (idx >> 4), q1 = (idx >> 1) & 7;
+        float2* u = v + q1 * R::S + n1;
+        float2 c[R::R2];
 #pragma unroll
-      for (int m = 0; m < R::R2; ++m) c[m] = u[STEP * m];
-      fft<R::R2, INV>(c);
+        for (int m = 0; m < R::R2; ++m) c[m] = u[STEP * m];
+        fft<R::R2, INV>(c);
 #pragma unroll
-      for (int m = 0; m < R::R2; ++m) {
-        if (!INV) u[STEP * m] = m == 0 ? c[0] : cmul(c[m], t.t2[STEP * m + n1]);
-        else u[STEP * m] = cmul(c[m], cconj(t.t1[q1 * R::S + n1 + STEP * m]));
+        for (int m = 0; m < R::R2; ++m) {
+          if (!INV) u[STEP * m] = m == 0 ? c[0] : cmul(c[m], t.t2[STEP * m + n1]);
+          else u[STEP * m] = cmul(c[m], cconj(t.t1[q1 * R::S + n1 + STEP * m]));
+        }
       }
     }
   };
@@ -211,7 +214,8 @@ __device__ __forceinline__ void gmid(float2* v, int h, const GTab& t, Sync&& syn
       }
     }
   };
-  if constexpr (R::R3 == 1) {
+  if constexpr (R::R2 == 1) {
+  } else if constexpr (R::R3 == 1) {
     pass2();
   } else if constexpr (INV) {
     pass3();
@@ -258,6 +262,21 @@ struct GridBar {
   int pad;
 };
 
+// the two halves, by one thread of each CTA
+__device__ __forceinline__ void grid_arrive(GridBar* gb) {
+  asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(&gb->count), "r"(1u) : "memory");
+}
+__device__ __forceinline__ bool grid_wait(GridBar* gb, unsigned int target) {
+  int ok = 0;
+  for (long it = 0; !ok && it < (1L << 22); ++it) {
+    unsigned int c;
+    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(c) : "l"(&gb->count) : "memory");
+    ok = int(c - target) >= 0;
+    if (!ok && (it & 255) == 255 && *reinterpret_cast<volatile int*>(&gb->err) != 0) break;
+  }
+  if (!ok) atomicExch(&gb->err, 7);  // WF_ERR_TIMEOUT
+  return ok != 0;
+}
 // opened(): run by thread 0 once the barrier has opened, before the CTA goes on
 template <class F>
 __device__ __forceinline__ bool grid_barrier(GridBar* gb, unsigned int nblocks, unsigned int& target, F&& opened) {
@@ -265,16 +284,9 @@ __device__ __forceinline__ bool grid_barrier(GridBar* gb, unsigned int nblocks, 
   __shared__ int s_ok;
   target += nblocks;
   if (threadIdx.x == 0) {
-    asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(&gb->count), "r"(1u) : "memory");
-    int ok = 0;
-    for (long it = 0; !ok && it < (1L << 22); ++it) {
-      unsigned int c;
-      asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(c) : "l"(&gb->count) : "memory");
-      ok = int(c - target) >= 0;
-      if (!ok && (it & 255) == 255 && *reinterpret_cast<volatile int*>(&gb->err) != 0) break;
-    }
+    grid_arrive(gb);
+    const bool ok = grid_wait(gb, target);
     if (ok) opened();
-    else atomicExch(&gb->err, 7);  // WF_ERR_TIMEOUT
     s_ok = ok;
   }
   __syncthreads();

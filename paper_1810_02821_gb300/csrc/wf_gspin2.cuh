@@ -21,25 +21,23 @@ struct GSpin2Args {
   GridBar* bar;
 };
 
-// two columns c0, c0 + 1 of both components of one chain: transform, draw, transform back
-template <int N, bool DRAW>
-__device__ __forceinline__ void gcol_spin2(const GSpin2Args& a, float2* Z, int c0, uint32_t step, uint32_t chain) {
-  using G = GGeo<N>;
-  constexpr int H = G::H, LR = G::LR, BC = G::BC, E = G::E, A = G::A, NC = E / 8, WH = G::WH;
-  const int comp = threadIdx.x & 1, col = c0 + int(threadIdx.x % 4) / 2;
-  const int h = threadIdx.x / 4, hb = h == 0 ? BC / 2 : BC - h;
-  const GTab t = gtab<N, false>();
-  const float2* __restrict__ fgE = a.s.fgE;
-  const float2* __restrict__ fgB = a.s.fgB;
-  const uint32_t k0 = a.s.key0, k1 = a.s.key1;
-  float2* v = gsmem() + (threadIdx.x % 4) * G::VCOL;
-  float2* Zc = Z + (long long)comp * H * LR + (long long)(NC * h) * LR + col;
+// The thread's column `col` of component `comp` (its vector v): transform, draw, transform back. zc: rows of the
+// column from NC h on (ZCols::at); e: 2 H float2 for the pairs of column 0, edge: whether the CTA holds it; fE(ky, kx),
+// fB(ky, kx): the mode tables; draw(j, group, zE, zB): the normals of the thread's j-th pair, edraw(ky, zE, zB): those
+// of a pair of column 0. Components in neighbouring lanes, comp = tid & 1.
+template <int N, int RB, bool DRAW, class Z, class FE, class FB, class D, class X>
+__device__ __forceinline__ void gcol_spin2(const Z& zc, float2* v, float2* e, bool edge, int col, int h, FE&& fE,
+                                           FB&& fB, D&& draw, X&& edraw) {
+  using G = GGeo<N, RB>;
+  constexpr int H = G::H, BC = G::BC, E = G::E, A = G::A, NC = E / 8;
+  const int comp = threadIdx.x & 1, hb = h == 0 ? BC / 2 : BC - h;
+  const GTab t = gtab<N, false, RB>();
   {
     float2 x[E];
 #pragma unroll
     for (int m = 0; m < 8; ++m)
 #pragma unroll
-      for (int i = 0; i < NC; ++i) x[8 * i + m] = __ldcg(Zc + (long long)(H / 8 * m + i) * LR);
+      for (int i = 0; i < NC; ++i) x[8 * i + m] = zc.ld(H / 8 * m + i);
     gfwd1<H, E>(v, h, x, t);
   }
   __syncthreads();
@@ -50,8 +48,7 @@ __device__ __forceinline__ void gcol_spin2(const GSpin2Args& a, float2* Z, int c
     gfwd_unit<H, E>(v, h, p);
     gfwd_unit<H, E>(v, hb, q);
     if (h == 0) unit0_swap<A>(p, q);
-    float2* e = gsmem() + G::O_EDGE;  // parked pairs of column 0: component 0, then component 1 (H float2 each)
-    if (c0 == 0) {
+    if (edge) {  // the same in every thread of the CTA; e: component 0, then component 1 (H float2 each)
       if (col == 0) {
         float2* ec = e + comp * H;
 #pragma unroll
@@ -66,15 +63,12 @@ __device__ __forceinline__ void gcol_spin2(const GSpin2Args& a, float2* Z, int c
       for (int k = threadIdx.x; k < H / 2; k += G::T) {
         float2 y1a = e[2 * k], y2a = e[2 * k + 1], y1b = e[H + 2 * k], y2b = e[H + 2 * k + 1];
         float zE[4] = {0.f, 0.f, 0.f, 0.f}, zB[4] = {0.f, 0.f, 0.f, 0.f};
-        if (DRAW) {
-          normals4(uint32_t(k), step, chain, 1u, k0, k1, zE);
-          normals4(uint32_t(k), step, chain, 9u, k0, k1, zB);
-        }
+        if (DRAW) edraw(k, zE, zB);
         if (k == 0) {
           // four real modes, each on k = 0 or a Nyquist line: no rotation, real draws with variance g^2
           constexpr float R2 = 1.41421356237309505f;
           auto upd = [&](float& u, float& w, int ky, int kx, float ze, float zb) {
-            const float2 mE = __ldg(fgE + ky * WH + kx), mB = __ldg(fgB + ky * WH + kx);
+            const float2 mE = fE(ky, kx), mB = fB(ky, kx);
             u = fmaf(mE.x, u, R2 * mE.y * ze);
             w = fmaf(mB.x, w, R2 * mB.y * zb);
           };
@@ -87,10 +81,9 @@ __device__ __forceinline__ void gcol_spin2(const GSpin2Args& a, float2* Z, int c
           float2 A2 = cscale(cadd(y1b, cconj(y2b)), 0.5f), B2 = cmul_mi(cscale(csub(y1b, cconj(y2b)), 0.5f));
           float c, s;
           ks_rot<N>(k, 0, c, s);
-          spin2_mode(A1, A2, c, s, __ldg(fgE + k * WH), __ldg(fgB + k * WH), zE[0], zE[1], zB[0], zB[1]);
+          spin2_mode(A1, A2, c, s, fE(k, 0), fB(k, 0), zE[0], zE[1], zB[0], zB[1]);
           ks_rot<N>(k, G::W / 2, c, s);
-          spin2_mode(B1, B2, c, s, __ldg(fgE + k * WH + G::W / 2), __ldg(fgB + k * WH + G::W / 2), zE[2], zE[3], zB[2],
-                     zB[3]);
+          spin2_mode(B1, B2, c, s, fE(k, G::W / 2), fB(k, G::W / 2), zE[2], zE[3], zB[2], zB[3]);
           y1a = cadd(A1, cmul_i(B1));
           y2a = cadd(cconj(A1), cmul_i(cconj(B1)));
           y1b = cadd(A2, cmul_i(B2));
@@ -116,16 +109,12 @@ __device__ __forceinline__ void gcol_spin2(const GSpin2Args& a, float2* Z, int c
       float2 a2 = comp == 0 ? own2 : got2, b2 = comp == 0 ? got2 : own2;
       const int ky1 = lead + BC * j, ky2 = ky1 == 0 ? H / 2 : H - ky1;
       float zE[4] = {0.f, 0.f, 0.f, 0.f}, zB[4] = {0.f, 0.f, 0.f, 0.f};
-      if (DRAW) {
-        const uint32_t grp = uint32_t(col * (H / 2) + ky1);
-        normals4(grp, step, chain, 1u, k0, k1, zE);
-        normals4(grp, step, chain, 9u, k0, k1, zB);
-      }
+      if (DRAW) draw(j, uint32_t(col * (H / 2) + ky1), zE, zB);
       float c, s;
       ks_rot<N>(ky1, col, c, s);
-      spin2_mode(a1, b1, c, s, __ldg(fgE + ky1 * WH + col), __ldg(fgB + ky1 * WH + col), zE[0], zE[1], zB[0], zB[1]);
+      spin2_mode(a1, b1, c, s, fE(ky1, col), fB(ky1, col), zE[0], zE[1], zB[0], zB[1]);
       ks_rot<N>(ky2, col, c, s);
-      spin2_mode(a2, b2, c, s, __ldg(fgE + ky2 * WH + col), __ldg(fgB + ky2 * WH + col), zE[2], zE[3], zB[2], zB[3]);
+      spin2_mode(a2, b2, c, s, fE(ky2, col), fB(ky2, col), zE[2], zE[3], zB[2], zB[3]);
       const float2 back1 = swap1(comp == 0 ? b1 : a1), back2 = swap1(comp == 0 ? b2 : a2);
       if (comp == 0) {
         p[j] = a1;
@@ -139,7 +128,7 @@ __device__ __forceinline__ void gcol_spin2(const GSpin2Args& a, float2* Z, int c
         q[A - 1 - j] = back2;
       }
     }
-    if (c0 == 0) {
+    if (edge) {
       __syncthreads();
       if (col == 0) {
         const float2* ec = e + comp * H;
@@ -165,9 +154,29 @@ __device__ __forceinline__ void gcol_spin2(const GSpin2Args& a, float2* Z, int c
 #pragma unroll
     for (int m = 0; m < 8; ++m)
 #pragma unroll
-      for (int i = 0; i < NC; ++i) __stcg(Zc + (long long)(H / 8 * m + i) * LR, x[8 * i + m]);
+      for (int i = 0; i < NC; ++i) zc.st(H / 8 * m + i, x[8 * i + m]);
   }
   __syncthreads();
+}
+
+// two columns c0, c0 + 1 of both components of one chain in global memory
+template <int N, bool DRAW>
+__device__ __forceinline__ void gcols_spin2(const GSpin2Args& a, float2* Z, int c0, uint32_t step, uint32_t chain) {
+  using G = GGeo<N>;
+  constexpr int WH = G::WH;
+  const int vec = threadIdx.x % 4, col = c0 + vec / 2, h = threadIdx.x / 4;
+  const float2* __restrict__ fgE = a.s.fgE;
+  const float2* __restrict__ fgB = a.s.fgB;
+  auto draw = [&](uint32_t g, float (&zE)[4], float (&zB)[4]) {
+    normals4(g, step, chain, 1u, a.s.key0, a.s.key1, zE);
+    normals4(g, step, chain, 9u, a.s.key0, a.s.key1, zB);
+  };
+  gcol_spin2<N, 8, DRAW>(
+      ZCols<N>{Z + (long long)(vec & 1) * G::H * G::LR}.at((G::E / 8) * h, col), gsmem() + vec * G::VCOL,
+      gsmem() + G::O_EDGE, c0 == 0, col, h, [&](int ky, int kx) { return __ldg(fgE + ky * WH + kx); },
+      [&](int ky, int kx) { return __ldg(fgB + ky * WH + kx); },
+      [&](int, uint32_t g, float (&zE)[4], float (&zB)[4]) { draw(g, zE, zB); },
+      [&](int ky, float (&zE)[4], float (&zB)[4]) { draw(uint32_t(ky), zE, zB); });
 }
 
 template <int N>
@@ -207,7 +216,7 @@ __global__ void __launch_bounds__(GGeo<N>::T, GGeo<N>::MIN_CTAS) k_gspin2(const 
     if (!grid_barrier(a.bar, nb, target)) return;
     for (int it = blockIdx.x; it < col_items; it += nb) {
       const int ci = it / COL;
-      gcol_spin2<N, DRAW>(a, a.Z + 2LL * ci * nz, (it % COL) * 2, a.s.step0 + uint32_t(done),
+      gcols_spin2<N, DRAW>(a, a.Z + 2LL * ci * nz, (it % COL) * 2, a.s.step0 + uint32_t(done),
                           a.s.chain0 + uint32_t(ci));
     }
     if (!grid_barrier(a.bar, nb, target)) return;

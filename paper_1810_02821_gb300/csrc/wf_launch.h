@@ -3,6 +3,8 @@
 
 #include <cuda_runtime.h>
 
+#include <type_traits>
+
 #include "wf_gibbs.cuh"
 #include "wf_global.cuh"
 #include "wf_batch.cuh"
@@ -12,7 +14,7 @@
 #include "wf_bphase.cuh"
 #include "wf_core.cuh"
 #include "wf_gspin2.cuh"
-#include "wf_gcluster.cuh"
+#include "wf_few.cuh"
 
 namespace wf {
 
@@ -62,12 +64,17 @@ cudaError_t batch_grid(int n_items, int grid_pct, int* grid_out);
 template <int N>
 cudaError_t launch_global(const GlobalArgs& a, cudaStream_t st, LaunchTimer* t);
 
-// the same sampler (mode 0) and Wiener filter (mode 1) with each field in one cluster (N in {128, 256}; a.Z, a.bar, a.acc
-// and a.prev unused); gcluster_count: clusters resident at once on the current device, 0 if they cannot run
+// the same sampler (mode 0) and, from 128, Wiener filter (mode 1) for few fields (wf_few.cuh; N in {64 .. 1024}; a.prev
+// unused, a.Z, a.bar and a.acc up to 256 too). few_count: fields resident at once on the current device, 0 if it cannot run
 template <int N>
-cudaError_t launch_gcluster(const GlobalArgs& a, cudaStream_t st, LaunchTimer* t);
+cudaError_t launch_few(const GlobalArgs& a, cudaStream_t st, LaunchTimer* t);
 template <int N>
-cudaError_t gcluster_count(bool solve, int* clusters);
+cudaError_t few_count(bool solve, int* fields);
+// the spin-2 sampler and filter in the same way (N in {128, 256, 512}), natural table orders
+template <int N>
+cudaError_t launch_few2(const GSpin2Args& a, cudaStream_t st, LaunchTimer* t);
+template <int N>
+cudaError_t few2_count(bool quiet, int* pairs);
 
 // batched large images (N >= 256): one cooperative launch of k_gbatch<N> over all fields of a size class
 template <int N>
@@ -373,52 +380,98 @@ cudaError_t launch_gspin2(const GSpin2Args& a, cudaStream_t st, LaunchTimer* t) 
   template cudaError_t launch_gbatch<N>(const GBArgs&, cudaStream_t);
 #endif
 
-#if defined(WF_LAUNCH_DEFINE_GCLUSTER)
+#if defined(WF_LAUNCH_DEFINE_FEW)
+// launches of k_few and k_few2: one cluster per field, or a cooperative grid
+template <class X>
+struct FewLaunch {
+  cudaLaunchConfig_t cfg{};
+  cudaLaunchAttribute attr{};
+  template <class Kern>
+  cudaError_t set(Kern kern, int T, int smem, int n_fields, cudaStream_t st) {
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    if (e != cudaSuccess) return e;
+    if (X::CLUSTER) {
+      if (X::C > 8 &&
+          (e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1)) != cudaSuccess)
+        return e;
+      attr.id = cudaLaunchAttributeClusterDimension;
+      attr.val.clusterDim.x = unsigned(X::C);
+      attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+    } else {
+      attr.id = cudaLaunchAttributeCooperative;
+      attr.val.cooperative = 1;
+    }
+    cfg.gridDim = dim3(unsigned(n_fields) * unsigned(X::C));
+    cfg.blockDim = dim3(unsigned(T));
+    cfg.dynamicSmemBytes = size_t(smem);
+    cfg.stream = st;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    return cudaSuccess;
+  }
+  template <class Kern>
+  static cudaError_t count(Kern kern, int T, int smem, int* n) {
+    FewLaunch l;
+    cudaError_t e = l.set(kern, T, smem, 1, nullptr);
+    if (e != cudaSuccess) return e;
+    if (X::CLUSTER) return cudaOccupancyMaxActiveClusters(n, kern, &l.cfg);
+    int dev = 0, sms = 0, per_sm = 0;
+    if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
+    if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
+    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, T, smem)) != cudaSuccess) return e;
+    *n = per_sm * sms / X::C;
+    return cudaSuccess;
+  }
+  template <class Kern, class Args>
+  static cudaError_t run(Kern kern, int T, int smem, int n_fields, const Args& a, cudaStream_t st, LaunchTimer* t) {
+    FewLaunch l;
+    cudaError_t e = l.set(kern, T, smem, n_fields, st);
+    if (e != cudaSuccess) return e;
+    if (t) t->start();
+    e = cudaLaunchKernelEx(&l.cfg, kern, a);
+    if (t) t->stop();
+    return e != cudaSuccess ? e : cudaGetLastError();
+  }
+};
 template <int N>
-cudaError_t gcluster_config(bool solve, int n_fields, cudaStream_t st, cudaLaunchConfig_t* cfg,
-                            cudaLaunchAttribute* attr) {
-  using K = GCl<N>;
-  auto kern = solve ? k_gcluster<N, true> : k_gcluster<N, false>;
-  const int smem = solve ? K::SMEM_SOLVE : K::SMEM_SAMPLE;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-  if (e != cudaSuccess) return e;
-  if (K::C > 8 && (e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1)) != cudaSuccess)
-    return e;
-  attr->id = cudaLaunchAttributeClusterDimension;
-  attr->val.clusterDim.x = K::C;
-  attr->val.clusterDim.y = attr->val.clusterDim.z = 1;
-  *cfg = cudaLaunchConfig_t{};
-  cfg->gridDim = dim3(unsigned(n_fields) * K::C);
-  cfg->blockDim = dim3(K::T);
-  cfg->dynamicSmemBytes = smem;
-  cfg->stream = st;
-  cfg->attrs = attr;
-  cfg->numAttrs = 1;
-  return cudaSuccess;
+using FewX = std::conditional_t<N <= 256, XCluster<N, 1>, XGrid<N, 1>>;
+template <int N>
+using FewX2 = std::conditional_t<N <= 128, XCluster<N, 2>, XGrid<N, 2>>;
+template <int N>
+cudaError_t few_count(bool solve, int* fields) {
+  using X = FewX<N>;
+  using K = FewGeo<N, X>;
+  if constexpr (N >= 128)
+    if (solve) return FewLaunch<X>::count(k_few<N, X, true>, K::T, K::SMEM_SOLVE, fields);
+  return FewLaunch<X>::count(k_few<N, X, false>, K::T, K::SMEM_SAMPLE, fields);
 }
 template <int N>
-cudaError_t gcluster_count(bool solve, int* clusters) {
-  cudaLaunchConfig_t cfg;
-  cudaLaunchAttribute attr;
-  const cudaError_t e = gcluster_config<N>(solve, 1, nullptr, &cfg, &attr);
-  if (e != cudaSuccess) return e;
-  return solve ? cudaOccupancyMaxActiveClusters(clusters, k_gcluster<N, true>, &cfg)
-               : cudaOccupancyMaxActiveClusters(clusters, k_gcluster<N, false>, &cfg);
+cudaError_t launch_few(const GlobalArgs& a, cudaStream_t st, LaunchTimer* t) {
+  using X = FewX<N>;
+  using K = FewGeo<N, X>;
+  if constexpr (N >= 128)
+    if (a.mode == 1) return FewLaunch<X>::run(k_few<N, X, true>, K::T, K::SMEM_SOLVE, a.n_fields, a, st, t);
+  return FewLaunch<X>::run(k_few<N, X, false>, K::T, K::SMEM_SAMPLE, a.n_fields, a, st, t);
 }
 template <int N>
-cudaError_t launch_gcluster(const GlobalArgs& a, cudaStream_t st, LaunchTimer* t) {
-  cudaLaunchConfig_t cfg;
-  cudaLaunchAttribute attr;
-  cudaError_t e = gcluster_config<N>(a.mode == 1, a.n_fields, st, &cfg, &attr);
-  if (e != cudaSuccess) return e;
-  if (t) t->start();
-  e = a.mode == 1 ? cudaLaunchKernelEx(&cfg, k_gcluster<N, true>, a) : cudaLaunchKernelEx(&cfg, k_gcluster<N, false>, a);
-  if (t) t->stop();
-  return e != cudaSuccess ? e : cudaGetLastError();
+cudaError_t few2_count(bool quiet, int* pairs) {
+  using X = FewX2<N>;
+  using K = FewGeo<N, X>;
+  return FewLaunch<X>::count(quiet ? k_few2<N, X, false> : k_few2<N, X, true>, K::T, K::SMEM_SAMPLE, pairs);
 }
-#define WF_INSTANTIATE_GCLUSTER(N)                                                          \
-  template cudaError_t gcluster_count<N>(bool, int*);                                        \
-  template cudaError_t launch_gcluster<N>(const GlobalArgs&, cudaStream_t, LaunchTimer*);
+template <int N>
+cudaError_t launch_few2(const GSpin2Args& a, cudaStream_t st, LaunchTimer* t) {
+  using X = FewX2<N>;
+  using K = FewGeo<N, X>;
+  return FewLaunch<X>::run(a.s.quiet ? k_few2<N, X, false> : k_few2<N, X, true>, K::T, K::SMEM_SAMPLE, a.s.n_chains, a,
+                           st, t);
+}
+#define WF_INSTANTIATE_FEW(N)                       \
+  template cudaError_t few_count<N>(bool, int*);     \
+  template cudaError_t launch_few<N>(const GlobalArgs&, cudaStream_t, LaunchTimer*);
+#define WF_INSTANTIATE_FEW2(N)                      \
+  template cudaError_t few2_count<N>(bool, int*);    \
+  template cudaError_t launch_few2<N>(const GSpin2Args&, cudaStream_t, LaunchTimer*);
 #endif
 
 #if defined(WF_LAUNCH_DEFINE_CLUSTER)

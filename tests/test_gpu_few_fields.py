@@ -1,6 +1,6 @@
-"""Few fields of 128^2 and 256^2: one thread-block cluster per field against the same arithmetic with the fields in
-global memory (the same passes in the same order: equal bit for bit), up to and past the number of resident clusters."""
-import numpy as np
+"""Few large fields, a block of rows and columns per CTA for the whole launch (up to 256^2 in thread-block clusters),
+against the same passes in the same order with several blocks per CTA: equal bit for bit, up to and past the number of
+resident fields."""
 import pytest
 
 from gpu_common import need_gpu, rel, to_dev, torch
@@ -21,9 +21,10 @@ def in_global():
 
 
 @pytest.mark.parametrize("H,chains", [(128, 1), (128, 15), (128, 35), (128, 48), (128, 49), (256, 1), (256, 7),
-                                      (256, 8), (256, 14), (256, 15)])
+                                      (256, 8), (256, 14), (256, 15), (512, 1), (512, 4), (512, 5), (1024, 1),
+                                      (1024, 2)])
 @pytest.mark.parametrize("dtype", ["float32", "bfloat16"])
-def test_clusters_equal_global_memory(in_global, H, chains, dtype):
+def test_samples_equal_global_memory(in_global, H, chains, dtype):
     need_gpu()
     build.build()
     p = synth.make_problem(H, seed=H + chains, mask_frac=0.1)
@@ -43,9 +44,9 @@ def test_clusters_equal_global_memory(in_global, H, chains, dtype):
         assert torch.equal(a, b)
 
 
-@pytest.mark.parametrize("H", [128, 256])
+@pytest.mark.parametrize("H", [128, 256, 512, 1024])
 @pytest.mark.parametrize("check,refine", [(1, 0), (3, 0), (10, 2)])
-def test_filter_in_a_cluster(in_global, H, check, refine):
+def test_filter_equals_global_memory(in_global, H, check, refine):
     need_gpu()
     build.build()
     p = synth.make_problem(H, seed=H, mask_frac=0.2, k0=1 / 32)
@@ -59,3 +60,48 @@ def test_filter_in_a_cluster(in_global, H, check, refine):
         assert torch.equal(a.s, b.s)
     else:  # the FP64 residual's sums come from atomics
         assert rel(a.s.cpu().numpy(), b.s.cpu().numpy()) < 1e-6
+
+
+@pytest.mark.parametrize("H,chains", [(128, 1), (128, 15), (128, 30), (256, 1), (256, 4), (256, 9), (256, 10), (512, 1), (512, 2),
+                                      (512, 3)])
+def test_shear_samples_equal_global_memory(in_global, H, chains):
+    need_gpu()
+    build.build()
+    p, q = synth.make_problem(H, seed=H, mask_frac=0.1), synth.make_problem(H, seed=H + 1, mask_frac=0.1)
+    d, N, m, P = to_dev(p)
+    d2, N2 = to_dev(q)[:2]
+    args = (d, d2, N, N2, m, P, (0.2 * P).contiguous())
+    call = lambda: wf.wf_sample_spin2(*args, seed=3, n_samples=2, n_chains=chains, chain_offset=5, burn_in=1, thin=2)
+    assert torch.equal(call(), in_global(call))
+
+
+@pytest.mark.parametrize("H", [128, 256, 512])
+def test_shear_filter_equals_global_memory(in_global, H):
+    need_gpu()
+    build.build()
+    p, q = synth.make_problem(H, seed=H, mask_frac=0.1), synth.make_problem(H, seed=H + 1, mask_frac=0.1)
+    d, N, m, P = to_dev(p)
+    d2, N2 = to_dev(q)[:2]
+    call = lambda: wf.wf_solve_spin2(d, d2, N, N2, m, P, (0.2 * P).contiguous(), tol=1e-5)
+    a, b = call(), in_global(call)
+    assert a.iters == b.iters and torch.equal(a.s, b.s)
+
+
+@pytest.mark.parametrize("chains", [1, 7, 114, 115])
+def test_64_in_clusters(chains):
+    """64^2 in clusters of 4 CTAs (rows of 32 points: no middle pass) against the on-chip kernel: the same draws, FP32
+    roundings apart; the sweeps contract, so the differences stay at a few units in the last place of the field."""
+    need_gpu()
+    build.build()
+    p = synth.make_problem(64, seed=chains, mask_frac=0.1)
+    dev = to_dev(p)
+    s0 = torch.randn(chains, 64, 64, device="cuda")
+    call = lambda: wf.wf_sample_ex(*dev, seed=3, n_samples=4, n_chains=chains, chain_offset=2, start_step=3, burn_in=1,
+                                   thin=2, init_s=s0)
+    a = call()
+    wf.wf_set_large_image_sampler("global")  # on chip below 128
+    try:
+        b = call()
+    finally:
+        wf.wf_set_large_image_sampler("auto")
+    assert rel(a.cpu().numpy(), b.cpu().numpy()) < 2e-6
