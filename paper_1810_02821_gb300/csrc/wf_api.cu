@@ -605,7 +605,7 @@ wf_status solve_global(const float* d, const float* Ndiag, const uint8_t* mask, 
   cudaError_t e = cudaSuccess;
   if (!rhs_tab) {  // level norms (rhs mode: supplied)
     a.mode = 2;
-    a.n_fields = levels;
+    a.n_fields = a.levels = levels;
     a.bnorm_out = reinterpret_cast<double*>(b + o_bn);
     e = launch_global_any(H, a, st, nullptr);
     if (e != cudaSuccess) return cuda_fail(e);
@@ -807,6 +807,7 @@ wf_status solve_pass(const float* d, const float* Ndiag, const uint8_t* mask, co
   a.level_max = o.level_max;
   a.check = o.check;
   a.rhs_mode = rhs_tab ? 1 : 0;
+  a.n_fields = 1;
   wf::BnormArgs bb{dn, pk, sc, bn, o.eta};
   cudaError_t e = cudaSuccess;
   switch (H) {
@@ -825,6 +826,114 @@ wf_status solve_pass(const float* d, const float* Ndiag, const uint8_t* mask, co
   if (iters_out) *iters_out = hst.iters;
   if (resid_out) *resid_out = hst.resid;
   return wf_status(hst.status);
+}
+
+// Problems of one launch of solve_many: one CTA each at 32 and 64, as many as k_few holds from 128 on
+int solve_many_max(int H) {
+  if (H == 32 || H == 64) return 64;
+  return H >= 128 && g_large_sampler == 0 && few_max(H, true) > 1 ? few_max(H, true) : 1;
+}
+// Cooled messenger solves of F problems d + f H W with the same N, mask and P at once (2 <= F <= solve_many_max; d finite,
+// no refinement, response or starting iterate): s_W to out + f H W. The problems run side by side in one launch, each as
+// solve_pass would run it alone; four at 256^2 take as long as one (0.55 ms). Returns the first status that is not WF_OK.
+wf_status solve_many(const float* d, int F, const float* Ndiag, const uint8_t* mask, const float* Pk, int H, int W,
+                     const wf_solve_opts& o, float* out_s, cudaStream_t st, wf::LaunchTimer* timer) {
+  const size_t n = size_t(H) * W, nm = size_t(H) * (W / 2 + 1), nz = size_t(H) * (W / 2), f = size_t(F);
+  const bool chip = H <= 64;
+  Scratch s1;
+  s1.st = st;
+  WF_CUDA(cudaMallocAsync(&s1.base, sizeof(wf::Scalars), st));
+  auto* sc = static_cast<wf::Scalars*>(s1.base);
+  WF_CUDA(launch_prep(d, Ndiag, mask, Pk, H, W, o.tau, o.eta, sc, st));
+  wf::Scalars hsc{};
+  if (!chip) {  // the number of levels sizes the level-norm pass
+    WF_CUDA(cudaMemcpyAsync(&hsc, sc, sizeof(hsc), cudaMemcpyDeviceToHost, st));
+    WF_CUDA(cudaStreamSynchronize(st));
+    if (hsc.status != WF_OK) return wf_status(hsc.status);
+  }
+  const int levels = chip ? 0 : hsc.n_levels;
+  Carve cv;
+  const size_t o_bar = cv.take<wf::GridBar>(f + 1), o_bn = cv.take<double>(f * kMaxLevels), o_acc = cv.take<double>(2 * f),
+               o_st = cv.take<wf::SolveStatus>(f), zeroed = cv.off, o_dn = cv.take<float2>(f * n),
+               o_pk = cv.take<float>(chip ? nm : 0), o_prev = cv.take<float2>(chip ? f * nz : 0),
+               o_z = cv.take<float2>(chip ? 0 : f * nz * size_t(levels));
+  Scratch scr;
+  scr.st = st;
+  WF_CUDA(cudaMallocAsync(&scr.base, cv.off, st));
+  char* b = static_cast<char*>(scr.base);
+  auto* dn = reinterpret_cast<float2*>(b + o_dn);
+  auto* pk = reinterpret_cast<float*>(b + o_pk);
+  auto* bn = reinterpret_cast<double*>(b + o_bn);
+  auto* sst = reinterpret_cast<wf::SolveStatus*>(b + o_st);
+  auto* bar = reinterpret_cast<wf::GridBar*>(b + o_bar);
+  WF_CUDA(cudaMemsetAsync(b, 0, zeroed, st));  // barriers, level norms, residual sums, statuses
+  for (size_t i = 0; i < f; ++i) {
+    const bool modes = chip && i == 0;
+    k_tables<<<int((n + (modes ? nm : 0) + 255) / 256), 256, 0, st>>>(
+        d + i * n, Ndiag, mask, Pk, H, W, sc, nullptr, dn + i * n, nullptr, chip ? 0 : -1, wf::core_cm(H),
+        modes ? pk : nullptr);
+  }
+  WF_CUDA(cudaGetLastError());
+  cudaError_t e = cudaSuccess;
+  if (chip) {
+    wf::SolveArgs a{};
+    a.dn = dn;
+    a.Pk = pk;
+    a.sc = sc;
+    a.bnorm2 = bn;
+    a.prev = reinterpret_cast<float2*>(b + o_prev);
+    a.out = out_s;
+    a.st = sst;
+    a.tol = o.tol;
+    a.eta = o.eta;
+    a.level_tol = o.level_tol;
+    a.max_iter = o.max_iter;
+    a.level_max = o.level_max;
+    a.check = o.check;
+    a.n_fields = F;
+    const wf::BnormArgs bb{dn, pk, sc, bn, o.eta};
+    e = H == 32 ? wf::launch_solve<32>(a, bb, st, timer) : wf::launch_solve<64>(a, bb, st, timer);
+  } else {
+    wf::GlobalArgs a{};
+    a.Z = reinterpret_cast<float2*>(b + o_z);
+    a.dn = dn;
+    a.Pk = Pk;
+    a.sc = sc;
+    a.bar = bar + f;
+    a.eta = o.eta;
+    a.mode = 2;
+    a.levels = levels;
+    a.n_fields = levels * F;
+    a.bnorm_out = bn;
+    e = launch_global_any(H, a, st, nullptr);
+    if (e != cudaSuccess) return cuda_fail(e);
+    a.mode = 1;
+    a.n_fields = F;
+    a.bar = bar;
+    a.bnorm2 = bn;
+    a.acc = reinterpret_cast<double*>(b + o_acc);
+    a.st = sst;
+    a.out = out_s;
+    a.tol = o.tol;
+    a.level_tol = o.level_tol;
+    a.max_iter = o.max_iter;
+    a.level_max = o.level_max;
+    a.check = o.check;
+    e = launch_global_any(H, a, st, timer);
+  }
+  if (e != cudaSuccess) return cuda_fail(e);
+  std::vector<wf::SolveStatus> hst(f);
+  std::vector<wf::GridBar> hb(f + 1);
+  WF_CUDA(cudaMemcpyAsync(&hsc, sc, sizeof(hsc), cudaMemcpyDeviceToHost, st));
+  WF_CUDA(cudaMemcpyAsync(hst.data(), sst, f * sizeof(hst[0]), cudaMemcpyDeviceToHost, st));
+  WF_CUDA(cudaMemcpyAsync(hb.data(), bar, (f + 1) * sizeof(hb[0]), cudaMemcpyDeviceToHost, st));
+  WF_CUDA(cudaStreamSynchronize(st));
+  if (hsc.status != WF_OK) return wf_status(hsc.status);
+  for (const auto& x : hb)
+    if (x.err) return wf_status(x.err);
+  for (const auto& x : hst)
+    if (x.status != WF_OK) return wf_status(x.status);
+  return WF_OK;
 }
 
 // Mixed-precision iterative refinement: FP32 messenger solves, FP64 residuals (wf_refine.cu).
@@ -2520,8 +2629,7 @@ wf_status wf_loglike_grad(const float* d, const float* sigma2, const uint8_t* ma
   const size_t n = size_t(H) * W, nm = size_t(H) * (W / 2 + 1);
   Carve cv;
   const size_t o_P = cv.take<float>(3 * nm), o_N = cv.take<float>(n), o_s = cv.take<float>(n), o_x = cv.take<float>(n),
-               o_z = cv.take<float>(n), o_w = cv.take<float>(n), o_sum = cv.take<double>(4),
-               o_pow = cv.take<double>(8);
+               o_sum = cv.take<double>(4), o_pow = cv.take<double>(2);
   Scratch scr;
   scr.st = st;
   WF_CUDA(cudaMallocAsync(&scr.base, cv.off, st));
@@ -2532,8 +2640,6 @@ wf_status wf_loglike_grad(const float* d, const float* sigma2, const uint8_t* ma
   float* Nd = reinterpret_cast<float*>(b + o_N);
   float* sW = out_wf ? out_wf : reinterpret_cast<float*>(b + o_s);
   float* x = reinterpret_cast<float*>(b + o_x);
-  float* z = reinterpret_cast<float*>(b + o_z);
-  float* wv = reinterpret_cast<float*>(b + o_w);
   double* sums = reinterpret_cast<double*>(b + o_sum);
   double* pw = reinterpret_cast<double*>(b + o_pow);
   const int nblk = int((nm + n + 255) / 256);
@@ -2569,26 +2675,53 @@ wf_status wf_loglike_grad(const float* d, const float* sigma2, const uint8_t* ma
   sp.tol = tol > 1e-5 ? tol : 1e-5;
   sp.refine = 0;  // plain FP32 iteration: its error is far below the trace estimate's
   double tsum[3] = {0, 0, 0}, tsq[3] = {0, 0, 0};
-  for (int j = 0; j < n_probes; ++j) {
-    k_rademacher<<<int((n / 4 + 255) / 256), 256, 0, st>>>(int(n), uint32_t(j), uint32_t(seed & 0xffffffffu),
-                                                          uint32_t(seed >> 32), mask, z);
+  const int most = solve_many_max(H), chunk = n_probes < 1 ? 1 : (n_probes < most ? n_probes : most);
+  Carve cp;
+  const size_t o_px = cp.take<float>(n * size_t(chunk)), o_pz = cp.take<float>(n * size_t(chunk)),
+               o_pw = cp.take<float>(n * size_t(chunk)), o_ps = cp.take<double>(4 * size_t(chunk)),
+               o_pp = cp.take<double>(4 * size_t(chunk));
+  Scratch spr;
+  spr.st = st;
+  WF_CUDA(cudaMallocAsync(&spr.base, cp.off, st));
+  char* pb = static_cast<char*>(spr.base);
+  float* xs = reinterpret_cast<float*>(pb + o_px);
+  float* zs = reinterpret_cast<float*>(pb + o_pz);
+  float* ws = reinterpret_cast<float*>(pb + o_pw);
+  double* psum = reinterpret_cast<double*>(pb + o_ps);
+  double* ppow = reinterpret_cast<double*>(pb + o_pp);
+  std::vector<double> hps(4 * size_t(chunk)), hpp(4 * size_t(chunk));
+  for (int j0 = 0; j0 < n_probes; j0 += chunk) {
+    const int F = n_probes - j0 < chunk ? n_probes - j0 : chunk;
+    for (int j = 0; j < F; ++j)
+      k_rademacher<<<int((n / 4 + 255) / 256), 256, 0, st>>>(int(n), uint32_t(j0 + j), uint32_t(seed & 0xffffffffu),
+                                                            uint32_t(seed >> 32), mask, zs + j * n);
     WF_CUDA(cudaGetLastError());
-    r = wf_solve_ex(z, Nd, mask, P, H, W, &sp, wv, &it, &rs, stream);  // wv = s_W(z)
+    if (F > 1) {
+      KernelTimer timer(st);
+      r = solve_many(zs, F, Nd, mask, P, H, W, sp, ws, st, &timer);
+      timer.collect();
+    } else {
+      r = wf_solve_ex(zs, Nd, mask, P, H, W, &sp, ws, &it, &rs, stream);  // ws = s_W(z)
+    }
     if (r != WF_OK) return r;
-    WF_CUDA(cudaMemsetAsync(sums, 0, 4 * sizeof(double), st));
-    k_xres<<<xb, 256, 0, st>>>(int(n), z, wv, Nd, sigma2, mask, x, sums);  // x = C^-1 z
+    WF_CUDA(cudaMemsetAsync(psum, 0, 4 * sizeof(double) * size_t(F), st));
+    for (int j = 0; j < F; ++j)  // x = C^-1 z
+      k_xres<<<xb, 256, 0, st>>>(int(n), zs + j * n, ws + j * n, Nd, sigma2, mask, xs + j * n, psum + 4 * j);
     WF_CUDA(cudaGetLastError());
     // w^T dS z = (|U(w+z)|^2_dP - |U(w-z)|^2_dP) / 4
-    if ((e = spectral_power_dev(x, z, 1.f, 1, dPa, 2, H, W, pw, st)) != cudaSuccess) return cuda_fail(e);
-    if ((e = spectral_power_dev(x, z, -1.f, 1, dPa, 2, H, W, pw + 2, st)) != cudaSuccess) return cuda_fail(e);
-    double hq[4];
-    WF_CUDA(cudaMemcpyAsync(hs, sums, 4 * sizeof(double), cudaMemcpyDeviceToHost, st));
-    WF_CUDA(cudaMemcpyAsync(hq, pw, 4 * sizeof(double), cudaMemcpyDeviceToHost, st));
+    if ((e = spectral_power_dev(xs, zs, 1.f, F, dPa, 2, H, W, ppow, st)) != cudaSuccess) return cuda_fail(e);
+    if ((e = spectral_power_dev(xs, zs, -1.f, F, dPa, 2, H, W, ppow + 2 * F, st)) != cudaSuccess) return cuda_fail(e);
+    WF_CUDA(cudaMemcpyAsync(hps.data(), psum, 4 * sizeof(double) * size_t(F), cudaMemcpyDeviceToHost, st));
+    WF_CUDA(cudaMemcpyAsync(hpp.data(), ppow, 4 * sizeof(double) * size_t(F), cudaMemcpyDeviceToHost, st));
     WF_CUDA(cudaStreamSynchronize(st));
-    const double t[3] = {0.25 * (hq[0] - hq[2]), 0.25 * (hq[1] - hq[3]), hs[1]};
-    for (int i = 0; i < 3; ++i) {
-      tsum[i] += t[i];
-      tsq[i] += t[i] * t[i];
+    for (int j = 0; j < F; ++j) {
+      const double* plus = hpp.data() + 2 * j;
+      const double* minus = plus + 2 * F;
+      const double t[3] = {0.25 * (plus[0] - minus[0]), 0.25 * (plus[1] - minus[1]), hps[4 * j + 1]};
+      for (int i = 0; i < 3; ++i) {
+        tsum[i] += t[i];
+        tsq[i] += t[i] * t[i];
+      }
     }
   }
   for (int i = 0; i < 3; ++i) {

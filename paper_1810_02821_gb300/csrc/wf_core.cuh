@@ -1231,19 +1231,22 @@ __device__ __forceinline__ int ksolve_sweeps(float2 (&x)[KGeo<N>::E], const floa
   }
 }
 
-// level norms of one problem, one CTA per level
+// level norms of the problems blockIdx.y (pixel tables dn + y H W), one CTA per level
 template <int N>
 __global__ void __launch_bounds__(KGeo<N>::T) k_mbnorm(BnormArgs a) {
   const Scalars sc = *a.sc;
   const int lev = blockIdx.x;
   if (sc.status != 0 || lev >= sc.n_levels) return;
   ktw_init<N>();
-  const double v = klevel_norm<N>(a.dn, a.Pk, float(level_lambda(sc, lev, a.eta) * sc.tau));
-  if (threadIdx.x == 0) a.bnorm2[lev] = v;
+  const double v = klevel_norm<N>(a.dn + blockIdx.y * (KGeo<N>::H * KGeo<N>::W), a.Pk,
+                                  float(level_lambda(sc, lev, a.eta) * sc.tau));
+  if (threadIdx.x == 0) a.bnorm2[blockIdx.y * kMaxLevels + lev] = v;
 }
 
-// one problem, one CTA (alone on its SM: up to 128 registers a thread)
-template <int N>
+// one problem per CTA (alone on its SM: up to 128 registers a thread): problem f on dn, out + f H W, bnorm2 + f kMaxLevels,
+// prev + f H W/2 and st + f; init_s only for a single problem. MANY false: one problem (with run-time offsets its sweeps
+// take 0.8% longer)
+template <int N, bool MANY>
 __global__ void __launch_bounds__(KGeo<N>::T, 1) k_msolve(SolveArgs a) {
   using G = KGeo<N>;
   const Scalars sc = *a.sc;
@@ -1253,13 +1256,15 @@ __global__ void __launch_bounds__(KGeo<N>::T, 1) k_msolve(SolveArgs a) {
   kload<N>(x, a.init_s);
   int it = 0;
   double rho = -1.0;
-  const int status = ksolve_sweeps<N>(x, a.dn, a.Pk, sc, a.bnorm2, a.prev, a.tol, a.eta, a.level_tol, a.max_iter,
+  const int f = MANY ? blockIdx.x : 0;
+  const int status = ksolve_sweeps<N>(x, a.dn + f * (G::H * G::W), a.Pk, sc, a.bnorm2 + f * kMaxLevels,
+                                      a.prev + f * (G::H * G::W / 2), a.tol, a.eta, a.level_tol, a.max_iter,
                                       a.level_max, a.check, it, rho, a.rhs_mode != 0);
-  kstore<N>(x, a.out, kOutF32);
+  kstore<N>(x, a.out + f * (G::H * G::W), kOutF32);
   if (threadIdx.x == 0) {
-    a.st->status = status;
-    a.st->iters = it;
-    a.st->resid = rho;
+    a.st[f].status = status;
+    a.st[f].iters = it;
+    a.st[f].resid = rho;
   }
 }
 

@@ -33,7 +33,7 @@ __device__ __forceinline__ void x_store(uint32_t addr, float2 v) {
 
 // How the CTAs of a field exchange the half spectrum: CTA b of a field owns rows RB b .. and columns CB b .. of each of
 // its NC components. row(comp, yl) and col(comp): accessors as ZRow and ZCols; arrive(), wait(): a barrier of the field's
-// CTAs (XGrid: of the grid) in two parts, stores before the arrival visible after the wait, false after a timeout.
+// CTAs (XGrid samplers: of the grid) in two parts, stores before the arrival visible after the wait, false after a timeout.
 template <int N, int NC_>
 struct XCluster {
   static constexpr int NC = NC_, RB = 16, C = N / RB, CB = N / 2 / C;
@@ -89,6 +89,7 @@ struct XGrid {
   float2* Z;  // of the field: [NC][H][W/2]
   int rank;
   GridBar* bar;
+  unsigned int count;  // CTAs that share the barrier
   unsigned int target;
   __device__ __forceinline__ ZRow row(int comp, int yl) const {
     return ZRow{Z + ((long long)comp * N + rank * RB + yl) * (N / 2)};
@@ -98,7 +99,7 @@ struct XGrid {
   }
   __device__ __forceinline__ void arrive() {
     __syncthreads();
-    target += gridDim.x;
+    target += count;
     if (threadIdx.x == 0) grid_arrive(bar);
   }
   __device__ __forceinline__ bool wait() const {
@@ -123,7 +124,7 @@ struct FewGeo {
   static_assert(X::NC * X::CB == G::CB && H / 2 <= 2 * T && O_X % 2 == 0 && O_PIX % 2 == 0, "geometry");
 };
 
-// scalar fields; a.mode 0 (chain blockIdx.x / C) or, with SOLVE, 1
+// scalar fields; a.mode 0 (chain blockIdx.x / C) or, with SOLVE, 1 (field blockIdx.x / C, each at its own pace)
 template <int N, class X, bool SOLVE>
 __global__ void __launch_bounds__(FewGeo<N, X>::T, FewGeo<N, X>::MIN_CTAS) k_few(const __grid_constant__ GlobalArgs a) {
   using K = FewGeo<N, X>;
@@ -131,13 +132,14 @@ __global__ void __launch_bounds__(FewGeo<N, X>::T, FewGeo<N, X>::MIN_CTAS) k_few
   constexpr int H = N, W = N, CB = X::CB, RB = X::RB, T = K::T, C = X::C, WH = W / 2 + 1, GR = X::NC * X::RB;
   const int rank = blockIdx.x % C, f = blockIdx.x / C;
   if (a.sc->status != 0) {  // uniform over the grid
-    if (SOLVE && blockIdx.x == 0 && threadIdx.x == 0) a.st->status = a.sc->status;
+    if (SOLVE && rank == 0 && threadIdx.x == 0) a.st[f].status = a.sc->status;
     return;
   }
   gtab_init<N, GR>();
   float2* s = gsmem();
   {
-    const float4* src = reinterpret_cast<const float4*>((SOLVE ? a.dn : a.aq) + rank * RB * W);
+    const float4* src = reinterpret_cast<const float4*>(
+        (SOLVE ? a.dn + (long long)f * H * W : a.aq) + rank * RB * W);
     for (int i = threadIdx.x; i < RB * W / 2; i += T) reinterpret_cast<float4*>(s + K::O_PIX)[i] = __ldg(src + i);
     float* P = reinterpret_cast<float*>(s + K::O_P);
     for (int i = threadIdx.x; i < H * CB; i += T) {
@@ -153,7 +155,7 @@ __global__ void __launch_bounds__(FewGeo<N, X>::T, FewGeo<N, X>::MIN_CTAS) k_few
   }
   X ex = [&] {
     if constexpr (X::CLUSTER) return X{s + K::O_X, rank};
-    else return X{a.Z + (long long)f * H * (W / 2), rank, a.bar, 0u};
+    else return X{a.Z + (long long)f * H * (W / 2), rank, SOLVE ? a.bar + f : a.bar, SOLVE ? unsigned(C) : gridDim.x, 0u};
   }();
   __syncthreads();
   if constexpr (X::CLUSTER) {  // every CTA has started: its shared memory may be stored to
@@ -261,7 +263,7 @@ __global__ void __launch_bounds__(FewGeo<N, X>::T, FewGeo<N, X>::MIN_CTAS) k_few
                          "d"(v)
                          : "memory");
         } else if (threadIdx.x == 0) {
-          atomicAdd(a.acc + parity, v);
+          atomicAdd(a.acc + 2 * f + parity, v);
         }
       }
       ex.arrive();
@@ -274,12 +276,12 @@ __global__ void __launch_bounds__(FewGeo<N, X>::T, FewGeo<N, X>::MIN_CTAS) k_few
 #pragma unroll
             for (int o = 8; o > 0; o >>= 1) tot += __shfl_xor_sync(0xffffffffu, tot, o);
           } else {
-            tot = __ldcg(a.acc + parity);
-            if (blockIdx.x == 0 && threadIdx.x == 0) a.acc[parity ^ 1] = 0.0;  // next check's accumulator
+            tot = __ldcg(a.acc + 2 * f + parity);
+            if (rank == 0 && threadIdx.x == 0) a.acc[2 * f + (parity ^ 1)] = 0.0;  // next check's accumulator
           }
           if (threadIdx.x == 0) {
             tot *= double(H) * W;
-            const double bn = a.bnorm2[a.rhs_mode ? 0 : lev], ref = bn > 0.0 ? bn : 1.0;
+            const double bn = a.bnorm2[a.rhs_mode ? 0 : f * kMaxLevels + lev], ref = bn > 0.0 ? bn : 1.0;
             GSolveState d{tot, ltau, lev, k, 1};
             if (!(tot == tot) || tot > 1e300 * ref) {
               d.status = 6;  // non-finite residual
@@ -292,7 +294,7 @@ __global__ void __launch_bounds__(FewGeo<N, X>::T, FewGeo<N, X>::MIN_CTAS) k_few
             } else if (tot < a.tol * a.tol * ref) {
               d.status = 0;
             }
-            if (blockIdx.x == 0) d.rho2 = tot / ref;
+            if (rank == 0) d.rho2 = tot / ref;
             dec = d;
           }
         }
@@ -308,11 +310,11 @@ __global__ void __launch_bounds__(FewGeo<N, X>::T, FewGeo<N, X>::MIN_CTAS) k_few
       grow_inv<N, GR>(zrow, x);
       if (status != 1) break;
     }
-    grow_store<N>(x, a.out, y, kOutF32);
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
-      a.st->status = status;
-      a.st->iters = it;
-      a.st->resid = rho2 >= 0.0 ? sqrt(rho2) : rho2;
+    grow_store<N>(x, a.out, (long long)f * H + y, kOutF32);
+    if (rank == 0 && threadIdx.x == 0) {
+      a.st[f].status = status;
+      a.st[f].iters = it;
+      a.st[f].resid = rho2 >= 0.0 ? sqrt(rho2) : rho2;
     }
   }
 }
@@ -348,7 +350,7 @@ __global__ void __launch_bounds__(FewGeo<N, X>::T, FewGeo<N, X>::MIN_CTAS) k_few
     }
   X ex = [&] {
     if constexpr (X::CLUSTER) return X{s + K::O_X, rank};
-    else return X{ga.Z + 2LL * f * H * (W / 2), rank, ga.bar, 0u};
+    else return X{ga.Z + 2LL * f * H * (W / 2), rank, ga.bar, gridDim.x, 0u};
   }();
   __syncthreads();
   if constexpr (X::CLUSTER) {  // every CTA has started: its shared memory may be stored to

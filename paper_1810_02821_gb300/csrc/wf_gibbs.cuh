@@ -1196,6 +1196,7 @@ struct SolveArgs {
   int level_max;
   int check;
   int rhs_mode;          // 1: solve (S^-1 + N^-1) s = r with the table's r (refinement correction)
+  int n_fields;          // host side: problems of the launch (k_msolve)
 };
 
 // The G -> 0 iteration with lambda-cooling for one field (one CTA of N threads). On entry c holds the

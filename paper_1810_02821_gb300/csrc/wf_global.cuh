@@ -316,7 +316,8 @@ struct GlobalArgs {
   uint32_t chain0;
   uint32_t step0;
   uint32_t key0, key1;
-  // Wiener filter (n_fields == 1)
+  // Wiener filter: k_global one field; k_few several, field f on the pixel table dn + f H W, the level norms
+  // bnorm2 + f kMaxLevels, out + f H W and bar, acc (2 each) and st from f on
   const double* bnorm2;    // level norms (rhs_mode: one norm for every level)
   double* acc;             // [2] residual accumulators (alternating)
   float2* prev;            // [H][W/2]
@@ -325,7 +326,8 @@ struct GlobalArgs {
   int max_iter, level_max, check;
   int rhs_mode;            // mode 1: dn holds (r, 1/N_bar), t = lambda tau r + w s (refinement correction)
   int mode;                // 0 sampler, 1 Wiener filter, 2 level norms (fields = levels), 3 weighted power
-  double* bnorm_out;       // mode 2: [n_fields]
+  int levels;              // mode 2: field f is level f % levels of pixel table f / levels
+  double* bnorm_out;       // mode 2: [n_fields / levels][kMaxLevels]
   // mode 3: fields v_f = va_f + vsign * vb_f, tables wts[nw][H][W/2+1], sums into wout[f*nw + j]
   const float* va;
   const float* vb;
@@ -569,8 +571,8 @@ __device__ void row_item(const GlobalArgs& a, int f, int y0, int done, bool firs
     return;
   }
   if (a.mode != 3)  // mode 3 transforms the field as loaded
-    pixel_update<N>(a.mode, x, y, a.aq, a.dn, a.step0 + uint32_t(done), a.chain0 + uint32_t(f), a.key0, a.key1,
-                    sc.sqrt_tau, ltau, a.rhs_mode, a.mode == 2 ? float(level_lambda(sc, f, a.eta) * sc.tau) : 0.f);
+    pixel_update<N>(a.mode, x, y, a.aq, a.mode == 2 ? a.dn + (long long)(f / a.levels) * G::H * G::W : a.dn, a.step0 + uint32_t(done), a.chain0 + uint32_t(f), a.key0, a.key1,
+                    sc.sqrt_tau, ltau, a.rhs_mode, a.mode == 2 ? float(level_lambda(sc, f % a.levels, a.eta) * sc.tau) : 0.f);
   grow_fwd<N>(x, z);
 }
 
@@ -904,7 +906,7 @@ __global__ void __launch_bounds__(GGeo<N>::T, GGeo<N>::MIN_CTAS) k_global(const 
   auto rows = [&](int done, bool first, bool emit_only, float ltau) {
     for (int it = blockIdx.x; it < row_items; it += nb) {
       const int f = it / G::ROW_ITEMS;
-      if (a.mode == 2 && f >= sc.n_levels) continue;  // level fields past the schedule
+      if (a.mode == 2 && f % a.levels >= sc.n_levels) continue;  // level fields past the schedule
       row_item<N>(a, f, (it % G::ROW_ITEMS) * G::RB, done, first, emit_only, ltau, sc);
     }
   };
@@ -950,9 +952,10 @@ __global__ void __launch_bounds__(GGeo<N>::T, GGeo<N>::MIN_CTAS) k_global(const 
     if (!grid_barrier(a.bar, nb, target)) return;
     for (int it = blockIdx.x; it < col_items; it += nb) {
       const int f = it / G::COL_ITEMS;
-      if (f >= sc.n_levels) continue;
+      if (f % a.levels >= sc.n_levels) continue;
       const double s = gblock_sum<G::T>(col(f, it, 0, 0.f, false, false), red);
-      if (threadIdx.x == 0) atomicAdd(a.bnorm_out + f, s / double(G::H * G::W));
+      if (threadIdx.x == 0)
+        atomicAdd(a.bnorm_out + (f / a.levels) * kMaxLevels + f % a.levels, s / double(G::H * G::W));
     }
     return;
   }

@@ -213,9 +213,12 @@ cudaError_t launch_solve(const SolveArgs& a, const BnormArgs& b, cudaStream_t st
   cudaError_t e = cudaSuccess;
   if constexpr (core_size(N)) {
     if (!a.rhs_mode)  // rhs mode: the level norms are supplied
-      e = launch_smem(k_mbnorm<N>, kMaxLevels, KGeo<N>::T, ksolve_smem<N>(), b, st, nullptr);
-    return e != cudaSuccess ? e : launch_smem(k_msolve<N>, 1, KGeo<N>::T, ksolve_smem<N>(), a, st, t);
+      e = launch_smem(k_mbnorm<N>, dim3(kMaxLevels, unsigned(a.n_fields)), KGeo<N>::T, ksolve_smem<N>(), b, st, nullptr);
+    if (e != cudaSuccess) return e;
+    return launch_smem(a.n_fields > 1 ? k_msolve<N, true> : k_msolve<N, false>, unsigned(a.n_fields), KGeo<N>::T,
+                       ksolve_smem<N>(), a, st, t);
   } else {
+    if (a.n_fields != 1) return cudaErrorInvalidValue;
     const int smem = Geo<N>::FIELD_BYTES + 33 * 8;
     if (!a.rhs_mode) e = launch_smem(k_bnorm<N>, kMaxLevels, N, smem, b, st, nullptr);
     return e != cudaSuccess ? e : launch_smem(k_solve<N>, 1, N, smem, a, st, t);

@@ -1,6 +1,7 @@
 """Few large fields, a block of rows and columns per CTA for the whole launch (up to 256^2 in thread-block clusters),
 against the same passes in the same order with several blocks per CTA: equal bit for bit, up to and past the number of
 resident fields."""
+import numpy as np
 import pytest
 
 from gpu_common import need_gpu, rel, to_dev, torch
@@ -105,3 +106,24 @@ def test_64_in_clusters(chains):
     finally:
         wf.wf_set_large_image_sampler("auto")
     assert rel(a.cpu().numpy(), b.cpu().numpy()) < 2e-6
+
+
+@pytest.mark.parametrize("H,probes", [(32, 3), (32, 64), (32, 65), (64, 2), (64, 67), (128, 2), (128, 49), (256, 7),
+                                      (256, 15), (512, 3)])
+def test_probes_solved_side_by_side(in_global, H, probes):
+    """The trace probes of the gradient, several solves in one launch (up to 64 on chip, else as many as are resident),
+    against the batched gradient's own solves, and from 128 on against one solve after the other (the same iterates)."""
+    need_gpu()
+    build.build()
+    p = synth.make_problem(H, seed=H, mask_frac=0.1, slope=-2.0, amp=1.2, k0=1.0 / H, sigma2=(0.01, 0.2))
+    d, s2, m = to_dev(p)[:3]
+    call = lambda: wf.wf_loglike_grad(d, s2, m, 1.2, -2.0, 1.0 / H, 1.0, n_probes=probes, seed=5, tol=1e-6)
+    a = call()
+    if H >= 128:
+        b = in_global(call)
+        np.testing.assert_allclose(a.grad, b.grad, rtol=1e-9)
+        np.testing.assert_allclose(a.grad_var, b.grad_var, rtol=1e-6)
+    c = wf.wf_loglike_grad_batch([(d, s2, m, 1.2, -2.0, 1.0 / H, 1.0, 5)], n_probes=probes, tol=1e-6)[0]
+    # both solve to a relative residual of 1e-5
+    sd = np.sqrt(a.grad_var) + 1e-12
+    assert np.all(np.abs(c.grad - a.grad) < 0.05 * sd + 1e-3 * np.abs(a.grad))
