@@ -2181,8 +2181,13 @@ wf_status record_batch(const BatchPlan& p, char* b, cudaStream_t st, ForkJoin& f
   WF_CUDA(cudaEventCreateWithFlags(&ready, cudaEventDisableTiming));
   fj.evs.push_back(ready);
   WF_CUDA(cudaEventRecord(ready, st));
-  auto new_stream = [&](cudaStream_t* out) -> cudaError_t {
-    cudaError_t e = cudaStreamCreateWithFlags(out, cudaStreamNonBlocking);
+  // Small classes come before the large ones in the GPU's order: a cooperative launch of a large class waits until the whole
+  // GPU is free, and CTAs of a small class not yet started by then would wait for its end (205 images of 128^2: the last
+  // 53 solves ran alone for 1.4 ms after it)
+  int prio_small = 0, prio_large = 0;
+  WF_CUDA(cudaDeviceGetStreamPriorityRange(&prio_large, &prio_small));
+  auto new_stream = [&](cudaStream_t* out, int prio) -> cudaError_t {
+    cudaError_t e = cudaStreamCreateWithPriority(out, cudaStreamNonBlocking, prio);
     if (e != cudaSuccess) return e;
     fj.side.push_back(*out);
     return cudaStreamWaitEvent(*out, ready, 0);
@@ -2190,7 +2195,7 @@ wf_status record_batch(const BatchPlan& p, char* b, cudaStream_t st, ForkJoin& f
   wf_status fail = WF_OK;
   for (size_t k = 0; k < p.small.size() && fail == WF_OK; ++k) {
     cudaStream_t s2;
-    cudaError_t e = new_stream(&s2);
+    cudaError_t e = new_stream(&s2, prio_small);
     if (e != cudaSuccess) { fail = cuda_fail(e); break; }
     fail = run_small(p.small[k], d_items, d_res, o, b, s2);
   }
@@ -2198,7 +2203,7 @@ wf_status record_batch(const BatchPlan& p, char* b, cudaStream_t st, ForkJoin& f
   for (int c = 0; c < 4 && fail == WF_OK && o.small_path == 1; ++c) {
     if (p.cls[c].empty()) continue;
     cudaStream_t s2;
-    cudaError_t e = new_stream(&s2);
+    cudaError_t e = new_stream(&s2, prio_small);
     if (e != cudaSuccess) { fail = cuda_fail(e); break; }
     wf::BatchArgs ba{};
     ba.items = d_items;
@@ -2223,7 +2228,7 @@ wf_status record_batch(const BatchPlan& p, char* b, cudaStream_t st, ForkJoin& f
   if (fail == WF_OK && p.nls) {
     std::vector<cudaStream_t> pool(p.nls);
     for (int k = 0; k < p.nls && fail == WF_OK; ++k) {
-      cudaError_t e = new_stream(&pool[k]);
+      cudaError_t e = new_stream(&pool[k], prio_large);
       if (e != cudaSuccess) fail = cuda_fail(e);
     }
     for (size_t k = 0; k < p.chunks.size() && fail == WF_OK; ++k) {
