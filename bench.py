@@ -10,7 +10,7 @@ Printed JSON line (rank 0):
   value      samples/s with inputs resident in HBM (events around each step; L2 flushed between steps)
   e2e        same metric through the same C call with host buffers: pinned H2D of the inputs, and every
              sample stored by the kernel into page-locked host memory, inside the timed region
-  roofline   the fused sampler kernel k_sample<128,1>: FFT flops (5 n log2 n per sweep) per launch over
+  roofline   the fused sampler kernel k_msample<128>: FFT flops (5 n log2 n per sweep) per launch over
              its event-timed duration, against the FP32 FMA throughput measured on the device
              (wf_measure_fp32_peak: every SM filled with independent FMA chains, CUDA events, best launch)
   cpu_baseline  the FP64 oracle on the host cores, on a bounded sample of the same workload
@@ -116,8 +116,8 @@ def aggregate_throughput(units_per_rank: int, world: int, max_ms: float) -> floa
     return units_per_rank * world / (max_ms / 1e3)
 
 
-# the sources k_sample<128,1> is compiled from (kernel, register FFT and RNG, launcher, translation unit)
-SAMPLE_KERNEL_SOURCES = ("wf_math.cuh", "wf_gibbs.cuh", "wf_launch.h", "wf_k128.cu")
+# the sources k_msample<128> is compiled from (kernel, register FFT and RNG, launcher, translation unit)
+SAMPLE_KERNEL_SOURCES = ("wf_math.cuh", "wf_gibbs.cuh", "wf_units.cuh", "wf_core.cuh", "wf_launch.h", "wf_k128.cu")
 
 
 def kernel_source_hash() -> str:
@@ -129,7 +129,7 @@ def kernel_source_hash() -> str:
 
 
 def profiled_traffic():
-    """DRAM bytes per launch of k_sample<128,1> from the committed ncu summary, if the kernel sources
+    """DRAM bytes per launch of k_msample<128> from the committed ncu summary, if the kernel sources
     are unchanged since it was taken (its 'csrc_hash' line); else None."""
     if not os.path.exists(PROFILE):
         return None
@@ -760,7 +760,7 @@ def main():
         "gibbs_steps_per_s": value,
         "roofline": {"bound": "alu", "achieved": achieved, "peak": FP32_PEAK_TFLOPS, "unit": "TFLOP/s",
                      "frac": achieved / FP32_PEAK_TFLOPS, "traffic": traffic,
-                     "kernel": "wf::k_sample<128,1>", "kernel_ms": kms,
+                     "kernel": "wf::k_msample<128>", "kernel_ms": kms,
                      "flops_per_launch": flops,
                      "peak_note": "of measured: FP32 FMA throughput of this GPU (fp32_peak); derived "
                                   f"{fp32_peak['sms']} SMs x {FP32_LANES} lanes x 2 x max clock = "

@@ -21,12 +21,12 @@
  *     the minimum observed Ndiag (max_k P_k if every pixel is missing). A tau above the minimum observed
  *     Ndiag is rejected with WF_ERR_TAU.
  *   - Supported sizes: H == W in {16, 32, 64, 128, 256, 512, 1024} (wf_supported_size). Up to 128 x 128
- *     a chain's field stays in one SM's shared memory for the whole call. At 256 x 256 and 512 x 512 the
- *     samplers and Wiener filters of many chains or images keep each field in the shared memory of one
- *     thread-block cluster (wf_set_large_image_sampler). Otherwise larger images keep the field in global
- *     memory and run as
+ *     a chain's field stays in one SM's shared memory for the whole call, or, for few fields of 64 x 64 to
+ *     256 x 256 and many of 256 x 256, in the shared memory of one thread-block cluster
+ *     (wf_set_large_image_sampler). Otherwise larger images keep the field in global memory and run as
  *     one cooperative launch (all CTAs co-resident) whose phases are separated by a bounded grid barrier
- *     (WF_ERR_TIMEOUT if a barrier wait gives up). For those sizes wf_solve_ex starts from zero
+ *     (WF_ERR_TIMEOUT if a barrier wait gives up; likewise the hand-over of a chain between two CTAs when
+ *     there are more chains than resident CTAs). From 256 x 256 up wf_solve_ex starts from zero
  *     (opts->init_s must be NULL).
  *   - Pointers named d, Ndiag, mask, Pk, out*, init_s are DEVICE pointers owned by the caller; pointers
  *     to iters_out / resid_out / opts are HOST pointers (may be NULL where stated).
@@ -452,8 +452,11 @@ double wf_last_kernel_ms(void);
  * and the global-memory kernels (fields in global memory, cooperative launches with many CTAs per field).
  * mode 0 (default, automatic): clusters when a call holds at least 400 chains at 256 x 256 (a batch as many
  * images) and the device can host the cluster, otherwise the global-memory kernels, which are faster for
- * fewer fields and at 512 x 512 (spin-2: clusters from 24 chains at 256 x 256); mode 1: always the global-memory kernels;
- * mode 2: clusters wherever the device can host them. Returns the previous mode.
+ * fewer fields and at 512 x 512 (spin-2: clusters from 24 chains at 256 x 256), and in their place, for as
+ * many fields as are resident at once (also at 64 x 64, 128 x 128 and 1024 x 1024), kernels of the same
+ * arithmetic that keep the tables, and up to 256 x 256 the field, in shared memory (equal bit for bit);
+ * mode 1: always the global-memory kernels; mode 2: clusters wherever the device can host them. Returns the
+ * previous mode.
  */
 int32_t wf_set_large_image_sampler(int32_t mode);
 
