@@ -9,7 +9,8 @@
 //             Alg. 1 from s_W, each image with its own tables, chain and key.
 // Each kernel holds one stage's code only (the fused kernel's instruction footprint stalled its warps on
 // instruction fetch), the block scheduler balances the unequal solves, and the sampler packs as many
-// fields per SM as the single-image sampler does.
+// fields per SM as the single-image sampler does. The kernels below run at 16 x 16; from 32 x 32 their forms with several
+// threads per row do (k_mblevels, k_mbsolve, k_mbsample).
 #pragma once
 
 #include "wf_gbatch.cuh"

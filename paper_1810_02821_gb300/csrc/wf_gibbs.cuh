@@ -494,7 +494,7 @@ struct SampleArgs {
 WF_HD int band_bytes(int n_bins) { return ((n_bins * 12 + 15) / 16) * 16; }
 
 // CTAs per SM the sample kernel is compiled for (register budget 65536 / (threads * CTAs)):
-// 128^2 fields are limited to three per SM by shared memory (66.5 KB each).
+// 128^2 fields (the fused batch kernel) are limited to three per SM by shared memory (66.5 KB each).
 // Philox calls in flight in the rolled pointwise-draw loops (the field registers are dead there)
 #ifndef WF_RNG_UNROLL
 #define WF_RNG_UNROLL 4

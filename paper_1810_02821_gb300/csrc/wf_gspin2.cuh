@@ -1,4 +1,5 @@
-// Spin-2 (shear) sweeps at 256^2 and 512^2 with the fields in global memory: both components of every chain as two
+// Spin-2 (shear) sweeps with the fields in global memory (256^2 and 512^2 beyond the pairs that k_few2 holds, 128^2 where
+// it cannot run): both components of every chain as two
 // fields of one persistent cooperative launch (the phases, transforms and barrier of wf_global.cuh).
 //   row phase    (CTA = 8 rows of one component): as the scalar sampler, the t-draw from stream 0 or 8;
 //   column phase (CTA = 2 columns of both components): thread tid holds component tid % 2 of column
