@@ -6,12 +6,19 @@
 // pixels) gives (I + S A N^-1 A) s - S A N^-1 d = -S r, so ||S r|| / ||S A N^-1 d|| is the relative residual used
 // everywhere else in the library, here evaluated in FP64.
 //
-// Two real fields a, b travel as one complex field z = a + i b: a_hat = (Z(k) + conj Z(-k)) / 2 and
-// i b_hat = (Z(k) - conj Z(-k)) / 2. Three kernels:
+// Complex fields (one real field, or the two components of a shear field, which share their unit) take three kernels:
 //   k_rows_fwd   forms z from the caller's arrays and transforms whole rows in shared memory;
-//   k_cols       transforms four whole columns in shared memory, two and their mirrors -kx, so that Z(k) and Z(-k)
-//                are both there for the pointwise step (a norm, or a new spectrum followed by the inverse transform);
+//   k_cols       transforms four whole columns in shared memory, then the pointwise step (a norm, or a new spectrum
+//                followed by the inverse transform);
 //   k_rows_inv   transforms the rows back and forms the caller's outputs.
+// The refinement residual has two real fields of different units, the iterate s and N^-1 (d - s), which goes with
+// 1 / s: in one complex field the rounding errors of the larger would fall on the smaller. So only their row transforms
+// share a complex one, with the second field scaled by a power of two to the first (exact, chosen by each CTA
+// from its own rows); k_rows_residual separates the two there and leaves the half spectra (kx <= N/2), and the columns of
+// each are transforms of their own: as many columns in all as the packed form has. k_cols_residual forms the norm, k_cols_divp
+// and k_rows_half the correction's S^-1 s. Every error is then relative to its own field, in any unit of the data. Against
+// both fields packed through the columns too, device us at 1024^2: a residual 217 -> 204, a correction's right-hand side (the
+// columns of s alone) 303 -> 208; at 64^2, launch-bound, 21.6 -> 21.5 and 27.2 -> 26.0.
 // A norm is two launches and an application of an operator three. The transforms are radix-4 Stockham passes
 // (self-sorting; Govindaraju et al., "High performance discrete Fourier transforms on graphics processors", SC'08)
 // with the twiddles from a table. Bound: the FP64 rate of this GPU (two lanes per SM and clock) at 512^2 and above, the
@@ -169,14 +176,13 @@ __device__ __forceinline__ double2 ks_rot_d(int N, int ky, int kx) {
 }
 
 // ---- sources z(field, pixel) of the forward rows ----
-struct SrcResidual {  // s + i rpix, rpix = A N^-1 (d - A s) on observed pixels with A != 0 (A = 1 when null)
+struct SrcResidual {  // s, and rpix = A N^-1 (d - A s) on observed pixels with A != 0 (A = 1 when null)
   const float *d, *Nd, *A, *s;
   const uint8_t* mask;
   __device__ __forceinline__ double rpix(int i) const {
     const double a = A ? double(A[i]) : 1.0;
     return (mask[i] || a == 0.0) ? 0.0 : a * (double(d[i]) - a * double(s[i])) / double(Nd[i]);
   }
-  __device__ __forceinline__ double2 operator()(int, int i) const { return make_double2(double(s[i]), rpix(i)); }
 };
 struct SrcRhs {  // A N^-1 d on observed pixels with A != 0
   const float *d, *Nd, *A;
@@ -225,44 +231,21 @@ __global__ void __launch_bounds__(DGeo<N>::TR) k_rows_fwd(Src src, double2* Z, d
   for (int e = threadIdx.x; e < G::RB * N; e += G::TR) z[e] = buf[e];
 }
 
-// ---- pointwise steps of the columns: op(f, ky, kx, z, m) with z = Z(k) and m = conj Z(-k) ----
-struct OpResidualNorm {  // |P r_hat - s_hat|^2 / n where P > 0, else |s_hat|^2 / n
-  static constexpr bool kNorm = true;
-  const float* Pk;
-  template <int N>
-  __device__ __forceinline__ double norm(int ky, int kx, double2 z, double2 m) const {
-    const double p = p_full(Pk, N, ky, kx);
-    const double2 s = make_double2(0.5 * (z.x + m.x), 0.5 * (z.y + m.y));
-    const double2 ir = make_double2(0.5 * (z.x - m.x), 0.5 * (z.y - m.y));  // i r_hat
-    const double2 e = p > 0.0 ? make_double2(p * ir.y - s.x, -p * ir.x - s.y) : s;
-    return (e.x * e.x + e.y * e.y) * (1.0 / (double(N) * N));
-  }
-};
+// ---- pointwise steps of the columns: op.norm or op.map(ky, kx, Z(k)) ----
 struct OpPNorm {  // P^2 |z|^2 / n
   static constexpr bool kNorm = true;
   const float* Pk;
   template <int N>
-  __device__ __forceinline__ double norm(int ky, int kx, double2 z, double2) const {
+  __device__ __forceinline__ double norm(int ky, int kx, double2 z) const {
     const double p = p_full(Pk, N, ky, kx);
     return p * p * (z.x * z.x + z.y * z.y) * (1.0 / (double(N) * N));
-  }
-};
-struct OpDivP {  // s_hat / (n P) where P > 0, else 0
-  static constexpr bool kNorm = false;
-  const float* Pk;
-  template <int N>
-  __device__ __forceinline__ double2 map(int ky, int kx, double2 z, double2 m) const {
-    const double p = p_full(Pk, N, ky, kx);
-    if (!(p > 0.0)) return make_double2(0.0, 0.0);
-    const double q = 0.5 / (double(N) * N * p);
-    return make_double2(q * (z.x + m.x), q * (z.y + m.y));
   }
 };
 struct OpMulP {  // P z / n
   static constexpr bool kNorm = false;
   const float* Pk;
   template <int N>
-  __device__ __forceinline__ double2 map(int ky, int kx, double2 z, double2) const {
+  __device__ __forceinline__ double2 map(int ky, int kx, double2 z) const {
     const double p = p_full(Pk, N, ky, kx) * (1.0 / (double(N) * N));
     return make_double2(z.x * p, z.y * p);
   }
@@ -270,15 +253,15 @@ struct OpMulP {  // P z / n
 struct OpKsInverse {  // E_hat + i B_hat = (c - i s)(g1_hat + i g2_hat), over n
   static constexpr bool kNorm = false;
   template <int N>
-  __device__ __forceinline__ double2 map(int ky, int kx, double2 z, double2) const {
+  __device__ __forceinline__ double2 map(int ky, int kx, double2 z) const {
     const double2 r = ks_rot_d(N, ky, kx);
     const double2 o = dmul(z, dconj(r));
     return make_double2(o.x * (1.0 / (double(N) * N)), o.y * (1.0 / (double(N) * N)));
   }
 };
 
-// columns of CTA blockIdx.x of field blockIdx.y: transform, then the sum of op's norms added to *out, or op's new
-// spectrum transformed back in place
+// columns 4 g .. 4 g + 3 (g = blockIdx.x) of field blockIdx.y: transform, then the sum of op's norms added to *out, or op's
+// new spectrum transformed back in place
 template <int N, class Op>
 __global__ void __launch_bounds__(DGeo<N>::TC) k_cols(Op op, double2* Z, double* out) {
   using G = DGeo<N>;
@@ -287,7 +270,7 @@ __global__ void __launch_bounds__(DGeo<N>::TC) k_cols(Op op, double2* Z, double*
   double2* z = Z + (long long)blockIdx.y * N * N;
   for (int e = threadIdx.x; e < 4 * N; e += G::TC) {
     const int c = e % 4, y = e / 4;
-    buf[c * N + y] = z[(long long)y * N + dcol<N>(g, c)];
+    buf[c * N + y] = z[(long long)y * N + 4 * g + c];
   }
   __syncthreads();
   dfft<N, 4, G::TC, false>(buf);
@@ -297,7 +280,7 @@ __global__ void __launch_bounds__(DGeo<N>::TC) k_cols(Op op, double2* Z, double*
 #pragma unroll 4
     for (int i = 0; i < ITER; ++i) {
       const int e = threadIdx.x + i * G::TC, c = e / N, ky = e % N;
-      acc += op.template norm<N>(ky, dcol<N>(g, c), buf[e], dconj(buf[dmir(g, c) * N + (N - ky) % N]));
+      acc += op.template norm<N>(ky, 4 * g + c, buf[e]);
     }
     dadd_block<G::TC>(acc, out);
   } else {
@@ -305,7 +288,7 @@ __global__ void __launch_bounds__(DGeo<N>::TC) k_cols(Op op, double2* Z, double*
 #pragma unroll
     for (int i = 0; i < ITER; ++i) {
       const int e = threadIdx.x + i * G::TC, c = e / N, ky = e % N;
-      v[i] = op.template map<N>(ky, dcol<N>(g, c), buf[e], dconj(buf[dmir(g, c) * N + (N - ky) % N]));
+      v[i] = op.template map<N>(ky, 4 * g + c, buf[e]);
     }
     __syncthreads();
 #pragma unroll
@@ -314,8 +297,116 @@ __global__ void __launch_bounds__(DGeo<N>::TC) k_cols(Op op, double2* Z, double*
     dfft<N, 4, G::TC, true>(buf);
     for (int e = threadIdx.x; e < 4 * N; e += G::TC) {
       const int c = e % 4, y = e / 4;
-      z[(long long)y * N + dcol<N>(g, c)] = buf[c * N + y];
+      z[(long long)y * N + 4 * g + c] = buf[c * N + y];
     }
+  }
+}
+
+// Rows of s and of rpix: one complex transform a row, s + i beta rpix with beta a power of two that brings the CTA's
+// largest rpix to its largest s, separated into the half spectra Z[0][y][kx] and Z[1][y][kx], kx <= N/2; *zero = 0.
+template <int N>
+__global__ void __launch_bounds__(DGeo<N>::TR) k_rows_residual(SrcResidual src, double2* Z, double* zero) {
+  using G = DGeo<N>;
+  constexpr int E = G::RB * N / G::TR, WH = N / 2 + 1, NW = G::TR / 32;
+  static_assert(G::TR % 32 == 0, "whole warps");
+  __shared__ int top[2][NW];
+  double2* buf = dsmem();
+  const int base = int(blockIdx.x) * G::RB * N;
+  if (zero && blockIdx.x == 0 && threadIdx.x == 0) *zero = 0.0;
+  double2 x[E];
+  int hs = 0, hr = 0;  // high words of the largest magnitudes
+#pragma unroll
+  for (int i = 0; i < E; ++i) {
+    const int at = base + int(threadIdx.x) + i * G::TR;
+    x[i] = make_double2(double(src.s[at]), src.rpix(at));
+    hs = max(hs, __double2hiint(x[i].x) & 0x7fffffff);
+    hr = max(hr, __double2hiint(x[i].y) & 0x7fffffff);
+  }
+  hs = __reduce_max_sync(0xffffffffu, hs);
+  hr = __reduce_max_sync(0xffffffffu, hr);
+  if (threadIdx.x % 32 == 0) {
+    top[0][threadIdx.x / 32] = hs;
+    top[1][threadIdx.x / 32] = hr;
+  }
+  __syncthreads();
+#pragma unroll
+  for (int w = 0; w < NW; ++w) {
+    hs = max(hs, top[0][w]);
+    hr = max(hr, top[1][w]);
+  }
+  const int es = hs >> 20, er = hr >> 20;
+  // unscaled if a field is zero or not finite; FP32 inputs keep the difference far below 1000
+  int sh = es == 0 || er == 0 || es == 2047 || er == 2047 ? 0 : es - er;
+  sh = sh > 1000 ? 1000 : (sh < -1000 ? -1000 : sh);
+  const double beta = __hiloint2double((1023 + sh) << 20, 0), half_ib = 0.5 * __hiloint2double((1023 - sh) << 20, 0);
+#pragma unroll
+  for (int i = 0; i < E; ++i) buf[threadIdx.x + i * G::TR] = make_double2(x[i].x, beta * x[i].y);
+  __syncthreads();
+  dfft<N, G::RB, G::TR, false>(buf);
+  for (int e = threadIdx.x; e < G::RB * WH; e += G::TR) {
+    const int v = e / WH, kx = e % WH;
+    const double2 a = buf[v * N + kx], b = dconj(buf[v * N + (N - kx) % N]);
+    const double2 d = dsub(a, b);  // 2 i beta rpix_hat
+    const long long at = ((long long)blockIdx.x * G::RB + v) * WH + kx;
+    Z[at] = make_double2(0.5 * (a.x + b.x), 0.5 * (a.y + b.y));
+    Z[(long long)N * WH + at] = make_double2(half_ib * d.y, -half_ib * d.x);
+  }
+}
+
+// *out += ||S r||^2: columns kx = 2 g and 2 g + 1 (up to N/2) of both half spectra of k_rows_residual, transformed, then
+// |P rpix_hat - s_hat|^2 / n where P > 0, else |s_hat|^2 / n, twice for the columns whose mirror is left out
+template <int N>
+__global__ void __launch_bounds__(DGeo<N>::TC) k_cols_residual(const float* __restrict__ Pk, const double2* __restrict__ Z,
+                                                               double* out) {
+  using G = DGeo<N>;
+  constexpr int WH = N / 2 + 1;
+  double2* buf = dsmem();
+  const int k0 = 2 * int(blockIdx.x);
+  for (int e = threadIdx.x; e < 4 * N; e += G::TC) {
+    const int c = e % 4, y = e / 4, kx = k0 + c % 2;
+    buf[c * N + y] = kx <= N / 2 ? __ldg(Z + ((long long)(c / 2) * N + y) * WH + kx) : make_double2(0.0, 0.0);
+  }
+  __syncthreads();
+  dfft<N, 4, G::TC, false>(buf);
+  double acc = 0.0;
+#pragma unroll 4
+  for (int i = 0; i < 2 * N / G::TC; ++i) {
+    const int e = threadIdx.x + i * G::TC, kx = k0 + e / N, ky = e % N;
+    if (kx > N / 2) continue;
+    const double p = double(Pk[ky * WH + kx]);
+    const double2 s = buf[e], r = buf[2 * N + e];
+    const double2 v = p > 0.0 ? make_double2(p * r.x - s.x, p * r.y - s.y) : s;
+    acc += (v.x * v.x + v.y * v.y) * ((kx == 0 || kx == N / 2 ? 1.0 : 2.0) / (double(N) * N));
+  }
+  dadd_block<G::TC>(acc, out);
+}
+
+// q_hat = s_hat / (n P) where P > 0, else 0: columns kx = 4 g .. 4 g + 3 (up to N/2) of the half spectrum of s, transformed,
+// divided and transformed back in place
+template <int N>
+__global__ void __launch_bounds__(DGeo<N>::TC) k_cols_divp(const float* __restrict__ Pk, double2* Z) {
+  using G = DGeo<N>;
+  constexpr int WH = N / 2 + 1;
+  double2* buf = dsmem();
+  const int k0 = 4 * int(blockIdx.x);
+  for (int e = threadIdx.x; e < 4 * N; e += G::TC) {
+    const int c = e % 4, y = e / 4;
+    buf[c * N + y] = k0 + c <= N / 2 ? Z[(long long)y * WH + k0 + c] : make_double2(0.0, 0.0);
+  }
+  __syncthreads();
+  dfft<N, 4, G::TC, false>(buf);
+#pragma unroll 4
+  for (int i = 0; i < 4 * N / G::TC; ++i) {
+    const int e = threadIdx.x + i * G::TC, kx = k0 + e / N;
+    const double p = kx <= N / 2 ? double(Pk[(e % N) * WH + kx]) : 0.0;
+    const double q = p > 0.0 ? 1.0 / (double(N) * N * p) : 0.0;
+    buf[e] = p > 0.0 ? make_double2(q * buf[e].x, q * buf[e].y) : make_double2(0.0, 0.0);
+  }
+  __syncthreads();
+  dfft<N, 4, G::TC, true>(buf);
+  for (int e = threadIdx.x; e < 4 * N; e += G::TC) {
+    const int c = e % 4, y = e / 4;
+    if (k0 + c <= N / 2) Z[(long long)y * WH + k0 + c] = buf[c * N + y];
   }
 }
 
@@ -386,6 +477,24 @@ __global__ void __launch_bounds__(DGeo<N>::TR) k_rows_inv(const double2* __restr
   for (int e = threadIdx.x; e < G::RB * N; e += G::TR) dst(f, base + e, buf[e]);
 }
 
+// rows of a real field from its half spectrum
+template <int N, class Dst>
+__global__ void __launch_bounds__(DGeo<N>::TR) k_rows_half(const double2* __restrict__ Z, Dst dst) {
+  using G = DGeo<N>;
+  constexpr int WH = N / 2 + 1;
+  double2* buf = dsmem();
+  for (int e = threadIdx.x; e < G::RB * WH; e += G::TR) {
+    const int v = e / WH, kx = e % WH;
+    const double2 z = __ldg(Z + ((long long)blockIdx.x * G::RB + v) * WH + kx);
+    buf[v * N + kx] = z;
+    if (kx != 0 && kx != N / 2) buf[v * N + N - kx] = dconj(z);
+  }
+  __syncthreads();
+  dfft<N, G::RB, G::TR, true>(buf);
+  const int base = int(blockIdx.x) * G::RB * N;
+  for (int e = threadIdx.x; e < G::RB * N; e += G::TR) dst(0, base + e, buf[e]);
+}
+
 __global__ void k_add_f32(int n, float* s, const float* __restrict__ e) {
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) s[i] += e[i];
 }
@@ -438,7 +547,7 @@ cudaError_t by_size(int N, F&& f) {
 
 }  // namespace
 
-size_t refine_scratch_bytes(int H, int W) { return size_t(H) * W * sizeof(double2); }
+size_t refine_scratch_bytes(int H, int W) { return size_t(2) * H * (W / 2 + 1) * sizeof(double2); }
 
 cudaError_t refine_bnorm(const RefineArgs& a, cudaStream_t st) {
   auto* Z = static_cast<double2*>(a.scratch);
@@ -453,8 +562,13 @@ cudaError_t refine_residual(const RefineArgs& a, cudaStream_t st) {
   auto* Z = static_cast<double2*>(a.scratch);
   return by_size(a.H, [&](auto S) {
     constexpr int N = decltype(S)::value;
-    const cudaError_t e = rows_fwd<N>(SrcResidual{a.d, a.Nd, a.A, a.s, a.mask}, Z, 1, a.rnorm, st);
-    return e != cudaSuccess ? e : cols<N>(OpResidualNorm{a.Pk}, Z, 1, a.rnorm, st);
+    using G = DGeo<N>;
+    cudaError_t e = smem_attr(k_cols_residual<N>, 4 * N * 16);
+    if (e != cudaSuccess) return e;
+    k_rows_residual<N><<<N / G::RB, G::TR, G::RB * N * 16, st>>>(SrcResidual{a.d, a.Nd, a.A, a.s, a.mask}, Z, a.rnorm);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    k_cols_residual<N><<<N / 4 + 1, G::TC, 4 * N * 16, st>>>(a.Pk, Z, a.rnorm);
+    return cudaGetLastError();
   });
 }
 
@@ -462,9 +576,14 @@ cudaError_t refine_correction(const RefineArgs& a, cudaStream_t st) {
   auto* Z = static_cast<double2*>(a.scratch);
   return by_size(a.H, [&](auto S) {
     constexpr int N = decltype(S)::value;
-    const cudaError_t e = cols<N>(OpDivP{a.Pk}, Z, 1, nullptr, st);  // q_hat = s_hat / P
+    using G = DGeo<N>;
+    cudaError_t e = smem_attr(k_cols_divp<N>, 4 * N * 16);
     if (e != cudaSuccess) return e;
-    return rows_inv<N>(Z, DstCorrection<N>{SrcResidual{a.d, a.Nd, a.A, a.s, a.mask}, a.dn, a.rtab, a.row_major}, 1, st);
+    k_cols_divp<N><<<N / 8 + 1, G::TC, 4 * N * 16, st>>>(a.Pk, Z);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    k_rows_half<N><<<N / G::RB, G::TR, G::RB * N * 16, st>>>(
+        Z, DstCorrection<N>{SrcResidual{a.d, a.Nd, a.A, a.s, a.mask}, a.dn, a.rtab, a.row_major});
+    return cudaGetLastError();
   });
 }
 

@@ -26,7 +26,7 @@ struct RefineArgs {
 
 size_t refine_scratch_bytes(int H, int W);
 cudaError_t refine_bnorm(const RefineArgs& a, cudaStream_t st);
-// the norm of the current iterate's residual; leaves its row transforms in scratch
+// the norm of the current iterate's residual; leaves the row transforms of s in scratch
 cudaError_t refine_residual(const RefineArgs& a, cudaStream_t st);
 // after refine_residual: the right-hand side r = A N^-1 (d - A s) - S^-1 s of the correction solve into rtab
 cudaError_t refine_correction(const RefineArgs& a, cudaStream_t st);

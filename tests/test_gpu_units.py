@@ -1,0 +1,57 @@
+"""The refined Wiener filter does not depend on the unit of the data: with d in units of c, and the noise
+variance and the spectrum in units of c^2, the map scales by c and the relative residual stays."""
+import numpy as np
+import pytest
+
+from gpu_common import need_gpu, rel, to_dev, torch
+from oracle import messenger as M
+from paper_1810_02821_gb300 import build, synth, wf
+
+pytestmark = pytest.mark.gpu
+
+UNITS = [1e-7, 1e-5, 1e6]
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _lib():
+    need_gpu()
+    build.build()
+
+
+def _problem(H, c, amp=1.0):
+    p = synth.make_problem(H, seed=H, mask_frac=0.1, k0=1.0 / 32, amp=amp)
+    p.d = (p.d.astype(np.float64) * c).astype(np.float32)
+    p.Ndiag = (p.Ndiag.astype(np.float64) * c * c).astype(np.float32)
+    p.Pk = (p.Pk.astype(np.float64) * c * c).astype(np.float32)
+    return p
+
+
+@pytest.mark.parametrize("H", [16, 64, 128, 512])
+@pytest.mark.parametrize("c,amp", [(c, 1.0) for c in UNITS] + [(1.0, 1e-6)])
+def test_refined_filter_in_any_unit(H, c, amp):
+    """The FP32 map's own rounding leaves a residual of a few 1e-8 (tol 1e-7 is reached in every unit), and bounds the
+    difference of two units' maps: inputs and outputs are rounded once each in either unit (2^-24 = 6e-8 relative, times
+    the few that the filter of a signal of this spectrum lets through)."""
+    one = wf.wf_solve_ex(*to_dev(_problem(H, 1.0, amp)), tol=1e-7, refine=8)
+    p = _problem(H, c, amp)
+    r = wf.wf_solve_ex(*to_dev(p), tol=1e-7, refine=8, allow_not_converged=True)
+    assert r.status == 0 and r.resid < 1e-7, (r.status, r.resid)
+    s = r.s.double().cpu().numpy()
+    rho = M.residual(s, p.d, p.Ndiag, p.mask, p.Pk)
+    assert abs(rho - r.resid) <= 1e-3 * rho + 1e-13, (rho, r.resid)
+    assert rel(s / c, one.s.double().cpu().numpy()) < 1e-6
+
+
+@pytest.mark.parametrize("c", UNITS)
+def test_wiener_map_in_any_unit(c):
+    """The map of the differentiable form at its tolerance of 3e-8, with d, sigma2 and the amplitude in units of c, c^2, c^2."""
+    H = 64
+    p = synth.make_problem(H, seed=3, mask_frac=0.1, k0=1.0 / H, sigma2=(0.05, 0.3))
+
+    def call(u):
+        d = torch.from_numpy((p.d.astype(np.float64) * u).astype(np.float32)).cuda()
+        s2 = torch.from_numpy((p.Ndiag.astype(np.float64) * u * u).astype(np.float32)).cuda()
+        s, _ = wf.wf_wiener_vjp(d, s2, torch.from_numpy(p.mask).cuda(), 1.3 * u * u, -1.8, 1.0 / H, 0.9, tol=3e-8)
+        return s.double().cpu().numpy() / u
+
+    assert rel(call(c), call(1.0)) < 1e-6
