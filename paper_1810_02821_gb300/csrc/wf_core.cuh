@@ -1197,7 +1197,7 @@ __device__ __forceinline__ int ksolve_sweeps(float2 (&x)[KGeo<N>::E], const floa
         // rho = sqrt(tot / bn) against the tolerances, without the division and the root
         const double bn = bnorm2[rhs ? 0 : lev], ref = bn > 0.0 ? bn : 1.0;
         KSolveState d{tot, ltau, lev, k, 1};
-        if (!(tot == tot) || tot > 1e300 * ref) {
+        if (residual_nonfinite(tot, ref)) {
           d.status = 6;  // non-finite residual
         } else if (lev < last_level) {
           if (tot < level_tol * level_tol * ref || k >= level_max) {

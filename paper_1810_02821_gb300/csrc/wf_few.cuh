@@ -283,7 +283,7 @@ __global__ void __launch_bounds__(FewGeo<N, X>::T, FewGeo<N, X>::MIN_CTAS) k_few
             tot *= double(H) * W;
             const double bn = a.bnorm2[a.rhs_mode ? 0 : f * kMaxLevels + lev], ref = bn > 0.0 ? bn : 1.0;
             GSolveState d{tot, ltau, lev, k, 1};
-            if (!(tot == tot) || tot > 1e300 * ref) {
+            if (residual_nonfinite(tot, ref)) {
               d.status = 6;  // non-finite residual
             } else if (lev < last_level) {
               if (tot < a.level_tol * a.level_tol * ref || k >= a.level_max) {

@@ -175,7 +175,7 @@ __global__ void __launch_bounds__(GGeo<N>::T, GGeo<N>::MIN_CTAS) k_gbatch(const 
           const double ref = bn > 0.0 ? bn : 1.0;  // rho = sqrt(tot / ref), compared without division and root
           S.tot = tot;
           S.ref = ref;
-          if (!(tot == tot) || tot > 1e300 * ref) {
+          if (residual_nonfinite(tot, ref)) {
             S.status = 6;
           } else if (S.lev < sc.n_levels - 1) {
             if (tot < a.level_tol * a.level_tol * ref || S.k >= a.level_max) {

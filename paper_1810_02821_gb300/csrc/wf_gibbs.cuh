@@ -66,6 +66,9 @@ WF_HD float wf_weight(float lt, float inb) {
   return 1.0f / (1.0f + lt * inb);
 #endif
 }
+// whether a check's relative residual sqrt(tot / ref) (ref > 0) counts as not finite: tot / ref NaN or above 1e300, without
+// the division. An infinite tot is named by itself: 1e300 ref is infinite too once ref exceeds 1.8e8
+WF_HD bool residual_nonfinite(double tot, double ref) { return !(tot < INFINITY) || tot > 1e300 * ref; }
 // a / b with the fast device division (about 2 ulp); used where a few ulp do not matter
 WF_HD float wf_fdiv(float a, float b) {
 #if defined(__CUDA_ARCH__)

@@ -984,7 +984,7 @@ __global__ void __launch_bounds__(GGeo<N>::T, GGeo<N>::MIN_CTAS) k_global(const 
       const double bn = a.bnorm2[a.rhs_mode ? 0 : lev], ref = bn > 0.0 ? bn : 1.0;
       if (blockIdx.x == 0) a.acc[parity ^ 1] = 0.0;  // next check's accumulator
       GSolveState d{tot, ltau, lev, k, 1};
-      if (!(tot == tot) || tot > 1e300 * ref) {
+      if (residual_nonfinite(tot, ref)) {
         d.status = 6;  // non-finite residual
       } else if (lev < last_level) {
         if (tot < a.level_tol * a.level_tol * ref || k >= a.level_max) {
