@@ -234,8 +234,9 @@ wf_status wf_shear_to_convergence(const float* gamma, int64_t n, int32_t H, int3
  *     cooperative launch per size class with the fields in global memory, or, from 400 images of 256 x 256,
  *     one thread-block cluster per image that runs its whole pipeline with the field in distributed shared
  *     memory (wf_set_large_image_sampler forces either). The size classes, and the chunks of a class on
- *     clusters, run on their own streams (up to `large_streams`) and overlap. All of it is ordered after the
- *     work already on `stream` and the call returns when everything has finished.
+ *     clusters, run on their own streams (up to `large_streams`) and overlap, with the priority of `stream` (up to
+ *     128 x 128 one step above it). All of it is ordered after the work already on `stream` and the call returns
+ *     when everything has finished.
  *   - items: HOST array; the pointers inside are DEVICE pointers owned by the caller; out_wf may be NULL
  *     (then the filter is not written), out_samples may be NULL when n_samples == 0.
  *   - On return items[i].status / iters / resid hold each image's wf_status, solve sweeps and last

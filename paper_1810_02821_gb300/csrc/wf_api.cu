@@ -2183,9 +2183,12 @@ wf_status record_batch(const BatchPlan& p, char* b, cudaStream_t st, ForkJoin& f
   WF_CUDA(cudaEventRecord(ready, st));
   // Small classes come before the large ones in the GPU's order: a cooperative launch of a large class waits until the whole
   // GPU is free, and CTAs of a small class not yet started by then would wait for its end (205 images of 128^2: the last
-  // 53 solves ran alone for 1.4 ms after it)
-  int prio_small = 0, prio_large = 0;
-  WF_CUDA(cudaDeviceGetStreamPriorityRange(&prio_large, &prio_small));
+  // 53 solves ran alone for 1.4 ms after it). The large classes have the priority of `st` and the small ones a step more, so
+  // that the batch passes none of the caller's more urgent streams and waits for none of the less urgent ones
+  int least = 0, greatest = 0, prio_large = 0;
+  WF_CUDA(cudaDeviceGetStreamPriorityRange(&least, &greatest));
+  WF_CUDA(cudaStreamGetPriority(st, &prio_large));
+  const int prio_small = prio_large > greatest ? prio_large - 1 : greatest;  // lower numbers are more urgent
   auto new_stream = [&](cudaStream_t* out, int prio) -> cudaError_t {
     cudaError_t e = cudaStreamCreateWithPriority(out, cudaStreamNonBlocking, prio);
     if (e != cudaSuccess) return e;
