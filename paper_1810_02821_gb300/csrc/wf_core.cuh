@@ -723,9 +723,10 @@ __device__ __forceinline__ void ksweeps(float2 (&x)[KGeo<N>::E], const float2* _
 // pairs on 152 SMs: two rounds of 22.9 us a sweep). Here as many CTAs as are resident take equal shares of all chains'
 // sweeps, laid end to end: CTA i runs sweeps [i W / R, (i + 1) W / R) of the W in all. A share starts and ends inside a
 // chain. The CTA runs the start of its last chain first and hands the state over, then its whole chains, and the rest
-// of its first chain last, from the state that CTA i - 1 handed over at the start of the launch: nobody waits in
-// practice, and the wait is bounded (cooperative launch: all CTAs are resident). A share is at least as long as a chain,
-// so a chain has at most two parts, and the first ends before the second starts. Measured at 128^2, us per sweep of all
+// of its first chain last, from the state that CTA i - 1 handed over. A share is at least as long as a chain, so a chain has at
+// most two parts, and a CTA comes to the second part after as many sweeps of its own as the first part has, or one less (shares
+// differ by a sweep): it waits for that sweep and for the difference of the two CTAs' paces over the first part, and no longer.
+// The wait is bounded (kawait_polls; cooperative launch: all CTAs are resident). Measured at 128^2, us per sweep of all
 // chains: 200 shear pairs 45.8 -> 30.8; scalar 350 chains 27 -> 20.4, 1000 chains 59.0 -> 57.8.
 // ---------------------------------------------------------------------------------------------
 struct KBalance {
@@ -790,12 +791,18 @@ __device__ __forceinline__ void kpublish(const KBalance& b, int i) {
   if (threadIdx.x == 0)
     asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(b.flag + i), "r"(1u) : "memory");
 }
-// waits for slot i (2^22 polls at most); false: gave up
-__device__ __forceinline__ bool kawait(const KBalance& b, int i) {
+// Polls after which a wait for a first part of `sweeps` sweeps gives up: a few seconds, and on top of them time in
+// proportion to the part, since two CTAs' paces may differ by a share of it (a poll is an L2 round trip, 0.3 us at least, so a
+// sweep adds 0.3 ms, several times what the sweep itself takes). A fixed limit of a few seconds gave up on
+// a difference of 1% over parts of some ten million sweeps.
+WF_HD long long kawait_polls(int sweeps) { return (1LL << 22) + 1024LL * sweeps; }
+// waits for slot i, the state after `sweeps` sweeps; false: gave up
+__device__ __forceinline__ bool kawait(const KBalance& b, int i, int sweeps) {
   __shared__ int s_ok;
   if (threadIdx.x == 0) {
     unsigned int v = 0;
-    for (long it = 0; v == 0 && it < (1L << 22); ++it)
+    const long long most = kawait_polls(sweeps);
+    for (long long it = 0; v == 0 && it < most; ++it)
       asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(b.flag + i) : "memory");
     if (v == 0) atomicExch(b.err, 7);  // WF_ERR_TIMEOUT
     s_ok = v != 0;
@@ -835,7 +842,7 @@ __device__ __forceinline__ bool ksample_part(const SampleArgs& a, const KBalance
   using G = KGeo<N>;
   float2 x[G::E];
   if (p.load) {
-    if (!kawait(bal, blockIdx.x - 1)) return false;
+    if (!kawait(bal, blockIdx.x - 1, p.d0)) return false;
     kload<N, 1, false>(x, bal.slot + (blockIdx.x - 1LL) * bal.slot_floats);
   } else {
     kload<N>(x, a.init_s ? a.init_s + p.c * a.init_stride : nullptr);
@@ -941,7 +948,7 @@ __global__ void __launch_bounds__(KGeo<N>::T, kcore_min_ctas<N>()) k_mband(const
     float2 x[G::E];
     const float* P = a.P0;  // the part's band powers
     if (p.load) {
-      if (!kawait(bal, blockIdx.x - 1)) return false;
+      if (!kawait(bal, blockIdx.x - 1, p.d0)) return false;
       P = bal.slot + (blockIdx.x - 1LL) * bal.slot_floats + G::H * G::W;
     }
     for (int b = threadIdx.x; b < a.n_bins; b += G::T) {
@@ -1083,7 +1090,7 @@ __global__ void __launch_bounds__(2 * KGeo<N>::T, N == 64 ? 3 : (N == 32 ? 6 : 1
   kparts<BAL>(bal, a.n_chains, a.n_sweeps, [&](const auto& p) {
     float2 x[G::E];
     if (p.load) {
-      if (!kawait(bal, blockIdx.x - 1)) return false;
+      if (!kawait(bal, blockIdx.x - 1, p.d0)) return false;
       kload<N, 2, false>(x, bal.slot + (blockIdx.x - 1LL) * bal.slot_floats + (threadIdx.x / G::T) * n);
     } else {
       kload<N, 2>(x, a.init_s ? a.init_s + p.c * a.init_stride + (threadIdx.x / G::T) * n : nullptr);

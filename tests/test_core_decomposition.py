@@ -8,8 +8,15 @@
   pair (k, -k) once, in the pair pattern (p[j], q[A-1-j]), (q[j], p[A-1-j]) with the stated frequencies;
 * the slot order of the mode tables.
 """
+import os
+import shutil
+import subprocess
+import tempfile
+
 import numpy as np
 import pytest
+
+from paper_1810_02821_gb300 import build
 
 SIZES = [32, 64, 128]
 
@@ -123,3 +130,33 @@ def test_balanced_shares_cover_every_sweep_once_and_hand_over_in_time(R, n_chain
     for c, v in loads.items():
         assert v["start"][0] == v["ready"][0] + 1 and v["start"][1] >= v["ready"][1] - 1   # equal shares to one sweep
     assert max(length) - min(length) <= 1
+
+
+@pytest.fixture(scope="module")
+def kernel_part():
+    """part(R, n_chains, n_sweeps, [(i, s), ...]) -> rows (exists, chain, first, end, load, save, polls) from the kernels'
+    own share arithmetic, compiled for the host."""
+    if shutil.which("nvcc") is None and not os.path.exists("/usr/local/cuda/bin/nvcc"):
+        pytest.skip("nvcc not available to build the host driver")
+    tmp = tempfile.mkdtemp()
+    exe = os.path.join(tmp, "shares")
+    src = os.path.join(os.path.dirname(os.path.abspath(__file__)), "helpers", "shares_host.cu")
+    subprocess.run([build.nvcc_path(), *build.ARCH, "-std=c++17", "-o", exe, src], check=True, cwd=tmp, capture_output=True)
+
+    def part(R, n_chains, S, which):
+        inp = "".join(f"{R} {n_chains} {S} {i} {s}\n" for i, s in which)
+        out = subprocess.run([exe], input=inp, capture_output=True, text=True, check=True).stdout
+        return [tuple(int(v) for v in line.split()) for line in out.splitlines()]
+
+    yield part
+    shutil.rmtree(tmp, ignore_errors=True)
+
+
+@pytest.mark.parametrize("R,n_chains,S", [(304, 305, 7), (304, 305, 10 ** 7), (152, 200, 2 ** 31 - 1)])
+def test_the_wait_for_a_state_outlasts_its_sweeps(kernel_part, R, n_chains, S):
+    """A CTA may come to the rest of a chain a sweep before the state is ready, and its pace over that part may differ from
+    the other CTA's: the limit of the wait, at 0.3 us a poll or more, is a second and then 0.1 ms for every sweep waited for."""
+    for row in kernel_part(R, n_chains, S, [(i, s) for i in range(R) for s in range(4)]):
+        exists, _, first, _, load, _, polls = row
+        if exists and load:
+            assert polls * 0.3e-6 >= 1.0 + 0.1e-3 * first
