@@ -456,8 +456,9 @@ double wf_last_kernel_ms(void);
  * fewer fields and at 512 x 512 (spin-2: clusters from 24 chains at 256 x 256), and in their place, for as
  * many fields as are resident at once (also at 64 x 64, 128 x 128 and 1024 x 1024), kernels of the same
  * arithmetic that keep the tables, and up to 256 x 256 the field, in shared memory (equal bit for bit);
- * mode 1: always the global-memory kernels; mode 2: clusters wherever the device can host them. Returns the
- * previous mode.
+ * mode 1: always the global-memory kernels; mode 2: clusters wherever the device can host them. Up to
+ * 128 x 128, mode 2 runs what mode 0 runs, and mode 1 the on-chip kernels or, for few fields of 128 x 128, the
+ * global-memory kernels. Returns the previous mode.
  */
 int32_t wf_set_large_image_sampler(int32_t mode);
 

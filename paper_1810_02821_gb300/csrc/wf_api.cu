@@ -191,12 +191,14 @@ bool size_on_chip(int H) { return H <= 128; }
 // chains: sampler 64^2 clusters / on chip 1 chain 3.2 / 3.9, 114 chains 4.3 / 4.6, 152 chains 4.8 / 4.7; 128^2 clusters 3.8
 // for up to 14 chains, 4.8 for 36, 5.6 for the 48 that are resident at once, on chip 9.6 (60 chains, two rounds of
 // clusters: as long), k_global 6.4 to 9.2 for up to 36. A Wiener filter 64^2 3.3 / 3.1, 128^2 3.9 / 8.0 (from zero only: the
-// other paths take no starting iterate). Spin-2 128^2, k_few2 / on chip: 1 chain 5.7 / 22.9, 36 chains 8.2 / 22.9; without
+// other paths take no starting iterate). "cluster" on the large-image switch takes the clusters up to 128^2 as "auto" does,
+// "global" takes none of them. Spin-2 128^2, k_few2 / on chip: 1 chain 5.7 / 22.9, 36 chains 8.2 / 22.9; without
 // clusters k_gspin2 takes 7.6 for 1 chain, 20.6 for 39.
+bool few_allowed(int H) { return g_large_sampler == 0 || (g_large_sampler == 2 && size_on_chip(H)); }
 bool sample_on_chip(int H, int units) {
-  if (H == 64) return g_large_sampler != 0 || units >= kFew64 || units > few_max(64, false);
-  if (H != 128) return size_on_chip(H);
-  const int few = few_max(H, false);
+  if (H != 64 && H != 128) return size_on_chip(H);
+  const int few = few_allowed(H) ? few_max(H, false) : 0;
+  if (H == 64) return units >= kFew64 || units > few;
   return units > (few > 0 ? few : kFew128 - 1);
 }
 bool spin2_on_chip(int H, int units) { return size_on_chip(H) && !(H == 128 && units < kFewSpin2); }
@@ -405,7 +407,7 @@ int few2_max(int H, bool quiet) {
 }
 
 cudaError_t launch_global_any(int H, const wf::GlobalArgs& a, cudaStream_t st, wf::LaunchTimer* t) {
-  if (a.mode <= 1 && g_large_sampler == 0 && a.n_fields <= few_max(H, a.mode == 1)) {
+  if (a.mode <= 1 && few_allowed(H) && a.n_fields <= few_max(H, a.mode == 1)) {
     switch (H) {
       case 64: return wf::launch_few<64>(a, st, t);  // sampler only
       case 128: return wf::launch_few<128>(a, st, t);
@@ -831,7 +833,7 @@ wf_status solve_pass(const float* d, const float* Ndiag, const uint8_t* mask, co
 // Problems of one launch of solve_many: one CTA each at 32 and 64, as many as k_few holds from 128 on
 int solve_many_max(int H) {
   if (H == 32 || H == 64) return 64;
-  return H >= 128 && g_large_sampler == 0 && few_max(H, true) > 1 ? few_max(H, true) : 1;
+  return H >= 128 && few_allowed(H) && few_max(H, true) > 1 ? few_max(H, true) : 1;
 }
 // Cooled messenger solves of F problems d + f H W with the same N, mask and P at once (2 <= F <= solve_many_max; d finite,
 // no refinement, response or starting iterate): s_W to out + f H W. The problems run side by side in one launch, each as
@@ -1334,7 +1336,7 @@ struct Spin2Path {
 };
 Spin2Path spin2_path(int H, int chains, bool quiet) {
   Spin2Path p;
-  if (g_large_sampler == 0 && chains <= few2_max(H, quiet)) {
+  if (few_allowed(H) && chains <= few2_max(H, quiet)) {
     p.few = p.global = true;
     p.perm = -1;
     p.z_count = size_t(chains) * H * H;
