@@ -389,7 +389,8 @@ wf_status wf_loglike_grad_batch(wf_lik_item* items, int32_t n_items, int32_t n_p
  *   x = C^-1 d_o = N^-1 (d - s_W) on o,  y = C^-1 (S g)_o  (C is symmetric, so the adjoint of the solve
  *   is one more Wiener solve: y = N^-1 (S g - s_W(S g)) on o, with the Wiener filter of "data" S g).
  * The dS terms are cross spectral powers sum_k dP_k Re(conj(U a)_k (U b)_k), evaluated as in
- * wf_spectral_power; S g is applied with FP64 transforms.
+ * wf_spectral_power from a + c b and a - c b (c: the power of two that brings b to a's scale); S g is applied
+ * with FP64 transforms.
  *   s_w_in: device [H][W], the Wiener filter of d for these parameters kept from an earlier call (the
  *           checkpointed forward solve), or NULL: it is solved here.
  *   g:      device [H][W] cotangent, or NULL: only the forward map is computed (out_vjp untouched).

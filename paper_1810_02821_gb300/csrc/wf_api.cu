@@ -2541,23 +2541,45 @@ __global__ void k_rademacher(int n, uint32_t probe, uint32_t k0, uint32_t k1, co
   }
 }
 
-// v = g - y (all pixels; y is 0 on missing ones) and sum[0] += sum_o sigma2 y x
+// v = g - y (all pixels; y is 0 on missing ones), sum[0] += sum_o sigma2 y x, sum[1] += x.x and sum[2] += v.v
 __global__ void k_vjp_mix(int n, const float* __restrict__ g, const float* __restrict__ y, const float* __restrict__ x,
                           const float* __restrict__ sigma2, const uint8_t* __restrict__ mask, float* v, double* sum) {
-  double a = 0.0;
+  double a = 0.0, xx = 0.0, vv = 0.0;
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-    v[i] = g[i] - y[i];
-    if (mask[i] == 0) a += double(sigma2[i]) * double(y[i]) * double(x[i]);
+    const float vi = g[i] - y[i];
+    const double xd = x[i];
+    v[i] = vi;
+    if (mask[i] == 0) a += double(sigma2[i]) * double(y[i]) * xd;
+    xx += xd * xd;
+    vv += double(vi) * double(vi);
   }
-  for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
-  if ((threadIdx.x & 31) == 0) atomicAdd(sum, a);
+  for (int o = 16; o > 0; o >>= 1) {
+    a += __shfl_xor_sync(0xffffffffu, a, o);
+    xx += __shfl_xor_sync(0xffffffffu, xx, o);
+    vv += __shfl_xor_sync(0xffffffffu, vv, o);
+  }
+  if ((threadIdx.x & 31) == 0) {
+    atomicAdd(sum, a);
+    atomicAdd(sum + 1, xx);
+    atomicAdd(sum + 2, vv);
+  }
 }
+
+// Cross powers of x = C^-1 z and a probe z: z.x / n (k_xres's first sum) is the scale of x against z. n a power of two
+wf::PairScale probe_scale(const double* sums, size_t n) {
+  wf::PairScale p;
+  p.sums = sums;
+  while ((size_t(1) << p.shift) < n) ++p.shift;
+  return p;
+}
+// the cross power from the powers of a + 2^e b and a - 2^e b
+double cross_power(double plus, double minus, int e) { return std::ldexp(plus - minus, -2 - e); }
 
 // weighted spectral power into device memory dout[n_fields * nw]
 cudaError_t spectral_power_dev(const float* a, const float* b, float sgn, int n_fields, const float* w, int nw, int H,
-                               int W, double* dout, cudaStream_t st) {
+                               int W, double* dout, cudaStream_t st, const wf::PairScale& scale = wf::PairScale()) {
   if (size_on_chip(H)) {
-    wf::WpowerArgs p{a, b, sgn, n_fields, w, nw, dout};
+    wf::WpowerArgs p{a, b, sgn, n_fields, w, nw, dout, scale};
     switch (H) {
       case 16: return wf::launch_wpower<16>(p, st);
       case 32: return wf::launch_wpower<32>(p, st);
@@ -2595,6 +2617,7 @@ cudaError_t spectral_power_dev(const float* a, const float* b, float sgn, int n_
     g.va = a;
     g.vb = b;
     g.vsign = sgn;
+    g.vscale = scale;
     g.wts = w;
     g.nw = nw;
     g.wout = dout;
@@ -2718,16 +2741,19 @@ wf_status wf_loglike_grad(const float* d, const float* sigma2, const uint8_t* ma
     for (int j = 0; j < F; ++j)  // x = C^-1 z
       k_xres<<<xb, 256, 0, st>>>(int(n), zs + j * n, ws + j * n, Nd, sigma2, mask, xs + j * n, psum + 4 * j);
     WF_CUDA(cudaGetLastError());
-    // w^T dS z = (|U(w+z)|^2_dP - |U(w-z)|^2_dP) / 4
-    if ((e = spectral_power_dev(xs, zs, 1.f, F, dPa, 2, H, W, ppow, st)) != cudaSuccess) return cuda_fail(e);
-    if ((e = spectral_power_dev(xs, zs, -1.f, F, dPa, 2, H, W, ppow + 2 * F, st)) != cudaSuccess) return cuda_fail(e);
+    // w^T dS z = (|U(w + c z)|^2_dP - |U(w - c z)|^2_dP) / 4c
+    const wf::PairScale sc = probe_scale(psum, n);
+    if ((e = spectral_power_dev(xs, zs, 1.f, F, dPa, 2, H, W, ppow, st, sc)) != cudaSuccess) return cuda_fail(e);
+    if ((e = spectral_power_dev(xs, zs, -1.f, F, dPa, 2, H, W, ppow + 2 * F, st, sc)) != cudaSuccess)
+      return cuda_fail(e);
     WF_CUDA(cudaMemcpyAsync(hps.data(), psum, 4 * sizeof(double) * size_t(F), cudaMemcpyDeviceToHost, st));
     WF_CUDA(cudaMemcpyAsync(hpp.data(), ppow, 4 * sizeof(double) * size_t(F), cudaMemcpyDeviceToHost, st));
     WF_CUDA(cudaStreamSynchronize(st));
     for (int j = 0; j < F; ++j) {
       const double* plus = hpp.data() + 2 * j;
       const double* minus = plus + 2 * F;
-      const double t[3] = {0.25 * (plus[0] - minus[0]), 0.25 * (plus[1] - minus[1]), hps[4 * j + 1]};
+      const int ex = sc.exponent(hps[4 * j], 0.0);
+      const double t[3] = {cross_power(plus[0], minus[0], ex), cross_power(plus[1], minus[1], ex), hps[4 * j + 1]};
       for (int i = 0; i < 3; ++i) {
         tsum[i] += t[i];
         tsq[i] += t[i] * t[i];
@@ -2842,9 +2868,10 @@ wf_status wf_loglike_grad_batch(wf_lik_item* items, int32_t n_items, int32_t n_p
         float* wv = F(o_w[i]) + size_t(j) * n;
         k_xres<<<xb, 256, 0, st>>>(int(n), z, wv, F(o_N[i]), it.sigma2, it.mask, F(o_x[i]), sums + 4 * q);
         WF_CUDA(cudaGetLastError());
-        cudaError_t e = spectral_power_dev(F(o_x[i]), z, 1.f, 1, F(o_P[i]) + nm, 2, it.H, it.W, pws + 4 * q, st);
+        const wf::PairScale sc = probe_scale(sums + 4 * q, n);
+        cudaError_t e = spectral_power_dev(F(o_x[i]), z, 1.f, 1, F(o_P[i]) + nm, 2, it.H, it.W, pws + 4 * q, st, sc);
         if (e == cudaSuccess)
-          e = spectral_power_dev(F(o_x[i]), z, -1.f, 1, F(o_P[i]) + nm, 2, it.H, it.W, pws + 4 * q + 2, st);
+          e = spectral_power_dev(F(o_x[i]), z, -1.f, 1, F(o_P[i]) + nm, 2, it.H, it.W, pws + 4 * q + 2, st, sc);
         if (e != cudaSuccess) return cuda_fail(e);
       }
     }
@@ -2865,7 +2892,9 @@ wf_status wf_loglike_grad_batch(wf_lik_item* items, int32_t n_items, int32_t n_p
       double tsum[3] = {0, 0, 0}, tsq[3] = {0, 0, 0};
       for (int j = 0; j < n_probes; ++j) {
         const size_t q = size_t(n_items) + size_t(i) * n_probes + j;
-        const double t[3] = {0.25 * (hp[4 * q] - hp[4 * q + 2]), 0.25 * (hp[4 * q + 1] - hp[4 * q + 3]), hs[4 * q + 1]};
+        const int ex = probe_scale(nullptr, size_t(it.H) * it.W).exponent(hs[4 * q], 0.0);
+        const double t[3] = {cross_power(hp[4 * q], hp[4 * q + 2], ex), cross_power(hp[4 * q + 1], hp[4 * q + 3], ex),
+                             hs[4 * q + 1]};
         for (int k = 0; k < 3; ++k) {
           tsum[k] += t[k];
           tsq[k] += t[k] * t[k];
@@ -2939,19 +2968,23 @@ wf_status wf_wiener_vjp(const float* d, const float* sigma2, const uint8_t* mask
   if ((r = wf_solve_ex(bv, Nd, mask, P, H, W, &so, wv, &it, &rs, stream)) != WF_OK) return r;  // s_W(S g)
   k_xres<<<xb, 256, 0, st>>>(int(n), bv, wv, Nd, sigma2, mask, y, sums);  // y = C^-1 (S g)_o
   WF_CUDA(cudaGetLastError());
-  WF_CUDA(cudaMemsetAsync(sums, 0, sizeof(double), st));
+  WF_CUDA(cudaMemsetAsync(sums, 0, 3 * sizeof(double), st));
   k_vjp_mix<<<xb, 256, 0, st>>>(int(n), g, y, x, sigma2, mask, bv, sums);  // bv = g - y
   WF_CUDA(cudaGetLastError());
-  // (g - y)^T dS x = (|U(x + v)|^2_dP - |U(x - v)|^2_dP) / 4
-  if ((e = spectral_power_dev(x, bv, 1.f, 1, dPa, 2, H, W, pw, st)) != cudaSuccess) return cuda_fail(e);
-  if ((e = spectral_power_dev(x, bv, -1.f, 1, dPa, 2, H, W, pw + 2, st)) != cudaSuccess) return cuda_fail(e);
-  double hs, hq[4];
-  WF_CUDA(cudaMemcpyAsync(&hs, sums, sizeof(double), cudaMemcpyDeviceToHost, st));
+  // (g - y)^T dS x = (|U(x + c v)|^2_dP - |U(x - c v)|^2_dP) / 4c, c^2 about x.x / v.v
+  wf::PairScale sc;
+  sc.sums = sums + 1;
+  sc.ratio = true;
+  if ((e = spectral_power_dev(x, bv, 1.f, 1, dPa, 2, H, W, pw, st, sc)) != cudaSuccess) return cuda_fail(e);
+  if ((e = spectral_power_dev(x, bv, -1.f, 1, dPa, 2, H, W, pw + 2, st, sc)) != cudaSuccess) return cuda_fail(e);
+  double hs[3], hq[4];
+  WF_CUDA(cudaMemcpyAsync(hs, sums, 3 * sizeof(double), cudaMemcpyDeviceToHost, st));
   WF_CUDA(cudaMemcpyAsync(hq, pw, 4 * sizeof(double), cudaMemcpyDeviceToHost, st));
   WF_CUDA(cudaStreamSynchronize(st));
-  out_vjp[0] = 0.25 * (hq[0] - hq[2]);
-  out_vjp[1] = 0.25 * (hq[1] - hq[3]);
-  out_vjp[2] = -hs;
+  const int ex = sc.exponent(hs[1], hs[2]);
+  out_vjp[0] = cross_power(hq[0], hq[2], ex);
+  out_vjp[1] = cross_power(hq[1], hq[3], ex);
+  out_vjp[2] = -hs[0];
   return WF_OK;
 }
 

@@ -19,6 +19,7 @@
 
 #include <cmath>
 #include <cstdint>
+#include <cstring>
 #include <limits>
 #include <type_traits>
 
@@ -69,6 +70,15 @@ WF_HD float wf_weight(float lt, float inb) {
 // whether a check's relative residual sqrt(tot / ref) (ref > 0) counts as not finite: tot / ref NaN or above 1e300, without
 // the division. An infinite tot is named by itself: 1e300 ref is infinite too once ref exceeds 1.8e8
 WF_HD bool residual_nonfinite(double tot, double ref) { return !(tot < INFINITY) || tot > 1e300 * ref; }
+WF_HD unsigned long long wf_double_bits(double v) {
+#if defined(__CUDA_ARCH__)
+  return (unsigned long long)__double_as_longlong(v);
+#else
+  unsigned long long u;
+  std::memcpy(&u, &v, sizeof(u));
+  return u;
+#endif
+}
 // a / b with the fast device division (about 2 ulp); used where a few ulp do not matter
 WF_HD float wf_fdiv(float a, float b) {
 #if defined(__CUDA_ARCH__)
@@ -1362,7 +1372,33 @@ __global__ void __launch_bounds__(N) k_bnorm(BnormArgs a) {
   if (lt == 0) a.bnorm2[lev] = v;
 }
 
-// Weighted spectral power of real fields v_f = a_f + sgn * b_f (b may be null): out[f*nw + j] =
+// Scale of b in the spectral power of a_f + sgn scale b_f. A cross power, sum_k w Re(conj(U a) U b), is the difference of the
+// powers of a + b and a - b over four; the sums are FP32, so with fields of different units (x = C^-1 z goes with one over the
+// noise variance, z is +-1) the smaller would vanish in them. A power of two that brings b to a costs nothing and divides
+// out exactly: 2^e with, from sums on the device (4 per field, the first two used), e = log2 sums[0] - shift, or half of
+// log2(sums[0] / sums[1]) with `ratio`. No sums: 1.
+struct PairScale {
+  const double* sums = nullptr;
+  int shift = 0;
+  bool ratio = false;
+  WF_HD int exponent(double s0, double s1) const {
+    auto ex = [](double v) {  // floor(log2 |v|), or out of range for 0 and values that are not finite
+      const int h = int((wf_double_bits(v) >> 52) & 0x7ff);
+      return h == 0 || h == 2047 ? 1 << 20 : h - 1023;
+    };
+    const int a = ex(s0), b = ratio ? ex(s1) : 0;
+    if (a == 1 << 20 || b == 1 << 20) return 0;
+    const int e = ratio ? (a - b) / 2 : a - shift;
+    return e > 100 ? 100 : (e < -100 ? -100 : e);
+  }
+};
+#if defined(__CUDACC__)
+__device__ __forceinline__ float pair_scale(const PairScale& p, int f) {
+  return p.sums ? ldexpf(1.0f, p.exponent(p.sums[4 * f], p.ratio ? p.sums[4 * f + 1] : 0.0)) : 1.0f;
+}
+#endif
+
+// Weighted spectral power of real fields v_f = a_f + sgn * scale_f * b_f (b may be null): out[f*nw + j] =
 // sum_k w_j(k) |(U v_f)_k|^2 with U the unitary 2D DFT (one CTA per field).
 struct WpowerArgs {
   const float* a;
@@ -1372,6 +1408,7 @@ struct WpowerArgs {
   const float* w;
   int nw;
   double* out;
+  PairScale scale;
 };
 
 template <int N>
@@ -1383,12 +1420,13 @@ __global__ void __launch_bounds__(N) k_wpower(WpowerArgs p) {
   const int f = blockIdx.x, lt = threadIdx.x;
   const long long base = (long long)f * G::H * G::W + (long long)lt * G::W;
   float2 c[G::LR];
+  const float sgn = p.sgn * pair_scale(p.scale, f);
 #pragma unroll
   for (int m = 0; m < G::LR; ++m) {
     float2 v = reinterpret_cast<const float2*>(p.a + base)[m];
     if (p.b) {
       const float2 u = reinterpret_cast<const float2*>(p.b + base)[m];
-      v = make_float2(fmaf(p.sgn, u.x, v.x), fmaf(p.sgn, u.y, v.y));
+      v = make_float2(fmaf(sgn, u.x, v.x), fmaf(sgn, u.y, v.y));
     }
     c[m] = v;
   }

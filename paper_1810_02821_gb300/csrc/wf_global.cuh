@@ -328,10 +328,11 @@ struct GlobalArgs {
   int mode;                // 0 sampler, 1 Wiener filter, 2 level norms (fields = levels), 3 weighted power
   int levels;              // mode 2: field f is level f % levels of pixel table f / levels
   double* bnorm_out;       // mode 2: [n_fields / levels][kMaxLevels]
-  // mode 3: fields v_f = va_f + vsign * vb_f, tables wts[nw][H][W/2+1], sums into wout[f*nw + j]
+  // mode 3: fields v_f = va_f + vsign * vscale_f * vb_f, tables wts[nw][H][W/2+1], sums into wout[f*nw + j]
   const float* va;
   const float* vb;
   float vsign;
+  PairScale vscale;
   const float* wts;
   int nw;
   double* wout;
@@ -549,11 +550,13 @@ __device__ void row_item(const GlobalArgs& a, int f, int y0, int done, bool firs
   } else if (a.mode == 3) {
     const long long o = ((long long)f * G::H + y) * G::W;
     grow_load<N>(x, a.va + o);
-    if (a.vb)
+    if (a.vb) {
+      const float sgn = a.vsign * pair_scale(a.vscale, f);
       gpixels<N>(x, [&](float2& v, int e) {
         const float2 u = __ldg(reinterpret_cast<const float2*>(a.vb + o) + e);
-        v = make_float2(fmaf(a.vsign, u.x, v.x), fmaf(a.vsign, u.y, v.y));
+        v = make_float2(fmaf(sgn, u.x, v.x), fmaf(sgn, u.y, v.y));
       });
+    }
   } else {
     grow_load<N>(x, a.mode == 0 && a.init_s ? a.init_s + f * a.init_stride + (long long)y * G::W : nullptr);
   }

@@ -1,4 +1,4 @@
-"""The refined Wiener filter does not depend on the unit of the data: with d in units of c, and the noise
+"""The refined Wiener filter and its derivatives do not depend on the unit of the data: with d in units of c, and the noise
 variance and the spectrum in units of c^2, the map scales by c and the relative residual stays."""
 import numpy as np
 import pytest
@@ -55,3 +55,45 @@ def test_wiener_map_in_any_unit(c):
         return s.double().cpu().numpy() / u
 
     assert rel(call(c), call(1.0)) < 1e-6
+
+
+@pytest.mark.parametrize("c", UNITS)
+def test_vjp_in_any_unit(c):
+    """d, sigma2 and the amplitude in units of c, c^2 and c^2: the map scales by c, its derivatives by c (slope, alpha) and
+    1/c (amplitude). Solves to 3e-8, derivatives as sums over 64^2 modes and pixels of products of two such solutions."""
+    H = 64
+    p = synth.make_problem(H, seed=3, mask_frac=0.1, k0=1.0 / H, sigma2=(0.05, 0.3))
+    g = torch.from_numpy(np.random.default_rng(H).standard_normal((H, H)).astype(np.float32)).cuda()
+
+    def call(u):
+        d = torch.from_numpy((p.d.astype(np.float64) * u).astype(np.float32)).cuda()
+        s2 = torch.from_numpy((p.Ndiag.astype(np.float64) * u * u).astype(np.float32)).cuda()
+        s, v = wf.wf_wiener_vjp(d, s2, torch.from_numpy(p.mask).cuda(), 1.3 * u * u, -1.8, 1.0 / H, 0.9, g, tol=3e-8)
+        return s.double().cpu().numpy() / u, v * np.array([u, 1.0 / u, 1.0 / u])
+
+    (s1, v1), (s, v) = call(1.0), call(c)
+    assert rel(s, s1) < 1e-6
+    np.testing.assert_allclose(v, v1, rtol=1e-4, atol=1e-6 * np.abs(v1).max())
+
+
+@pytest.mark.parametrize("H", [16, 64, 256])
+@pytest.mark.parametrize("c", UNITS)
+def test_likelihood_gradient_in_any_unit(H, c):
+    """Gradients by amplitude, slope and alpha scale by 1/c^2, 1 and 1. The trace probes' solves stop at 1e-5 in either
+    unit (their sums agree to a few times that)."""
+    p = synth.make_problem(H, seed=4, mask_frac=0.1, k0=1.0 / H, sigma2=(0.05, 0.3))
+
+    def call(u, batch=False):
+        d = torch.from_numpy((p.d.astype(np.float64) * u).astype(np.float32)).cuda()
+        s2 = torch.from_numpy((p.Ndiag.astype(np.float64) * u * u).astype(np.float32)).cuda()
+        m = torch.from_numpy(p.mask).cuda()
+        par = (1.3 * u * u, -1.8, 1.0 / H, 0.9)
+        if batch:
+            r = wf.wf_loglike_grad_batch([(d, s2, m, *par, 1)], n_probes=3, tol=1e-6)[0]
+        else:
+            r = wf.wf_loglike_grad(d, s2, m, *par, n_probes=3, seed=1, tol=1e-6)
+        return r.grad * np.array([u * u, 1.0, 1.0])
+
+    one, got, batch = call(1.0), call(c), call(c, batch=True)
+    np.testing.assert_allclose(got, one, rtol=1e-4, atol=1e-4 * np.abs(one).max())
+    np.testing.assert_allclose(batch, one, rtol=1e-3, atol=1e-3 * np.abs(one).max())
