@@ -312,11 +312,11 @@ void wf_batch_graph_destroy(wf_batch_graph g);
 /*
  * Launch-shape autotuner of the batched form. Starting from *opts, it times graph replays of this batch
  * (one warm-up and `reps` timed replays per candidate, CUDA events on `stream`) and keeps, one knob at a
- * time, the fastest large_grid_pct in {100, 50, 25, 12}, large_streams in {1, 2, 4, 8, 16} (when the batch has
- * images above 128 x 128), large_cluster_rows in {32, 64} (when it has 512 x 512 images), small_path in {0, 1}
- * and then, for the fused path, small_grid_pct in {100, 50, 25} or, for the phased path,
- * small_fields_per_cta in {1, 2, 4, 8} (when it has images up to 128 x 128); the chosen values are written
- * back to *opts and the
+ * time, the fastest large_grid_pct in {100, 50, 25, 12} (when a class above 128 x 128 runs on the global-memory
+ * kernels), large_streams in {1, 2, 4, 8, 16} (when one runs on clusters, or there are several),
+ * large_cluster_rows in {32, 64} (when 512 x 512 images run on clusters), small_path in {0, 1} (when there are images
+ * up to 128 x 128) and then, for the fused path, small_grid_pct in {100, 50, 25} or, for the phased path with samples of
+ * 16 x 16 images, small_fields_per_cta in {1, 2, 4, 8}; the chosen values are written back to *opts and the
  * best replay time to *best_ms (HOST, may be NULL). The items' outputs are overwritten by the trial runs.
  * A representative subset of a large batch tunes faster than the whole batch.
  */

@@ -2399,8 +2399,9 @@ wf_status wf_batch_autotune(const wf_batch_item* items, int32_t n_items, wf_batc
   if (!opts || !items || n_items < 1 || reps < 1) return WF_ERR_ARG;
   if (!batch_opts_ok(*opts)) return WF_ERR_ARG;
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-  bool has_large = false;
-  for (int i = 0; i < n_items; ++i) has_large |= items[i].H > 128;
+  int count[7] = {};  // images per size class
+  for (int i = 0; i < n_items; ++i)
+    for (int c = 0; c < 7; ++c) count[c] += items[i].H == kBatchSizes[c];
   cudaEvent_t e0, e1;
   WF_CUDA(cudaEventCreate(&e0));
   if (cudaEventCreate(&e1) != cudaSuccess) {
@@ -2441,22 +2442,21 @@ wf_status wf_batch_autotune(const wf_batch_item* items, int32_t n_items, wf_batc
       }
     }
   };
-  bool has_512 = false;
-  for (int i = 0; i < n_items; ++i) has_512 |= items[i].H == 512;
-  if (has_large) {
-    try_knob(&wf_batch_opts::large_grid_pct, {100, 50, 25, 12});
-    try_knob(&wf_batch_opts::large_streams, {1, 2, 4, 8, 16});
+  // only the knobs that reach a kernel of this batch (a candidate costs a capture and its replays)
+  int large = 0, clusters = 0;  // classes above 128 x 128, and those of them on clusters
+  for (int c = 4; c < 7; ++c) {
+    large += count[c] > 0;
+    clusters += count[c] > 0 && use_cluster(kBatchSizes[c], count[c], best.large_cluster_rows);
   }
-  if (has_512) try_knob(&wf_batch_opts::large_cluster_rows, {32, 64});
-  bool has_small = false;
-  for (int i = 0; i < n_items; ++i) has_small |= items[i].H <= 128;
-  int min_small = 1024;
-  for (int i = 0; i < n_items; ++i)
-    if (items[i].H < min_small) min_small = items[i].H;
-  if (has_small) {
+  if (large > clusters) try_knob(&wf_batch_opts::large_grid_pct, {100, 50, 25, 12});
+  if (clusters || large > 1) try_knob(&wf_batch_opts::large_streams, {1, 2, 4, 8, 16});
+  if (count[5] && use_cluster(512, count[5], best.large_cluster_rows))
+    try_knob(&wf_batch_opts::large_cluster_rows, {32, 64});
+  if (count[0] + count[1] + count[2] + count[3]) {
     try_knob(&wf_batch_opts::small_path, {0, 1});
     if (best.small_path == 1) try_knob(&wf_batch_opts::small_grid_pct, {100, 50, 25});
-    if (best.small_path == 0 && min_small < 128) try_knob(&wf_batch_opts::small_fields_per_cta, {1, 2, 4, 8});
+    if (best.small_path == 0 && count[0] && best.n_samples > 0)
+      try_knob(&wf_batch_opts::small_fields_per_cta, {1, 2, 4, 8});
   }
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
