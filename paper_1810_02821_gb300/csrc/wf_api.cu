@@ -184,12 +184,12 @@ cudaError_t launch_prep(const float* d, const float* Ndiag, const uint8_t* mask,
 
 int few_max(int H, bool solve);
 
-constexpr int kFew64 = 115, kFew128 = 36, kFewSpin2 = 40;  // chains from which the on-chip kernels run
+constexpr int kFew64 = 115, kFew128 = 36, kFewSpin2 = 40;  // chains from which the on-chip kernels run, on 152 SMs
 bool size_on_chip(int H) { return H <= 128; }
 // Whether fields of an on-chip size run on the on-chip kernels, one CTA per field, or spread over several SMs (k_few:
 // clusters, where the device has them; else k_global at 128^2), with less latency for few fields. us per sweep of all
 // chains: sampler 64^2 clusters / on chip 1 chain 3.2 / 3.9, 114 chains 4.3 / 4.6, 152 chains 4.8 / 4.7; 128^2 clusters 3.8
-// for up to 14 chains, 4.8 for 36, 5.6 for the 48 that are resident at once, on chip 9.6 (60 chains, two rounds of
+// for up to 14 chains, 4.8 for 36, 5.6 for the 50 or so that are resident at once, on chip 9.6 (60 chains, two rounds of
 // clusters: as long), k_global 6.4 to 9.2 for up to 36. A Wiener filter 64^2 3.3 / 3.1, 128^2 3.9 / 8.0 (from zero only: the
 // other paths take no starting iterate). "cluster" on the large-image switch takes the clusters up to 128^2 as "auto" does,
 // "global" takes none of them. Spin-2 128^2, k_few2 / on chip: 1 chain 5.7 / 22.9, 36 chains 8.2 / 22.9; without
@@ -318,14 +318,6 @@ bool cluster_fits(int H, int rows) {
   return known[k][dev] == 1;
 }
 
-// Order of the sampler's mode table at an on-chip size (mode_pos), which selects its kernel: several threads per
-// row, except for more 64 x 64 chains than one wave of that kernel (5 CTAs on each of 152 SMs), where the
-// one-thread-per-row kernel runs with fewer instructions (us per sweep, one thread per row / several: 600 chains
-// 9.77 / 8.99, 900 chains 13.3 / 14.9, 1216 chains 17.1 / 17.6, 2048 chains 29.3 / 29.7; both kernels are then bound by
-// instruction dispatch). At 32 and 128 several threads per row are faster or equal at every count (128, 1000
-// chains: 65.4 / 60.0; 32, 4864 chains: 17.0 / 16.8).
-int sample_cm(int H, int n_chains) { return H == 64 && n_chains > 760 ? 0 : wf::core_cm(H); }
-
 // An output the kernels may store to: device or managed memory, or page-locked host memory that is
 // mapped into the device address space at the same address (cudaHostAlloc, or cudaHostRegister with
 // mapping, under unified addressing). Page-locked memory without that mapping cannot be written by a
@@ -367,6 +359,18 @@ int resident_fields(std::mutex& mu, int (&known)[64], F&& query) {
     known[dev] = n + 1;
   }
   return known[dev] - 1;
+}
+
+// Order of the sampler's mode table at an on-chip size (mode_pos), which selects its kernel: several threads per
+// row, except for more 64 x 64 chains than one wave of that kernel (on 152 SMs with 5 CTAs each 760), where the
+// one-thread-per-row kernel runs with fewer instructions (us per sweep, one thread per row / several: 600 chains
+// 9.77 / 8.99, 900 chains 13.3 / 14.9, 1216 chains 17.1 / 17.6, 2048 chains 29.3 / 29.7; both kernels are then bound by
+// instruction dispatch). At 32 and 128 several threads per row are faster or equal at every count (128, 1000
+// chains: 65.4 / 60.0; 32, 4864 chains: 17.0 / 16.8).
+int sample_cm(int H, int n_chains) {
+  static std::mutex mu;
+  static int known[64] = {};
+  return H == 64 && n_chains > resident_fields(mu, known, wf::sample_wave<64>) ? 0 : wf::core_cm(H);
 }
 
 // Fields of a launch up to which k_few takes the place of k_global: as many as are resident at once on the device (0: it

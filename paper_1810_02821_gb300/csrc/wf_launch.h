@@ -34,6 +34,10 @@ constexpr int fields_per_cta() { return N >= 128 ? 1 : 128 / N; }
 template <int N>
 cudaError_t launch_sample(const SampleArgs& a, cudaStream_t st, LaunchTimer* t, int* timeout);
 
+// chains of one wave of the sampler with several threads per row (N in {32, 64, 128}) on the current device
+template <int N>
+cudaError_t sample_wave(int* chains);
+
 template <int N>
 cudaError_t launch_sample_band(const SampleArgs& a, cudaStream_t st, LaunchTimer* t, int* timeout);
 
@@ -170,6 +174,22 @@ cudaError_t launch_chains(Kern whole, Kern balanced, int n_chains, int threads, 
 }
 
 template <int N>
+cudaError_t sample_wave(int* chains) {
+  *chains = 0;
+  if constexpr (core_size(N)) {
+    int dev = 0, sms = 0, per_sm = 0;
+    cudaError_t e = cudaFuncSetAttribute(k_msample<N, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, KGeo<N>::SMEM);
+    if (e != cudaSuccess) return e;
+    if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
+    if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_msample<N, false>, KGeo<N>::T, KGeo<N>::SMEM);
+    *chains = per_sm * sms;
+    return e;
+  }
+  return cudaErrorInvalidValue;
+}
+
+template <int N>
 cudaError_t launch_sample(const SampleArgs& a, cudaStream_t st, LaunchTimer* t, int* timeout) {
   if constexpr (core_size(N)) {
     if (a.cm != 0)
@@ -301,6 +321,7 @@ cudaError_t launch_wpower(const WpowerArgs& p, cudaStream_t st) {
 
 #define WF_INSTANTIATE(N)                                                              \
   template cudaError_t launch_sample<N>(const SampleArgs&, cudaStream_t, LaunchTimer*, int*); \
+  template cudaError_t sample_wave<N>(int*);                                             \
   template cudaError_t launch_sample_band<N>(const SampleArgs&, cudaStream_t, LaunchTimer*, int*); \
   template cudaError_t launch_sample_spin2<N>(const Spin2Args&, cudaStream_t, LaunchTimer*, int*); \
   template cudaError_t launch_solve<N>(const SolveArgs&, const BnormArgs&, cudaStream_t, LaunchTimer*); \
