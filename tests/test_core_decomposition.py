@@ -93,45 +93,6 @@ def test_slot_order_of_the_mode_tables(N):
         assert slot // A + BR * (slot % A) == kx
 
 
-def _parts(i, R, n_chains, S):
-    """Parts (chain, first sweep, end, load, save) of CTA i, in the order it runs them."""
-    W = n_chains * S
-    q, r = divmod(W, R)
-    a, b = q * i + r * i // R, q * (i + 1) + r * (i + 1) // R
-    out = []
-    if b % S:
-        out.append((b // S, 0, b % S, False, True))
-    out += [(c, 0, S, False, False) for c in range((a + S - 1) // S, b // S)]
-    if a % S:
-        out.append((a // S, a % S, S, True, False))
-    return out
-
-
-@pytest.mark.parametrize("R,n_chains,S", [(152, 200, 30), (304, 1000, 7), (304, 305, 1), (5, 6, 100), (7, 13, 3), (3, 3, 4)])
-def test_balanced_shares_cover_every_sweep_once_and_hand_over_in_time(R, n_chains, S):
-    """Equal shares of all chains' sweeps: every sweep once, at most two parts a chain, the first part of a split chain
-    at the start of its CTA and the second at the end of the next one, never before the first has finished."""
-    seen, loads, length = {}, {}, []
-    for i in range(R):
-        t = 0
-        for k, (c, d0, d1, load, save) in enumerate(_parts(i, R, n_chains, S)):
-            assert d0 < d1
-            seen.setdefault(c, []).append((d0, d1))
-            if save:
-                assert k == 0
-                loads.setdefault(c, {})["ready"] = (i, d1)
-            if load:
-                loads.setdefault(c, {})["start"] = (i, t)
-            t += d1 - d0
-        length.append(t)
-    for c in range(n_chains):
-        spans = sorted(seen[c])
-        assert len(spans) <= 2 and spans[0][0] == 0 and spans[-1][1] == S and all(x[1] == y[0] for x, y in zip(spans, spans[1:]))
-    for c, v in loads.items():
-        assert v["start"][0] == v["ready"][0] + 1 and v["start"][1] >= v["ready"][1] - 1   # equal shares to one sweep
-    assert max(length) - min(length) <= 1
-
-
 @pytest.fixture(scope="module")
 def kernel_part():
     """part(R, n_chains, n_sweeps, [(i, s), ...]) -> rows (exists, chain, first, end, load, save, polls) from the kernels'
@@ -150,6 +111,69 @@ def kernel_part():
 
     yield part
     shutil.rmtree(tmp, ignore_errors=True)
+
+
+def _parts(i, R, n_chains, S):
+    """Parts (chain, first sweep, end, load, save) of CTA i, in the order it runs them."""
+    W = n_chains * S
+    q, r = divmod(W, R)
+    a, b = q * i + r * i // R, q * (i + 1) + r * (i + 1) // R
+    out = []
+    if b % S:
+        out.append((b // S, 0, b % S, False, True))
+    out += [(c, 0, S, False, False) for c in range((a + S - 1) // S, b // S)]
+    if a % S:
+        out.append((a // S, a % S, S, True, False))
+    return out
+
+
+@pytest.mark.parametrize("R,n_chains,S", [(152, 200, 30), (304, 1000, 7), (304, 305, 1), (5, 6, 100), (7, 13, 3), (3, 3, 4)])
+def test_balanced_shares_cover_every_sweep_once_and_hand_over_in_time(kernel_part, R, n_chains, S):
+    """Equal shares of all chains' sweeps: every sweep once, at most two parts a chain, the first part of a split chain
+    at the start of its CTA and the second at the end of the next one, one sweep before the first has finished at the
+    earliest. The kernels' own parts (kpart_of, compiled for the host) are the ones checked here."""
+    parts = [_parts(i, R, n_chains, S) for i in range(R)]
+    got = iter(kernel_part(R, n_chains, S, [(i, s) for i in range(R) for s in range(len(parts[i]) + 1)]))
+    for own in parts:
+        assert [row[:6] for row in (next(got) for _ in own)] == [(1, c, d0, d1, int(load), int(save)) for c, d0, d1, load, save in own]
+        assert next(got)[0] == 0   # and no further part
+    seen, loads, length = {}, {}, []
+    for i in range(R):
+        t = 0
+        for k, (c, d0, d1, load, save) in enumerate(parts[i]):
+            assert d0 < d1
+            seen.setdefault(c, []).append((d0, d1))
+            if save:
+                assert k == 0
+                loads.setdefault(c, {})["ready"] = (i, d1)
+            if load:
+                loads.setdefault(c, {})["start"] = (i, t)
+            t += d1 - d0
+        length.append(t)
+    for c in range(n_chains):
+        spans = sorted(seen[c])
+        assert len(spans) <= 2 and spans[0][0] == 0 and spans[-1][1] == S and all(x[1] == y[0] for x, y in zip(spans, spans[1:]))
+    for c, v in loads.items():
+        assert v["start"][0] == v["ready"][0] + 1 and v["start"][1] >= v["ready"][1] - 1   # equal shares to one sweep
+    assert max(length) - min(length) <= 1
+
+
+@pytest.mark.parametrize("R,n_chains,S", [(304, 2 ** 31 - 1, 2 ** 31 - 1), (760, 2 ** 31 - 5, 2 ** 31 - 1), (152, 2 ** 31 - 1, 2 ** 30)])
+def test_share_arithmetic_near_the_largest_sweep_count(kernel_part, R, n_chains, S):
+    """n_chains n_sweeps close to 2^62: the first and last parts of each share, in exact integers."""
+    W = n_chains * S
+    q, r = divmod(W, R)
+    for i in (0, 1, 2, R // 2, R - 2, R - 1):
+        a, b = q * i + r * i // R, q * (i + 1) + r * (i + 1) // R
+        head = int(b % S > 0)
+        whole = b // S - (a + S - 1) // S
+        rows = kernel_part(R, n_chains, S, [(i, s) for s in (0, head, head + whole - 1, head + whole, head + whole + 1)])
+        if head:
+            assert rows[0][:6] == (1, b // S, 0, b % S, 0, 1)
+        assert rows[1][:6] == (1, (a + S - 1) // S, 0, S, 0, 0) and rows[2][:6] == (1, b // S - 1, 0, S, 0, 0)
+        if a % S:
+            assert rows[3][:6] == (1, a // S, a % S, S, 1, 0)
+        assert rows[3][0] == int(a % S > 0) and rows[4][0] == 0
 
 
 @pytest.mark.parametrize("R,n_chains,S", [(304, 305, 7), (304, 305, 10 ** 7), (152, 200, 2 ** 31 - 1)])
