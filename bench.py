@@ -57,7 +57,7 @@ FP32_LANES = 128   # FP32 FMA lanes per SM (for the derived figure shown beside 
 # (set in main); the derived SMs x lanes x 2 x max clock figure is reported only as a note
 FP32_PEAK_TFLOPS = None
 WORKLOAD = "paper-shaped 128x128 image, 1024 independent chains x 100 posterior samples per step"
-PROFILE = os.path.join(ROOT, "profiles", "k_sample_128_paper128.txt")
+PROFILE = os.path.join(ROOT, "profiles", "k_msample_128.txt")
 
 
 def parse():
@@ -552,7 +552,7 @@ def spin2_sampler(dev, n_chains: int = 512):
            "roofline": {"bound": "alu", "achieved": 2 * FLOPS_PER_SWEEP * n_chains * N_SAMPLES / (kms / 1e3) / 1e12,
                         "peak": FP32_PEAK_TFLOPS, "unit": "TFLOP/s",
                         "frac": 2 * FLOPS_PER_SWEEP * n_chains * N_SAMPLES / (kms / 1e3) / 1e12 / FP32_PEAK_TFLOPS}}
-    # 256^2 and 512^2: both components of a chain in one thread-block cluster
+    # 256^2: both components of a chain in one thread-block cluster; 512^2: both in global memory
     for Hl, chains, ns in ((256, 228, 20), (512, 36, 10)):
         q = synth.make_problem(Hl, seed=Hl, mask_frac=0.1, slope=-2.0, k0=1.0 / 32, sigma2=(0.05, 0.5))
         d2l = np.where(q.mask == 1, 0.0, rng.standard_normal(q.d.shape)).astype(np.float32)
@@ -565,8 +565,9 @@ def spin2_sampler(dev, n_chains: int = 512):
             wf.wf_sample_spin2(*argl, seed=2 + i, n_samples=ns, n_chains=chains)
             ks.append(wf.wf_last_kernel_ms())
         kl = statistics.mean(ks)
+        where = "one thread-block cluster" if Hl == 256 else "global memory"
         res[f"{Hl}x{Hl}"] = {"workload": f"{Hl}x{Hl} shear pair, {chains} chains x {ns} sweeps (all kept), "
-                                         "both components of a chain in one thread-block cluster",
+                                         f"both components of a chain in {where}",
                              "samples_per_s": chains * ns / (kl / 1e3), "kernel_ms": kl,
                              "roofline": _fft_roofline(Hl, chains * ns, kl, fields=2)}
     return res
