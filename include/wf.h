@@ -452,9 +452,10 @@ double wf_last_kernel_ms(void);
  * rounding): thread-block clusters, each holding one chain's or image's field in distributed shared memory
  * (N / 64 or N / 32 CTAs; a batch image runs its level norms, cooled solve and samples in one cluster),
  * and the global-memory kernels (fields in global memory, cooperative launches with many CTAs per field).
- * mode 0 (default, automatic): clusters when a call holds at least 400 chains at 256 x 256 (a batch as many
- * images) and the device can host the cluster, otherwise the global-memory kernels, which are faster for
- * fewer fields and at 512 x 512 (spin-2: clusters from 24 chains at 256 x 256), and in their place, for as
+ * mode 0 (default, automatic): clusters for the chains of a 256 x 256 call that fill the clusters' last round
+ * well (about 86 to 110 chains, 180 to 220, 290 to 330 and nearly all counts above) and for batches of 400 images of
+ * that size or more, where the device can host the cluster, otherwise the global-memory kernels, which are faster for
+ * few fields and at 512 x 512 (spin-2: clusters from 24 chains at 256 x 256), and in their place, for as
  * many fields as are resident at once (also at 64 x 64, 128 x 128 and 1024 x 1024), kernels of the same
  * arithmetic that keep the tables, and up to 256 x 256 the field, in shared memory (equal bit for bit);
  * mode 1: always the global-memory kernels; mode 2: clusters wherever the device can host them. Up to

@@ -258,14 +258,30 @@ bool size_ok(int H, int W) {
 
 bool cluster_fits(int H, int rows = 0);
 
-// Path for `units` independent fields (chains or images) of H x H, H in {256, 512}: one thread-block cluster per
-// field, or the global-memory kernels. Automatic choice, measured on GB300 (us per sampler sweep of all chains,
-// global-memory / cluster): 256^2: 16 chains 11.9 / 29.4, 64 chains 34.4 / 33.3, 228 chains 88 / 100, 342 chains
-// 131 / 136, 400 chains 161 / 147, 1000 chains 380 / 354; 512^2: 4 chains 12.5 / 25.2, 50 chains 90 / 134, 152 chains
-// 265 / 370, 600 chains 1005 / 1443. So clusters from 400 fields at 256^2 (every SM full of clusters either way, and
-// the fields no longer fit L2 with their tables) and the global-memory kernels at every count at 512^2. A batch's
-// classes cross over at the same counts (Wiener solve and 16 samples, ms: 77 images of 256^2 5.5 / 7.3, 307 images
-// 17.5 / 17.6; 102 images of 512^2 21.9 / 26.4).
+// fields resident at once on the current device, queried once per device (known: fields + 1)
+template <class F>
+int resident_fields(std::mutex& mu, int (&known)[64], F&& query) {
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) {
+    cudaGetLastError();
+    return 0;
+  }
+  std::lock_guard<std::mutex> lock(mu);
+  if (known[dev] == 0) {
+    int n = 0;
+    if (query(&n) != cudaSuccess) {
+      cudaGetLastError();
+      n = 0;
+    }
+    known[dev] = n + 1;
+  }
+  return known[dev] - 1;
+}
+
+// Path for a batch class of `units` images of H x H, H in {256, 512}: one thread-block cluster per image, or the
+// global-memory kernels. Wiener solve and 16 samples, ms, global-memory / clusters: 77 images of 256^2 5.5 / 7.3, 307 images
+// 17.5 / 17.6; 102 images of 512^2 21.9 / 26.4. So clusters from 400 images of 256^2 (every SM full of clusters either way, and
+// the fields no longer fit L2 with their tables) and the global-memory kernels at every count at 512^2.
 int cluster_min_units(int H) { return H == 256 ? 400 : 1 << 30; }
 
 // Path of the spin-2 sampler and filter at 256 and 512: the global-memory kernels, or clusters from 24 chains at 256^2
@@ -293,29 +309,34 @@ cudaError_t launch_cpipe_any(int H, int rows, const wf::CBArgs& a, cudaStream_t 
   return rows == 64 ? wf::launch_cpipe<512, 64>(a, st, t) : wf::launch_cpipe<512, 32>(a, st, t);
 }
 
+// sampler clusters of that geometry resident at once on the current device, and whether there is one
+int cluster_resident(int H, int rows = 0) {
+  static std::mutex mu;
+  static int known[3][64] = {};
+  const int r = cluster_rows_of(H, rows);
+  return resident_fields(mu, known[H == 256 ? 0 : (r == 64 ? 2 : 1)], [=](int* n) { return csample_clusters_any(H, r, n); });
+}
+bool cluster_fits(int H, int rows) { return cluster_resident(H, rows) > 0; }
+
 bool use_cluster(int H, int units, int rows = 0) {
   if ((H != 256 && H != 512) || g_large_sampler == 1 || !cluster_fits(H, rows)) return false;
   return g_large_sampler == 2 || units >= cluster_min_units(H);
 }
 
-// whether at least one sampler cluster of that geometry fits on the current device (queried once per device)
-bool cluster_fits(int H, int rows) {
-  static std::mutex mu;
-  static int known[3][64] = {};  // 0 unknown, 1 fits, 2 does not
-  int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) {
-    cudaGetLastError();
-    return false;
-  }
-  const int k = H == 256 ? 0 : (cluster_rows_of(H, rows) == 64 ? 2 : 1);
-  std::lock_guard<std::mutex> lock(mu);
-  if (known[k][dev] == 0) {
-    int clusters = 0;
-    const cudaError_t e = csample_clusters_any(H, cluster_rows_of(H, rows), &clusters);
-    if (e != cudaSuccess) cudaGetLastError();
-    known[k][dev] = (e == cudaSuccess && clusters > 0) ? 1 : 2;
-  }
-  return known[k][dev] == 1;
+// The same for a sampler call of `chains` chains. Clusters run in rounds of the R resident ones (110 here), and a round takes
+// almost as long when it is half empty; the global-memory kernel's sweep grows in small steps. So at 256^2 clusters where
+// their last round is well filled, the more rounds the less so. us per sweep of all chains, global-memory / clusters:
+// 34 chains 24.4 / 29.4, 52 26.2 / 32.7, 64 34.4 / 33.0, 84 36.4 / 39.0, 88 45.0 / 39.1, 110 46.6 / 39.4, 112 46.8 / 62.5, 170 67.6 /
+// 69.3, 200 80.8 / 77.2, 220 86.5 / 78.3, 228 88.6 / 99.1, 270 107 / 111, 300 118 / 115, 330 129 / 117, 340 131 / 136, 350 140 / 137,
+// 450 172 / 171, 1000 379 / 353. 512^2: the global-memory kernels at every count (4 chains 12.5 / 25.2, 50 chains 90 / 134, 152
+// chains 265 / 370, 600 chains 1005 / 1443).
+bool sample_on_clusters(int H, int chains) {
+  if (H != 256 || g_large_sampler != 0) return use_cluster(H, chains);
+  const int R = cluster_resident(H);
+  if (R == 0) return false;
+  const int rounds = chains / R, fill = int(32LL * (chains % R) / R);  // of the last round, in 32nds
+  if (rounds == 0) return fill >= 25 || (fill >= 17 && fill < 21);
+  return chains % R == 0 || rounds >= 4 || fill >= (rounds < 3 ? 20 : 4);
 }
 
 // An output the kernels may store to: device or managed memory, or page-locked host memory that is
@@ -339,26 +360,6 @@ bool out_ptr_ok(const void* p) {
     return pageable != 0;
   }
   return true;
-}
-
-// fields resident at once on the current device, queried once per device (known: fields + 1)
-template <class F>
-int resident_fields(std::mutex& mu, int (&known)[64], F&& query) {
-  int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) {
-    cudaGetLastError();
-    return 0;
-  }
-  std::lock_guard<std::mutex> lock(mu);
-  if (known[dev] == 0) {
-    int n = 0;
-    if (query(&n) != cudaSuccess) {
-      cudaGetLastError();
-      n = 0;
-    }
-    known[dev] = n + 1;
-  }
-  return known[dev] - 1;
 }
 
 // Order of the sampler's mode table at an on-chip size (mode_pos), which selects its kernel: several threads per
@@ -1091,8 +1092,8 @@ wf_status wf_sample_ex(const float* d, const float* Ndiag, const uint8_t* mask, 
     Ndiag = resp.Nd;
     mask = resp.mask;
   }
-  // 256 and 512: one cluster per chain when the device can host the cluster, else the field in global memory
-  const bool cluster = use_cluster(H, o.n_chains);
+  // 256 and 512: one cluster per chain, or the field in global memory
+  const bool cluster = sample_on_clusters(H, o.n_chains);
   if (!sample_on_chip(H, o.n_chains) && !cluster) {
     KernelTimer gt(st);
     const wf_status r = sample_global(d, Ndiag, mask, Pk, H, W, seed, o, sweeps, out, st, &gt);
