@@ -123,11 +123,33 @@ cudaError_t launch_smem(Kern kern, dim3 grid, int threads, int smem, const Args&
   if (t) t->stop();
   return cudaGetLastError();
 }
-// One CTA per chain, or, with more chains than are resident at once, a cooperative launch of equal shares (KBalance)
-// whose scratch (slots, flags) comes from st's memory pool. A last round of 0.92 to 1 CTA per SM at two CTAs per SM
-// keeps one CTA per chain: alone on their SMs those run at twice the pace, and shares would not be faster.
-template <class Kern, class Args>
-cudaError_t launch_chains(Kern whole, Kern balanced, int n_chains, int threads, int smem, int slot_floats,
+// Whether equal shares (KBalance) are faster than one CTA per chain for n chains of N x N fields, `sweeps` sweeps each, on
+// `sms` SMs with per_sm resident CTAs. In units of a full round's sweep: one CTA per chain takes its full rounds and, for
+// the last one, the share of an SM's places that its fullest SM has taken, but not less than `lat` (a CTA alone on its SM: 0.27
+// of a round at 32^2, 0.24 to 0.37 for shear pairs; 0.33 to 0.6 with the band statistics). Shares take n / R rounds, a few
+// percent slower per sweep, and `fixed` sweeps a call more (allocation, flags, cooperative launch: 10 to 40 us, 50 to 120 with
+// the band statistics). Measured, ms a call, one CTA per chain / shares: 128^2 100 sweeps 350 chains 2.94 / 2.36, 440 2.93 / 2.89,
+// 607 3.79 / 3.87, 1000 6.34 / 6.17, 1500 8.93 / 9.11; 300 shear pairs 4.93 / 5.01; 32^2 1521 chains 0.95 / 0.87, 3000 1.35 / 1.44,
+// 5000 2.07 / 2.20; 64^2 bands 20 sweeps 761 chains 0.91 / 0.83, 1500 1.20 / 1.39; 4 sweeps of 600 128^2 chains 0.42 / 0.45.
+struct BalanceCost {
+  double lat, fixed;
+};
+template <int N>
+constexpr BalanceCost balance_cost(bool band) {
+  return band ? BalanceCost{0.6, N == 32 ? 3.0 : 8.0} : BalanceCost{0.3, N == 32 ? 6.0 : 2.0};
+}
+WF_HD bool balance_pays(int N, const BalanceCost& c, long long n, int per_sm, int sms, long long sweeps) {
+  const long long R = (long long)per_sm * sms;
+  if (R <= 0 || n <= R || n % R == 0) return false;
+  const double layers = double((n % R + sms - 1) / sms) / per_sm;
+  const double whole = double(n / R) + (layers > c.lat ? layers : c.lat);
+  const double shares = double(n) / double(R) * (N == 32 ? 1.08 : (N == 64 ? 1.06 : 1.03));
+  return (whole - shares) * double(sweeps) > c.fixed;
+}
+// One CTA per chain, or a cooperative launch of equal shares where these are faster, whose scratch (slots, flags) comes
+// from st's memory pool
+template <int N, class Kern, class Args>
+cudaError_t launch_chains(Kern whole, Kern balanced, const BalanceCost& cost, int n_chains, int threads, int smem, int slot_floats,
                           const Args& a, cudaStream_t st, LaunchTimer* t, int* timeout) {
   cudaError_t e = cudaFuncSetAttribute(balanced, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (e != cudaSuccess) return e;
@@ -135,11 +157,11 @@ cudaError_t launch_chains(Kern whole, Kern balanced, int n_chains, int threads, 
   if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
   if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
   if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, balanced, threads, smem)) != cudaSuccess) return e;
-  const int R = per_sm * sms, over = R > 0 ? n_chains % R : 0;
+  const int R = per_sm * sms;
   KBalance b{};
   void* base = nullptr;
   const size_t flags = (size_t(R) + 1) * sizeof(unsigned int), off = (flags + 255) / 256 * 256;
-  bool bal = timeout && R > 0 && n_chains > R && over != 0 && !(per_sm == 2 && over <= sms && over > sms - sms / 12);
+  bool bal = timeout && balance_pays(N, cost, n_chains, per_sm, sms, a.n_sweeps);
   if (bal) {
     e = cudaMallocAsync(&base, off + size_t(R) * size_t(slot_floats) * sizeof(float), st);
     if (e == cudaErrorMemoryAllocation) {  // no room for the states handed over: one CTA per chain needs none
@@ -193,8 +215,8 @@ template <int N>
 cudaError_t launch_sample(const SampleArgs& a, cudaStream_t st, LaunchTimer* t, int* timeout) {
   if constexpr (core_size(N)) {
     if (a.cm != 0)
-      return launch_chains(k_msample<N, false>, k_msample<N, true>, a.n_chains, KGeo<N>::T, KGeo<N>::SMEM, N * N, a, st,
-                           t, timeout);
+      return launch_chains<N>(k_msample<N, false>, k_msample<N, true>, balance_cost<N>(false), a.n_chains, KGeo<N>::T,
+                              KGeo<N>::SMEM, N * N, a, st, t, timeout);
   }
   if constexpr (N == 16 || N == 64) {
     constexpr int FPC = fields_per_cta<N>();
@@ -206,8 +228,8 @@ cudaError_t launch_sample(const SampleArgs& a, cudaStream_t st, LaunchTimer* t, 
 template <int N>
 cudaError_t launch_sample_band(const SampleArgs& a, cudaStream_t st, LaunchTimer* t, int* timeout) {
   if constexpr (core_size(N)) {
-    return launch_chains(k_mband<N, false>, k_mband<N, true>, a.n_chains, KGeo<N>::T,
-                         KGeo<N>::SMEM + band_bytes(a.n_bins), N * N + (a.n_bins + 3) / 4 * 4, a, st, t, timeout);
+    return launch_chains<N>(k_mband<N, false>, k_mband<N, true>, balance_cost<N>(true), a.n_chains, KGeo<N>::T,
+                            KGeo<N>::SMEM + band_bytes(a.n_bins), N * N + (a.n_bins + 3) / 4 * 4, a, st, t, timeout);
   } else {
     constexpr int FPC = fields_per_cta<N>();
     return launch_smem(k_sample_band<N, FPC>, (a.n_chains + FPC - 1) / FPC, N * FPC,
@@ -219,8 +241,8 @@ template <int N>
 cudaError_t launch_sample_spin2(const Spin2Args& a, cudaStream_t st, LaunchTimer* t, int* timeout) {
   if constexpr (core_size(N)) {
     // the filter (quiet) is one chain
-    return launch_chains(a.quiet ? k_mspin2<N, false, false> : k_mspin2<N, true, false>, k_mspin2<N, true, true>,
-                         a.n_chains, 2 * KGeo<N>::T, kspin2_smem<N>(), 2 * N * N, a, st, t, a.quiet ? nullptr : timeout);
+    return launch_chains<N>(a.quiet ? k_mspin2<N, false, false> : k_mspin2<N, true, false>, k_mspin2<N, true, true>,
+                            balance_cost<N>(false), a.n_chains, 2 * KGeo<N>::T, kspin2_smem<N>(), 2 * N * N, a, st, t, a.quiet ? nullptr : timeout);
   } else {
     constexpr int FPC = fields_per_cta<N>();  // images per CTA; two component fields each
     return launch_smem(k_sample_spin2<N, FPC>, (a.n_chains + FPC - 1) / FPC, 2 * N * FPC,
