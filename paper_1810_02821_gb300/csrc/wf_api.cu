@@ -1455,7 +1455,7 @@ wf_status wf_sample_spin2(const float* d1, const float* d2, const float* N1, con
   a.out_dtype = o.out_dtype;
   KernelTimer timer(st);
   auto* bar = reinterpret_cast<wf::GridBar*>(b + o_bar);
-  WF_CUDA(cudaMemsetAsync(bar, 0, sizeof(wf::GridBar), st));
+  if (path.global) WF_CUDA(cudaMemsetAsync(bar, 0, sizeof(wf::GridBar), st));
   int timeout = 0;
   const cudaError_t e = launch_spin2_any(H, path, a, reinterpret_cast<float2*>(b + o_z), bar, st, &timer, &timeout);
   if (e != cudaSuccess) return cuda_fail(e);
@@ -1571,7 +1571,7 @@ wf_status wf_solve_spin2(const float* d1, const float* d2, const float* N1, cons
   a.out = out; a.n_samples = 1; a.n_chains = 1; a.burn_in = 0; a.thin = 1; a.out_dtype = 0;
   a.quiet = 1;
   auto* bar = reinterpret_cast<wf::GridBar*>(b + o_bar);
-  WF_CUDA(cudaMemsetAsync(bar, 0, sizeof(wf::GridBar), st));
+  if (path.global) WF_CUDA(cudaMemsetAsync(bar, 0, sizeof(wf::GridBar), st));
   const int cm = path.cm, perm = path.perm;
   int timeout = 0;  // one chain: never a balanced launch
   auto run = [&](double lam, int sweeps) -> wf_status {
