@@ -554,7 +554,7 @@ __device__ __forceinline__ double ccol_p2(cooperative_groups::cluster_group& cl,
                                           const float* __restrict__ Pk) {
   using G = CGeo<N, MR>;
   constexpr int WH = G::WH;
-  auto p2 = [](float P, float re, float im) -> float { return P * P * fmaf(re, re, im * im); };
+  auto p2 = [](float P, float re, float im) -> float { return fmaf(P * re, P * re, (P * im) * (P * im)); };
   float acc = 0.0f;
   ccol_units<N, MR, false>(cl, rows, g, [&](int K, int t, float2& y1, float2& y2, int ky1, int ky2) {
     if (K != 0) {

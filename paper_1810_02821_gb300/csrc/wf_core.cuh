@@ -621,7 +621,7 @@ __device__ __forceinline__ float ks_p2(const KCol<N>& t, float2 (&p)[KGeo<N>::A]
   using G = KGeo<N>;
   constexpr int L = G::L, HL = G::H * G::L;
   float acc = 0.0f;
-  auto p2 = [](float P, float re, float im) -> float { return P * P * fmaf(re, re, im * im); };
+  auto p2 = [](float P, float re, float im) -> float { return fmaf(P * re, P * re, (P * im) * (P * im)); };
   kpairs<N>(
       t, p, q,
       [&](float2& y1, float2& y2, int ky1, int ky2) {

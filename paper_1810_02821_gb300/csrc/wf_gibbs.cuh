@@ -385,7 +385,8 @@ WF_HD void rhs_row(float2 (&c)[N / 2], int y, const float2* __restrict__ dn, flo
 // ---------------------------------------------------------------------------------------------
 // Fourier-space updates (Alg. 1 s-update) on the modes held by a column thread
 // ---------------------------------------------------------------------------------------------
-// sum over the full spectrum of P^2 |V|^2 for the forward transform V held by this thread
+// sum over the full spectrum of |P V|^2 (P V squared, not P: P^2 leaves the range of FP32 for maps in units of 1e-10 or 1e9) for
+// the forward transform V held by this thread
 // (edge columns separated into kx = 0 and kx = W/2)
 template <int N>
 WF_HD double p2_power(const float2 (&x)[N / 2], int lt, const float* __restrict__ Pk) {
@@ -393,7 +394,7 @@ WF_HD double p2_power(const float2 (&x)[N / 2], int lt, const float* __restrict_
   constexpr int WH = G::WH;
   const int col = lt % G::LC, r = lt / G::LC;
   float acc = 0.0f;  // the thread's LC modes in FP32; the caller sums the threads in FP64
-  auto p2 = [](float P, float re, float im) -> float { return P * P * fmaf(re, re, im * im); };
+  auto p2 = [](float P, float re, float im) -> float { return fmaf(P * re, P * re, (P * im) * (P * im)); };
   for_mode_pairs<N>(r, [&](auto KP, auto KQ, int ky1, int ky2, auto ZG) {
     constexpr int kp = decltype(KP)::value, kq = decltype(KQ)::value;
     constexpr bool zero_group = decltype(ZG)::value != 0;

@@ -796,7 +796,7 @@ __device__ __forceinline__ float gcol_update(int mode, const Z& z, int c0, FG&& 
           });
     });
   } else {
-    auto p2 = [](float P, float re, float im) -> float { return P * P * fmaf(re, re, im * im); };
+    auto p2 = [](float P, float re, float im) -> float { return fmaf(P * re, P * re, (P * im) * (P * im)); };
     gcol<N, false, RB>(z, c0, [&](float2 (&p)[G::A], float2 (&q)[G::A], int col, int h, int hb) {
       gpairs<N, RB>(
           p, q, col, h, hb, c0,

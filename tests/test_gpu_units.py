@@ -97,3 +97,34 @@ def test_likelihood_gradient_in_any_unit(H, c):
     one, got, batch = call(1.0), call(c), call(c, batch=True)
     np.testing.assert_allclose(got, one, rtol=1e-4, atol=1e-4 * np.abs(one).max())
     np.testing.assert_allclose(batch, one, rtol=1e-3, atol=1e-3 * np.abs(one).max())
+
+
+@pytest.mark.parametrize("H,mode", [(16, "auto"), (64, "auto"), (128, "auto"), (128, "global"), (256, "auto"), (256, "global"),
+                                    (256, "cluster"), (512, "auto"), (512, "cluster"), (1024, "auto")])
+@pytest.mark.parametrize("c", [1e-12, 1e10])
+def test_unrefined_filter_in_any_unit(H, mode, c):
+    """The FP32 iteration stops by the level norms ||S N^-1 d||^2, which have the unit of the map squared. Two maps that stop
+    at a residual of 1e-5 differ by a few times that."""
+    wf.wf_set_large_image_sampler(mode)
+    try:
+        one = wf.wf_solve_ex(*to_dev(_problem(H, 1.0)), tol=1e-5, refine=0)
+        r = wf.wf_solve_ex(*to_dev(_problem(H, c)), tol=1e-5, refine=0)
+    finally:
+        wf.wf_set_large_image_sampler("auto")
+    assert abs(r.iters - one.iters) <= 4, (r.iters, one.iters)
+    assert rel(r.s.double().cpu().numpy() / c, one.s.double().cpu().numpy()) < 1e-4
+
+
+@pytest.mark.parametrize("small_path", [0, 1])
+@pytest.mark.parametrize("c", [1e-12, 1e10])
+def test_batch_in_any_unit(small_path, c):
+    sizes = [16, 32, 64, 128, 256, 512]
+
+    def call(u):
+        images = [wf.BatchImage(*to_dev(_problem(H, u))) for H in sizes]
+        wf.wf_batch_run(images, small_path=small_path)
+        return images
+
+    for a, b in zip(call(c), call(1.0)):
+        assert abs(a.iters - b.iters) <= 4, (a.iters, b.iters)
+        assert rel(a.out_wf.double().cpu().numpy() / c, b.out_wf.double().cpu().numpy()) < 1e-4
