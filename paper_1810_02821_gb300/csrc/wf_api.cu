@@ -1612,6 +1612,12 @@ wf_status wf_solve_spin2(const float* d1, const float* d2, const float* N1, cons
     if (!(rho == rho)) { status = WF_ERR_NONFINITE; break; }
     if (rho < o.tol) { status = WF_OK; break; }
   }
+  if (path.global && rho < 0.0) {  // max_iter ended within the cooling levels: no check has looked at their barriers yet
+    wf::GridBar hb{};
+    WF_CUDA(cudaMemcpyAsync(&hb, bar, sizeof(hb), cudaMemcpyDeviceToHost, st));
+    WF_CUDA(cudaStreamSynchronize(st));
+    if (hb.err) return wf_status(hb.err);
+  }
   if (iters_out) *iters_out = iters;
   if (resid_out) *resid_out = rho;
   return status;
